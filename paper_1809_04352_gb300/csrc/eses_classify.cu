@@ -11,12 +11,19 @@
 //      with an empty set labels its 32 points outside at once; otherwise every
 //      lane tests its point against the set: inside a van der Waals ball -> 1,
 //      in no expanded ball -> 0, else a shell point;
-//   3. shell points go to a per-tile queue; when there are any, the block
-//      builds the staged atoms' neighbour sets (expanded spheres that meet)
-//      and works through the queue: free triple points within r_p, convex
-//      witnesses of the containing balls, saddle witnesses of the pairs of
-//      the containing balls, each witness tested for freeness against the
-//      neighbours of its atoms only.
+//   3. shell points go to a per-tile queue, brick by brick; when there are
+//      any, the block builds the staged atoms' neighbour sets (expanded spheres
+//      that meet) and works through the queue, a warp at a time on neighbouring
+//      points (shell_points): free triple points within r_p, convex witnesses
+//      of the containing balls, saddle witnesses of the circles near the warp's
+//      points, each witness tested for freeness against the neighbours of its
+//      atoms only.
+//   Bound by instruction issue and the latency of a tile's slowest points.  One
+//   thread per point walking its own balls' circles (12.9 active lanes, 65 % of
+//   the kernel in this phase, 59,000 cycles a tile on the 5,000-atom globule at
+//   h 0.25) became all lanes on one patch at a time: 2.19 -> 1.30 ms there,
+//   8.2 -> 5.0 ms at 20,000 atoms, 3.6 -> 2.2 ms on 32 molecules at h 0.5,
+//   1.30 -> 0.64 ms in FP64 on 200 atoms (single-tile queue pops included).
 //   T = double, FILT = false is the plain FP64 form; T = float, FILT = true
 //   is the filtered form, whose undecided points get LABEL_BAND and are
 //   counted per tile.
@@ -29,6 +36,11 @@ namespace eses {
 
 constexpr int CLS_THREADS = 256;
 constexpr int NBRICK = 16;     // 2x4x4-point bricks per tile
+// lanes per shell point: doubled while points x lanes stays within this (one
+// lane per point above it), so a tile of few points still uses its warps.
+// Measured at 256 / 512 / 1,024: 1.61 / 1.39 / 1.54 ms on the 5,000-atom globule
+// (216 points a tile), 2.74 / 2.30 / 2.36 ms at h 0.5
+constexpr int CLS_SPLIT = 2 * CLS_THREADS;
 
 template <class CP>
 struct ClsSmem {
@@ -36,13 +48,9 @@ struct ClsSmem {
     int hkey[HS];                  // staged-atom lookup (pair_slots)
     short hval[HS];
     short2 pslot[CP::P];           // staged slots of each pair's atoms (-1: not staged)
-    int inc_start[CP::A + 1];      // incident pairs per staged atom (CSR)
-    int inc_fill[CP::A];
-    short inc[2 * CP::P];
     unsigned bmask[NBRICK][AWC];   // per-brick sets of the atoms whose expanded ball reaches the brick
     unsigned nbm[CP::A * AWC];     // neighbour set of every staged atom (build_neighbour_sets)
-    int bcount[NBRICK];
-    short queue[TILE_PTS];         // shell points
+    short queue[TILE_PTS];         // shell points, brick by brick
     int nq, band, next;            // queue length, band points, next queue position to take
 };
 
@@ -72,115 +80,140 @@ __device__ __forceinline__ T pt_coord(const Grid &G, int k)
     else return (double)k * G.h;
 }
 
-// per-atom incident pair lists (whole block)
-template <class T, class CP>
-__device__ void build_incidence(const TileS<T, CP> &S, ClsSmem<CP> &C)
+// Freeness of a witness against the staged atoms in m0 & m1 (m1 may be null),
+// as free_set, inlined: the lanes of a warp test witnesses of one patch, so
+// they walk the same atoms.
+template <bool FILT, class T, class CP>
+__device__ __forceinline__ int witness_free(const TileS<T, CP> &S, T qx, T qy, T qz, const unsigned *m0,
+                                            const unsigned *m1, int nw, T rp, T delta, int &nt)
 {
-    constexpr int A_CAP = CP::A;
-    for (int a = threadIdx.x; a < A_CAP + 1; a += blockDim.x) C.inc_start[a] = 0;
-    pair_slots<T>(S, C.hkey, C.hval, C.pslot);
-    for (int p = threadIdx.x; p < S.np; p += blockDim.x) {
-        const short2 sl = C.pslot[p];
-        if (sl.x >= 0 && sl.y >= 0) {
-            atomicAdd(&C.inc_start[sl.x + 1], 1);
-            atomicAdd(&C.inc_start[sl.y + 1], 1);
+    int res = 1;
+    for (int w = 0; w < nw; ++w) {
+        unsigned bits = m1 ? (m0[w] & m1[w]) : m0[w];
+        while (bits) {
+            const int k = (w << 5) + __ffs(bits) - 1;
+            bits &= bits - 1;
+            ++nt;
+            const P4<T> c = S.atom[k];
+            const T dx = qx - c.x, dy = qy - c.y, dz = qz - c.z;
+            const T R = c.w + rp;
+            const int t = lt_sq<FILT>(dx * dx + dy * dy + dz * dz, R * R, R, delta);
+            if (t == 1) return 0;
+            if (t < 0) res = -1;
         }
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {  // inclusive scan of inc_start[1..A_CAP] by one warp
-        const int lane = threadIdx.x;
-        const int per = (A_CAP + 31) / 32;
-        const int base = 1 + lane * per;
-        int s = 0;
-        for (int k = 0; k < per; ++k)
-            if (base + k <= A_CAP) s += C.inc_start[base + k];
-        int inc = s;
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += t;
-        }
-        int run = inc - s;
-        for (int k = 0; k < per; ++k)
-            if (base + k <= A_CAP) {
-                run += C.inc_start[base + k];
-                C.inc_start[base + k] = run;
-            }
-    }
-    __syncthreads();
-    for (int a = threadIdx.x; a < A_CAP; a += blockDim.x) C.inc_fill[a] = C.inc_start[a];
-    __syncthreads();
-    for (int p = threadIdx.x; p < S.np; p += blockDim.x) {
-        short2 sl = C.pslot[p];
-        if (sl.x >= 0 && sl.y >= 0) {
-            C.inc[atomicAdd(&C.inc_fill[sl.x], 1)] = (short)p;
-            C.inc[atomicAdd(&C.inc_fill[sl.y], 1)] = (short)p;
-        }
-    }
-    __syncthreads();
+    return res;
 }
 
-// Shell point: witnesses among free triple points, the containing balls and
-// their pairs.  A group of G lanes (G a power of two) shares one point: the
-// candidates (triple points; per containing ball its face, then its incident
-// pairs) are numbered and lane r of the group tests those numbered r mod G.
-// Returns this lane's part: 0 a free witness within r_p (certain), 2 one is
-// undecided, 1 none; the group's label is 0 if any part is 0, else 2 if any
-// part is 2, else 1 -- the label of one lane testing every candidate.  nt
-// counts the atom tests of the witnesses' freeness.
+// Shell points of one warp: 32 / G points, G lanes (a power of two) each;
+// `code` is the lane's queue entry (-1: none), (x, y, z) its point, r its rank
+// among the point's lanes.  Every patch that could hold a witness of some
+// point of the warp is taken in turn, triple points, then convex, then
+// saddle patches: lanes test their own point against the same patch, so its
+// data and the atoms that could cover its witness are broadcast reads and the
+// lanes stay together (rank r of G takes every G-th patch).  Circles are
+// first culled against the box of the points still undecided, lanes over
+// circles; a circle that meets no containing ball of a point is no nearer
+// than r_p with a free witness unless the point is outside, so testing it
+// changes no decision.  Returns the point's label on each of its lanes:
+// 0 a free witness within r_p (certain), 2 undecided, 1 none.
 template <bool FILT, class T, class CP>
-__device__ int shell_part(const TileS<T, CP> &S, const ClsSmem<CP> &C, int brick, T x, T y, T z, T rp, T d0, int r,
-                          int G, int &nt)
+__device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem<CP> &C, int code, T x, T y, T z, T rp,
+                                            T d0, float hf, int r, int G, int &nt)
 {
-    SmemAcc<T, CP> A(S);
+    constexpr unsigned full = 0xffffffffu;
     constexpr int aw = ClsSmem<CP>::AWC;
-    bool unsure = false;
-    const T thr = rp, thr2 = rp * rp;
-    for (int v = r; v < S.nv; v += G) {
-        P4<T> q = S.vq[v];
-        T dx = x - q.x, dy = y - q.y, dz = z - q.z;
-        int t = lt_sq<FILT>(dx * dx + dy * dy + dz * dz, thr2, thr, d0);
-        if (t == 1) return 0;
-        if (t < 0) unsure = true;
+    const int lane = threadIdx.x & 31;
+    const SmemAcc<T, CP> A(S);
+    // every G-th bit from r: this lane's share of a 32-patch word
+    const unsigned share = (G == 32 ? 1u : full / ((1u << G) - 1u)) << r;
+    const unsigned gmask = (G == 32 ? full : ((1u << G) - 1u)) << (lane & ~(G - 1));
+    bool done = code < 0, hit = false, unsure = false;
+    // a point is settled once any of its lanes has a witness
+    auto settle = [&]() {
+        const unsigned h = __ballot_sync(full, hit);  // every lane votes
+        done = done || (h & gmask) != 0u;
+        return __all_sync(full, done);
+    };
+    const T rp2 = rp * rp;
+    for (int v = r; v < S.nv && !done; v += G) {
+        const P4<T> q = S.vq[v];
+        const T dx = x - q.x, dy = y - q.y, dz = z - q.z;
+        const int t = lt_sq<FILT>(dx * dx + dy * dy + dz * dz, rp2, rp, d0);
+        if (t == 1) hit = done = true;
+        else if (t < 0) unsure = true;
     }
     const int nw = (S.na + 31) >> 5;
-    int u = 0;  // candidate number
-    for (int wd = 0; wd < nw; ++wd) {
-      unsigned bits = C.bmask[brick][wd];
-      while (bits) {
-        const int a = (wd << 5) + __ffs(bits) - 1;
-        bits &= bits - 1;
-        P4<T> c = S.atom[a];
-        T dx = x - c.x, dy = y - c.y, dz = z - c.z;
-        T R = c.w + rp;
-        if (lt_sq<FILT>(dx * dx + dy * dy + dz * dz, R * R, R, d0) == 0) continue;  // ball does not hold x
-        if ((u & (G - 1)) == r) {
-            int w = face_witness<FILT>(A, a, x, y, z, rp, thr, d0, C.nbm, aw, nt);
-            if (w == 1) return 0;
-            if (w < 0) unsure = true;
-        }
-        ++u;
-        const int k0 = C.inc_start[a], k1 = C.inc_start[a + 1];
-        for (int k = k0 + ((r - u) & (G - 1)); k < k1; k += G) {
-            const int p = (int)C.inc[k];
-            const short2 sl = C.pslot[p];
-            // a pair whose other ball holds x too is tested once, under the
-            // lower slot (the balls are taken in slot order; the same test
-            // decides whether that ball is taken)
-            const int b = sl.x == a ? sl.y : sl.x;
-            if (b >= 0 && b < a && ((C.bmask[brick][b >> 5] >> (b & 31)) & 1u)) {
-                const P4<T> cb = S.atom[b];
-                const T ex = x - cb.x, ey = y - cb.y, ez = z - cb.z;
-                const T Rb = cb.w + rp;
-                if (lt_sq<FILT>(ex * ex + ey * ey + ez * ez, Rb * Rb, Rb, d0) != 0) continue;
+    if (!settle()) {
+        // convex patches of the balls that reach the points' bricks
+        const unsigned *bm = C.bmask[(code >> 9) & 15];
+        for (int wd = 0; wd < nw; ++wd) {
+            unsigned bits = __reduce_or_sync(full, done ? 0u : bm[wd]) & share;
+            while (bits && !done) {
+                const int a = (wd << 5) + __ffs(bits) - 1;
+                bits &= bits - 1;
+                T qx, qy, qz, dq;
+                int e0, e1;
+                const int tw = face_proposal<FILT>(A, a, x, y, z, rp, rp, d0, qx, qy, qz, dq, e0, e1);
+                if (tw == 0) continue;
+                if (tw == -2) {
+                    unsure = true;
+                    continue;
+                }
+                const int f = witness_free<FILT>(S, qx, qy, qz, C.nbm + a * aw, (const unsigned *)nullptr, nw, rp,
+                                                 dq + d0, nt);
+                if (f == 1 && tw == 1) hit = done = true;
+                else if (f != 0) unsure = true;
             }
-            int ws = saddle_witness<FILT>(A, p, x, y, z, rp, thr, d0, C.nbm, aw, (int)sl.x, (int)sl.y, nt);
-            if (ws == 1) return 0;
-            if (ws < 0) unsure = true;
         }
-        u += k1 - k0;
-      }
     }
-    return unsure ? 2 : 1;
+    if (!settle()) {
+        // box of the undecided points, then the circles that come within r_p of it
+        const int li = (code >> 6) & 7, lj = (code >> 3) & 7, lk = code & 7;
+        const int i0 = __reduce_min_sync(full, done ? 8 : li), i1 = __reduce_max_sync(full, done ? -1 : li);
+        const int j0 = __reduce_min_sync(full, done ? 8 : lj), j1 = __reduce_max_sync(full, done ? -1 : lj);
+        const int k0 = __reduce_min_sync(full, done ? 8 : lk), k1 = __reduce_max_sync(full, done ? -1 : lk);
+        const float hh = 0.5f * hf;
+        const float cx = hh * (float)(i0 + i1), cy = hh * (float)(j0 + j1), cz = hh * (float)(k0 + k1);
+        const float ex = (float)(i1 - i0), ey = (float)(j1 - j0), ez = (float)(k1 - k0);
+        // 2e-3 A covers the FP32 rounding of the distance (as in the prefilters)
+        const float reach = (float)rp + hh * sqrtf(ex * ex + ey * ey + ez * ez) + 2e-3f;
+        for (int p0 = 0; p0 < S.np; p0 += 32) {
+            bool near = false;
+            if (p0 + lane < S.np) {
+                const P4<T> o = S.po[p0 + lane], u = S.pu[p0 + lane];
+                const short2 sl = C.pslot[p0 + lane];
+                const float yx = cx - (float)o.x, yy = cy - (float)o.y, yz = cz - (float)o.z;
+                const float ux = (float)u.x, uy = (float)u.y, uz = (float)u.z;
+                const float zc = yx * ux + yy * uy + yz * uz;
+                const float wx = yx - zc * ux, wy = yy - zc * uy, wz = yz - zc * uz;
+                const float e = sqrtf(wx * wx + wy * wy + wz * wz) - (float)o.w;
+                // (an atom that is not staged is too far for the circle's points near the tile)
+                near = e * e + zc * zc < reach * reach && sl.x >= 0 && sl.y >= 0;
+            }
+            unsigned bits = __ballot_sync(full, near) & share;
+            while (bits && !done) {
+                const int p = p0 + __ffs(bits) - 1;
+                bits &= bits - 1;
+                T qx, qy, qz, dq;
+                int e0, e1;
+                const int t = saddle_proposal<FILT>(A, p, x, y, z, rp, rp, d0, qx, qy, qz, dq, e0, e1);
+                if (t == 0) continue;
+                if (t == -2) {
+                    unsure = true;
+                    continue;
+                }
+                const short2 sl = C.pslot[p];
+                const int f = witness_free<FILT>(S, qx, qy, qz, C.nbm + sl.x * aw, C.nbm + sl.y * aw, nw, rp, dq + d0,
+                                                 nt);
+                if (f == 1 && t == 1) hit = done = true;
+                else if (f != 0) unsure = true;
+            }
+            if (settle()) break;
+        }
+    }
+    const unsigned h = __ballot_sync(full, hit), u = __ballot_sync(full, unsure);
+    return (h & gmask) ? 0 : ((u & gmask) ? 2 : 1);
 }
 
 // bytes of a CTA's staging (TileS, then ClsSmem 16-byte aligned), rounded up to
@@ -225,6 +258,11 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
         int8_t *__restrict__ labels = labels_all + G.lab0;
         const T d0 = FILT ? (T)G.d0 : T(0);
         const T h = (T)G.h;
+        if (threadIdx.x == 0) {  // before stage_tile's barriers, after the last tile's closing one
+            C.nq = 0;
+            C.band = 0;
+            C.next = 0;
+        }
         double x0[3];
         stage_tile<T>(M, G, mol, tile, S, x0);
         if (!BIG && (S.flags & ERR_CAP_ANY)) {  // uniform: set before stage_tile's last barrier
@@ -235,12 +273,7 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
         // (the global-memory tier classifies even a tile that overflows it,
         // with its lists cut at capacity, so every label is written; the
         // error bit makes the run report ESES_ECAPACITY)
-        if (threadIdx.x == 0) {
-            C.nq = 0;
-            C.band = 0;
-            C.next = 0;
-            if (S.flags) atomicOr(err, S.flags);
-        }
+        if (threadIdx.x == 0 && S.flags) atomicOr(err, S.flags);
         int t[3];
         tile_coords(G, tile, t);
         if (S.na == 0) {  // no atom within reach: every point is free
@@ -255,9 +288,9 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
             __syncthreads();
             continue;
         }
-        build_incidence<T, CP>(S, C);
-        // phase 1: bricks
-        for (int brick = warp; brick < NBRICK; brick += CLS_THREADS / 32) {
+        // phase 1: bricks, two neighbours per warp
+        static_assert(NBRICK == 2 * (CLS_THREADS / 32), "two bricks per warp");
+        for (int brick = 2 * warp; brick < 2 * warp + 2; ++brick) {
             int li, lj, lk;
             brick_point(brick, 0, li, lj, lk);
             const T b0x = (T)li * h, b0y = (T)lj * h, b0z = (T)lk * h;
@@ -278,7 +311,6 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
                 if (lane == 0) C.bmask[brick][base >> 5] = m;
                 cnt += __popc(m);
             }
-            if (lane == 0) C.bcount[brick] = cnt;
             __syncwarp();
             brick_point(brick, lane, li, lj, lk);
             long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
@@ -311,9 +343,14 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
                 else if (!sas) lab = sas_u ? LABEL_BAND : LABEL_OUT;
                 else lab = -1;  // shell point
             }
+            // the brick's shell points, one after the other
+            const unsigned shell = __ballot_sync(0xffffffffu, valid && lab == -1);
+            int at = 0;
+            if (lane == 0 && shell) at = atomicAdd(&C.nq, __popc(shell));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(shell & ((1u << lane) - 1u));
             if (valid) {
                 if (lab == -1) {
-                    C.queue[atomicAdd(&C.nq, 1)] = (short)((li << 6) | (lj << 3) | lk | (brick << 9));
+                    C.queue[at] = (short)((li << 6) | (lj << 3) | lk | (brick << 9));
                 } else {
                     labels[(gi * G.dims[1] + gj) * G.dims[2] + gk] = (int8_t)lab;
                     if (FILT && lab == LABEL_BAND) atomicAdd(&C.band, 1);
@@ -322,38 +359,29 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
         }
         __syncthreads();
         const int nq = C.nq;
-        if (nq > 0) {  // neighbour sets for the witnesses' freeness tests
+        if (nq > 0) {  // neighbour sets and pair slots for the witnesses' freeness tests
             build_neighbour_sets<T, CP>(S, C.nbm, rp);
-            __syncthreads();
+            pair_slots<T>(S, C.hkey, C.hval, C.pslot);
         }
-        // phase 2: shell points, the whole block; with few points, groups of
-        // up to 32 lanes share one (so a tile's last point is not left to one
-        // lane).  A thread (or group) takes the next point from a block counter
-        // when it is done, so the slow points do not pile up on a few threads.
+        // phase 2: shell points, 32 / gs at a time per warp from a block counter
         int gs = 1;
-        while (gs < 32 && nq * gs * 2 <= CLS_THREADS) gs <<= 1;
-        const int r = lane & (gs - 1);
-        const unsigned gmask = (gs == 32 ? 0xffffffffu : ((1u << gs) - 1u)) << (lane & ~(gs - 1));
-        for (;;) {
+        while (gs < 32 && nq * gs * 2 <= CLS_SPLIT) gs <<= 1;
+        const int r = lane & (gs - 1), per = 32 / gs;
+        while (nq > 0) {
             int k = 0;
-            if (r == 0) k = atomicAdd(&C.next, 1);
-            k = __shfl_sync(gmask, k, lane & ~(gs - 1));
+            if (lane == 0) k = atomicAdd(&C.next, per);
+            k = __shfl_sync(0xffffffffu, k, 0);
             if (k >= nq) break;
-            int code = C.queue[k];
-            int brick = (code >> 9) & 15;
-            int li = (code >> 6) & 7, lj = (code >> 3) & 7, lk = code & 7;
-            T x = pt_coord<T>(G, li), y = pt_coord<T>(G, lj), z = pt_coord<T>(G, lk);
-            int part = shell_part<FILT, T, CP>(S, C, brick, x, y, z, rp, d0, r, gs, ntests);
-            // group label: 0 if any part found a witness, else 2 if any is undecided, else 1
-            for (int o = 1; o < gs; o <<= 1) {
-                const int q = __shfl_xor_sync(gmask, part, o);
-                part = (part == 0 || q == 0) ? 0 : max(part, q);
-            }
-            if (r == 0) {
-                long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
-                          gk = (long long)TILE * t[2] + lk;
-                labels[(gi * G.dims[1] + gj) * G.dims[2] + gk] = (int8_t)part;
-                if (FILT && part == LABEL_BAND) atomicAdd(&C.band, 1);
+            k += lane / gs;
+            const int code = k < nq ? C.queue[k] : -1;
+            const int li = (code >> 6) & 7, lj = (code >> 3) & 7, lk = code & 7;
+            const T x = pt_coord<T>(G, li), y = pt_coord<T>(G, lj), z = pt_coord<T>(G, lk);
+            const int lab = shell_points<FILT, T, CP>(S, C, code, x, y, z, rp, d0, (float)G.h, r, gs, ntests);
+            if (r == 0 && code >= 0) {
+                const long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
+                                gk = (long long)TILE * t[2] + lk;
+                labels[(gi * G.dims[1] + gj) * G.dims[2] + gk] = (int8_t)lab;
+                if (FILT && lab == LABEL_BAND) atomicAdd(&C.band, 1);
             }
         }
         __syncthreads();

@@ -485,7 +485,8 @@ __device__ void pair_slots(const TileS<T, C> &S, int *hkey, short *hval, short2 
     __syncthreads();
 }
 
-// Neighbour sets of the staged atoms (whole block): bit b of nbm[a * aw + w]
+// Neighbour sets of the staged atoms (whole block, one warp per atom and word,
+// lanes over the other atoms): bit b of nbm[a * aw + w]
 // (b = 32 w + bit) is set when the expanded spheres of staged atoms a != b
 // come within 1e-3 A of meeting (the margin covers the rounding of staged
 // FP32 positions, so no true neighbour is left out).
@@ -493,20 +494,20 @@ template <class T, class C>
 __device__ __forceinline__ void build_neighbour_sets(const TileS<T, C> &S, unsigned *nbm, T rp)
 {
     constexpr int aw = atom_words<C>();
-    const int na = S.na, nw = (na + 31) >> 5;
-    for (int it = threadIdx.x; it < na * nw; it += blockDim.x) {
-        const int a = it / nw, w = it - a * nw;
+    const int na = S.na, nw = (na + 31) >> 5, lane = threadIdx.x & 31;
+    for (int it = threadIdx.x >> 5; it < na * nw; it += blockDim.x >> 5) {
+        const int a = it / nw, w = it - a * nw, b = (w << 5) + lane;
         const P4<T> ca = S.atom[a];
         const T Ra = ca.w + rp + T(1e-3);
-        unsigned bits = 0u;
-        const int b0 = w << 5, b1 = min(na, b0 + 32);
-        for (int b = b0; b < b1; ++b) {
+        bool meet = false;
+        if (b < na && b != a) {
             const P4<T> cb = S.atom[b];
             const T dx = ca.x - cb.x, dy = ca.y - cb.y, dz = ca.z - cb.z;
             const T reach = Ra + cb.w + rp;
-            if (b != a && dx * dx + dy * dy + dz * dz < reach * reach) bits |= 1u << (b - b0);
+            meet = dx * dx + dy * dy + dz * dz < reach * reach;
         }
-        nbm[a * aw + w] = bits;
+        const unsigned bits = __ballot_sync(0xffffffffu, meet);
+        if (lane == 0) nbm[a * aw + w] = bits;
     }
 }
 
@@ -598,40 +599,6 @@ __device__ __forceinline__ int saddle_proposal(const Acc &A, int p, T x, T y, T 
     e0 = ij.x;
     e1 = ij.y;
     return t;
-}
-
-// Convex witness of staged atom a at x: 1 free projection at distance < thr,
-// 0 none, -1 undecided.  nbm: the staged atoms' neighbour sets; the
-// projection's freeness is tested against a's neighbours (free_set).
-template <bool FILT, class Acc, class T>
-__device__ __noinline__ int face_witness(const Acc &A, int a, T x, T y, T z, T rp, T thr, T d0, const unsigned *nbm,
-                                         int aw, int &nt)
-{
-    T qx, qy, qz, dq;
-    int e0, e1;
-    const int tw = face_proposal<FILT>(A, a, x, y, z, rp, thr, d0, qx, qy, qz, dq, e0, e1);
-    if (tw == 0) return 0;
-    if (tw == -2) return -1;
-    int f = free_set<FILT>(A, qx, qy, qz, nbm + a * aw, (const unsigned *)nullptr, rp, dq + d0, nt);
-    if (f == 1 && tw == 1) return 1;
-    return f == 0 ? 0 : -1;
-}
-
-// Saddle witness of pair p at x: nearest point of its circle; its freeness
-// is tested against the common neighbours of the pair's staged atoms (slots
-// sa, sb).
-template <bool FILT, class Acc, class T>
-__device__ __noinline__ int saddle_witness(const Acc &A, int p, T x, T y, T z, T rp, T thr, T d0, const unsigned *nbm,
-                                           int aw, int sa, int sb, int &nt)
-{
-    T qx, qy, qz, dq;
-    int e0, e1;
-    const int t = saddle_proposal<FILT>(A, p, x, y, z, rp, thr, d0, qx, qy, qz, dq, e0, e1);
-    if (t == 0) return 0;
-    if (t == -2) return -1;
-    int f = free_set<FILT>(A, qx, qy, qz, nbm + sa * aw, nbm + sb * aw, rp, dq + d0, nt);
-    if (f == 1 && t == 1) return 1;
-    return f == 0 ? 0 : -1;
 }
 
 // Freeness of q (the same on every lane) against every staged atom but e0,
