@@ -26,3 +26,39 @@ def test_shell_points_of_few_and_many_lanes(n, h, prec):
     finally:
         eses.eses_destroy(ctx)
 
+
+def _edges(lab):
+    """Crossing edges per axis: 8x8x8 tiles in C order, then point order."""
+    out = []
+    for a in range(3):
+        g = np.argwhere(np.diff(lab.astype(np.int16), axis=a) != 0)
+        t, l = g // 8, g % 8
+        nt = [-(-d // 8) for d in lab.shape]
+        key = ((t[:, 0] * nt[1] + t[:, 1]) * nt[2] + t[:, 2]) * 512 + (l[:, 0] * 8 + l[:, 1]) * 8 + l[:, 2]
+        g = g[np.argsort(key, kind="stable")]
+        out.append((g[:, 0] * lab.shape[1] + g[:, 1]) * lab.shape[2] + g[:, 2])
+    return out
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (1, 1, 9), (3, 2, 5), (8, 8, 8), (9, 9, 9), (17, 8, 16), (7, 65, 33),
+                                  (33, 130, 257), (160, 170, 300)])
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_noalloc_rows_at_every_alignment(dims, shift):
+    """Label rows at every alignment of the first label and of a row (odd
+    lengths), grids smaller than a word, one and several tiles per warp."""
+    import torch
+
+    libbuild.build()
+    rng = np.random.default_rng(sum(dims) + shift)
+    lab = (rng.random(dims) < 0.4).astype(np.int8)
+    if max(dims) > 100:
+        lab[: dims[0] // 2] = 1  # whole tiles without edges
+    store = torch.full((lab.size + shift,), 1, dtype=torch.int8, device="cuda")
+    store[shift:] = torch.from_numpy(lab.reshape(-1)).cuda()
+    ref = _edges(lab)
+    outs = [torch.full((len(r) + 1,), -1, dtype=torch.int64, device="cuda") for r in ref]
+    counts = eses.eses_crossing_edges_noalloc(store.data_ptr() + shift, dims, *outs, [len(r) for r in ref])
+    for a in range(3):
+        assert counts[a] == len(ref[a])
+        got = outs[a].cpu().numpy()
+        assert np.array_equal(got[:-1], ref[a]) and got[-1] == -1, a
