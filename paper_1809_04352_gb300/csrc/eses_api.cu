@@ -130,10 +130,10 @@ struct eses_ctx {
     Batch B{};
     // device buffers
     DBuf xyz, rad, in_mol, grid_d, cg_d, tile_off_d, atom_mol, vert_mol, medge, term, queue;
-    DBuf cell_id, cell_count, cell_start, cursor, atom_orig, atom;
+    DBuf cell_id, cell_count, cell_start, cursor, atom_scat, atom_cell, atom_orig, atom;
     DBuf nb_count, nb_start, nb_list, circle_count, contained, face;
     DBuf pair_count, pair_start, pair_o, pair_u, pair_ij, pair_free;
-    DBuf vert_count, vert_start, vert, vert_atoms;
+    DBuf vert_count, vert_start, vert, vert_atoms, arc_list, arc_whole;
     DBuf pbin_count, pbin_start, pbin_cursor, pbin_cell, pbin_list;
     DBuf vbin_count, vbin_start, vbin_cursor, vbin_cell, vbin_list;
     DBuf labels, tile_band, tile_edges, edge_start, tile_inside;
@@ -225,6 +225,18 @@ int list_total(eses_ctx *c, const int *start, long long n, int &planned)
     ck(cudaStreamSynchronize(c->stream), "synchronize");
     planned = v;
     return v;
+}
+
+// two list totals, read with one wait
+void list_totals(eses_ctx *c, const int *a, int &pa, const int *b, int &pb)
+{
+    if (g_capturing) return;
+    int v[2] = {0, 0};
+    ck(cudaMemcpyAsync(&v[0], a, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "read list total");
+    ck(cudaMemcpyAsync(&v[1], b, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "read list total");
+    ck(cudaStreamSynchronize(c->stream), "synchronize");
+    pa = v[0];
+    pb = v[1];
 }
 
 int validate(const double *xyz, const double *r, int64_t n, double rp, double h, double margin, std::string &msg)
@@ -586,7 +598,9 @@ int run_device(eses_ctx *c)
     int *cell_count = ensure<int>(c->cell_count, ncell);
     int *cell_start = ensure<int>(c->cell_start, ncell + 1);
     int *cursor = ensure<int>(c->cursor, ncell);
+    int *scat = ensure<int>(c->atom_scat, n);
     int *orig = ensure<int>(c->atom_orig, n);
+    int *atom_cell = ensure<int>(c->atom_cell, n);
     double4 *atom = ensure<double4>(c->atom, n);
     int *atom_mol = ensure<int>(c->atom_mol, n);
     ck(cudaMemsetAsync(cell_count, 0, sizeof(int) * ncell, st), "memset");
@@ -594,49 +608,45 @@ int run_device(eses_ctx *c)
     nl += launch_cell_count((const double *)c->xyz.p, (const int *)c->in_mol.p, n, M.cg, M.cell, cell_id, cell_count,
                             st);
     nl += scan(c, cell_count, cell_start, ncell);
-    nl += launch_cell_scatter(nullptr, nullptr, n, cell_id, cell_start, cursor, orig, st);
+    float4 *ahi = ensure<float4>(c->atom_hi, n), *alo = ensure<float4>(c->atom_lo, n);
+    nl += launch_cell_scatter(nullptr, nullptr, n, cell_id, cell_start, cursor, scat, st);
     nl += launch_cell_finish((const double *)c->xyz.p, (const double *)c->rad.p, (const int *)c->in_mol.p, (int)ncell,
-                             cell_start, orig, atom, atom_mol, st);
+                             cell_start, scat, B.grid, orig, atom, atom_mol, atom_cell, ahi, alo, st);
     M.atom = atom;
     M.atom_orig = orig;
     M.atom_mol = atom_mol;
+    M.atom_cell = atom_cell;
     M.cell_start = cell_start;
-    float4 *ahi = ensure<float4>(c->atom_hi, n), *alo = ensure<float4>(c->atom_lo, n);
-    nl += launch_model_f32(M, 0, B.grid, ahi, alo, nullptr, st);
     M.atom_hi = ahi;
     M.atom_lo = alo;
 
     mark(c, ST_PAIRS);
-    // 2. neighbours
+    // 2. neighbours and circle pairs
     int *nb_count = ensure<int>(c->nb_count, n);
     int *circle_count = ensure<int>(c->circle_count, n);
     uint8_t *contained = ensure<uint8_t>(c->contained, n);
     int *nb_start = ensure<int>(c->nb_start, n + 1);
-    nl += launch_nb_count(M, nb_count, circle_count, contained, st);
-    nl += scan(c, nb_count, nb_start, n);
-    const int n_nb = list_total(c, nb_start, n, c->n_nb);
-    int *nb_list = ensure<int>(c->nb_list, std::max(n_nb, 1));
-    M.nb_start = nb_start;
-    M.nb_list = nb_list;
-    nl += launch_nb_fill(M, nb_list, st);
-
-    // 3. circle pairs
     int *pair_count = ensure<int>(c->pair_count, n);
     int *pair_start = ensure<int>(c->pair_start, n + 1);
-    nl += launch_pair_count(M, pair_count, st);
+    nl += launch_nb_count(M, nb_count, circle_count, pair_count, contained, st);
+    nl += scan(c, nb_count, nb_start, n);
     nl += scan(c, pair_count, pair_start, n);
-    const int np = list_total(c, pair_start, n, c->n_pairs);
-    M.n_pairs = np;
+    list_totals(c, nb_start + n, c->n_nb, pair_start + n, c->n_pairs);
+    const int n_nb = c->n_nb, np = c->n_pairs;
+    int *nb_list = ensure<int>(c->nb_list, std::max(n_nb, 1));
+    int2 *pair_ij = ensure<int2>(c->pair_ij, std::max(np, 1));
     double4 *pair_o = ensure<double4>(c->pair_o, std::max(np, 1));
     double4 *pair_u = ensure<double4>(c->pair_u, std::max(np, 1));
-    int2 *pair_ij = ensure<int2>(c->pair_ij, std::max(np, 1));
-    nl += launch_pair_fill(M, pair_start, pair_o, pair_u, pair_ij, st);
-    M.pair_o = pair_o;
-    M.pair_u = pair_u;
-    M.pair_ij = pair_ij;
     float4 *phi = ensure<float4>(c->pair_hi, std::max(np, 1)), *plo = ensure<float4>(c->pair_lo, std::max(np, 1));
     float4 *pu32 = ensure<float4>(c->pair_u32, std::max(np, 1));
-    nl += launch_model_f32(M, 1, B.grid, phi, plo, pu32, st);
+    M.nb_start = nb_start;
+    M.nb_list = nb_list;
+    M.n_pairs = np;
+    M.pair_ij = pair_ij;
+    nl += launch_nb_fill(M, nb_list, pair_start, pair_ij, st);
+    nl += launch_pair_geom(M, B.grid, pair_o, pair_u, phi, plo, pu32, st);
+    M.pair_o = pair_o;
+    M.pair_u = pair_u;
     M.pair_hi = phi;
     M.pair_lo = plo;
     M.pair_u32 = pu32;
@@ -646,7 +656,14 @@ int run_device(eses_ctx *c)
     uint8_t *pair_free = ensure<uint8_t>(c->pair_free, std::max(np, 1));
     int *vert_count = ensure<int>(c->vert_count, std::max(np, 1));
     int *vert_start = ensure<int>(c->vert_start, np + 1);
-    nl += launch_arcs(M, pair_free, vert_count, st);
+    // free triple points per circle are few (14 in 100 circles of the globules, fewer when packed): a list as
+    // long as the circles holds them, and a circle that finds it full is emitted whole
+    ArcList AL;
+    AL.cap = std::max(np, 1) + 4096;
+    AL.e = ensure<int4>(c->arc_list, (size_t)AL.cap);
+    AL.whole = ensure<int>(c->arc_whole, std::max(np, 1));
+    AL.n = misc + 16;
+    nl += launch_arcs(M, pair_free, vert_count, AL, st);
     M.pair_free = pair_free;
     nl += scan(c, vert_count, vert_start, np);
     const int nv = list_total(c, vert_start, np, c->n_verts);
@@ -654,9 +671,13 @@ int run_device(eses_ctx *c)
     double4 *vert = ensure<double4>(c->vert, std::max(nv, 1));
     int *vert_mol = ensure<int>(c->vert_mol, std::max(nv, 1));
     int4 *vert_atoms = ensure<int4>(c->vert_atoms, std::max(nv, 1));
-    nl += launch_arcs_emit(M, vert_start, vert, vert_mol, vert_atoms, st);
+    float4 *vhi = ensure<float4>(c->vert_hi, std::max(nv, 1)), *vlo = ensure<float4>(c->vert_lo, std::max(nv, 1));
+    const VertOut VO{vert, vert_mol, vert_atoms, vhi, vlo, B.grid};
+    nl += launch_arcs_emit(M, vert_start, AL, VO, st);
     M.vert = vert;
     M.vert_mol = vert_mol;
+    M.vert_hi = vhi;
+    M.vert_lo = vlo;
 
     if (n >= (1 << 27) || np >= (1 << 27) || nv >= (1 << 27))
         throw std::string("more than 2^27 atoms, circle pairs or triple points");
@@ -691,10 +712,6 @@ int run_device(eses_ctx *c)
     M.pcell_list = plist;
     M.vcell_start = vstart;
     M.vcell_list = vlist;
-    float4 *vhi = ensure<float4>(c->vert_hi, std::max(nv, 1)), *vlo = ensure<float4>(c->vert_lo, std::max(nv, 1));
-    nl += launch_model_f32(M, 2, B.grid, vhi, vlo, nullptr, st);
-    M.vert_hi = vhi;
-    M.vert_lo = vlo;
 
     // 7. classification (+ FP64 band re-evaluation), persistent over all tiles;
     //    with the proposer, certified far tiles are filled first and only the
@@ -1899,7 +1916,7 @@ void eses_destroy(eses_ctx *c)
     if (!c) return;
     DBuf *bufs[] = {&c->xyz, &c->rad, &c->in_mol, &c->grid_d, &c->cg_d, &c->tile_off_d, &c->atom_mol, &c->vert_mol,
                     &c->medge, &c->term, &c->queue, &c->cell_id, &c->cell_count, &c->cell_start, &c->cursor,
-                    &c->atom_orig, &c->atom, &c->nb_count, &c->nb_start, &c->nb_list, &c->circle_count,
+                    &c->atom_scat, &c->atom_cell, &c->atom_orig, &c->atom, &c->arc_list, &c->arc_whole, &c->nb_count, &c->nb_start, &c->nb_list, &c->circle_count,
                     &c->contained, &c->face, &c->pair_count, &c->pair_start, &c->pair_o, &c->pair_u, &c->pair_ij,
                     &c->pair_free, &c->vert_count, &c->vert_start, &c->vert, &c->vert_atoms, &c->pbin_count, &c->pbin_start,
                     &c->pbin_cursor, &c->pbin_cell, &c->pbin_list, &c->vbin_count, &c->vbin_start, &c->vbin_cursor,

@@ -74,6 +74,7 @@ struct Model {
     const CellGrid *cg;           // per molecule
     const int *atom_mol;          // molecule of each sorted atom
     const double4 *atom;          // sorted atoms (x, y, z, r)
+    const int *atom_cell;         // cell of each sorted atom
     const int *atom_orig;         // original index of each sorted atom (in the batch)
     const uint8_t *atom_face;     // 1: expanded sphere keeps a free face
     double cell;                  // cell edge (all molecules)

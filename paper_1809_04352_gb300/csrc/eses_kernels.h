@@ -20,21 +20,34 @@ int launch_cell_count(const double *xyz, const int *in_mol, int n, const CellGri
                       int *cell_count, cudaStream_t st);
 int launch_cell_scatter(const double *xyz, const double *r, int n, const int *cell_id, const int *cell_start,
                          int *cursor, int *sorted_orig, cudaStream_t st);
+// scattered: the atoms of every cell in any order; the sorted atoms with their FP32 copies come out
 int launch_cell_finish(const double *xyz, const double *r, const int *in_mol, int ncell, const int *cell_start,
-                       int *sorted_orig, double4 *atom, int *atom_mol, cudaStream_t st);
-int launch_nb_count(const Model &M, int *nb_count, int *circle_count, uint8_t *contained, cudaStream_t st);
-int launch_nb_fill(const Model &M, int *nb_list, cudaStream_t st);
-int launch_pair_count(const Model &M, int *pair_count, cudaStream_t st);
-int launch_pair_fill(const Model &M, const int *pair_start, double4 *pair_o, double4 *pair_u, int2 *pair_ij,
-                      cudaStream_t st);
-int launch_arcs(const Model &M, uint8_t *pair_free, int *vert_count, cudaStream_t st);
-int launch_arcs_emit(const Model &M, const int *vert_start, double4 *vert, int *vert_mol, int4 *vert_atoms,
-                     cudaStream_t st);
+                       const int *scattered, const Grid *grids, int *sorted_orig, double4 *atom, int *atom_mol,
+                       int *atom_cell, float4 *hi, float4 *lo, cudaStream_t st);
+int launch_nb_count(const Model &M, int *nb_count, int *circle_count, int *pair_count, uint8_t *contained,
+                    cudaStream_t st);
+int launch_nb_fill(const Model &M, int *nb_list, const int *pair_start, int2 *pair_ij, cudaStream_t st);
+int launch_pair_geom(const Model &M, const Grid *grids, double4 *pair_o, double4 *pair_u, float4 *hi, float4 *lo,
+                     float4 *u32, cudaStream_t st);
+// free end points that the arc kernel lists for the emission of triple points
+struct ArcList {
+    int4 *e;     // (circle, third atom, end point, place among the circle's), any order; circle -1: dead
+    int *n;      // [0] entries, [1] circles in `whole` (both zero before launch_arcs)
+    int *whole;  // circles emitted whole by a warp each (room for every circle)
+    int cap;
+};
+// triple points: position and third atom, molecule, atoms, FP32 copies relative to the molecule's grid origin
+struct VertOut {
+    double4 *vert;
+    int *mol;
+    int4 *atoms;
+    float4 *hi, *lo;
+    const Grid *grids;
+};
+int launch_arcs(const Model &M, uint8_t *pair_free, int *vert_count, const ArcList &L, cudaStream_t st);
+int launch_arcs_emit(const Model &M, const int *vert_start, const ArcList &L, const VertOut &O, cudaStream_t st);
 int launch_faces(const Model &M, const int *circle_count, const uint8_t *contained, uint8_t *face, cudaStream_t st);
 int launch_bin_count(const Model &M, int which, bool cull, int *count, int *item_cell, cudaStream_t st);
-// FP32 double-float copies: which 0 atoms (hi, lo), 1 circles (hi, lo, axis), 2 triple points (hi, lo)
-int launch_model_f32(const Model &M, int which, const Grid *grids, float4 *hi, float4 *lo_, float4 *u32,
-                     cudaStream_t st);
 int launch_bin_scatter(const Model &M, int which, const int *item_cell, const int *start, int *cursor, int *list,
                         cudaStream_t st);
 

@@ -18,6 +18,8 @@
 // (§5) -- the same set as step 3.
 #include <math.h>
 
+#include <algorithm>
+
 #include "eses_kernels.h"
 
 namespace eses {
@@ -80,58 +82,91 @@ int launch_cell_scatter(const double *, const double *, int n, const int *cell_i
     return 1;
 }
 
-// order every cell by original atom index (deterministic layout), then gather
-__global__ void k_cell_finish(const double *__restrict__ xyz, const double *__restrict__ r,
-                              const int *__restrict__ in_mol, int ncell, const int *__restrict__ cell_start,
-                              int *__restrict__ sorted_orig, double4 *__restrict__ atom, int *__restrict__ atom_mol)
+// Every cell's atoms ordered by original atom index (deterministic layout),
+// gathered with their FP32 copies.  One warp per cell, an atom's place its rank
+// among the cell's indices (one thread's insertion sort in global memory held
+// the launch to 85 us on 26 atoms a cell; 6 us now).
+constexpr int CELL_WARPS = 4;
+
+__global__ void __launch_bounds__(CELL_WARPS * 32) k_cell_finish(
+    const double *__restrict__ xyz, const double *__restrict__ r, const int *__restrict__ in_mol, int ncell,
+    const int *__restrict__ cell_start, const int *__restrict__ scattered, const Grid *__restrict__ grids,
+    int *__restrict__ sorted_orig, double4 *__restrict__ atom, int *__restrict__ atom_mol,
+    int *__restrict__ atom_cell, float4 *__restrict__ hi, float4 *__restrict__ lo)
 {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncell) return;
-    int s = cell_start[c], e = cell_start[c + 1];
-    for (int a = s + 1; a < e; ++a) {
-        int v = sorted_orig[a];
-        int b = a - 1;
-        while (b >= s && sorted_orig[b] > v) {
-            sorted_orig[b + 1] = sorted_orig[b];
-            --b;
+    const int lane = threadIdx.x & 31;
+    for (long long c = (long long)blockIdx.x * CELL_WARPS + (threadIdx.x >> 5); c < ncell;
+         c += (long long)gridDim.x * CELL_WARPS) {
+        const int s = cell_start[c], e = cell_start[c + 1];
+        for (int a = s + lane; a < e; a += 32) {
+            const int o = scattered[a];
+            int rank = 0;
+            for (int b = s; b < e; ++b) rank += scattered[b] < o ? 1 : 0;
+            const int k = s + rank, mol = in_mol[o];
+            const double4 at = make_double4(xyz[3 * o], xyz[3 * o + 1], xyz[3 * o + 2], r[o]);
+            sorted_orig[k] = o;
+            atom[k] = at;
+            atom_mol[k] = mol;
+            atom_cell[k] = (int)c;
+            const double *L = grids[mol].lo;
+            float hx, hy, hz, ex, ey, ez;
+            split_df(at.x - L[0], hx, ex);
+            split_df(at.y - L[1], hy, ey);
+            split_df(at.z - L[2], hz, ez);
+            hi[k] = make_float4(hx, hy, hz, (float)at.w);
+            lo[k] = make_float4(ex, ey, ez, 0.0f);
         }
-        sorted_orig[b + 1] = v;
-    }
-    for (int a = s; a < e; ++a) {
-        int o = sorted_orig[a];
-        atom[a] = make_double4(xyz[3 * o], xyz[3 * o + 1], xyz[3 * o + 2], r[o]);
-        atom_mol[a] = in_mol[o];
     }
 }
 
 int launch_cell_finish(const double *xyz, const double *r, const int *in_mol, int ncell, const int *cell_start,
-                       int *sorted_orig, double4 *atom, int *atom_mol, cudaStream_t st)
+                       const int *scattered, const Grid *grids, int *sorted_orig, double4 *atom, int *atom_mol,
+                       int *atom_cell, float4 *hi, float4 *lo, cudaStream_t st)
 {
-    k_cell_finish<<<(ncell + 255) / 256, 256, 0, st>>>(xyz, r, in_mol, ncell, cell_start, sorted_orig, atom, atom_mol);
+    const int nb = (ncell + CELL_WARPS - 1) / CELL_WARPS;
+    k_cell_finish<<<nb < 65536 ? nb : 65536, CELL_WARPS * 32, 0, st>>>(xyz, r, in_mol, ncell, cell_start, scattered,
+                                                                       grids, sorted_orig, atom, atom_mol, atom_cell,
+                                                                       hi, lo);
     return 1;
 }
 
 // --------------------------------------------------------------------------
-// neighbour iteration over the 27 cells around a sorted atom (in the cells of
-// its own molecule), one warp: f(j, valid) on every lane for 32 consecutive
-// atoms of a cell at a time, so the lanes visit the atoms in cell order and
-// ballots over `valid` keep that order
+// The atoms of the 27 cells around sorted atom i (in the cells of its own
+// molecule) in cell order, one warp: f(j, valid) on every lane, 32 atoms at a
+// time.  The three cells along the last axis hold consecutive atoms, so the
+// walk is over 9 runs laid end to end (a cell of the globules holds 3 atoms:
+// cell by cell, 27 steps of 3 lanes).
 // --------------------------------------------------------------------------
 template <class F>
-__device__ __forceinline__ void warp_neighbour_cells(const Model &M, int mol, double px, double py, double pz, F f)
+__device__ __forceinline__ void warp_neighbour_cells(const Model &M, int i, F f)
 {
+    const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const CellGrid g = M.cg[mol];
-    const int ca = cell_coord(px, g.clo[0], M.cell, g.cn[0]);
-    const int cb = cell_coord(py, g.clo[1], M.cell, g.cn[1]);
-    const int cc = cell_coord(pz, g.clo[2], M.cell, g.cn[2]);
-    for (int a = max(ca - 1, 0); a <= min(ca + 1, g.cn[0] - 1); ++a)
-        for (int b = max(cb - 1, 0); b <= min(cb + 1, g.cn[1] - 1); ++b)
-            for (int c = max(cc - 1, 0); c <= min(cc + 1, g.cn[2] - 1); ++c) {
-                const int id = g.coff + (a * g.cn[1] + b) * g.cn[2] + c;
-                const int s0 = M.cell_start[id], s1 = M.cell_start[id + 1];
-                for (int j0 = s0; j0 < s1; j0 += 32) f(j0 + lane, j0 + lane < s1);
-            }
+    const CellGrid &g = M.cg[M.atom_mol[i]];
+    const int c = M.atom_cell[i] - g.coff, n1 = g.cn[1], n2 = g.cn[2];
+    const int cc = c % n2, cb = (c / n2) % n1, ca = c / (n2 * n1);
+    int start = 0, len = 0;
+    if (lane < 9) {
+        const int a = ca - 1 + lane / 3, b = cb - 1 + lane % 3;
+        if (a >= 0 && b >= 0 && a < g.cn[0] && b < n1) {
+            const int row = g.coff + (a * n1 + b) * n2;
+            start = M.cell_start[row + max(cc - 1, 0)];
+            len = M.cell_start[row + min(cc + 1, n2 - 1) + 1] - start;
+        }
+    }
+    int end = len;  // inclusive prefix over the runs
+    for (int o = 1; o < 16; o <<= 1) {
+        const int v = __shfl_up_sync(full, end, o);
+        if (lane >= o) end += v;
+    }
+    const int total = __shfl_sync(full, end, 8);
+    start -= end - len;  // atom of position t in run r: start[r] + t
+    for (int t0 = 0; t0 < total; t0 += 32) {
+        const int t = t0 + lane;
+        int r = 0;
+        for (int q = 0; q < 8; ++q) r += t >= __shfl_sync(full, end, q) ? 1 : 0;
+        f(__shfl_sync(full, start, r) + t, t < total);
+    }
 }
 
 constexpr int NB_WARPS = 4;  // warps (atoms) per block of the neighbour and pair kernels
@@ -172,153 +207,134 @@ __device__ __forceinline__ bool circle_canon(const Model &M, int i, int j, const
     return circle_of(sw ? cj : ci, sw ? Rj : Ri, sw ? ci : cj, sw ? Ri : Rj, o, u, rho);
 }
 
-// One warp per atom: neighbours (expanded spheres that overlap), circles, and
-// whether the expanded ball lies inside another one.
+// Sorted atom j next to atom i: 0 the expanded spheres do not overlap, 1 they
+// do without meeting in a circle (`within`: ball i lies inside ball j), 2 they
+// meet in a circle.  Taken in FP32 from the double-float copies when the
+// distance clears every limit by 1e-3 A + 1e-5 S (the copies' difference is
+// good to 1e-6 A and the radii to 6e-8 S), else in FP64 with the circle's own
+// arithmetic -- FP64 here costs an SM one warp instruction per 16 cycles.
+__device__ __forceinline__ int nb_class(const Model &M, int i, int j, const float4 &ih, const float4 &il, bool &within)
+{
+    const float4 jh = M.atom_hi[j], jl = M.atom_lo[j];
+    const float dx = (jh.x - ih.x) + (jl.x - il.x), dy = (jh.y - ih.y) + (jl.y - il.y),
+                dz = (jh.z - ih.z) + (jl.z - il.z);
+    const float rpf = (float)M.rp, Ri = ih.w + rpf, Rj = jh.w + rpf;
+    const float d2 = dx * dx + dy * dy + dz * dz, S = Ri + Rj, m = 1e-3f + 1e-5f * S;
+    if (d2 > (S + m) * (S + m)) return 0;
+    const float inner = fabsf(Ri - Rj) + m;
+    if (S > m && d2 < (S - m) * (S - m) && d2 > inner * inner) return 2;
+    const double4 ci = M.atom[i], cj = M.atom[j];
+    const double Rd = ci.w + M.rp, Re = cj.w + M.rp;
+    const double ex = cj.x - ci.x, ey = cj.y - ci.y, ez = cj.z - ci.z;
+    const double D2 = ex * ex + ey * ey + ez * ez, Sd = Rd + Re;
+    if (!(D2 < Sd * Sd)) return 0;
+    double3 o, u;
+    double rho;
+    if (circle_canon(M, i, j, ci, Rd, cj, Re, o, u, rho)) return 2;
+    if (Re >= Rd && sqrt(D2) <= Re - Rd) within = true;
+    return 1;
+}
+
+// One warp per atom: neighbours (expanded spheres that overlap), circles,
+// circles with later atoms (the atom's pairs), and whether the expanded ball
+// lies inside another one.
 __global__ void __launch_bounds__(NB_WARPS * 32) k_nb_count(Model M, int *__restrict__ nb_count,
                                                            int *__restrict__ circle_count,
+                                                           int *__restrict__ pair_count,
                                                            uint8_t *__restrict__ contained)
 {
     const int i = blockIdx.x * NB_WARPS + (threadIdx.x >> 5);
     if (i >= M.n_atoms) return;  // uniform per warp
-    const double4 ci = M.atom[i];
-    const double Ri = ci.w + M.rp;
-    int nb = 0, nc = 0;
+    const float4 ih = M.atom_hi[i], il = M.atom_lo[i];
+    int nb = 0, nc = 0, np = 0;
     bool inside = false;
-    warp_neighbour_cells(M, M.atom_mol[i], ci.x, ci.y, ci.z, [&](int j, bool valid) {
+    warp_neighbour_cells(M, i, [&](int j, bool valid) {
         if (!valid || j == i) return;
-        const double4 cj = M.atom[j];
-        const double Rj = cj.w + M.rp;
-        const double dx = cj.x - ci.x, dy = cj.y - ci.y, dz = cj.z - ci.z;
-        const double D2 = dx * dx + dy * dy + dz * dz;
-        const double S = Ri + Rj;
-        if (D2 < S * S) {
-            ++nb;
-            double3 o, u;
-            double rho;
-            if (circle_canon(M, i, j, ci, Ri, cj, Rj, o, u, rho)) ++nc;
-            else if (Rj >= Ri && sqrt(D2) <= Rj - Ri) inside = true;  // ball i inside ball j
-        }
+        const int k = nb_class(M, i, j, ih, il, inside);
+        nb += k > 0 ? 1 : 0;
+        nc += k == 2 ? 1 : 0;
+        np += k == 2 && j > i ? 1 : 0;
     });
-    for (int o = 16; o > 0; o >>= 1) {
-        nb += __shfl_xor_sync(0xffffffffu, nb, o);
-        nc += __shfl_xor_sync(0xffffffffu, nc, o);
-    }
+    nb = __reduce_add_sync(0xffffffffu, nb);
+    nc = __reduce_add_sync(0xffffffffu, nc);
+    np = __reduce_add_sync(0xffffffffu, np);
     inside = __any_sync(0xffffffffu, inside);
     if ((threadIdx.x & 31) == 0) {
         nb_count[i] = nb;
         circle_count[i] = nc;
+        pair_count[i] = np;
         contained[i] = inside ? 1 : 0;
     }
 }
 
-int launch_nb_count(const Model &M, int *nb_count, int *circle_count, uint8_t *contained, cudaStream_t st)
+int launch_nb_count(const Model &M, int *nb_count, int *circle_count, int *pair_count, uint8_t *contained,
+                    cudaStream_t st)
 {
     if (M.n_atoms <= 0) return 0;
-    k_nb_count<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, nb_count, circle_count, contained);
+    k_nb_count<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, nb_count, circle_count, pair_count,
+                                                                              contained);
     return 1;
 }
 
-// One warp per atom: the neighbour list in cell order (the same order as a
-// serial walk over the 27 cells).
-__global__ void __launch_bounds__(NB_WARPS * 32) k_nb_fill(Model M, int *__restrict__ nb_list)
+// One warp per atom i: the neighbour list in cell order (the same order as a
+// serial walk over the 27 cells), and its pairs -- the circles with neighbours
+// j > i -- in that order.
+__global__ void __launch_bounds__(NB_WARPS * 32) k_nb_fill(Model M, int *__restrict__ nb_list,
+                                                          const int *__restrict__ pair_start,
+                                                          int2 *__restrict__ pair_ij)
 {
     const int i = blockIdx.x * NB_WARPS + (threadIdx.x >> 5);
     if (i >= M.n_atoms) return;
-    const int lane = threadIdx.x & 31;
-    const double4 ci = M.atom[i];
-    const double Ri = ci.w + M.rp;
-    int w = M.nb_start[i];
-    warp_neighbour_cells(M, M.atom_mol[i], ci.x, ci.y, ci.z, [&](int j, bool valid) {
-        bool keep = false;
-        if (valid && j != i) {
-            const double4 cj = M.atom[j];
-            const double Rj = cj.w + M.rp;
-            const double dx = cj.x - ci.x, dy = cj.y - ci.y, dz = cj.z - ci.z;
-            const double S = Ri + Rj;
-            keep = dx * dx + dy * dy + dz * dz < S * S;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (keep) nb_list[w + __popc(m & ((1u << lane) - 1))] = j;
+    const unsigned full = 0xffffffffu, below = (1u << (threadIdx.x & 31)) - 1;
+    const float4 ih = M.atom_hi[i], il = M.atom_lo[i];
+    int w = M.nb_start[i], wp = pair_start[i];
+    warp_neighbour_cells(M, i, [&](int j, bool valid) {
+        bool within = false;
+        const int k = valid && j != i ? nb_class(M, i, j, ih, il, within) : 0;
+        const unsigned m = __ballot_sync(full, k > 0), mp = __ballot_sync(full, k == 2 && j > i);
+        if (k > 0) nb_list[w + __popc(m & below)] = j;
+        if (k == 2 && j > i) pair_ij[wp + __popc(mp & below)] = make_int2(i, j);
         w += __popc(m);
+        wp += __popc(mp);
     });
 }
 
-int launch_nb_fill(const Model &M, int *nb_list, cudaStream_t st)
+int launch_nb_fill(const Model &M, int *nb_list, const int *pair_start, int2 *pair_ij, cudaStream_t st)
 {
     if (M.n_atoms <= 0) return 0;
-    k_nb_fill<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, nb_list);
+    k_nb_fill<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, nb_list, pair_start, pair_ij);
     return 1;
 }
 
-// One warp per atom i: circles with neighbours j > i.
-__global__ void __launch_bounds__(NB_WARPS * 32) k_pair_count(Model M, int *__restrict__ pair_count)
+// One thread per pair (full warps of FP64 work): its circle, and the FP32 copies.
+__global__ void k_pair_geom(Model M, const Grid *__restrict__ grids, double4 *__restrict__ pair_o,
+                            double4 *__restrict__ pair_u, float4 *__restrict__ hi, float4 *__restrict__ lo,
+                            float4 *__restrict__ u32)
 {
-    const int i = blockIdx.x * NB_WARPS + (threadIdx.x >> 5);
-    if (i >= M.n_atoms) return;
-    const double4 ci = M.atom[i];
-    const double Ri = ci.w + M.rp;
-    int c = 0;
-    for (int t = M.nb_start[i] + (threadIdx.x & 31); t < M.nb_start[i + 1]; t += 32) {
-        const int j = M.nb_list[t];
-        if (j <= i) continue;
-        const double4 cj = M.atom[j];
-        double3 o, u;
-        double rho;
-        if (circle_canon(M, i, j, ci, Ri, cj, cj.w + M.rp, o, u, rho)) ++c;
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0) pair_count[i] = c;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= M.n_pairs) return;
+    const int2 ij = M.pair_ij[k];
+    const double4 ci = M.atom[ij.x], cj = M.atom[ij.y];
+    double3 o = make_double3(0.0, 0.0, 0.0), u = o;
+    double rho = 0.0;
+    circle_canon(M, ij.x, ij.y, ci, ci.w + M.rp, cj, cj.w + M.rp, o, u, rho);
+    pair_o[k] = make_double4(o.x, o.y, o.z, rho);
+    pair_u[k] = make_double4(u.x, u.y, u.z, 0.0);
+    const double *L = grids[M.atom_mol[ij.x]].lo;
+    float hx, hy, hz, ex, ey, ez;
+    split_df(o.x - L[0], hx, ex);
+    split_df(o.y - L[1], hy, ey);
+    split_df(o.z - L[2], hz, ez);
+    hi[k] = make_float4(hx, hy, hz, (float)rho);
+    lo[k] = make_float4(ex, ey, ez, 0.0f);
+    u32[k] = make_float4((float)u.x, (float)u.y, (float)u.z, 0.0f);
 }
 
-int launch_pair_count(const Model &M, int *pair_count, cudaStream_t st)
+int launch_pair_geom(const Model &M, const Grid *grids, double4 *pair_o, double4 *pair_u, float4 *hi, float4 *lo,
+                     float4 *u32, cudaStream_t st)
 {
-    if (M.n_atoms <= 0) return 0;
-    k_pair_count<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, pair_count);
-    return 1;
-}
-
-// One warp per atom i: the circles with neighbours j > i, in neighbour-list order.
-__global__ void __launch_bounds__(NB_WARPS * 32) k_pair_fill(Model M, const int *__restrict__ pair_start,
-                                                            double4 *__restrict__ pair_o, double4 *__restrict__ pair_u,
-                                                            int2 *__restrict__ pair_ij)
-{
-    const int i = blockIdx.x * NB_WARPS + (threadIdx.x >> 5);
-    if (i >= M.n_atoms) return;
-    const int lane = threadIdx.x & 31;
-    const double4 ci = M.atom[i];
-    const double Ri = ci.w + M.rp;
-    int w = pair_start[i];
-    const int t1 = M.nb_start[i + 1];
-    for (int t0 = M.nb_start[i]; t0 < t1; t0 += 32) {
-        const int t = t0 + lane;
-        bool keep = false;
-        double3 o, u;
-        double rho = 0.0;
-        int j = -1;
-        if (t < t1) {
-            j = M.nb_list[t];
-            if (j > i) {
-                const double4 cj = M.atom[j];
-                keep = circle_canon(M, i, j, ci, Ri, cj, cj.w + M.rp, o, u, rho);
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-            const int k = w + __popc(m & ((1u << lane) - 1));
-            pair_o[k] = make_double4(o.x, o.y, o.z, rho);
-            pair_u[k] = make_double4(u.x, u.y, u.z, 0.0);
-            pair_ij[k] = make_int2(i, j);
-        }
-        w += __popc(m);
-    }
-}
-
-int launch_pair_fill(const Model &M, const int *pair_start, double4 *pair_o, double4 *pair_u, int2 *pair_ij,
-                      cudaStream_t st)
-{
-    if (M.n_atoms <= 0) return 0;
-    k_pair_fill<<<(M.n_atoms + NB_WARPS - 1) / NB_WARPS, NB_WARPS * 32, 0, st>>>(M, pair_start, pair_o, pair_u,
-                                                                               pair_ij);
+    if (M.n_pairs <= 0) return 0;
+    k_pair_geom<<<(M.n_pairs + 127) / 128, 128, 0, st>>>(M, grids, pair_o, pair_u, hi, lo, u32);
     return 1;
 }
 
@@ -448,8 +464,10 @@ __device__ void arcs_of_pair(const Model &M, int p, uint8_t *pair_free, int *ver
 // end point covered -- is taken in FP32 when it clears its error bound and in
 // FP64 otherwise, so the decisions are those of the FP64 form.  FP32 end
 // points carry a propagated error bound (the FP64 end point is used when that
-// bound exceeds 2e-4 A); emitted triple points are always computed in FP64.
+// bound exceeds 2e-2 A, or past 2e-4 A when its first-order form may not hold);
+// emitted triple points are always computed in FP64 (k_verts).
 constexpr int ARC_MAXN = 256;
+constexpr int ARC_CODES = 64;  // free end points of one circle listed for k_verts (more: the circle is emitted whole)
 
 // 1: d2 < t^2 certain, 0: d2 >= t^2 certain, -1 undecided (delta: error of the vector)
 __device__ __forceinline__ int arc_lt(float d2, float t, float delta)
@@ -464,16 +482,25 @@ __device__ __forceinline__ int arc_lt(float d2, float t, float delta)
 // The lanes gather the common neighbours (ballot compaction, list order;
 // circles with more than ARC_MAXN take the FP64 form on one lane), then each
 // lane takes candidates a = lane, lane + 32, ...: its cover of the circle, its
-// end points and their freeness against every other candidate.  Emitted triple points keep the order (a, end point).
+// end points and their freeness against every other candidate.  Emitted triple points keep the order (a, end point):
+// the count pass lists them (2 k + end point) for k_verts, which computes them one thread each.
+// Bound by FP64 issue wherever a lane needs an exact end point (one warp
+// instruction per 16 cycles per SM): with FP64 end points past a bound of 2e-4 A
+// about one lane in two circles took them (2.0 ms on 5,000 atoms at 0.1
+// atoms/A^3, 1.4 ms on 32 molecules at h 0.5; 0.62 and 0.52 ms now, bound by
+// issue: half the candidates of a circle cover nothing of it and are dropped
+// before the pairwise tests, each of which is two multiply-adds in the plane).
 constexpr int ARC_WARPS = 4;
+constexpr int ARC_CTAS = 8;  // resident blocks asked for: 64 registers, the FP64 fallbacks' values spilled (106: 4 blocks)
 
 struct ArcWarp {
     float4 nb[ARC_MAXN];
     int nbk[ARC_MAXN];
+    int code[ARC_CODES];
 };
 
 template <bool EMIT>
-__device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pair_free, int *vert_count,
+__device__ int arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pair_free, int *vert_count,
                                   const int *vert_start, double4 *vert)
 {
     const unsigned full_mask = 0xffffffffu;
@@ -527,20 +554,33 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
     }
     __syncwarp();
     if (n > ARC_MAXN) {  // very crowded circle: the FP64 form, one lane
-        if (lane == 0) arcs_of_pair<EMIT>(M, p, pair_free, vert_count, vert_start, vert);
-        __syncwarp();
-        return;
+        int listed = 0;
+        if (lane == 0) {
+            arcs_of_pair<EMIT>(M, p, pair_free, vert_count, vert_start, vert);
+            if (!EMIT && vert_count[p] > 0) listed = ARC_CODES + 1;  // emitted whole
+        }
+        return __shfl_sync(full_mask, listed, 0);
     }
     CircleFrame f;
     bool have64 = false;
     // 2. a candidate that covers the whole circle ends the work before any
     //    end point is tested (at protein packing most circles are buried
     //    this way): the same cover decisions as below, FP64 when undecided
+    //    Each candidate is left in the circle's plane: its centre (d1, d2), num
+    //    = rho^2 + |d|^2 - R^2 (a circle point q is covered iff 2 q.d > num)
+    //    and the error bound en + ed of either side.
+    //    A candidate that certainly covers nothing of the circle is dropped:
+    //    it covers no end point either.
     bool full = false;
-    for (int r = 0; r * 32 < n && !full; ++r) {
+    float amax = 0.0f, emax = 0.0f;  // the lanes' largest |(d1, d2)| and error bound
+    const int n_common = n;
+    n = 0;
+    for (int r = 0; r * 32 < n_common && !full; ++r) {
         const int a = r * 32 + lane;
-        bool whole = false;
-        if (a < n) {
+        bool whole = false, keep = false;
+        float4 flat = make_float4(0.f, 0.f, 0.f, 0.f);
+        int ka = 0;
+        if (a < n_common) {
             const float4 c = W.nb[a];
             const float d1 = c.x * v1x + c.y * v1y + c.z * v1z;
             const float d2 = c.x * v2x + c.y * v2y + c.z * v2z;
@@ -551,6 +591,13 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
             const float en = 2.0f * dk * dlt + 2e-6f * (rho * rho + dd + c.w * c.w);
             const float ed = 2.0f * rho * (dlt + 3e-7f * dk) + 2e-6f * den;
             const float err = 2.0f * (en + ed);
+            keep = num < den + err;
+            flat = make_float4(d1, d2, num, en + ed);
+            ka = W.nbk[a];
+            if (keep) {
+                amax = fmaxf(amax, A);
+                emax = fmaxf(emax, en + ed);
+            }
             if (num < -den - err) {
                 whole = true;
             } else if (num < -den + err) {  // undecided near a whole cover: FP64
@@ -558,22 +605,39 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
                     f = frame_of(M.pair_o[p], M.pair_u[p]);
                     have64 = true;
                 }
-                const double4 ck = M.atom[W.nbk[a]];
+                const double4 ck = M.atom[ka];
                 double3 qa, qb;
                 whole = cover_of(f, ck, ck.w + M.rp, qa, qb) == 2;
             }
         }
         full = __any_sync(full_mask, whole);
+        // (places at or below the ones just read: the votes stand between reads and writes)
+        const unsigned m = __ballot_sync(full_mask, keep);
+        if (keep) {
+            const int at = n + __popc(m & ((1u << lane) - 1));
+            W.nb[at] = flat;
+            W.nbk[at] = ka;
+        }
+        n += __popc(m);
+        __syncwarp();
     }
     if (full) {
         if (!EMIT && lane == 0) {
             pair_free[p] = 0;
             vert_count[p] = 0;
         }
-        __syncwarp();
-        return;
+        return 0;
     }
-    // 3. candidates a = lane + 32 r: covers, end points and their freeness
+    for (int o = 16; o > 0; o >>= 1) {
+        amax = fmaxf(amax, __shfl_xor_sync(full_mask, amax, o));
+        emax = fmaxf(emax, __shfl_xor_sync(full_mask, emax, o));
+    }
+    __syncwarp();
+    // 3. candidates a = lane + 32 r: covers, end points and their freeness.  An
+    //    end point q (in the plane) is tested against every other candidate with
+    //    two multiply-adds and one bound for all of them: 2 q.d - num against
+    //    2 |dq| max |d| + 2 max(en + ed).  Only an end point that no candidate
+    //    covers for certain and some could is taken to FP64.
     int n_partial = 0, n_free_end = 0, n_emit_total = 0;
     const int w0 = EMIT ? vert_start[p] : 0;
     for (int r = 0; r * 32 < n; ++r) {
@@ -584,16 +648,9 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
         bool e64 = false;
         if (a < n) {
             const float4 c = W.nb[a];
-            const float d1 = c.x * v1x + c.y * v1y + c.z * v1z;
-            const float d2 = c.x * v2x + c.y * v2y + c.z * v2z;
-            const float dd = c.x * c.x + c.y * c.y + c.z * c.z;
-            const float A = sqrtf(d1 * d1 + d2 * d2);
-            const float num = rho * rho + dd - c.w * c.w, den = 2.0f * rho * A;
-            const float dk = sqrtf(dd);
-            const float en = 2.0f * dk * dlt + 2e-6f * (rho * rho + dd + c.w * c.w);
-            const float ed = 2.0f * rho * (dlt + 3e-7f * dk) + 2e-6f * den;
-            const float err = 2.0f * (en + ed);
-            float qf[2][3];
+            const float A = sqrtf(c.x * c.x + c.y * c.y);
+            const float num = c.z, den = 2.0f * rho * A, err = 2.0f * c.w;
+            float q1[2] = {0.0f, 0.0f}, q2[2] = {0.0f, 0.0f};
             float dq = 1.0f;
             if (num >= den + err) {
                 status = 0;
@@ -604,21 +661,21 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
                 if (num < den - err && num > -den + err) {  // partial for certain: FP32 end points
                     const float T = num / den;
                     const float sT = sqrtf(fmaxf(0.0f, 1.0f - T * T));
-                    const float iA = 1.0f / A;
-                    const float epx = (d1 * v1x + d2 * v2x) * iA, epy = (d1 * v1y + d2 * v2y) * iA,
-                                epz = (d1 * v1z + d2 * v2z) * iA;
-                    const float enx = uy * epz - uz * epy, eny = uz * epx - ux * epz, enz = ux * epy - uy * epx;
+                    const float iA = 1.0f / A, e1 = c.x * iA, e2 = c.y * iA;
                     for (int e = 0; e < 2; ++e) {
-                        const float sg = e == 0 ? 1.0f : -1.0f;
-                        qf[e][0] = rho * (T * epx + sg * sT * enx);
-                        qf[e][1] = rho * (T * epy + sg * sT * eny);
-                        qf[e][2] = rho * (T * epz + sg * sT * enz);
+                        const float sg = e == 0 ? sT : -sT;
+                        q1[e] = rho * (T * e1 - sg * e2);
+                        q2[e] = rho * (T * e2 + sg * e1);
                     }
-                    const float dT = (en + fabsf(T) * ed) / den;
+                    // (c.w bounds num's error and den's together, so also |T| of den's)
+                    const float dT = c.w / den;
                     dq = rho * (dT * (1.0f + fabsf(T) / fmaxf(sT, 1e-6f)) + 2.0f * (dlt / fmaxf(A, 1e-6f) + 3e-7f)) +
                          1e-6f;
+                    // past 2e-4 A the bound still holds to a tenth while dT << sT^2 (the second-order part of
+                    // the end point's shift is dT / (2 sT^2) of the first-order one)
+                    if (dq > 2e-4f) dq = dT < 0.05f * sT * sT && dq < 1.8e-2f ? 1.1f * dq : 1.0f;
                 }
-                if (dq > 2e-4f) {  // undecided cover or loose FP32 end points: FP64
+                if (dq > 2e-2f) {  // undecided cover or loose FP32 end points: FP64
                     if (!have64) {
                         f = frame_of(M.pair_o[p], M.pair_u[p]);
                         have64 = true;
@@ -628,41 +685,50 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
                     status = cov;
                     if (cov == 1) {
                         for (int e = 0; e < 2; ++e) {
-                            qf[e][0] = (float)(qe[e].x - f.o.x);
-                            qf[e][1] = (float)(qe[e].y - f.o.y);
-                            qf[e][2] = (float)(qe[e].z - f.o.z);
+                            const float qx = (float)(qe[e].x - f.o.x), qy = (float)(qe[e].y - f.o.y),
+                                        qz = (float)(qe[e].z - f.o.z);
+                            q1[e] = qx * v1x + qy * v1y + qz * v1z;
+                            q2[e] = qx * v2x + qy * v2y + qz * v2z;
                         }
-                        dq = 1e-6f;
+                        dq = 1e-6f + 1e-6f * rho;
                         e64 = true;
                     }
                 }
             }
             if (status == 1) {
+                const float E = 2.0f * (dq * amax + emax);
+                bool cov0 = false, cov1 = false, und0 = false, und1 = false;
+                const float x0 = 2.0f * q1[0], y0 = 2.0f * q2[0], x1 = 2.0f * q1[1], y1 = 2.0f * q2[1];
+                for (int b = 0; b < n && !(cov0 && cov1); ++b) {
+                    const float4 cb = W.nb[b];
+                    const float g0 = fmaf(x0, cb.x, fmaf(y0, cb.y, -cb.z)), g1 = fmaf(x1, cb.x, fmaf(y1, cb.y, -cb.z));
+                    if (b == a) continue;
+                    cov0 = cov0 || g0 > E;
+                    cov1 = cov1 || g1 > E;
+                    und0 = und0 || g0 >= -E;
+                    und1 = und1 || g1 >= -E;
+                }
+                fr[0] = !cov0;
+                fr[1] = !cov1;
                 for (int e = 0; e < 2; ++e) {
-                    bool free_ = true;
-                    for (int b = 0; b < n && free_; ++b) {
-                        if (b == a) continue;
-                        const float4 cb = W.nb[b];
-                        const float ex = qf[e][0] - cb.x, ey = qf[e][1] - cb.y, ez = qf[e][2] - cb.z;
-                        int t = arc_lt(ex * ex + ey * ey + ez * ez, cb.w, dq + dlt);
-                        if (t < 0) {  // FP64: the exact end point against the exact ball
-                            if (!e64) {
-                                if (!have64) {
-                                    f = frame_of(M.pair_o[p], M.pair_u[p]);
-                                    have64 = true;
-                                }
-                                const double4 ck = M.atom[W.nbk[a]];
-                                cover_of(f, ck, ck.w + M.rp, qe[0], qe[1]);
-                                e64 = true;
-                            }
-                            const double4 c64 = M.atom[W.nbk[b]];
-                            const double Rb = c64.w + M.rp;
-                            const double gx = qe[e].x - c64.x, gy = qe[e].y - c64.y, gz = qe[e].z - c64.z;
-                            t = (gx * gx + gy * gy + gz * gz < Rb * Rb) ? 1 : 0;
+                    if (!(fr[e] && (e == 0 ? und0 : und1))) continue;
+                    if (!e64) {  // the exact end point against the exact balls that could cover it
+                        if (!have64) {
+                            f = frame_of(M.pair_o[p], M.pair_u[p]);
+                            have64 = true;
                         }
-                        if (t == 1) free_ = false;
+                        const double4 ck = M.atom[W.nbk[a]];
+                        cover_of(f, ck, ck.w + M.rp, qe[0], qe[1]);
+                        e64 = true;
                     }
-                    fr[e] = free_;
+                    for (int b = 0; b < n && fr[e]; ++b) {
+                        const float4 cb = W.nb[b];
+                        if (b == a || 2.0f * (q1[e] * cb.x + q2[e] * cb.y) - cb.z < -1.5f * E) continue;
+                        const double4 c64 = M.atom[W.nbk[b]];
+                        const double Rb = c64.w + M.rp;
+                        const double gx = qe[e].x - c64.x, gy = qe[e].y - c64.y, gz = qe[e].z - c64.z;
+                        if (gx * gx + gy * gy + gz * gz < Rb * Rb) fr[e] = false;
+                    }
                 }
             }
         }
@@ -680,6 +746,14 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
             if (lane >= o) inc += u;
         }
         const int tot = __shfl_sync(full_mask, inc, 31);
+        if (!EMIT && ne_ > 0) {
+            int at = n_emit_total + inc - ne_;
+            for (int e = 0; e < 2; ++e)
+                if (fr[e]) {
+                    if (at < ARC_CODES) W.code[at] = 2 * W.nbk[a] + e;
+                    ++at;
+                }
+        }
         if (EMIT && ne_ > 0) {
             if (!e64) {
                 if (!have64) {
@@ -708,53 +782,94 @@ __device__ void arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pa
         vert_count[p] = full ? 0 : n_emit_total;
     }
     __syncwarp();
+    return full ? 0 : n_emit_total;
 }
 
-__global__ void __launch_bounds__(ARC_WARPS * 32) k_arcs(Model M, uint8_t *__restrict__ pair_free,
-                                                         int *__restrict__ vert_count)
-{
-    __shared__ ArcWarp W[ARC_WARPS];
-    const int warp = threadIdx.x >> 5;
-    const int p = blockIdx.x * ARC_WARPS + warp;
-    if (p >= M.n_pairs) return;  // uniform per warp
-    arcs_of_pair_warp<false>(M, p, W[warp], pair_free, vert_count, nullptr, nullptr);
-}
-
-// emits the free triple points of circle p (xyz, third atom in w), their
-// molecule and their three atoms (i, j of the circle, k; sorted indices)
-__global__ void __launch_bounds__(ARC_WARPS * 32) k_arcs_emit(Model M, const int *__restrict__ vert_start,
-                                                              double4 *__restrict__ vert, int *__restrict__ vert_mol,
-                                                              int4 *__restrict__ vert_atoms)
+// Free end points to emit, listed while their circle is at hand: entry (circle,
+// third atom, end point, place among the circle's).  A circle with more than
+// ARC_CODES, or whose run does not fit the list, goes to `whole`.
+__global__ void __launch_bounds__(ARC_WARPS * 32, ARC_CTAS) k_arcs(Model M, uint8_t *__restrict__ pair_free,
+                                                         int *__restrict__ vert_count, ArcList L)
 {
     __shared__ ArcWarp W[ARC_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = blockIdx.x * ARC_WARPS + warp;
-    if (p >= M.n_pairs) return;
-    if (vert_start[p + 1] == vert_start[p]) return;
-    arcs_of_pair_warp<true>(M, p, W[warp], nullptr, nullptr, vert_start, vert);
-    __syncwarp();
-    const int2 ij = M.pair_ij[p];
+    if (p >= M.n_pairs) return;  // uniform per warp
+    const int n = arcs_of_pair_warp<false>(M, p, W[warp], pair_free, vert_count, nullptr, nullptr);
+    if (n == 0) return;
+    int off = L.cap;
+    if (lane == 0 && n <= ARC_CODES) off = atomicAdd(L.n, n);
+    off = __shfl_sync(0xffffffffu, off, 0);
+    const bool fits = n <= ARC_CODES && off >= 0 && off <= L.cap - n;
+    if (!fits && lane == 0) L.whole[atomicAdd(L.n + 1, 1)] = p;
+    for (int k = lane; k < n && off >= 0 && off + k < L.cap; k += 32)  // (a slot no run fills is dead)
+        L.e[off + k] = fits ? make_int4(p, W[warp].code[k] >> 1, W[warp].code[k] & 1, k) : make_int4(-1, 0, 0, 0);
+}
+
+// one triple point's molecule, atoms and FP32 copies
+__device__ __forceinline__ void vert_out(const Model &M, const VertOut &O, const double4 &v, int2 ij, int at)
+{
     const int mol = M.atom_mol[ij.x];
-    for (int k = vert_start[p] + lane; k < vert_start[p + 1]; k += 32) {
-        vert_mol[k] = mol;
-        vert_atoms[k] = make_int4(ij.x, ij.y, (int)vert[k].w, 0);
+    O.mol[at] = mol;
+    O.atoms[at] = make_int4(ij.x, ij.y, (int)v.w, 0);
+    const double *L = O.grids[mol].lo;
+    float hx, hy, hz, ex, ey, ez;
+    split_df(v.x - L[0], hx, ex);
+    split_df(v.y - L[1], hy, ey);
+    split_df(v.z - L[2], hz, ez);
+    O.hi[at] = make_float4(hx, hy, hz, 0.0f);
+    O.lo[at] = make_float4(ex, ey, ez, 0.0f);
+}
+
+// The listed triple points in FP64, one thread each (full warps of FP64 work;
+// a warp per circle with a lane or two in FP64 took 0.77 ms for 64,000 points).
+__global__ void __launch_bounds__(128) k_verts(Model M, const int *__restrict__ vert_start, ArcList L, VertOut O)
+{
+    const int n = min(*L.n, L.cap);
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+        const int4 e = L.e[q];
+        if (e.x < 0) continue;
+        const CircleFrame f = frame_of(M.pair_o[e.x], M.pair_u[e.x]);
+        const double4 ck = M.atom[e.y];
+        double3 qe[2];
+        cover_of(f, ck, ck.w + M.rp, qe[0], qe[1]);
+        const double3 x = e.z ? qe[1] : qe[0];
+        const int at = vert_start[e.x] + e.w;
+        const double4 v = make_double4(x.x, x.y, x.z, (double)e.y);
+        O.vert[at] = v;
+        vert_out(M, O, v, M.pair_ij[e.x], at);
     }
 }
 
-int launch_arcs(const Model &M, uint8_t *pair_free, int *vert_count, cudaStream_t st)
+// the circles that were not listed: a warp each emits its triple points
+__global__ void __launch_bounds__(ARC_WARPS * 32) k_arcs_emit(Model M, const int *__restrict__ vert_start, ArcList L,
+                                                              VertOut O)
+{
+    __shared__ ArcWarp W[ARC_WARPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n = L.n[1];
+    for (int q = blockIdx.x * ARC_WARPS + warp; q < n; q += gridDim.x * ARC_WARPS) {
+        const int p = L.whole[q];
+        arcs_of_pair_warp<true>(M, p, W[warp], nullptr, nullptr, vert_start, O.vert);
+        __syncwarp();
+        for (int k = vert_start[p] + lane; k < vert_start[p + 1]; k += 32) vert_out(M, O, O.vert[k], M.pair_ij[p], k);
+        __syncwarp();
+    }
+}
+
+int launch_arcs(const Model &M, uint8_t *pair_free, int *vert_count, const ArcList &L, cudaStream_t st)
 {
     if (M.n_pairs <= 0) return 0;
-    k_arcs<<<(M.n_pairs + ARC_WARPS - 1) / ARC_WARPS, ARC_WARPS * 32, 0, st>>>(M, pair_free, vert_count);
+    k_arcs<<<(M.n_pairs + ARC_WARPS - 1) / ARC_WARPS, ARC_WARPS * 32, 0, st>>>(M, pair_free, vert_count, L);
     return 1;
 }
 
-int launch_arcs_emit(const Model &M, const int *vert_start, double4 *vert, int *vert_mol, int4 *vert_atoms,
-                     cudaStream_t st)
+int launch_arcs_emit(const Model &M, const int *vert_start, const ArcList &L, const VertOut &O, cudaStream_t st)
 {
-    if (M.n_pairs <= 0) return 0;
-    k_arcs_emit<<<(M.n_pairs + ARC_WARPS - 1) / ARC_WARPS, ARC_WARPS * 32, 0, st>>>(M, vert_start, vert, vert_mol,
-                                                                                  vert_atoms);
-    return 1;
+    if (M.n_verts <= 0) return 0;
+    k_verts<<<(M.n_verts + 127) / 128, 128, 0, st>>>(M, vert_start, L, O);
+    k_arcs_emit<<<std::min(64, (M.n_pairs + ARC_WARPS - 1) / ARC_WARPS), ARC_WARPS * 32, 0, st>>>(M, vert_start, L, O);
+    return 2;
 }
 
 __global__ void k_faces_init(int n, const int *__restrict__ circle_count, const uint8_t *__restrict__ contained,
@@ -820,67 +935,6 @@ __global__ void k_bin_scatter(int n, const int *__restrict__ item_cell, const in
     int id = item_cell[p];
     if (id < 0) return;
     list[start[id] + atomicAdd(&cursor[id], 1)] = p;
-}
-
-__global__ void k_f32_atoms(Model M, const Grid *__restrict__ grids, float4 *__restrict__ hi, float4 *__restrict__ lo)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= M.n_atoms) return;
-    const double *L = grids[M.atom_mol[k]].lo;
-    const double lx = L[0], ly = L[1], lz = L[2];
-    float hx, hy, hz, ex, ey, ez;
-    double4 a = M.atom[k];
-    split_df(a.x - lx, hx, ex);
-    split_df(a.y - ly, hy, ey);
-    split_df(a.z - lz, hz, ez);
-    hi[k] = make_float4(hx, hy, hz, (float)a.w);
-    lo[k] = make_float4(ex, ey, ez, 0.0f);
-}
-
-__global__ void k_f32_pairs(Model M, const Grid *__restrict__ grids, float4 *__restrict__ hi, float4 *__restrict__ lo,
-                            float4 *__restrict__ u32)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= M.n_pairs) return;
-    const double *L = grids[M.atom_mol[M.pair_ij[k].x]].lo;
-    const double lx = L[0], ly = L[1], lz = L[2];
-    float hx, hy, hz, ex, ey, ez;
-    double4 o = M.pair_o[k];
-    double4 u = M.pair_u[k];
-    split_df(o.x - lx, hx, ex);
-    split_df(o.y - ly, hy, ey);
-    split_df(o.z - lz, hz, ez);
-    hi[k] = make_float4(hx, hy, hz, (float)o.w);
-    lo[k] = make_float4(ex, ey, ez, 0.0f);
-    u32[k] = make_float4((float)u.x, (float)u.y, (float)u.z, 0.0f);
-}
-
-__global__ void k_f32_verts(Model M, const Grid *__restrict__ grids, float4 *__restrict__ hi, float4 *__restrict__ lo)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= M.n_verts) return;
-    const double *L = grids[M.vert_mol[k]].lo;
-    const double lx = L[0], ly = L[1], lz = L[2];
-    float hx, hy, hz, ex, ey, ez;
-    double4 v = M.vert[k];
-    split_df(v.x - lx, hx, ex);
-    split_df(v.y - ly, hy, ey);
-    split_df(v.z - lz, hz, ez);
-    hi[k] = make_float4(hx, hy, hz, 0.0f);
-    lo[k] = make_float4(ex, ey, ez, 0.0f);
-}
-
-// which: 0 atoms, 1 circles (centre and axis), 2 triple points; relative to
-// the grid origin of each item's molecule
-int launch_model_f32(const Model &M, int which, const Grid *grids, float4 *hi, float4 *lo_, float4 *u32,
-                     cudaStream_t st)
-{
-    int n = which == 0 ? M.n_atoms : (which == 1 ? M.n_pairs : M.n_verts);
-    if (n <= 0) return 0;
-    if (which == 0) k_f32_atoms<<<(n + 255) / 256, 256, 0, st>>>(M, grids, hi, lo_);
-    else if (which == 1) k_f32_pairs<<<(n + 255) / 256, 256, 0, st>>>(M, grids, hi, lo_, u32);
-    else k_f32_verts<<<(n + 255) / 256, 256, 0, st>>>(M, grids, hi, lo_);
-    return 1;
 }
 
 int launch_bin_count(const Model &M, int which, bool cull, int *count, int *item_cell, cudaStream_t st)

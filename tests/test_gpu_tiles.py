@@ -62,3 +62,35 @@ def test_noalloc_rows_at_every_alignment(dims, shift):
         assert counts[a] == len(ref[a])
         got = outs[a].cpu().numpy()
         assert np.array_equal(got[:-1], ref[a]) and got[-1] == -1, a
+
+
+def test_circle_with_many_free_end_points():
+    """Two large balls whose circle carries 35 small ones, none touching the
+    next: 70 free triple points on one circle, more than the arc kernel lists
+    for one thread each, so the circle is emitted whole by a warp."""
+    libbuild.build()
+    rho = np.sqrt((30.0 + 1.4) ** 2 - 10.0 ** 2)
+    phi = 2.0 * np.pi * np.arange(35) / 35
+    ring = np.stack([np.zeros(35), rho * np.cos(phi), rho * np.sin(phi)], 1)
+    xyz = np.concatenate([[[-10.0, 0.0, 0.0], [10.0, 0.0, 0.0]], ring])
+    rad = np.concatenate([[30.0, 30.0], np.full(35, 0.5)])
+    ref = oracle.run(xyz, rad, 1.4, 1.5, 1.6)
+    ctx = eses.eses_create(xyz, rad, 1.4, 1.5, 1.6)
+    try:
+        eses.eses_set_option(ctx, eses.ESES_OPT_GRAPH, 1)
+        for _ in range(3):  # planned, captured, replayed
+            eses.eses_run(ctx)
+            patch = eses.eses_patch_data(ctx)
+            v = patch["vertices"]
+            # every triple point on both large spheres and on one small one
+            d = np.linalg.norm(v[:, None, :] - xyz[None], axis=2) - (rad + 1.4)
+            assert np.abs(d[:, :2]).max() < 1e-9 and np.abs(d[:, 2:]).min(1).max() < 1e-9
+            assert len(v) == 70
+            assert np.array_equal(eses.eses_labels(ctx), ref.labels)
+            for a in range(3):
+                g = eses.eses_intersections(ctx, a)
+                o = np.argsort(g["idx"])
+                assert np.array_equal(g["idx"][o], ref.idx[a])
+                assert np.abs(g["tau"][o] - ref.tau[a]).max() * 1.5 < 1e-6
+    finally:
+        eses.eses_destroy(ctx)
