@@ -32,7 +32,9 @@
 //   k_edge_pick: one thread per edge: the first root when the end point is
 //     inside or one candidate is left and the FP32 bounds order the
 //     candidates; the other edges are listed;
-//   k_edge_hard: one warp per listed edge: near ties broken on FP64 roots; at
+//   k_edge_settle: one thread per listed edge: the outside end points that the
+//     candidates' own witnesses decide;
+//   k_edge_hard: one warp per edge left: near ties broken on FP64 roots; at
 //     an outside end point each earlier candidate tested first against the
 //     later candidates' witnesses, then by the full witness search, whose
 //     undecided items are re-tested in FP64.
@@ -731,26 +733,38 @@ __device__ __noinline__ void torus_piece_exact(const Acc &X, RootSink &out, int 
     for (int k = 0; k < n; ++k) torus_root_exact(X, out, pi, s64, axis, h, rp, inside, r64[k]);
 }
 
-// Can item `it` (staged atom, vertex or pair, in that order) put a root on the
-// edge from s along axis?  Spheres |y - c| = rad: only if the distance from c
-// to the segment takes the value rad (its minimum and maximum over the
-// segment bracket rad); tori: the 1-Lipschitz distance to the circle is
-// within h/2 of r_p at the edge's midpoint.  mg widens both for FP32.
+// Can item `it` (staged atom, vertex or pair, in that order) put an accepted
+// root on the edge from s along axis (`inside`: the label at s)?
+// Spheres |y - c| = rad: the segment comes within rad of c, and its far end
+// (for a root where the line leaves the ball) or near end (where it enters)
+// is not inside the ball.  The line must leave a van der Waals ball and enter
+// a probe ball after an inside end, the other way round after an outside one;
+// an atom whose expanded sphere keeps no free face has no free witness.
+// Tori, D the distance to the circle along the edge, g = D - r_p: D is
+// 1-Lipschitz, so |g| at the midpoint is at most h/2; and where the circle and
+// its axis stay away (|g''| <= C = 1 / min(D, |w|) over the edge) |g| is at
+// most |g'| h/2 + C h^2/8, and g' keeps its sign when |g'| > C h/2, which must
+// be falling after an inside end, rising after an outside one.
+// mg widens every test for FP32.  (The Lipschitz test alone, and spheres by
+// their distance range only, left 1.50 M sphere and 4.31 M torus candidates on
+// 1.14 M edges of the 5,000-atom globule; see k_roots_torus.)
 template <class T, class CP>
-__device__ __forceinline__ bool cand_test(const TileS<T, CP> &S, const T *s, int axis, int it, T hT, T rpT, T mg)
+__device__ __forceinline__ bool cand_test(const TileS<T, CP> &S, const T *s, int axis, bool inside, int it, T hT, T rpT,
+                                          T mg)
 {
     const int na = S.na, nv = S.nv;
     if (it < na + nv) {
-        const P4<T> c = it < na ? S.atom[it] : S.vq[it - na];
-        const T rad = it < na ? c.w : rpT;
+        const bool vdw = it < na;
+        const P4<T> c = vdw ? S.atom[it] : S.vq[it - na];
+        const T rad = vdw ? c.w : rpT;
         const T d0 = s[0] - c.x, d1 = s[1] - c.y, d2 = s[2] - c.z;
         const T dd = d0 * d0 + d1 * d1 + d2 * d2;
         const T da = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
         const T tc = fmin(fmax(-da, T(0)), hT);         // nearest point of the segment
         const T dmin2 = dd + tc * (tc + T(2) * da);
-        const T dmax2 = dd + fmax(T(0), hT * (hT + T(2) * da));
+        const T end2 = vdw == inside ? dd + hT * (hT + T(2) * da) : dd;
         const T rhi = rad + mg, rlo = fmax(rad - mg, T(0));
-        return dmin2 <= rhi * rhi && dmax2 >= rlo * rlo;
+        return dmin2 <= rhi * rhi && end2 >= rlo * rlo && (!vdw || S.aface[it] != 0);
     }
     const int pi = it - na - nv;
     const P4<T> o = S.po[pi];
@@ -759,9 +773,16 @@ __device__ __forceinline__ bool cand_test(const TileS<T, CP> &S, const T *s, int
     m[axis] += T(0.5) * hT;
     const T zc = m[0] * u.x + m[1] * u.y + m[2] * u.z;
     const T w2 = fmax(m[0] * m[0] + m[1] * m[1] + m[2] * m[2] - zc * zc, T(0));
-    const T e1 = sqrt(w2) - o.w;
-    const T gm = sqrt(e1 * e1 + zc * zc) - rpT;
-    return fabs(gm) <= T(0.5) * hT + mg;
+    const T nw = sqrt(w2), e1 = nw - o.w;
+    const T D = sqrt(e1 * e1 + zc * zc), gm = fabs(D - rpT), half = T(0.5) * hT + mg;
+    if (gm > half) return false;
+    const T low = fmin(D, nw) - half;
+    if (low < T(0.1)) return true;
+    const T ua = axis == 0 ? u.x : (axis == 1 ? u.y : u.z);
+    const T bend = half / low;  // C h/2: g' moves by at most this over the edge
+    const T dg = (e1 * (m[axis] - zc * ua) / nw + zc * ua) / D;
+    if (gm > fabs(dg) * half + T(0.5) * bend * half + mg + T(1e-9)) return false;
+    return !((inside ? dg : -dg) > bend + T(1e-2));
 }
 
 // Roots of one (edge, piece) candidate that can be the surface on that edge:
@@ -1320,7 +1341,7 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
             int cs = 0, ct = 0;
             for (int i0 = 0; i0 < nitem; i0 += 32) {
                 const int it = i0 + lane;
-                const bool hit = it < nitem && cand_test<T, CP>(S, s, R.axis, it, hT, rpT, mg);
+                const bool hit = it < nitem && cand_test<T, CP>(S, s, R.axis, R.lab == LABEL_IN, it, hT, rpT, mg);
                 const unsigned m = __ballot_sync(0xffffffffu, hit), sm = sphere_bits(i0 >> 5, nsph);
                 cs += __popc(m & sm);
                 ct += __popc(m & ~sm);
@@ -1442,7 +1463,7 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
                     const int it = i0 + lane;
                     const unsigned m =
                         keep ? E.hmask[e * nwd + (i0 >> 5)]
-                             : __ballot_sync(0xffffffffu, it < nitem && cand_test<T, CP>(S, s, R.axis, it, hT, rpT, mg));
+                             : __ballot_sync(0xffffffffu, it < nitem && cand_test<T, CP>(S, s, R.axis, R.lab == LABEL_IN, it, hT, rpT, mg));
                     const bool hit = (m >> lane) & 1u;
                     const unsigned sm = sphere_bits(i0 >> 5, nsph), ms = m & sm, mt = m & ~sm;
                     const long long qs = ps + __popc(ms & below), qt = pt + __popc(mt & below);
@@ -1778,7 +1799,154 @@ __global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Batch B, RootWork W,
     }
 }
 
-// 5. The listed edges: one warp per edge (grid-stride over the list).  The
+// 4b. FP32 form only: the listed edges that the targeted test settles, one
+// thread each.  At an outside end point the candidates go in order of t; one
+// whose point is closer than r_p to the free witness of another remaining
+// candidate is strictly outside M and dropped, and the last one left is the
+// root -- warp_select's first test with its tolerances, so an edge takes the
+// same candidate on either path.  A tie that the FP32 bounds cannot order, a
+// test that is not certain, an inside end point or more than SETTLE_MAX
+// candidates leave the edge to the warp selection (W.hard2).
+// On the 5,000-atom globule 388 k of the warps' 653 k iterations were this
+// test, 545 warp instructions for one lane's work each.
+constexpr int SETTLE_MAX = 6;
+constexpr int SETTLE_THREADS = 128;
+
+__global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B, RootWork W,
+                                                                const int *__restrict__ edge_start, EdgeOut out)
+{
+    const long long nt = B.n_tiles;
+    const int lane = threadIdx.x & 31;
+    const long long nh = (long long)W.ctr[3], stride = (long long)gridDim.x * SETTLE_THREADS;
+    const float rp = (float)M.rp;
+    for (long long q0 = (long long)blockIdx.x * SETTLE_THREADS + (threadIdx.x & ~31); q0 < nh; q0 += stride) {
+        const long long q = q0 + lane;
+        bool left = false;
+        int g = 0;
+        if (q < nh) {
+            g = W.hard[q];
+            const int4 inf = W.einfo[g];
+            const int cnt = W.ecnt[g];
+            const int ns = cnt & 0xffff, nq = (cnt >> 16) & 0xffff;
+            const int pk = inf.y, axis = pk_axis(pk), lab = pk_label(pk), p = pk_point(pk);
+            left = true;
+            if (!pk_dropped(pk) && lab != LABEL_IN) {
+                const unsigned char *sl = W.slab + ((size_t)(unsigned)inf.x << 4);
+                const SlabHdr *hd = reinterpret_cast<const SlabHdr *>(sl);
+                const Grid &G = B.grid[__ldg(&hd->mol)];
+                float s[3], hT;
+                edge_point<float>(G, p, s, hT);
+                const float d0 = G.d0, tie = 1e-6f * hT;
+                const SlabAcc<float> A(sl);
+                const int na = A.na();
+                // the candidates: root, error bound, best position on the edge and what it adds to d0, piece
+                float t[SETTLE_MAX], err[SETTLE_MAX], tp[SETTLE_MAX], dp[SETTLE_MAX];
+                int kind[SETTLE_MAX], id[SETTLE_MAX];
+                int n = 0;
+                for (int j = 0; j < ns + nq; ++j) {
+                    const bool sph = j < ns;
+                    const int k = sph ? inf.z + j : inf.w + (j - ns);
+                    const int nr = sph ? W.nsph[k] : W.ntor[k];
+                    for (int r = 0; r < nr; ++r) {
+                        const RootRec c = sph ? W.rsph[(size_t)SPH_SLOTS * k + r] : W.rtor[(size_t)TOR_SLOTS * k + r];
+                        if (!(c.t < INFINITY) || c.err < 0.0f) continue;  // rejected (or never settled)
+                        const int it = sph ? W.csph[k].y : W.ctor[k].y;
+#pragma unroll
+                        for (int z = 0; z < SETTLE_MAX; ++z)
+                            if (z == n) {
+                                t[z] = c.t;
+                                err[z] = c.err;
+                                tp[z] = c.t64 == c.t64 ? (float)c.t64 : c.t;
+                                dp[z] = c.t64 == c.t64 ? 2e-7f : c.err;
+                                kind[z] = sph ? (it < na ? 0 : 2) : 1;
+                                id[z] = sph && it >= na ? it - na : it;
+                            }
+                        ++n;
+                    }
+                }
+                unsigned alive = n >= 1 && n <= SETTLE_MAX ? (1u << n) - 1u : 0u;
+                int pick = -1;
+                while (alive) {
+                    // the first candidate left, and whether the bounds order it before the others
+                    int k = -1, kk = 0, ki = 0;
+                    float tk = INFINITY, ek = 0.0f, dk = 0.0f, yk = 0.0f;
+#pragma unroll
+                    for (int z = 0; z < SETTLE_MAX; ++z)
+                        if (((alive >> z) & 1u) && t[z] < tk) {
+                            k = z;
+                            tk = t[z];
+                            ek = err[z];
+                            yk = tp[z];
+                            dk = d0 + dp[z];
+                            kk = kind[z];
+                            ki = id[z];
+                        }
+                    if (k < 0) break;
+                    bool tied = false;
+#pragma unroll
+                    for (int z = 0; z < SETTLE_MAX; ++z)
+                        if (((alive >> z) & 1u) && z != k && t[z] - tk <= err[z] + ek + tie) tied = true;
+                    if (tied) break;
+                    const unsigned rest = alive & ~(1u << k);
+                    if (rest == 0u) {
+                        pick = k;
+                        break;
+                    }
+                    float y[3] = {s[0], s[1], s[2]};
+                    y[0] += axis == 0 ? yk : 0.0f;
+                    y[1] += axis == 1 ? yk : 0.0f;
+                    y[2] += axis == 2 ? yk : 0.0f;
+                    bool outside = false;
+#pragma unroll
+                    for (int z = 0; z < SETTLE_MAX; ++z) {
+                        if (!((rest >> z) & 1u) || outside || (kind[z] == kk && id[z] == ki)) continue;
+                        if (kind[z] == 2) {
+                            const P4<float> v = A.vq(id[z]);
+                            const float dx = y[0] - v.x, dy = y[1] - v.y, dz = y[2] - v.z;
+                            outside = lt_sq<true>(dx * dx + dy * dy + dz * dz, rp * rp, rp, dk) == 1;
+                            continue;
+                        }
+                        float qx, qy, qz, dq;
+                        int e0, e1, tw, sa = id[z], sb = -1;
+                        if (kind[z] == 0) {
+                            tw = face_proposal<true>(A, id[z], y[0], y[1], y[2], rp, rp, dk, qx, qy, qz, dq, e0, e1);
+                        } else {
+                            tw = saddle_proposal<true>(A, id[z], y[0], y[1], y[2], rp, rp, dk, qx, qy, qz, dq, e0, e1);
+                            const short2 ps = A.pslot(id[z]);
+                            sa = ps.x;
+                            sb = ps.y;
+                        }
+                        outside = tw == 1 && free_witness<true>(A, qx, qy, qz, sa, sb, e0, e1, rp, dq + dk) == 1;
+                    }
+                    if (!outside) break;  // not certain: the full search decides
+                    alive = rest;
+                }
+                if (pick >= 0) {
+                    left = false;
+                    float tr = 0.0f;
+                    int pkind = 0, pid = 0;
+#pragma unroll
+                    for (int z = 0; z < SETTLE_MAX; ++z)
+                        if (z == pick) {
+                            tr = tp[z];
+                            pkind = kind[z];
+                            pid = id[z];
+                        }
+                    const int o = g - edge_start[axis * nt];
+                    code_out(out, axis, o, 0, tr, pkind, A.model_index(pkind, pid), lab);
+                }
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, left);
+        int base = 0;
+        if (lane == 0 && m) base = (int)atomicAdd(W.ctr + 5, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (left) W.hard2[base + __popc(m & ((1u << lane) - 1))] = g;
+    }
+}
+
+// 5. The listed edges: one warp per edge (grid-stride over the list: in the
+// FP32 form those that 4b left).  The
 // edge's accepted roots are gathered in candidate order into the warp's
 // buffer in shared memory (at most WCAND; more is a capacity error), then
 // chosen by warp_select.  A failure is logged with its candidates.
@@ -1791,13 +1959,14 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
     __shared__ WCand cand[HARD_THREADS / 32][WCAND];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long nt = B.n_tiles;
-    const long long nh = (long long)W.ctr[3];
+    const long long nh = (long long)W.ctr[FILT ? 5 : 3];
+    const int *__restrict__ list = FILT ? W.hard2 : W.hard;
     const double rp = M.rp;
     const T rpT = (T)rp;
     WCand *c = cand[warp];
     for (long long q = (long long)blockIdx.x * (HARD_THREADS / 32) + warp; q < nh;
          q += (long long)gridDim.x * (HARD_THREADS / 32)) {
-        const int g = W.hard[q];
+        const int g = list[q];
         const int4 inf = W.einfo[g];
         const int cnt = W.ecnt[g];
         const int ns = cnt & 0xffff, nq = (cnt >> 16) & 0xffff;
@@ -1888,16 +2057,40 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
 }
 
 // One thread per crossing edge, over the three axes: FP64 root of the chosen
-// piece next to the recorded FP32 root, normal, outputs, area/volume terms
-// (block partial sums in fixed order).
+// piece next to the recorded FP32 root, normal, outputs, area/volume terms.
+// Bound by FP64 issue (one warp instruction per 16 cycles per SM).  The
+// block's edges are first ordered by kind, tori before spheres, so nearly
+// every warp runs one of the two paths instead of both, and 1 / h comes from
+// the host: 513 -> 326 us on 1.2 M edges.
 __global__ void __launch_bounds__(POLISH_THREADS) k_edge_polish(Model M, Batch B, EdgeOut out,
                                                                 const long long *__restrict__ medge,
                                                                 double2 *__restrict__ term)
 {
-    const long long e = (long long)blockIdx.x * POLISH_THREADS + threadIdx.x;
+    __shared__ short order[POLISH_THREADS];
+    __shared__ int n_tor[POLISH_THREADS / 32];
+    const long long e0 = (long long)blockIdx.x * POLISH_THREADS;
     const int nm = B.n_mol;
     const long long n0 = medge[nm], n1 = medge[2 * nm + 1], n2 = medge[3 * nm + 2];
     const double rp = M.rp;
+    {
+        const long long e = e0 + threadIdx.x;
+        const int a = e < n0 ? 0 : (e < n0 + n1 ? 1 : 2);
+        const long long o = e - (a == 0 ? 0 : (a == 1 ? n0 : n0 + n1));
+        const bool tor = e < n0 + n1 + n2 && ((out.code[a][o].y >> 29) & 3) == 1;
+        const unsigned m = __ballot_sync(0xffffffffu, tor);
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        if (lane == 0) n_tor[warp] = __popc(m);
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int w = 0; w < POLISH_THREADS / 32; ++w) {
+            if (w < warp) before += n_tor[w];
+            all += n_tor[w];
+        }
+        before += __popc(m & ((1u << lane) - 1));
+        order[tor ? before : all + (int)threadIdx.x - before] = (short)threadIdx.x;
+        __syncthreads();
+    }
+    const long long e = e0 + order[threadIdx.x];
     if (e < n0 + n1 + n2) {
         const int a = e < n0 ? 0 : (e < n0 + n1 ? 1 : 2);
         const long long o = e - (a == 0 ? 0 : (a == 1 ? n0 : n0 + n1));
@@ -1919,30 +2112,25 @@ __global__ void __launch_bounds__(POLISH_THREADS) k_edge_polish(Model M, Batch B
         // the recorded piece must exist (a kind and index out of range is treated as a failed root)
         const bool bad = kind == 3 || (kind == 0 && mid >= M.n_atoms) || (kind == 1 && mid >= M.n_pairs) ||
                          (kind == 2 && mid >= M.n_verts);
-        long long gi, gj, gk;  // full-grid point of the lower index
+        double s[3];  // full-grid point of the lower index
         if (idx < (1LL << 32) && G.full[1] * G.full[2] < (1LL << 32)) {  // 32-bit division where it fits
             const unsigned i32 = (unsigned)idx, d2 = (unsigned)G.full[2], d1 = (unsigned)G.full[1];
             const unsigned q = i32 / d2;
-            gk = i32 - q * d2;
-            gj = q % d1;
-            gi = q / d1;
+            s[0] = G.lo[0] + h * (double)(q / d1);
+            s[1] = G.lo[1] + h * (double)(q % d1);
+            s[2] = G.lo[2] + h * (double)(i32 - q * d2);
         } else {
-            gi = idx / (G.full[1] * G.full[2]);
-            gj = (idx / G.full[2]) % G.full[1];
-            gk = idx % G.full[2];
+            s[0] = G.lo[0] + h * (double)(idx / (G.full[1] * G.full[2]));
+            s[1] = G.lo[1] + h * (double)((idx / G.full[2]) % G.full[1]);
+            s[2] = G.lo[2] + h * (double)(idx % G.full[2]);
         }
-        const double s[3] = {G.lo[0] + h * (double)gi, G.lo[1] + h * (double)gj, G.lo[2] + h * (double)gk};
         double t = 0.5 * h, n[3] = {0.0, 0.0, 0.0};
         if (!failed && !bad) {
             double c[3], u[3] = {0.0, 0.0, 0.0}, rho = 0.0;
-            if (kind == 0) {
-                double4 g = M.atom[mid];
+            if (kind != 1) {
+                const double4 g = kind == 0 ? M.atom[mid] : M.vert[mid];
                 c[0] = g.x; c[1] = g.y; c[2] = g.z;
-                t = exact_root_sphere(c, g.w, s, a, (double)t32);
-            } else if (kind == 2) {
-                double4 g = M.vert[mid];
-                c[0] = g.x; c[1] = g.y; c[2] = g.z;
-                t = exact_root_sphere(c, rp, s, a, (double)t32);
+                t = exact_root_sphere(c, kind == 0 ? g.w : rp, s, a, (double)t32);
             } else {
                 double4 g = M.pair_o[mid];
                 double4 q = M.pair_u[mid];
@@ -1956,7 +2144,7 @@ __global__ void __launch_bounds__(POLISH_THREADS) k_edge_polish(Model M, Batch B
             y[a] += t;
             exact_normal(kind, c, u, rho, y, n);
         }
-        const double tau = t * (1.0 / h);
+        const double tau = t * G.ih;
         out.tau[a][o] = tau;
         out.nrm[a][3 * o + 0] = n[0];
         out.nrm[a][3 * o + 1] = n[1];
@@ -2170,13 +2358,17 @@ static void roots_launch(const Model &M, const Batch &B, int threads, EdgeOut ou
     const int gs = std::max(g_occ_roots[P][0][ts], 1) * g_edge_n_sm;
     const int gq = std::max(g_occ_roots[P][1][ts], 1) * g_edge_n_sm;
     k_roots_sphere<T, FILT><<<gs, tb, 0, st>>>(M, B, W, err);
-    cudaMemsetAsync(W.ctr + 3, 0, 2 * sizeof(unsigned long long), st);  // hard edges, FP64 jobs
+    cudaMemsetAsync(W.ctr + 3, 0, 3 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, hard edges
     k_roots_torus<T, FILT><<<gq, tb, 0, st>>>(M, B, W, err);
     if (FILT)
         k_roots_torus_exact<T, FILT><<<std::max(g_occ_exact[P], 1) * g_edge_n_sm, tb, 0, st>>>(M, B, W, err);
     const long long pb = std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, PICK_THREADS), 1),
                                              8LL * g_edge_n_sm);
     k_edge_pick<T><<<(unsigned)pb, PICK_THREADS, 0, st>>>(B, W, edge_start, ne_all, out, err);
+    if (FILT)
+        k_edge_settle<<<(unsigned)std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, 4 * SETTLE_THREADS), 1),
+                                                      8LL * g_edge_n_sm),
+                        SETTLE_THREADS, 0, st>>>(M, B, W, edge_start, out);
     k_edge_hard<T, FILT><<<std::max(g_occ_hard[P], 1) * g_edge_n_sm, HARD_THREADS, 0, st>>>(
         M, B, W, edge_start, out, n_fail, err, fail_log);
 }
@@ -2202,7 +2394,7 @@ int launch_edge_roots(const Model &M, const Batch &B, int precision, int threads
         roots_launch<double, false>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
     else
         roots_launch<float, true>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
-    return precision == 0 ? 4 : 5;
+    return precision == 0 ? 4 : 6;
 }
 
 long long polish_blocks(long long n_edges) { return n_edges > 0 ? ceil_div_ll(n_edges, POLISH_THREADS) : 0; }

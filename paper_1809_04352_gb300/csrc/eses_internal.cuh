@@ -114,7 +114,7 @@ struct Model {
 // toff = 0 and own = dims = full.
 struct Grid {
     double lo[3];                 // origin of the full grid
-    double h;
+    double h, ih;                 // spacing and 1 / h
     long long dims[3];            // points of the computed box
     long long own[3];             // owned points from the box origin
     long long full[3];            // points of the full grid (output lower indices index it)
