@@ -136,7 +136,7 @@ struct eses_ctx {
     DBuf vert_count, vert_start, vert, vert_atoms, arc_list, arc_whole;
     DBuf pbin_count, pbin_start, pbin_cursor, pbin_cell, pbin_list;
     DBuf vbin_count, vbin_start, vbin_cursor, vbin_cell, vbin_list;
-    DBuf labels, tile_band, tile_edges, edge_start, tile_inside;
+    DBuf labels, band, tile_edges, edge_start, tile_inside;
     DBuf out_idx[3], out_tau[3], out_nrm[3], out_tau32[3], out_nrm32[3], out_code[3];
     DBuf scan_tmp, misc, av, counts, red_d, red_i;  // misc: err, n_fail
     DBuf fail_log;
@@ -719,7 +719,7 @@ int run_device(eses_ctx *c)
     //    with the proposer, certified far tiles are filled first and only the
     //    others are classified
     int8_t *labels = ensure<int8_t>(c->labels, c->n_points);
-    int *tile_band = ensure<int>(c->tile_band, nt);
+    int *band = ensure<int>(c->band, (size_t)nt + 1);  // count, then the tiles with undecided points
     int *prop_counts = ensure<int>(c->prop_counts, 4);
     ck(cudaMemsetAsync(prop_counts, 0, 4 * sizeof(int), st), "memset");
     mark(c, ST_CLASSIFY);
@@ -729,8 +729,7 @@ int run_device(eses_ctx *c)
         int *pos = ensure<int>(c->need_pos, nt + 1);
         int *list = ensure<int>(c->tile_list, nt);
         nl += launch_propose(M, B, c->proposer, (const float *)c->mlp_params.p, c->z_far, labels,
-                             c->precision == ESES_PREC_FP64 ? nullptr : tile_band, need, prop_counts, d_err,
-                             c->tc_wait, st);
+                             need, prop_counts, d_err, c->tc_wait, st);
         nl += scan(c, need, pos, nt);
         nl += launch_compact(nt, need, pos, list, st);
         cq.list = list;
@@ -740,9 +739,9 @@ int run_device(eses_ctx *c)
     ck(cudaMemsetAsync(ovf, 0, sizeof(int), st), "memset");
     unsigned char *big = ensure<unsigned char>(c->big, std::max(classify_big_bytes(), edges_big_bytes()));
     nl += launch_classify(M, B, c->precision, cq, grid_of(c, c->cls, classify_ctas_per_sm(c->precision)), labels,
-                          c->precision == ESES_PREC_FP64 ? nullptr : tile_band, d_err, ovf, big, d_tests, st);
+                          c->precision == ESES_PREC_FP64 ? nullptr : band, d_err, ovf, big, d_tests, st);
     mark(c, ST_BAND);
-    if (c->precision != ESES_PREC_FP64) nl += launch_band(M, B, labels, tile_band, d_err, ovf, big, st);
+    if (c->precision != ESES_PREC_FP64) nl += launch_band(M, B, labels, band, d_err, ovf, big, st);
     c->n_cavity = 0;
     c->ext_sweeps = 0;
     if (c->exterior) {  // cavities filled: sweeps until one reaches nothing new (never under capture)
@@ -1279,7 +1278,7 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
         Batch &B = c->B;
         int *misc = (int *)c->misc.p;
         int8_t *labels = (int8_t *)c->labels.p;
-        int *tile_band = (int *)c->tile_band.p;
+        int *band = (int *)c->band.p;
         auto time_it = [&](auto &&launch) {
             launch();
             ck(cudaEventRecord(e0, st), "record");
@@ -1303,13 +1302,13 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                 float ms = time_it([&] {
                     ck(cudaMemsetAsync(c->queue.p, 0, 4 * sizeof(unsigned long long), st), "memset");
                     launch_classify(M, B, c->precision, sched_of(c, s, 0), grid_of(c, s, cls_max), labels,
-                                    c->precision == ESES_PREC_FP64 ? nullptr : tile_band, misc, (int *)c->ovf.p,
+                                    c->precision == ESES_PREC_FP64 ? nullptr : band, misc, (int *)c->ovf.p,
                                     (unsigned char *)c->big.p, nullptr, st);
                 });
                 if (ms < best_cls_ms) best_cls_ms = ms, best_cls = s;
             }
         if (c->precision != ESES_PREC_FP64)
-            launch_band(M, B, labels, tile_band, misc, (int *)c->ovf.p, (unsigned char *)c->big.p, st);
+            launch_band(M, B, labels, band, misc, (int *)c->ovf.p, (unsigned char *)c->big.p, st);
         // root solve: staging CTAs per SM x tiles per pop x root-kernel threads per block
         Shape best_edge = c->edge;
         float best_edge_ms = INFINITY;
@@ -1924,7 +1923,7 @@ void eses_destroy(eses_ctx *c)
                     &c->contained, &c->face, &c->pair_count, &c->pair_start, &c->pair_o, &c->pair_u, &c->pair_ij,
                     &c->pair_free, &c->vert_count, &c->vert_start, &c->vert, &c->vert_atoms, &c->pbin_count, &c->pbin_start,
                     &c->pbin_cursor, &c->pbin_cell, &c->pbin_list, &c->vbin_count, &c->vbin_start, &c->vbin_cursor,
-                    &c->vbin_cell, &c->vbin_list, &c->labels, &c->tile_band, &c->tile_edges, &c->edge_start,
+                    &c->vbin_cell, &c->vbin_list, &c->labels, &c->band, &c->tile_edges, &c->edge_start,
                     &c->tile_inside, &c->scan_tmp, &c->misc, &c->av, &c->counts, &c->red_d, &c->red_i, &c->fail_log,
                     &c->ovf, &c->big, &c->r_einfo, &c->r_ecnt, &c->r_csph, &c->r_ctor, &c->r_nsph, &c->r_ntor,
                     &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_hard2, &c->r_jobs, &c->atom_hi,

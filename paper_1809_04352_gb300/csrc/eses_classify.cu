@@ -25,10 +25,12 @@
 //   8.2 -> 5.0 ms at 20,000 atoms, 3.6 -> 2.2 ms on 32 molecules at h 0.5,
 //   1.30 -> 0.64 ms in FP64 on 200 atoms (single-tile queue pops included).
 //   T = double, FILT = false is the plain FP64 form; T = float, FILT = true
-//   is the filtered form, whose undecided points get LABEL_BAND and are
-//   counted per tile.
+//   is the filtered form, whose undecided points get LABEL_BAND and whose
+//   tiles with such points are listed.
 // k_band: re-labels the undecided points of the tiles that have any, in FP64:
 //   one warp per point runs the witness search over every staged item.
+#include <algorithm>
+
 #include "eses_kernels.h"
 #include "eses_tile.cuh"
 
@@ -230,7 +232,7 @@ __host__ __device__ constexpr size_t cls_bytes()
 // that too is a capacity error.
 template <class T, bool FILT, class CP, bool BIG>
 __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, TileSched Q, int8_t *__restrict__ labels_all,
-                                                          int *__restrict__ tile_band, int *__restrict__ err,
+                                                          int *__restrict__ band, int *__restrict__ err,
                                                           int *__restrict__ ovf, unsigned char *__restrict__ big,
                                                           unsigned long long *__restrict__ n_tests)
 {
@@ -284,7 +286,6 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
                 if (gi < G.dims[0] && gj < G.dims[1] && gk < G.dims[2])
                     labels[(gi * G.dims[1] + gj) * G.dims[2] + gk] = LABEL_OUT;
             }
-            if (threadIdx.x == 0 && tile_band) tile_band[gt] = 0;
             __syncthreads();
             continue;
         }
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0 && tile_band) tile_band[gt] = C.band;
+        if (threadIdx.x == 0 && band && C.band > 0) band[1 + atomicAdd(&band[0], 1)] = (int)gt;
         __syncthreads();
       }
     }
@@ -451,36 +452,26 @@ __host__ __device__ constexpr size_t band_bytes()
     return (sizeof(TileS<double, CP>) + 255) & ~(size_t)255;
 }
 
-// CapSmall: chunks of CLS_THREADS tiles, the threads pick out the tiles with
-// undecided points, then the block re-labels them one after the other.
-// CapBig (BIG): the tiles listed in ovf, staged in global memory.
+// CapSmall: the tiles that the classification listed (band[0] of them, any
+// order), a block each.  CapBig (BIG): the tiles listed in ovf, staged in
+// global memory.  Bound by the latency of a tile's FP64 staging and witness
+// search; blocks that picked the tiles out of 256-tile chunks took a chunk's
+// listed tiles one after the other (95-130 us at any size; 25-35 us now).
 template <class CP, bool BIG>
 __global__ void __launch_bounds__(CLS_THREADS) k_band(Model M, Batch B, int8_t *__restrict__ labels_all,
-                                                      const int *__restrict__ tile_band, int *__restrict__ err,
+                                                      const int *__restrict__ band, int *__restrict__ err,
                                                       int *__restrict__ ovf, unsigned char *__restrict__ big)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *store = BIG ? big + (size_t)blockIdx.x * band_bytes<CP>() : smem_raw;
     TileS<double, CP> &S = *reinterpret_cast<TileS<double, CP> *>(store);
     __shared__ Grid sG;
-    __shared__ int s_list[CLS_THREADS];
     __shared__ short s_pts[TILE_PTS];
-    __shared__ int s_n, s_np;
-    if (BIG) {
-        const int n = ovf[1];
-        for (int k = blockIdx.x; k < n; k += gridDim.x) band_tile<CP>(M, B, ovf[2 + k], labels_all, S, sG, s_pts, s_np,
-                                                                     err, ovf, true);
-        return;
-    }
-    for (long long c0 = (long long)blockIdx.x * CLS_THREADS; c0 < B.n_tiles; c0 += (long long)gridDim.x * CLS_THREADS) {
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        if (c0 + threadIdx.x < B.n_tiles && tile_band[c0 + threadIdx.x] != 0) s_list[atomicAdd(&s_n, 1)] = threadIdx.x;
-        __syncthreads();
-        const int nband = s_n;
-        for (int q = 0; q < nband; ++q)
-            band_tile<CP>(M, B, c0 + s_list[q], labels_all, S, sG, s_pts, s_np, err, ovf, false);
-    }
+    __shared__ int s_np;
+    const int *list = BIG ? ovf + 1 : band;
+    const int n = list[0];
+    for (int k = blockIdx.x; k < n; k += gridDim.x)
+        band_tile<CP>(M, B, list[1 + k], labels_all, S, sG, s_pts, s_np, err, ovf, BIG);
 }
 
 static long long g_band_grid = 1;  // resident k_band CTAs on the device
@@ -531,35 +522,35 @@ int classify_ctas_per_sm(int precision)
 // the shared-memory tier over the scheduled tiles, then the global-memory
 // tier over the tiles that overflowed it (ovf: count, then tiles)
 int launch_classify(const Model &M, const Batch &B, int precision, const TileSched &Q, int grid, int8_t *labels,
-                    int *tile_band, int *err, int *ovf, unsigned char *big, unsigned long long *n_tests,
+                    int *band, int *err, int *ovf, unsigned char *big, unsigned long long *n_tests,
                     cudaStream_t st)
 {
     if (grid < 1) grid = 1;
+    if (band) cudaMemsetAsync(band, 0, sizeof(int), st);
     cudaMemsetAsync(ovf + 1, 0, sizeof(int), st);
     TileSched QB{nullptr, 1, ovf + 2, ovf + 1};
     if (precision == 0) {
         k_classify<double, false, CapMid, false><<<grid, CLS_THREADS, cls_bytes<double, CapMid>(), st>>>(
-            M, B, Q, labels, tile_band, err, ovf, nullptr, n_tests);
-        k_classify<double, false, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, tile_band, err, ovf,
+            M, B, Q, labels, band, err, ovf, nullptr, n_tests);
+        k_classify<double, false, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
                                                                                big, n_tests);
     } else {
         k_classify<float, true, CapMid, false><<<grid, CLS_THREADS, cls_bytes<float, CapMid>(), st>>>(
-            M, B, Q, labels, tile_band, err, ovf, nullptr, n_tests);
-        k_classify<float, true, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, tile_band, err, ovf,
+            M, B, Q, labels, band, err, ovf, nullptr, n_tests);
+        k_classify<float, true, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
                                                                              big, n_tests);
     }
     return 2;
 }
 
-int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *tile_band, int *err, int *ovf,
+int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *band, int *err, int *ovf,
                 unsigned char *big, cudaStream_t st)
 {
-    const long long chunks = (B.n_tiles + CLS_THREADS - 1) / CLS_THREADS;
-    const long long grid = chunks < 1 ? 1 : (chunks < g_band_grid ? chunks : g_band_grid);
+    const long long grid = std::max(1LL, std::min(B.n_tiles, g_band_grid));
     cudaMemsetAsync(ovf + 1, 0, sizeof(int), st);
-    k_band<CapSmall, false><<<(int)grid, CLS_THREADS, band_bytes<CapSmall>(), st>>>(M, B, labels, tile_band, err, ovf,
+    k_band<CapSmall, false><<<(int)grid, CLS_THREADS, band_bytes<CapSmall>(), st>>>(M, B, labels, band, err, ovf,
                                                                                  nullptr);
-    k_band<CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, labels, tile_band, err, ovf, big);
+    k_band<CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, labels, band, err, ovf, big);
     return 2;
 }
 

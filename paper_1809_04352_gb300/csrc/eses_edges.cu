@@ -1084,51 +1084,75 @@ __device__ int warp_select(const AccT &A, const AccX &X, WCand *c, int n, const 
 
 // Per tile and axis: crossing edges (end labels differ) and inside edges (both
 // ends inside) leaving the tile's points in + direction, and the tile's inside
-// points.  One warp per tile, 16 points per lane, warp sums (no block barrier).
+// points.  One warp per tile.  Bound by the label reads: a row of 8 + 1 labels
+// is read as three aligned words (byte by byte where those would pass the
+// molecule's end) and kept as 9 bits, bit 15 set for a row on the grid; the
+// counts are then popcounts of rows against their neighbours.  Byte loads per
+// point and axis took 153 us on 38 M points (250 GB/s) and 939 us on 198 M.
 constexpr int COUNT_WARPS = 8;
 
 __global__ void __launch_bounds__(COUNT_WARPS * 32) k_edge_count(Batch B, const int8_t *__restrict__ labels_all,
                                                                 int *__restrict__ tile_edges,
                                                                 int *__restrict__ tile_inside)
 {
+    __shared__ uint16_t rows[COUNT_WARPS][81];
     const int lane = threadIdx.x & 31;
+    uint16_t *row = rows[threadIdx.x >> 5];
     const long long nt = B.n_tiles;
     const long long nw = (long long)gridDim.x * COUNT_WARPS;
     for (long long gt = (long long)blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); gt < nt; gt += nw) {
         const Grid &G = B.grid[mol_of_tile(B, gt)];
-        const long long dims[3] = {G.dims[0], G.dims[1], G.dims[2]};
-        const long long own[3] = {G.own[0], G.own[1], G.own[2]};
-        const int8_t *__restrict__ labels = labels_all + G.lab0;
-        const long long st1 = dims[2], st0 = dims[1] * dims[2];
+        const long long d0 = G.dims[0], d1 = G.dims[1], d2 = G.dims[2], np = d0 * d1 * d2;
+        const uint8_t *__restrict__ labels = reinterpret_cast<const uint8_t *>(labels_all) + G.lab0;
         int t[3];
         tile_coords(G, gt - G.tile0, t);
-        int ce[3] = {0, 0, 0}, ci[3] = {0, 0, 0}, npin = 0;
-        for (int p = lane; p < TILE_PTS; p += 32) {
-            const long long g[3] = {(long long)TILE * t[0] + (p >> 6), (long long)TILE * t[1] + ((p >> 3) & 7),
-                                    (long long)TILE * t[2] + (p & 7)};
-            if (g[0] >= own[0] || g[1] >= own[1] || g[2] >= own[2]) continue;  // not owned (or not in the grid)
-            const long long idx = g[0] * st0 + g[1] * st1 + g[2];
-            const int l0 = labels[idx];
-            npin += l0;
-            const long long str[3] = {st0, st1, 1};
-            for (int a = 0; a < 3; ++a) {
-                if (g[a] + 1 >= dims[a]) continue;
-                const int l1 = labels[idx + str[a]];
-                if (l0 != l1) ++ce[a];
-                else if (l0) ++ci[a];
+        const long long gk = (long long)TILE * t[2];
+        for (int r = lane; r < 81; r += 32) {
+            const int i = r / 9, j = r - 9 * i;
+            const long long gi = (long long)TILE * t[0] + i, gj = (long long)TILE * t[1] + j;
+            unsigned m = 0u;
+            if (gi < d0 && gj < d1) {
+                const long long at = (gi * d1 + gj) * d2 + gk;
+                const uint8_t *p = labels + at;
+                if (at + 12 <= np) {
+                    const int off = (int)(reinterpret_cast<uintptr_t>(p) & 3);
+                    const unsigned *q = reinterpret_cast<const unsigned *>(p - off);
+                    const unsigned a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2);
+                    const unsigned w0 = __funnelshift_r(a0, a1, 8 * off), w1 = __funnelshift_r(a1, a2, 8 * off);
+                    m = ((w0 & 0x01010101u) * 0x01020408u >> 24) | (((w1 & 0x01010101u) * 0x01020408u >> 24) << 4) |
+                        (((a2 >> (8 * off)) & 1u) << 8);
+                } else {
+                    for (int k = 0; k < 9 && gk + k < d2; ++k) m |= (unsigned)(p[k] & 1) << k;
+                }
+                m |= 0x8000u;
             }
+            row[r] = (uint16_t)m;
         }
-        for (int a = 0; a < 3; ++a) {
-            ce[a] = __reduce_add_sync(0xffffffffu, ce[a]);
-            ci[a] = __reduce_add_sync(0xffffffffu, ci[a]);
+        __syncwarp();
+        // (points past the grid hold the next row's labels: masked by the row lengths)
+        const int n_on = (int)min(9LL, d2 - gk), n_own = (int)max(0LL, min(8LL, G.own[2] - gk));
+        const unsigned own = (1u << n_own) - 1u, ownz = own & ((1u << (n_on - 1)) - 1u);
+        unsigned c[3] = {0u, 0u, 0u}, npin = 0u;  // crossing | inside edges << 16
+        for (int q = 0; q < 2; ++q) {
+            const int i = (2 * lane + q) >> 3, j = (2 * lane + q) & 7, r = 9 * i + j;
+            if ((long long)TILE * t[0] + i >= G.own[0] || (long long)TILE * t[1] + j >= G.own[1]) continue;
+            const unsigned m = row[r], x = row[r + 9], y = row[r + 1], z = (m & 0x1ffu) >> 1;
+            const unsigned ox = (x & 0x8000u) ? own : 0u, oy = (y & 0x8000u) ? own : 0u;
+            c[0] += __popc((m ^ x) & ox) | (__popc(m & x & ox) << 16);
+            c[1] += __popc((m ^ y) & oy) | (__popc(m & y & oy) << 16);
+            c[2] += __popc((m ^ z) & ownz) | (__popc(m & z & ownz) << 16);
+            npin += __popc(m & own);
         }
+        for (int a = 0; a < 3; ++a) c[a] = __reduce_add_sync(0xffffffffu, c[a]);
         npin = __reduce_add_sync(0xffffffffu, npin);
         if (lane < 3) {
-            tile_edges[lane * nt + gt] = lane == 0 ? ce[0] : (lane == 1 ? ce[1] : ce[2]);
-            tile_inside[lane * nt + gt] = lane == 0 ? ci[0] : (lane == 1 ? ci[1] : ci[2]);
+            const unsigned v = lane == 0 ? c[0] : (lane == 1 ? c[1] : c[2]);
+            tile_edges[lane * nt + gt] = (int)(v & 0xffffu);
+            tile_inside[lane * nt + gt] = (int)(v >> 16);
         } else if (lane == 3) {
-            tile_inside[3 * nt + gt] = npin;
+            tile_inside[3 * nt + gt] = (int)npin;
         }
+        __syncwarp();
     }
 }
 

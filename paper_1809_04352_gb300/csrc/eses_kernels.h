@@ -58,12 +58,13 @@ int classify_ctas_per_sm(int precision);
 // ovf: int[2 + tiles] scratch (tiles sent to the global-memory tier over the
 // run, the stage's count, then the tiles that overflowed the shared-memory
 // staging); big: classify_big_bytes() of global scratch for that tier
+// band (null: FP64 form): int[1 + tiles], the number of tiles with undecided points, then those tiles;
 // n_tests (may be null): adds up the atom tests of the shell points' witness freeness
 int launch_classify(const Model &M, const Batch &B, int precision, const TileSched &Q, int grid, int8_t *labels,
-                    int *tile_band, int *err, int *ovf, unsigned char *big, unsigned long long *n_tests,
+                    int *band, int *err, int *ovf, unsigned char *big, unsigned long long *n_tests,
                     cudaStream_t st);
 size_t classify_big_bytes();
-int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *tile_band, int *err, int *ovf,
+int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *band, int *err, int *ovf,
                 unsigned char *big, cudaStream_t st);
 // exterior-only surface (eses_exterior.cu): state init, one sweep (sets *changed
 // when it reached new points), cavity points relabelled inside (counted)
@@ -170,7 +171,7 @@ int launch_tile_targets(const Batch &B, const int8_t *labels, uint8_t *target, c
 // tiles left to the exact classification; counts[0..1] += proposed, certified;
 // wait_limit: polls of each tensor-core wait (< 0: the default limit)
 int launch_propose(const Model &M, const Batch &B, int mode, const float *P, float z_far, int8_t *labels,
-                   int *tile_band, int *need, int *counts, int *err, long long wait_limit, cudaStream_t st);
+                   int *need, int *counts, int *err, long long wait_limit, cudaStream_t st);
 // the proposer's tensor-core MLP on n rows of features (err |= ERR_TIMEOUT on a wait that ran out)
 int launch_mlp_forward_tc(const float *X, int n, const float *P, float *z, int *err, cudaStream_t st);
 int launch_compact(long long n, const int *need, const int *pos, int *list, cudaStream_t st);

@@ -341,7 +341,7 @@ __device__ int certify_tile(const Model &M, const Grid &G, int mol, long long ti
 // classification.  mode 1: MLP + certificate; mode 2: certificate on every tile.
 __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int mode, const float *__restrict__ Pg,
                                                           float z_far, int8_t *__restrict__ labels_all,
-                                                          int *__restrict__ tile_band, int *__restrict__ need,
+                                                          int *__restrict__ need,
                                                           int *__restrict__ counts, int *__restrict__ err,
                                                           long long wait_limit)
 {
@@ -391,7 +391,6 @@ __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int 
                 }
                 if (lane == 0) {
                     need[g2] = 0;
-                    if (tile_band) tile_band[g2] = 0;
                 }
             }
             if (lane == 0) {
@@ -498,9 +497,9 @@ static int tc_grid(long long rows)
 }
 
 int launch_propose(const Model &M, const Batch &B, int mode, const float *P, float z_far, int8_t *labels,
-                   int *tile_band, int *need, int *counts, int *err, long long wait_limit, cudaStream_t st)
+                   int *need, int *counts, int *err, long long wait_limit, cudaStream_t st)
 {
-    k_propose<<<tc_grid(B.n_tiles), PROP_THREADS, sizeof(TcSmem), st>>>(M, B, mode, P, z_far, labels, tile_band, need,
+    k_propose<<<tc_grid(B.n_tiles), PROP_THREADS, sizeof(TcSmem), st>>>(M, B, mode, P, z_far, labels, need,
                                                                        counts, err, wait_limit);
     return 1;
 }
