@@ -745,44 +745,64 @@ __device__ __noinline__ void torus_piece_exact(const Acc &X, RootSink &out, int 
 // its axis stay away (|g''| <= C = 1 / min(D, |w|) over the edge) |g| is at
 // most |g'| h/2 + C h^2/8, and g' keeps its sign when |g'| > C h/2, which must
 // be falling after an inside end, rising after an outside one.
-// mg widens every test for FP32.  (The Lipschitz test alone, and spheres by
+// The test is FP32 in either form (a superset of the pieces with roots: every
+// comparison is widened by 2e-3 A).  (The Lipschitz test alone, and spheres by
 // their distance range only, left 1.50 M sphere and 4.31 M torus candidates on
-// 1.14 M edges of the 5,000-atom globule; see k_roots_torus.)
+// 1.14 M edges of the 5,000-atom globule, 1.0 M and 1.6 M now.)
+struct CandItem {  // one staged piece, held by a lane over many edges
+    float x, y, z, r;  // sphere: centre, radius; circle: centre, rho
+    float ux, uy, uz;  // circle: axis
+    int kind;          // 0 van der Waals sphere, 1 probe sphere, 2 circle, -1 none
+};
+
 template <class T, class CP>
-__device__ __forceinline__ bool cand_test(const TileS<T, CP> &S, const T *s, int axis, bool inside, int it, T hT, T rpT,
-                                          T mg)
+__device__ __forceinline__ CandItem cand_item(const TileS<T, CP> &S, int it, int nitem, float rp)
 {
-    const int na = S.na, nv = S.nv;
-    if (it < na + nv) {
-        const bool vdw = it < na;
-        const P4<T> c = vdw ? S.atom[it] : S.vq[it - na];
-        const T rad = vdw ? c.w : rpT;
-        const T d0 = s[0] - c.x, d1 = s[1] - c.y, d2 = s[2] - c.z;
-        const T dd = d0 * d0 + d1 * d1 + d2 * d2;
-        const T da = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
-        const T tc = fmin(fmax(-da, T(0)), hT);         // nearest point of the segment
-        const T dmin2 = dd + tc * (tc + T(2) * da);
-        const T end2 = vdw == inside ? dd + hT * (hT + T(2) * da) : dd;
-        const T rhi = rad + mg, rlo = fmax(rad - mg, T(0));
-        return dmin2 <= rhi * rhi && end2 >= rlo * rlo && (!vdw || S.aface[it] != 0);
+    const int na = S.na, nsph = S.na + S.nv;
+    CandItem c{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, -1};
+    if (it >= nitem) return c;
+    const P4<T> o = it < na ? S.atom[it] : (it < nsph ? S.vq[it - na] : S.po[it - nsph]);
+    c.x = (float)o.x;
+    c.y = (float)o.y;
+    c.z = (float)o.z;
+    c.r = it < na || it >= nsph ? (float)o.w : rp;
+    c.kind = it < na ? (S.aface[it] != 0 ? 0 : -1) : (it < nsph ? 1 : 2);
+    if (it >= nsph) {
+        const P4<T> u = S.pu[it - nsph];
+        c.ux = (float)u.x;
+        c.uy = (float)u.y;
+        c.uz = (float)u.z;
     }
-    const int pi = it - na - nv;
-    const P4<T> o = S.po[pi];
-    const P4<T> u = S.pu[pi];
-    T m[3] = {s[0] - o.x, s[1] - o.y, s[2] - o.z};
-    m[axis] += T(0.5) * hT;
-    const T zc = m[0] * u.x + m[1] * u.y + m[2] * u.z;
-    const T w2 = fmax(m[0] * m[0] + m[1] * m[1] + m[2] * m[2] - zc * zc, T(0));
-    const T nw = sqrt(w2), e1 = nw - o.w;
-    const T D = sqrt(e1 * e1 + zc * zc), gm = fabs(D - rpT), half = T(0.5) * hT + mg;
-    if (gm > half) return false;
-    const T low = fmin(D, nw) - half;
-    if (low < T(0.1)) return true;
-    const T ua = axis == 0 ? u.x : (axis == 1 ? u.y : u.z);
-    const T bend = half / low;  // C h/2: g' moves by at most this over the edge
-    const T dg = (e1 * (m[axis] - zc * ua) / nw + zc * ua) / D;
-    if (gm > fabs(dg) * half + T(0.5) * bend * half + mg + T(1e-9)) return false;
-    return !((inside ? dg : -dg) > bend + T(1e-2));
+    return c;
+}
+
+__device__ __forceinline__ bool cand_test(const CandItem &c, const float *s, int axis, bool inside, float h, float rp)
+{
+    constexpr float mg = 2e-3f;
+    const float d0 = s[0] - c.x, d1 = s[1] - c.y, d2 = s[2] - c.z;
+    if (c.kind < 2) {
+        const float dd = d0 * d0 + d1 * d1 + d2 * d2;
+        const float da = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
+        const float tc = fminf(fmaxf(-da, 0.0f), h);         // nearest point of the segment
+        const float dmin2 = dd + tc * (tc + 2.0f * da);
+        const float end2 = (c.kind == 0) == inside ? dd + h * (h + 2.0f * da) : dd;
+        const float rhi = c.r + mg, rlo = fmaxf(c.r - mg, 0.0f);
+        return c.kind >= 0 && dmin2 <= rhi * rhi && end2 >= rlo * rlo;
+    }
+    const float half = 0.5f * h;
+    const float m0 = axis == 0 ? d0 + half : d0, m1 = axis == 1 ? d1 + half : d1, m2 = axis == 2 ? d2 + half : d2;
+    const float zc = m0 * c.ux + m1 * c.uy + m2 * c.uz;
+    const float w2 = fmaxf(m0 * m0 + m1 * m1 + m2 * m2 - zc * zc, 0.0f);
+    const float nw = sqrtf(w2), e1 = nw - c.r;
+    const float D = sqrtf(e1 * e1 + zc * zc), gm = fabsf(D - rp), H = half + mg;
+    if (gm > H) return false;
+    const float low = fminf(D, nw) - H;
+    if (low < 0.1f) return true;
+    const float ua = axis == 0 ? c.ux : (axis == 1 ? c.uy : c.uz), ma = axis == 0 ? m0 : (axis == 1 ? m1 : m2);
+    const float bend = __fdividef(H, low);  // C h/2: g' moves by at most this over the edge
+    const float dg = __fdividef(e1 * __fdividef(ma - zc * ua, nw) + zc * ua, D);
+    if (gm > fabsf(dg) * H + 0.5f * bend * H + mg) return false;
+    return !((inside ? dg : -dg) > bend + 1e-2f);
 }
 
 // Roots of one (edge, piece) candidate that can be the surface on that edge:
@@ -1269,7 +1289,7 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
     __shared__ Grid sG;
     const long long nt = B.n_tiles;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const T rpT = (T)M.rp, mg = FILT ? T(2e-3) : T(0);
+    const T rpT = (T)M.rp;
     long long iter = 0;
     const long long npos = sched_count(Q, nt);
     for (;;) {
@@ -1288,8 +1308,6 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
         const int8_t *__restrict__ labels = labels_all + G.lab0;
         const long long st1 = G.dims[2], st0 = G.dims[1] * G.dims[2];
         const long long fst1 = G.full[2], fst0 = G.full[1] * G.full[2];  // strides of the output indices
-        const double h = G.h;
-        const T hT = (T)h;
         double x0[3];
         stage_tile<T>(M, G, mol, tile, S, x0);
         if (!BIG && (S.flags & ERR_CAP_ANY)) {  // uniform: set before stage_tile's last barrier
@@ -1354,26 +1372,25 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
                 (long long)(TILE * (t[0] + G.toff[0]) + li) * fst0 + (long long)(TILE * (t[1] + G.toff[1]) + lj) * fst1 +
                 (TILE * (t[2] + G.toff[2]) + lk);
         }
-        // (edge, item) pairs that pass the prefilter, counted: one warp per edge,
-        // lanes over items; the hit masks kept when they fit
+        // (edge, item) pairs that pass the prefilter, counted: lanes over items,
+        // an item kept in registers while its warp goes through the warp's
+        // edges; the hit masks kept when they fit
         const int nwd = (nitem + 31) >> 5;
         const bool keep = (long long)ne * nwd <= HMASK_WORDS;
-        for (int e = warp; e < ne; e += EDGE_WARPS) {
-            const EdgeRef R = edge_ref(E, e);
-            T s[3], hs;
-            edge_point<T>(G, R.p, s, hs);
-            int cs = 0, ct = 0;
-            for (int i0 = 0; i0 < nitem; i0 += 32) {
-                const int it = i0 + lane;
-                const bool hit = it < nitem && cand_test<T, CP>(S, s, R.axis, R.lab == LABEL_IN, it, hT, rpT, mg);
-                const unsigned m = __ballot_sync(0xffffffffu, hit), sm = sphere_bits(i0 >> 5, nsph);
-                cs += __popc(m & sm);
-                ct += __popc(m & ~sm);
-                if (keep && lane == 0) E.hmask[e * nwd + (i0 >> 5)] = m;
-            }
-            if (lane == 0) {
-                E.cs[e] = cs;
-                E.ct[e] = ct;
+        const float rpf = (float)M.rp;
+        for (int i0 = 0; i0 < max(nitem, 1); i0 += 32) {
+            const CandItem item = cand_item<T, CP>(S, i0 + lane, nitem, rpf);
+            const unsigned sm = sphere_bits(i0 >> 5, nsph);
+            for (int e = warp; e < ne; e += EDGE_WARPS) {
+                const EdgeRef R = edge_ref(E, e);
+                float s[3], hs;
+                edge_point<float>(G, R.p, s, hs);
+                const unsigned m = __ballot_sync(0xffffffffu, cand_test(item, s, R.axis, R.lab == LABEL_IN, hs, rpf));
+                if (lane == 0) {  // (the same lane for every word of an edge)
+                    E.cs[e] = (i0 ? E.cs[e] : 0) + __popc(m & sm);
+                    E.ct[e] = (i0 ? E.ct[e] : 0) + __popc(m & ~sm);
+                    if (keep) E.hmask[e * nwd + (i0 >> 5)] = m;
+                }
             }
         }
         __syncthreads();
@@ -1478,16 +1495,20 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
             for (int e = warp; e < ne; e += EDGE_WARPS) {
                 const EdgeRef R = edge_ref(E, e);
                 const int g = E.gbase[R.axis] + (e - E.estart[R.axis]);
-                T s[3], hs;
-            edge_point<T>(G, R.p, s, hs);
+                float s[3], hs;
+                edge_point<float>(G, R.p, s, hs);
                 long long ps = E.sb + E.cs[e], pt = E.tb + E.ct[e];
                 const long long ps1 = E.sb + E.cs[e + 1], pt1 = E.tb + E.ct[e + 1];
                 const unsigned below = (1u << lane) - 1;
                 for (int i0 = 0; i0 < nitem; i0 += 32) {
                     const int it = i0 + lane;
-                    const unsigned m =
-                        keep ? E.hmask[e * nwd + (i0 >> 5)]
-                             : __ballot_sync(0xffffffffu, it < nitem && cand_test<T, CP>(S, s, R.axis, R.lab == LABEL_IN, it, hT, rpT, mg));
+                    unsigned m;
+                    if (keep) {
+                        m = E.hmask[e * nwd + (i0 >> 5)];
+                    } else {  // tested again
+                        const CandItem item = cand_item<T, CP>(S, it, nitem, rpf);
+                        m = __ballot_sync(0xffffffffu, cand_test(item, s, R.axis, R.lab == LABEL_IN, hs, rpf));
+                    }
                     const bool hit = (m >> lane) & 1u;
                     const unsigned sm = sphere_bits(i0 >> 5, nsph), ms = m & sm, mt = m & ~sm;
                     const long long qs = ps + __popc(ms & below), qt = pt + __popc(mt & below);
@@ -1634,6 +1655,14 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus(Model M, Batch
         } else {
             const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
             const SlabExact<T> X(A, M, x0);
+            // (a candidate that the certified isolation finds without a root near the edge has none in FP64)
+            const P4<T> o = A.po(c.y), u = A.pu(c.y);
+            const float q0[3] = {(float)(s64[0] - o.x), (float)(s64[1] - o.y), (float)(s64[2] - o.z)};
+            const float uu[3] = {(float)u.x, (float)u.y, (float)u.z};
+            float rt[4];
+            int nr = 0;
+            if (!torus_roots32(q0, uu, (float)o.w, rpf, pk_axis(pk), -1e-4f, (float)h + 1e-4f, B.grid[mol].d0, rt, nr) ||
+                nr > 0)
             torus_roots<T, FILT>(A, X, c.y, s64, pk_axis(pk), pk_label(pk) == LABEL_IN, h, rp, d0, out);
         }
         if (out.n > TOR_SLOTS) atomicOr(err, ERR_CAP_CAND);
