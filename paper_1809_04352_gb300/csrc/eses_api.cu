@@ -728,6 +728,7 @@ int run_device(eses_ctx *c)
         int *need = ensure<int>(c->need, nt);
         int *pos = ensure<int>(c->need_pos, nt + 1);
         int *list = ensure<int>(c->tile_list, nt);
+        ck(cudaMemsetAsync(labels, LABEL_OUT, c->n_points, st), "memset");
         nl += launch_propose(M, B, c->proposer, (const float *)c->mlp_params.p, c->z_far, labels,
                              need, prop_counts, d_err, c->tc_wait, st);
         nl += scan(c, need, pos, nt);

@@ -290,7 +290,7 @@ __global__ void k_tile_targets(Batch B, const int8_t *__restrict__ labels_all, u
 __device__ int certify_tile(const Model &M, const Grid &G, int mol, long long tile)
 {
     const int lane = threadIdx.x & 31;
-    const CellGrid cg = M.cg[mol];
+    const CellGrid &cg = M.cg[mol];
     int tc[3];
     tile_coords(G, tile, tc);
     float th[3], tl[3];
@@ -312,24 +312,52 @@ __device__ int certify_tile(const Model &M, const Grid &G, int mol, long long ti
         c1[a] = min((int)floorf(u + reach), cg.cn[a] - 1);
     }
     bool not_out = false, in = false;
-    // per (x, y) cell column, the atoms of its z cells are contiguous
-    for (int a = c0[0]; a <= c1[0]; ++a)
-        for (int b = c0[1]; b <= c1[1]; ++b) {
-            if (c0[2] > c1[2]) continue;
-            const int id0 = cg.coff + (a * cg.cn[1] + b) * cg.cn[2];
-            const int e = M.cell_start[id0 + c1[2] + 1];
-            for (int k = M.cell_start[id0 + c0[2]] + lane; k < e; k += 32) {
-                const float4 hi = M.atom_hi[k], lo = M.atom_lo[k];
-                const float dx = (hi.x - th[0]) + (lo.x - tl[0]);
-                const float dy = (hi.y - th[1]) + (lo.y - tl[1]);
-                const float dz = (hi.z - th[2]) + (lo.z - tl[2]);
-                const float d2 = dx * dx + dy * dy + dz * dz;
-                const float to = hi.w + rp + delta + slack;  // outside needs d >= R + delta
-                if (d2 * rel_lo < to * to) not_out = true;
-                const float ti = hi.w - delta - slack;  // inside needs d < r - delta
-                if (ti > 0.0f && d2 * rel_hi < ti * ti) in = true;
-            }
+    auto test = [&](int k) {
+        const float4 hi = M.atom_hi[k], lo = M.atom_lo[k];
+        const float dx = (hi.x - th[0]) + (lo.x - tl[0]);
+        const float dy = (hi.y - th[1]) + (lo.y - tl[1]);
+        const float dz = (hi.z - th[2]) + (lo.z - tl[2]);
+        const float d2 = dx * dx + dy * dy + dz * dz;
+        const float to = hi.w + rp + delta + slack;  // outside needs d >= R + delta
+        if (d2 * rel_lo < to * to) not_out = true;
+        const float ti = hi.w - delta - slack;  // inside needs d < r - delta
+        if (ti > 0.0f && d2 * rel_hi < ti * ti) in = true;
+    };
+    // per (x, y) cell column, the atoms of its z cells are contiguous: one lane
+    // per column reads its range and the lanes walk the ranges laid end to end
+    // (column by column, two dependent loads each, cost a far tile nine round
+    // trips to find no atom)
+    const int n0 = c1[0] - c0[0] + 1, n1 = c1[1] - c0[1] + 1;
+    if (n0 <= 0 || n1 <= 0 || c0[2] > c1[2]) return 0;
+    if ((long long)n0 * n1 <= 32) {
+        int start = 0, len = 0;
+        if (lane < n0 * n1) {
+            const int id0 = cg.coff + ((c0[0] + lane / n1) * cg.cn[1] + c0[1] + lane % n1) * cg.cn[2];
+            start = M.cell_start[id0 + c0[2]];
+            len = M.cell_start[id0 + c1[2] + 1] - start;
         }
+        int end = len;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        start -= end - len;  // atom of position t in column r: start[r] + t
+        const int total = __shfl_sync(0xffffffffu, end, 31);
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            int r = 0;  // columns that end at or before t
+            for (int q = 0; q < n0 * n1 - 1; ++q) r += t >= __shfl_sync(0xffffffffu, end, q) ? 1 : 0;
+            const int k = __shfl_sync(0xffffffffu, start, r) + t;
+            if (t < total) test(k);
+        }
+    } else {
+        for (int a = c0[0]; a <= c1[0]; ++a)
+            for (int b = c0[1]; b <= c1[1]; ++b) {
+                const int id0 = cg.coff + (a * cg.cn[1] + b) * cg.cn[2];
+                const int e = M.cell_start[id0 + c1[2] + 1];
+                for (int k = M.cell_start[id0 + c0[2]] + lane; k < e; k += 32) test(k);
+            }
+    }
     if (!__any_sync(0xffffffffu, not_out)) return 0;
     if (__any_sync(0xffffffffu, in)) return 1;
     return -1;
@@ -337,8 +365,11 @@ __device__ int certify_tile(const Model &M, const Grid &G, int mol, long long ti
 
 // Proposer: features and tensor-core score per tile (thread per tile, 128
 // tiles per CTA step), then the certificate for the tiles scored far (warp
-// per tile); certified tiles are filled, the others flagged for the exact
-// classification.  mode 1: MLP + certificate; mode 2: certificate on every tile.
+// per tile); tiles certified inside are filled (the labels start as outside
+// everywhere), the others flagged for the exact classification.  mode 1: MLP +
+// certificate; mode 2: certificate on every tile.  Bound by the latency of the
+// cell look-ups; filling the outside tiles here, 8-byte rows at any alignment,
+// cost more than clearing all labels at HBM speed does.
 __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int mode, const float *__restrict__ Pg,
                                                           float z_far, int8_t *__restrict__ labels_all,
                                                           int *__restrict__ need,
@@ -351,6 +382,7 @@ __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int 
     __shared__ int n_far;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t phase = 0;
+    int proposed = 0, certified = 0;  // the warp's tiles
     if (mode == 1) tc_setup(T, Pg, wait_limit);
     for (long long base = (long long)blockIdx.x * PROP_THREADS; base < B.n_tiles;
          base += (long long)gridDim.x * PROP_THREADS) {
@@ -379,7 +411,7 @@ __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int 
             const Grid &G = B.grid[mol];
             const long long tile = g2 - G.tile0;
             const int r = certify_tile(M, G, mol, tile);
-            if (r >= 0) {
+            if (r == 1) {
                 int8_t *labels = labels_all + G.lab0;
                 int tc[3];
                 tile_coords(G, tile, tc);
@@ -389,16 +421,16 @@ __global__ void __launch_bounds__(PROP_THREADS) k_propose(Model M, Batch B, int 
                     if (g0 < G.dims[0] && g1 < G.dims[1] && gz < G.dims[2])
                         labels[(g0 * G.dims[1] + g1) * G.dims[2] + gz] = (int8_t)r;
                 }
-                if (lane == 0) {
-                    need[g2] = 0;
-                }
             }
-            if (lane == 0) {
-                atomicAdd(&counts[0], 1);                // tiles proposed far
-                if (r >= 0) atomicAdd(&counts[1], 1);    // certified
-            }
+            if (r >= 0 && lane == 0) need[g2] = 0;
+            proposed += 1;
+            certified += r >= 0 ? 1 : 0;
         }
         __syncthreads();
+    }
+    if (lane == 0 && proposed) {
+        atomicAdd(&counts[0], proposed);
+        atomicAdd(&counts[1], certified);
     }
     if (mode == 1) tc_teardown(T, phase);
 }
