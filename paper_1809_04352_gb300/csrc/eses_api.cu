@@ -747,7 +747,7 @@ int run_device(eses_ctx *c)
     c->ext_sweeps = 0;
     if (c->exterior) {  // cavities filled: sweeps until one reaches nothing new (never under capture)
         if (g_capturing) throw std::string("the exterior-only surface is not captured in a graph");
-        uint8_t *ext = ensure<uint8_t>(c->ext, c->n_points);
+        uint16_t *ext = ensure<uint16_t>(c->ext, 64 * (size_t)nt);
         uint8_t *open = ensure<uint8_t>(c->ext_open, nt);
         // em[0..1]: four ints (three sweep flags, the sweep count), em[2]: filled points
         unsigned long long *em = ensure<unsigned long long>(c->ext_misc, 3);
@@ -760,7 +760,7 @@ int run_device(eses_ctx *c)
         if (coop == 1) {  // one launch for every sweep
             ++nl;
         } else {  // no cooperative launch on this device: one launch per sweep, driven from the host
-            const int sweep_grid = (int)std::min<long long>(std::max<long long>(nt, 1), 8LL * c->n_sm);
+            const int sweep_grid = (int)std::min<long long>(std::max<long long>(ceil_div_ll(nt, 8), 1), 8LL * c->n_sm);
             for (long long it = 0; it <= nt; ++it) {
                 ck(cudaMemsetAsync(flags, 0, sizeof(int), st), "memset");
                 nl += launch_ext_sweep(B, ext, open, flags, sweep_grid, st);

@@ -1122,33 +1122,11 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32) k_edge_count(Batch B, const 
     const long long nw = (long long)gridDim.x * COUNT_WARPS;
     for (long long gt = (long long)blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); gt < nt; gt += nw) {
         const Grid &G = B.grid[mol_of_tile(B, gt)];
-        const long long d0 = G.dims[0], d1 = G.dims[1], d2 = G.dims[2], np = d0 * d1 * d2;
-        const uint8_t *__restrict__ labels = reinterpret_cast<const uint8_t *>(labels_all) + G.lab0;
+        const long long d2 = G.dims[2];
         int t[3];
         tile_coords(G, gt - G.tile0, t);
         const long long gk = (long long)TILE * t[2];
-        for (int r = lane; r < 81; r += 32) {
-            const int i = r / 9, j = r - 9 * i;
-            const long long gi = (long long)TILE * t[0] + i, gj = (long long)TILE * t[1] + j;
-            unsigned m = 0u;
-            if (gi < d0 && gj < d1) {
-                const long long at = (gi * d1 + gj) * d2 + gk;
-                const uint8_t *p = labels + at;
-                if (at + 12 <= np) {
-                    const int off = (int)(reinterpret_cast<uintptr_t>(p) & 3);
-                    const unsigned *q = reinterpret_cast<const unsigned *>(p - off);
-                    const unsigned a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2);
-                    const unsigned w0 = __funnelshift_r(a0, a1, 8 * off), w1 = __funnelshift_r(a1, a2, 8 * off);
-                    m = ((w0 & 0x01010101u) * 0x01020408u >> 24) | (((w1 & 0x01010101u) * 0x01020408u >> 24) << 4) |
-                        (((a2 >> (8 * off)) & 1u) << 8);
-                } else {
-                    for (int k = 0; k < 9 && gk + k < d2; ++k) m |= (unsigned)(p[k] & 1) << k;
-                }
-                m |= 0x8000u;
-            }
-            row[r] = (uint16_t)m;
-        }
-        __syncwarp();
+        tile_rows(G, labels_all, t, row);
         // (points past the grid hold the next row's labels: masked by the row lengths)
         const int n_on = (int)min(9LL, d2 - gk), n_own = (int)max(0LL, min(8LL, G.own[2] - gk));
         const unsigned own = (1u << n_own) - 1u, ownz = own & ((1u << (n_on - 1)) - 1u);
