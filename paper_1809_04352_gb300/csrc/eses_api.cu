@@ -164,7 +164,7 @@ struct eses_ctx {
     bool exterior = false;
     DBuf ext, ext_open, ext_misc;
     // triangle mesh of the last run (eses_mesh_count / eses_mesh)
-    DBuf mesh_mask, mesh_tile, mesh_off, mesh_keys, mesh_xyz, mesh_err;
+    DBuf mesh_mask, mesh_tile, mesh_off, mesh_keys, mesh_xyz, mesh_err, mesh_tot;
     long long n_tri = -1;  // -1: not made for the current results
     long long n_cavity = 0;
     int ext_sweeps = 0;
@@ -1803,19 +1803,16 @@ int eses_mesh_count(eses_ctx *c, int64_t *n_tri)
             cudaStream_t st = c->stream;
             const long long nt = c->n_tiles;
             const Batch &B = c->B;
-            uint32_t *mask = ensure<uint32_t>(c->mesh_mask, (size_t)nt * 3 * (TILE_PTS / 32));
+            uint32_t *mask = ensure<uint32_t>(c->mesh_mask, mesh_mask_words(nt));
             int *tile = ensure<int>(c->mesh_tile, nt);
             int *off = ensure<int>(c->mesh_off, nt + 1);
             int *derr = ensure<int>(c->mesh_err, 1);
-            launch_mesh_masks(B, (const int8_t *)c->labels.p, mask, st);
-            launch_mesh_count(B, (const int8_t *)c->labels.p, tile, st);
             // the total in 64 bits first: the offsets are 32-bit
-            std::vector<int> per_tile((size_t)nt);
-            ck(cudaMemcpyAsync(per_tile.data(), tile, sizeof(int) * (size_t)nt, cudaMemcpyDeviceToHost, st), "read");
+            unsigned long long *dtot = ensure<unsigned long long>(c->mesh_tot, 1), total = 0;
+            launch_mesh_count(B, (const int8_t *)c->labels.p, mask, tile, dtot, st);
+            ck(cudaMemcpyAsync(&total, dtot, sizeof(total), cudaMemcpyDeviceToHost, st), "read");
             ck(cudaStreamSynchronize(st), "synchronize");
-            long long total = 0;
-            for (int v : per_tile) total += v;
-            if (total >= (1LL << 31)) return fail(c, ESES_EINVAL, "mesh of 2^31 triangles or more");
+            if (total >= (1ULL << 31)) return fail(c, ESES_EINVAL, "mesh of 2^31 triangles or more");
             scan(c, tile, off, nt);
             const int tot = (int)total;
             EdgeOut eo{};
@@ -1931,7 +1928,7 @@ void eses_destroy(eses_ctx *c)
                     &c->atom_lo, &c->pair_hi, &c->pair_lo, &c->pair_u32, &c->vert_hi, &c->vert_lo,
                     &c->mlp_params, &c->need, &c->need_pos, &c->tile_list, &c->prop_counts, &c->features,
                     &c->targets, &c->ext, &c->ext_open, &c->ext_misc, &c->mesh_mask, &c->mesh_tile, &c->mesh_off,
-                    &c->mesh_keys, &c->mesh_xyz, &c->mesh_err};
+                    &c->mesh_keys, &c->mesh_xyz, &c->mesh_err, &c->mesh_tot};
     if (c->own_stream) cudaStreamSynchronize(c->own_stream);
     drop_graph(c);
     for (DBuf *b : bufs) free_buf(*b);

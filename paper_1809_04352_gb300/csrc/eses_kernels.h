@@ -139,8 +139,9 @@ int launch_edge_polish(const Model &M, const Batch &B, EdgeOut out, long long n_
 // triangles per tile, and the triangles (keys and FP64 points)
 int mesh_init();
 int mesh_table_host(int8_t *tri, uint8_t *n, int max_tri);
-int launch_mesh_masks(const Batch &B, const int8_t *labels, uint32_t *mask, cudaStream_t st);
-int launch_mesh_count(const Batch &B, const int8_t *labels, int *tile_tri, cudaStream_t st);
+size_t mesh_mask_words(long long n_tiles);  // 32-bit words of the masks
+int launch_mesh_count(const Batch &B, const int8_t *labels, uint32_t *mask, int *tile_tri, unsigned long long *total,
+                      cudaStream_t st);
 int launch_mesh_emit(const Batch &B, const int8_t *labels, const uint32_t *mask, const int *edge_start,
                      const EdgeOut &out, const int *tile_off, long long *keys, double *xyz, int *err, cudaStream_t st);
 // part_d / part_i: reduce_scratch(n_mol) doubles / int64 each
