@@ -30,7 +30,7 @@
 
 namespace eses {
 
-constexpr int GRAD_S = 64;        // samples per block of the gradient kernel
+constexpr int GRAD_S = 32;        // samples per block of the gradient kernel
 constexpr int GRAD_THREADS = 256;
 constexpr int PROP_THREADS = 128;  // tiles per block of the proposer kernel
 
@@ -75,16 +75,65 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const float *__restrict__ X
 // every parameter; per-block partial sums in fixed order, then a fixed-order
 // reduction over blocks (deterministic)
 // ---------------------------------------------------------------------------
+// 32 samples per block (4,096 samples: 128 blocks, one wave on 152 SMs) and every
+// layer as a register tile: a thread takes 2 samples x 4 units of an
+// activation, 4 x 4 (2 x 4) weights of a gradient, so each 16-byte word from
+// shared memory feeds 4 to 8 multiply-adds (one output per thread, two 4-byte
+// words per multiply-add, took 45 us on 64 blocks).  Bound by shared-memory
+// bandwidth and the block's five barriers.
 struct GradSmem {
-    float P[MLP_NPARAM];
+    float P[MLP_NPARAM + 3];               // rounded to 16 bytes
+    float W2T[MLP_H][MLP_H + 4];           // W2 transposed
     float X[GRAD_S][MLP_IN];
-    float H1[GRAD_S][MLP_H];
-    float H2[GRAD_S][MLP_H];
-    float D1[GRAD_S][MLP_H];
-    float D2[GRAD_S][MLP_H];
-    float dz[GRAD_S];
-    float loss[GRAD_S];
+    float H1[GRAD_S][MLP_H], H2[GRAD_S][MLP_H];
+    float D1[GRAD_S][MLP_H], D2[GRAD_S][MLP_H];
+    float dz[GRAD_S], loss[GRAD_S];
 };
+static_assert(MLP_NPARAM % 4 == 1 && P_B1 % 4 == 0 && P_W2 % 4 == 0 && P_B2 % 4 == 0 && P_W3 % 4 == 0,
+              "16-byte parameter rows");
+static_assert(GRAD_THREADS == (GRAD_S / 2) * (MLP_H / 4), "two samples x four units a thread");
+
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+// (the caller's scratch is aligned to a float only)
+__device__ __forceinline__ void st4(float *p, const float4 &v)
+{
+    p[0] = v.x;
+    p[1] = v.y;
+    p[2] = v.z;
+    p[3] = v.w;
+}
+__device__ __forceinline__ void fma4(float4 &a, float x, const float4 &w)
+{
+    a.x = fmaf(x, w.x, a.x);
+    a.y = fmaf(x, w.y, a.y);
+    a.z = fmaf(x, w.z, a.z);
+    a.w = fmaf(x, w.w, a.w);
+}
+
+// a[q] += sum_k A[s + q][k] * W[k][j .. j + 3] for the thread's two samples
+template <int K, int LD>
+__device__ __forceinline__ void rows_times(const float (*A)[K], const float *W, int s, int j, float4 a[2])
+{
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        const float4 x0 = ld4(&A[s][k]), x1 = ld4(&A[s + 1][k]);
+        const float4 w0 = ld4(W + (k + 0) * LD + j), w1 = ld4(W + (k + 1) * LD + j), w2 = ld4(W + (k + 2) * LD + j),
+                     w3 = ld4(W + (k + 3) * LD + j);
+        fma4(a[0], x0.x, w0);
+        fma4(a[1], x1.x, w0);
+        fma4(a[0], x0.y, w1);
+        fma4(a[1], x1.y, w1);
+        fma4(a[0], x0.z, w2);
+        fma4(a[1], x1.z, w2);
+        fma4(a[0], x0.w, w3);
+        fma4(a[1], x1.w, w3);
+    }
+}
+
+__device__ __forceinline__ float4 relu4(const float4 &a)
+{
+    return make_float4(fmaxf(a.x, 0.0f), fmaxf(a.y, 0.0f), fmaxf(a.z, 0.0f), fmaxf(a.w, 0.0f));
+}
 
 __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad_part(const float *__restrict__ X,
                                                                 const float *__restrict__ y,
@@ -97,93 +146,113 @@ __global__ void __launch_bounds__(GRAD_THREADS) k_mlp_grad_part(const float *__r
     const int tid = threadIdx.x;
     const int s0 = blockIdx.x * GRAD_S;
     const int ns = min(GRAD_S, n - s0);
-    for (int k = tid; k < MLP_NPARAM; k += GRAD_THREADS) G.P[k] = Pg[k];
+    for (int k = tid; k < MLP_NPARAM; k += GRAD_THREADS) {
+        const float p = Pg[k];
+        G.P[k] = p;
+        if (k >= P_W2 && k < P_B2) G.W2T[(k - P_W2) % MLP_H][(k - P_W2) / MLP_H] = p;
+    }
     for (int k = tid; k < GRAD_S * MLP_IN; k += GRAD_THREADS) {
         const int s = k / MLP_IN, i = k % MLP_IN;
         G.X[s][i] = s < ns ? X[(size_t)(s0 + s) * MLP_IN + i] : 0.0f;
     }
     __syncthreads();
-    for (int k = tid; k < GRAD_S * MLP_H; k += GRAD_THREADS) {
-        const int s = k / MLP_H, j = k % MLP_H;
-        float a = G.P[P_B1 + j];
-        for (int i = 0; i < MLP_IN; ++i) a = fmaf(G.X[s][i], G.P[P_W1 + i * MLP_H + j], a);
-        G.H1[s][j] = fmaxf(a, 0.0f);
-    }
+    // the thread's samples and units
+    const int s = 2 * (tid / (MLP_H / 4)), j = 4 * (tid % (MLP_H / 4));
+    float4 h[2];
+    h[0] = h[1] = ld4(G.P + P_B1 + j);
+    rows_times<MLP_IN, MLP_H>(G.X, G.P + P_W1, s, j, h);
+    for (int q = 0; q < 2; ++q) *reinterpret_cast<float4 *>(&G.H1[s + q][j]) = relu4(h[q]);
     __syncthreads();
-    for (int k = tid; k < GRAD_S * MLP_H; k += GRAD_THREADS) {
-        const int s = k / MLP_H, j = k % MLP_H;
-        float a = G.P[P_B2 + j];
-        for (int i = 0; i < MLP_H; ++i) a = fmaf(G.H1[s][i], G.P[P_W2 + i * MLP_H + j], a);
-        G.H2[s][j] = fmaxf(a, 0.0f);
+    h[0] = h[1] = ld4(G.P + P_B2 + j);
+    rows_times<MLP_H, MLP_H>(G.H1, G.P + P_W2, s, j, h);
+    // z: the 16 threads of a sample pair are neighbouring lanes
+    const float4 w3 = ld4(G.P + P_W3 + j);
+    float z[2];
+    for (int q = 0; q < 2; ++q) {
+        h[q] = relu4(h[q]);
+        *reinterpret_cast<float4 *>(&G.H2[s + q][j]) = h[q];
+        z[q] = fmaf(h[q].x, w3.x, fmaf(h[q].y, w3.y, fmaf(h[q].z, w3.z, h[q].w * w3.w)));
+        for (int o = 1; o < MLP_H / 4; o <<= 1) z[q] += __shfl_xor_sync(0xffffffffu, z[q], o);
+        z[q] += G.P[P_B3];
     }
-    __syncthreads();
-    if (tid < GRAD_S) {
-        const int s = tid;
+    for (int q = 0; q < 2; ++q) {
         float dz = 0.0f, l = 0.0f;
-        if (s < ns) {
-            float z = G.P[P_B3];
-            for (int k = 0; k < MLP_H; ++k) z = fmaf(G.H2[s][k], G.P[P_W3 + k], z);
-            const float yy = y[s0 + s], ww = w[s0 + s];
-            const float sg = 1.0f / (1.0f + expf(-z));
+        if (s + q < ns) {
+            const float yy = y[s0 + s + q], ww = w[s0 + s + q];
+            const float sg = 1.0f / (1.0f + expf(-z[q]));
             dz = ww * (sg - yy);
-            l = ww * (fmaxf(z, 0.0f) - z * yy + log1pf(expf(-fabsf(z))));
+            l = ww * (fmaxf(z[q], 0.0f) - z[q] * yy + log1pf(expf(-fabsf(z[q]))));
         }
-        G.dz[s] = dz;
-        G.loss[s] = l;
+        if (j == 0) {
+            G.dz[s + q] = dz;
+            G.loss[s + q] = l;
+        }
+        *reinterpret_cast<float4 *>(&G.D2[s + q][j]) =
+            make_float4(h[q].x > 0.0f ? dz * w3.x : 0.0f, h[q].y > 0.0f ? dz * w3.y : 0.0f,
+                        h[q].z > 0.0f ? dz * w3.z : 0.0f, h[q].w > 0.0f ? dz * w3.w : 0.0f);
     }
     __syncthreads();
-    for (int k = tid; k < GRAD_S * MLP_H; k += GRAD_THREADS) {
-        const int s = k / MLP_H, j = k % MLP_H;
-        G.D2[s][j] = G.H2[s][j] > 0.0f ? G.dz[s] * G.P[P_W3 + j] : 0.0f;
+    h[0] = h[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    rows_times<MLP_H, MLP_H + 4>(G.D2, &G.W2T[0][0], s, j, h);
+    for (int q = 0; q < 2; ++q) {
+        const float4 a = ld4(&G.H1[s + q][j]);
+        *reinterpret_cast<float4 *>(&G.D1[s + q][j]) =
+            make_float4(a.x > 0.0f ? h[q].x : 0.0f, a.y > 0.0f ? h[q].y : 0.0f, a.z > 0.0f ? h[q].z : 0.0f,
+                        a.w > 0.0f ? h[q].w : 0.0f);
     }
     __syncthreads();
-    for (int k = tid; k < GRAD_S * MLP_H; k += GRAD_THREADS) {
-        const int s = k / MLP_H, j = k % MLP_H;
-        float a = 0.0f;
-        if (G.H1[s][j] > 0.0f)
-            for (int q = 0; q < MLP_H; ++q) a = fmaf(G.D2[s][q], G.P[P_W2 + j * MLP_H + q], a);
-        G.D1[s][j] = a;
-    }
-    __syncthreads();
+    // weight gradients: rows r .. of W2 (4) and of W1 (2), columns c .. c + 3
     float *out = part + (size_t)blockIdx.x * (MLP_NPARAM + 1);
-    for (int q = tid; q < MLP_NPARAM; q += GRAD_THREADS) {
-        float g = 0.0f;
-        if (q < P_B1) {
-            const int i = q / MLP_H, j = q % MLP_H;
-            for (int s = 0; s < GRAD_S; ++s) g = fmaf(G.X[s][i], G.D1[s][j], g);
-        } else if (q < P_W2) {
-            const int j = q - P_B1;
-            for (int s = 0; s < GRAD_S; ++s) g += G.D1[s][j];
-        } else if (q < P_B2) {
-            const int j = (q - P_W2) / MLP_H, k = (q - P_W2) % MLP_H;
-            for (int s = 0; s < GRAD_S; ++s) g = fmaf(G.H1[s][j], G.D2[s][k], g);
-        } else if (q < P_W3) {
-            const int k = q - P_B2;
-            for (int s = 0; s < GRAD_S; ++s) g += G.D2[s][k];
-        } else if (q < P_B3) {
-            const int k = q - P_W3;
-            for (int s = 0; s < GRAD_S; ++s) g = fmaf(G.dz[s], G.H2[s][k], g);
-        } else {
-            for (int s = 0; s < GRAD_S; ++s) g += G.dz[s];
-        }
-        out[q] = g;
+    const int c = 4 * (tid % 16), r = tid / 16;
+    float4 g2[4], g1[2];
+    for (int q = 0; q < 4; ++q) g2[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    g1[0] = g1[1] = g2[0];
+#pragma unroll 4
+    for (int k = 0; k < GRAD_S; ++k) {
+        const float4 d2 = ld4(&G.D2[k][c]), d1 = ld4(&G.D1[k][c]), a = ld4(&G.H1[k][4 * r]);
+        const float2 x = *reinterpret_cast<const float2 *>(&G.X[k][2 * r]);
+        fma4(g2[0], a.x, d2);
+        fma4(g2[1], a.y, d2);
+        fma4(g2[2], a.z, d2);
+        fma4(g2[3], a.w, d2);
+        fma4(g1[0], x.x, d1);
+        fma4(g1[1], x.y, d1);
     }
-    if (tid == 0) {
-        float l = 0.0f;
-        for (int s = 0; s < GRAD_S; ++s) l += G.loss[s];
-        out[MLP_NPARAM] = l;
+    for (int q = 0; q < 4; ++q) st4(out + P_W2 + (4 * r + q) * MLP_H + c, g2[q]);
+    for (int q = 0; q < 2; ++q) st4(out + P_W1 + (2 * r + q) * MLP_H + c, g1[q]);
+    // biases, w3 and the loss: one sum per thread
+    if (tid < 3 * MLP_H + 2) {
+        const int u = tid % MLP_H, kind = tid / MLP_H;
+        float g = 0.0f;
+        for (int k = 0; k < GRAD_S; ++k) {
+            if (kind == 0) g += G.D1[k][u];
+            else if (kind == 1) g += G.D2[k][u];
+            else if (kind == 2) g = fmaf(G.dz[k], G.H2[k][u], g);
+            else g += u == 0 ? G.dz[k] : G.loss[k];
+        }
+        out[kind == 0 ? P_B1 + u : (kind == 1 ? P_B2 + u : (kind == 2 ? P_W3 + u : P_B3 + u))] = g;
     }
 }
 
-__global__ void k_mlp_grad_reduce(const float *__restrict__ part, int nblocks, float *__restrict__ grad,
-                                  float *__restrict__ loss)
+// sums of the blocks' parts in a fixed order: warps take every eighth block, lanes neighbouring parameters
+constexpr int RED_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * RED_WARPS) k_mlp_grad_reduce(const float *__restrict__ part, int nblocks,
+                                                                   float *__restrict__ grad, float *__restrict__ loss)
 {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q > MLP_NPARAM) return;
+    __shared__ float sum[RED_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = blockIdx.x * 32 + lane;
     float g = 0.0f;
-    for (int b = 0; b < nblocks; ++b) g += part[(size_t)b * (MLP_NPARAM + 1) + q];
-    if (q < MLP_NPARAM) grad[q] = g;
-    else if (loss) *loss = g;
+    if (q <= MLP_NPARAM)
+        for (int b = warp; b < nblocks; b += RED_WARPS) g += part[(size_t)b * (MLP_NPARAM + 1) + q];
+    sum[warp][lane] = g;
+    __syncthreads();
+    if (warp == 0 && q <= MLP_NPARAM) {
+        for (int k = 1; k < RED_WARPS; ++k) g += sum[k][lane];
+        if (q < MLP_NPARAM) grad[q] = g;
+        else if (loss) *loss = g;
+    }
 }
 
 __global__ void k_adam(float *__restrict__ P, const float *__restrict__ g, float *__restrict__ m,
@@ -492,7 +561,7 @@ int launch_mlp_grad(const float *X, const float *y, const float *w, int n, const
     if (n <= 0) return 0;
     const int nb = (n + GRAD_S - 1) / GRAD_S;
     k_mlp_grad_part<<<nb, GRAD_THREADS, grad_smem(), st>>>(X, y, w, n, P, part);
-    k_mlp_grad_reduce<<<(MLP_NPARAM + 1 + 255) / 256, 256, 0, st>>>(part, nb, grad, loss);
+    k_mlp_grad_reduce<<<(MLP_NPARAM + 1 + 31) / 32, 32 * RED_WARPS, 0, st>>>(part, nb, grad, loss);
     return 2;
 }
 
