@@ -136,7 +136,7 @@ struct eses_ctx {
     DBuf vert_count, vert_start, vert, vert_atoms, arc_list, arc_whole;
     DBuf pbin_count, pbin_start, pbin_cursor, pbin_cell, pbin_list;
     DBuf vbin_count, vbin_start, vbin_cursor, vbin_cell, vbin_list;
-    DBuf labels, band, tile_edges, edge_start, tile_inside;
+    DBuf labels, band, cls_list, etiles, tile_edges, edge_start, tile_inside;
     DBuf out_idx[3], out_tau[3], out_nrm[3], out_tau32[3], out_nrm32[3], out_code[3];
     DBuf scan_tmp, misc, av, counts, red_d, red_i;  // misc: err, n_fail
     DBuf fail_log;
@@ -539,6 +539,18 @@ TileSched sched_of(eses_ctx *c, const Shape &s, int which)
     return q;
 }
 
+// the tiles that the classification takes: those the proposer left, or those an atom's cell reaches
+void cls_tiles(const eses_ctx *c, TileSched &q)
+{
+    if (c->proposer != ESES_PROPOSER_OFF) {
+        q.list = (const int *)c->tile_list.p;
+        q.list_n = (const int *)c->need_pos.p + c->n_tiles;
+    } else {
+        q.list = (const int *)c->cls_list.p + 1;
+        q.list_n = (const int *)c->cls_list.p;
+    }
+}
+
 // Buffers of the phased root solve.  Planning: capacities from a first
 // estimate per crossing edge (grown by run_device when the staging pass needs
 // more); capturing: the planned capacities.
@@ -733,9 +745,13 @@ int run_device(eses_ctx *c)
                              need, prop_counts, d_err, c->tc_wait, st);
         nl += scan(c, need, pos, nt);
         nl += launch_compact(nt, need, pos, list, st);
-        cq.list = list;
-        cq.list_n = pos + nt;
+    } else {
+        // labels start as outside; tiles that no atom's cell reaches keep that and are not taken
+        int *list = ensure<int>(c->cls_list, (size_t)nt + 1);
+        ck(cudaMemsetAsync(labels, LABEL_OUT, c->n_points, st), "memset");
+        nl += launch_tile_list(M, B, list, st);
     }
+    cls_tiles(c, cq);
     int *ovf = ensure<int>(c->ovf, (size_t)nt + 2);
     ck(cudaMemsetAsync(ovf, 0, sizeof(int), st), "memset");
     unsigned char *big = ensure<unsigned char>(c->big, std::max(classify_big_bytes(), edges_big_bytes()));
@@ -785,7 +801,8 @@ int run_device(eses_ctx *c)
     int *tile_inside = ensure<int>(c->tile_inside, 4 * nt);
     long long *medge = ensure<long long>(c->medge, 3 * ((size_t)c->n_mol + 1));
     mark(c, ST_EDGE_COUNT);
-    nl += launch_edge_count(B, labels, tile_edges, tile_inside, st);
+    int *etiles = ensure<int>(c->etiles, (size_t)nt + 1);
+    nl += launch_edge_count(B, labels, tile_edges, tile_inside, etiles, st);
     nl += scan(c, tile_edges, edge_start, 3 * nt);
     nl += launch_mol_edges(B, edge_start, medge, st);
     if (!g_capturing) {
@@ -813,7 +830,9 @@ int run_device(eses_ctx *c)
     long long *fail_log = ensure<long long>(c->fail_log, FAIL_LOG * FAIL_REC);
     mark(c, ST_EDGE_SOLVE);
     RootWork W = root_work(c, ne_all);
-    const TileSched eq = sched_of(c, c->edge, 1);
+    TileSched eq = sched_of(c, c->edge, 1);
+    eq.list = etiles + 1;
+    eq.list_n = etiles;
     const int eg = grid_of(c, c->edge, edge_ctas_per_sm(c->precision));
     nl += launch_edge_stage(M, B, c->precision, eq, eg, labels, edge_start, eo, d_err, ovf, big, W, st);
     if (!g_capturing) {  // planning: the totals the staging pass needed; a full buffer is grown and the pass rerun
@@ -1302,7 +1321,9 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                 s.pop_set = true;
                 float ms = time_it([&] {
                     ck(cudaMemsetAsync(c->queue.p, 0, 4 * sizeof(unsigned long long), st), "memset");
-                    launch_classify(M, B, c->precision, sched_of(c, s, 0), grid_of(c, s, cls_max), labels,
+                    TileSched q = sched_of(c, s, 0);
+                    cls_tiles(c, q);
+                    launch_classify(M, B, c->precision, q, grid_of(c, s, cls_max), labels,
                                     c->precision == ESES_PREC_FP64 ? nullptr : band, misc, (int *)c->ovf.p,
                                     (unsigned char *)c->big.p, nullptr, st);
                 });
@@ -1351,7 +1372,10 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                     s.pop_set = true;
                     s.threads = threads;
                     float ms = time_it([&] {
-                        launch_edge_stage(M, B, c->precision, sched_of(c, s, 1), grid_of(c, s, edge_max), labels,
+                        TileSched q = sched_of(c, s, 1);
+                        q.list = (const int *)c->etiles.p + 1;
+                        q.list_n = (const int *)c->etiles.p;
+                        launch_edge_stage(M, B, c->precision, q, grid_of(c, s, edge_max), labels,
                                           (const int *)c->edge_start.p, eo, misc, (int *)c->ovf.p,
                                           (unsigned char *)c->big.p, W, st);
                         launch_edge_roots(M, B, c->precision, threads, eo, (const int *)c->edge_start.p, ne_all,
@@ -1921,7 +1945,7 @@ void eses_destroy(eses_ctx *c)
                     &c->contained, &c->face, &c->pair_count, &c->pair_start, &c->pair_o, &c->pair_u, &c->pair_ij,
                     &c->pair_free, &c->vert_count, &c->vert_start, &c->vert, &c->vert_atoms, &c->pbin_count, &c->pbin_start,
                     &c->pbin_cursor, &c->pbin_cell, &c->pbin_list, &c->vbin_count, &c->vbin_start, &c->vbin_cursor,
-                    &c->vbin_cell, &c->vbin_list, &c->labels, &c->band, &c->tile_edges, &c->edge_start,
+                    &c->vbin_cell, &c->vbin_list, &c->labels, &c->band, &c->cls_list, &c->etiles, &c->tile_edges, &c->edge_start,
                     &c->tile_inside, &c->scan_tmp, &c->misc, &c->av, &c->counts, &c->red_d, &c->red_i, &c->fail_log,
                     &c->ovf, &c->big, &c->r_einfo, &c->r_ecnt, &c->r_csph, &c->r_ctor, &c->r_nsph, &c->r_ntor,
                     &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_hard2, &c->r_jobs, &c->atom_hi,

@@ -278,14 +278,7 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
         if (threadIdx.x == 0 && S.flags) atomicOr(err, S.flags);
         int t[3];
         tile_coords(G, tile, t);
-        if (S.na == 0) {  // no atom within reach: every point is free
-            for (int p = threadIdx.x; p < TILE_PTS; p += CLS_THREADS) {
-                int li = p >> 6, lj = (p >> 3) & 7, lk = p & 7;
-                long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
-                          gk = (long long)TILE * t[2] + lk;
-                if (gi < G.dims[0] && gj < G.dims[1] && gk < G.dims[2])
-                    labels[(gi * G.dims[1] + gj) * G.dims[2] + gk] = LABEL_OUT;
-            }
+        if (S.na == 0) {  // no atom within reach: every point is free (the labels start as outside)
             __syncthreads();
             continue;
         }
@@ -472,6 +465,53 @@ __global__ void __launch_bounds__(CLS_THREADS) k_band(Model M, Batch B, int8_t *
     const int n = list[0];
     for (int k = blockIdx.x; k < n; k += gridDim.x)
         band_tile<CP>(M, B, list[1 + k], labels_all, S, sG, s_pts, s_np, err, ovf, BIG);
+}
+
+// The tiles whose staging range of cells holds an atom, one thread per tile
+// (the range of stage_tile): the others are outside everywhere, and a CTA that
+// staged them spent 13,000 cycles to find out (half the tiles of a molecule's
+// box at h 0.5).
+__global__ void __launch_bounds__(256) k_tile_list(Model M, Batch B, int *__restrict__ list)
+{
+    const int lane = threadIdx.x & 31;
+    for (long long g0 = (long long)blockIdx.x * 256 + (threadIdx.x & ~31); g0 < B.n_tiles;
+         g0 += (long long)gridDim.x * 256) {
+        const long long gt = g0 + lane;
+        bool any = false;
+        if (gt < B.n_tiles) {
+            const int mol = mol_of_tile(B, gt);
+            const Grid &G = B.grid[mol];
+            const CellGrid &CG = M.cg[mol];
+            int t[3], c0[3], c1[3];
+            tile_coords(G, gt - G.tile0, t);
+            const float icell = 1.0f / (float)M.cell, halo = (float)G.halo + 1e-2f;
+            for (int a = 0; a < 3; ++a) {
+                const double fx0 = G.lo[a] + G.h * (double)(TILE * (t[a] + G.toff[a]));
+                const double fx1 = fx0 + G.h * (double)TILE;
+                c0[a] = max((int)floorf(((float)(fx0 - CG.clo[a]) - halo) * icell), 0);
+                c1[a] = min((int)floorf(((float)(fx1 - CG.clo[a]) + halo) * icell), CG.cn[a] - 1);
+            }
+            if (c0[2] <= c1[2])
+                for (int x = c0[0]; x <= c1[0] && !any; ++x)
+                    for (int y = c0[1]; y <= c1[1] && !any; ++y) {
+                        const int id = CG.coff + (x * CG.cn[1] + y) * CG.cn[2];
+                        any = M.cell_start[id + c1[2] + 1] > M.cell_start[id + c0[2]];
+                    }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, any);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(&list[0], __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (any) list[1 + base + __popc(m & ((1u << lane) - 1u))] = (int)gt;
+    }
+}
+
+int launch_tile_list(const Model &M, const Batch &B, int *list, cudaStream_t st)
+{
+    cudaMemsetAsync(list, 0, sizeof(int), st);
+    const long long nb = ceil_div_ll(std::max(B.n_tiles, 1LL), 256);
+    k_tile_list<<<(unsigned)std::min(nb, 65536LL), 256, 0, st>>>(M, B, list);
+    return 1;
 }
 
 static long long g_band_grid = 1;  // resident k_band CTAs on the device

@@ -55,6 +55,8 @@ int launch_bin_scatter(const Model &M, int which, const int *item_cell, const in
 // persistent: `grid` CTAs take tiles in the order of Q (labels of the whole batch)
 void classify_init();
 int classify_ctas_per_sm(int precision);
+// the tiles that some atom's cell reaches: list = int[1 + tiles], their number, then the tiles (any order)
+int launch_tile_list(const Model &M, const Batch &B, int *list, cudaStream_t st);
 // ovf: int[2 + tiles] scratch (tiles sent to the global-memory tier over the
 // run, the stage's count, then the tiles that overflowed the shared-memory
 // staging); big: classify_big_bytes() of global scratch for that tier
@@ -75,7 +77,8 @@ int launch_ext_fill(const Batch &B, uint16_t *ext, uint8_t *tile_open, int *flag
 int launch_ext_apply(const Batch &B, int8_t *labels, const uint16_t *ext, unsigned long long *filled, cudaStream_t st);
 
 // ---- crossing edges, roots, area/volume (eses_edges.cu) ------------------
-int launch_edge_count(const Batch &B, const int8_t *labels, int *tile_edges, int *tile_inside_edges,
+// etiles: int[1 + tiles], the number of tiles with crossing edges, then those tiles
+int launch_edge_count(const Batch &B, const int8_t *labels, int *tile_edges, int *tile_inside_edges, int *etiles,
                       cudaStream_t st);
 // medge[a * (n_mol + 1) + m]: first edge of molecule m in axis a's output
 int launch_mol_edges(const Batch &B, const int *edge_start, long long *medge, cudaStream_t st);
