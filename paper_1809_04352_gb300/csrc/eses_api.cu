@@ -38,6 +38,27 @@ namespace {
 struct DBuf {
     void *p = nullptr;
     size_t cap = 0;
+    bool pooled = false;  // lies in a block of the context's pool
+};
+
+// A context's device memory.  A run takes about a hundred buffers, most of a
+// few kB; a cudaMalloc and a cudaFree each (13 us apiece) were 2.6 ms of the
+// 4.9 ms in which a 1,501-atom molecule is created, run, read and destroyed.
+// Buffers up to POOL_MAX bytes lie in blocks that the context allocates, each
+// as large as everything it holds so far (POOL_MIN .. POOL_MAX: up to there a
+// block costs the same 80 us to take and 60 us to give back; so at most half
+// of a large context's pool is unused), and larger ones are allocated alone.
+// What a grown buffer leaves is taken again by the next one that fits.  One
+// thread uses a context at a time; destroying it gives every block back.
+constexpr size_t POOL_MIN = (size_t)16 << 20, POOL_MAX = (size_t)128 << 20, POOL_ALIGN = 512;
+struct Pool {
+    struct Span {
+        char *p;
+        size_t n;
+    };
+    std::vector<void *> blocks;
+    std::vector<Span> left;  // unused spans
+    size_t total = 0;
 };
 
 struct CudaError {
@@ -51,12 +72,58 @@ void ck(cudaError_t e, const char *what)
 }
 
 struct CaptureGrow {};  // a buffer would have to grow during graph capture
+struct NeedBig {};      // a tile overflows the shared-memory staging and the global-memory tier's scratch is not there yet
 
 thread_local bool g_capturing = false;
 // allocation-failure injection (ESES_OPT_FAIL_ALLOC): the calling context's
 // countdown while one of its entry points runs; the allocation that brings it
 // to zero fails before cudaMalloc is called
 thread_local long long *g_fail_countdown = nullptr;
+// the calling context's pool while one of its entry points runs
+thread_local Pool *g_pool = nullptr;
+
+void *device_alloc(size_t bytes)
+{
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        throw std::bad_alloc();
+    }
+    return p;
+}
+
+// `bytes` (a multiple of POOL_ALIGN) from the smallest unused span that holds
+// them, or from a new block
+void *pool_take(Pool &P, size_t bytes)
+{
+    size_t best = P.left.size();
+    for (size_t k = 0; k < P.left.size(); ++k)
+        if (P.left[k].n >= bytes && (best == P.left.size() || P.left[k].n < P.left[best].n)) best = k;
+    if (best == P.left.size()) {
+        const size_t n = std::max(bytes, std::min(std::max(P.total, POOL_MIN), POOL_MAX));
+        P.blocks.reserve(P.blocks.size() + 1);  // (nothing may throw once the block is there)
+        P.left.reserve(P.left.size() + 1);
+        char *b = (char *)device_alloc(n);
+        P.blocks.push_back(b);
+        P.total += n;
+        P.left.push_back(Pool::Span{b, n});
+    }
+    Pool::Span &s = P.left[best];
+    void *p = s.p;
+    s.p += bytes;
+    s.n -= bytes;
+    if (s.n == 0) {
+        s = P.left.back();
+        P.left.pop_back();
+    }
+    return p;
+}
+
+void free_buf(DBuf &b)
+{
+    if (b.p && !b.pooled) cudaFree(b.p);
+    b = DBuf();
+}
 
 template <class T>
 T *ensure(DBuf &b, size_t count)
@@ -64,18 +131,17 @@ T *ensure(DBuf &b, size_t count)
     size_t bytes = std::max<size_t>(count * sizeof(T), 16);
     if (b.cap < bytes) {
         if (g_capturing) throw CaptureGrow{};
-        if (b.p) cudaFree(b.p);
-        b.p = nullptr;
-        b.cap = 0;
-        size_t want = bytes + bytes / 4;
-        if (g_fail_countdown && *g_fail_countdown > 0 && --*g_fail_countdown == 0) throw std::bad_alloc();
-        cudaError_t e = cudaMalloc(&b.p, want);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            b.p = nullptr;
+        const size_t want = (bytes + bytes / 4 + POOL_ALIGN - 1) / POOL_ALIGN * POOL_ALIGN;
+        if (g_fail_countdown && *g_fail_countdown > 0 && --*g_fail_countdown == 0) {
+            if (!b.pooled) free_buf(b);
             throw std::bad_alloc();
         }
+        if (b.pooled && g_pool) g_pool->left.push_back(Pool::Span{(char *)b.p, b.cap});
+        free_buf(b);
+        const bool pooled = g_pool && want <= POOL_MAX;
+        b.p = pooled ? pool_take(*g_pool, want) : device_alloc(want);
         b.cap = want;
+        b.pooled = pooled;
     }
     return (T *)b.p;
 }
@@ -129,6 +195,7 @@ struct eses_ctx {
     Model M{};
     Batch B{};
     // device buffers
+    Pool pool;
     DBuf xyz, rad, in_mol, grid_d, cg_d, tile_off_d, atom_mol, vert_mol, medge, term, queue;
     DBuf cell_id, cell_count, cell_start, cursor, atom_scat, atom_cell, atom_orig, atom;
     DBuf nb_count, nb_start, nb_list, circle_count, contained, face;
@@ -140,6 +207,7 @@ struct eses_ctx {
     DBuf out_idx[3], out_tau[3], out_nrm[3], out_tau32[3], out_nrm32[3], out_code[3];
     DBuf scan_tmp, misc, av, counts, red_d, red_i;  // misc: err, n_fail
     DBuf fail_log;
+    bool use_big = false;  // a run of this context had a tile for the global-memory tier
     DBuf ovf, big;  // tiles that overflow the shared-memory staging, and the global-memory tier's scratch
     // phased root solve: edge records, candidates, their roots, staged tiles (slabs), counters, hard edges
     DBuf r_einfo, r_ecnt, r_csph, r_ctor, r_nsph, r_ntor, r_rsph, r_rtor, r_slab, r_ctr, r_hard, r_hard2, r_jobs;
@@ -166,6 +234,7 @@ struct eses_ctx {
     // triangle mesh of the last run (eses_mesh_count / eses_mesh)
     DBuf mesh_mask, mesh_tile, mesh_off, mesh_keys, mesh_xyz, mesh_err, mesh_tot;
     long long n_tri = -1;  // -1: not made for the current results
+    bool mesh_ready = false;
     long long n_cavity = 0;
     int ext_sweeps = 0;
     // learned tile proposer
@@ -209,6 +278,23 @@ void drop_graph(eses_ctx *c)
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
 }
+
+// points allocations at the context's pool and failure countdown for one entry
+// point (nested ones keep theirs)
+struct AllocScope {
+    Pool *pool;
+    long long *countdown;
+    explicit AllocScope(eses_ctx *c) : pool(g_pool), countdown(g_fail_countdown)
+    {
+        g_pool = &c->pool;
+        g_fail_countdown = &c->fail_alloc;
+    }
+    ~AllocScope()
+    {
+        g_pool = pool;
+        g_fail_countdown = countdown;
+    }
+};
 
 int scan(eses_ctx *c, const int *in, int *out, long long n)
 {
@@ -451,13 +537,13 @@ int create_common(const double *hxyz, const double *hr, const int64_t *counts, i
             c->given_dims[a] = grid_dims[a];
         }
     }
+    AllocScope scope(c);
     try {
         ck(cudaGetDevice(&c->device), "cudaGetDevice");
         ck(cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device), "device attribute");
         classify_init();
         edges_init();
         mlp_init();
-        if (mesh_init() != 0) throw CudaError{cudaErrorInvalidValue, "mesh case table"};
         ck(cudaGetLastError(), "kernel attributes");
         ck(cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking), "cudaStreamCreate");
         c->stream = c->own_stream;
@@ -504,13 +590,6 @@ int create_common(const double *hxyz, const double *hr, const int64_t *counts, i
     }
     *out = c;
     return ESES_OK;
-}
-
-void free_buf(DBuf &b)
-{
-    if (b.p) cudaFree(b.p);
-    b.p = nullptr;
-    b.cap = 0;
 }
 
 void mark(eses_ctx *c, int k)
@@ -754,7 +833,10 @@ int run_device(eses_ctx *c)
     cls_tiles(c, cq);
     int *ovf = ensure<int>(c->ovf, (size_t)nt + 2);
     ck(cudaMemsetAsync(ovf, 0, sizeof(int), st), "memset");
-    unsigned char *big = ensure<unsigned char>(c->big, std::max(classify_big_bytes(), edges_big_bytes()));
+    // the global-memory tier's scratch (tens of MB) is taken once a run has had
+    // a tile for it (NeedBig); until then its launches are left out
+    unsigned char *big = nullptr;
+    if (c->use_big) big = ensure<unsigned char>(c->big, std::max(classify_big_bytes(), edges_big_bytes()));
     nl += launch_classify(M, B, c->precision, cq, grid_of(c, c->cls, classify_ctas_per_sm(c->precision)), labels,
                           c->precision == ESES_PREC_FP64 ? nullptr : band, d_err, ovf, big, d_tests, st);
     mark(c, ST_BAND);
@@ -810,7 +892,10 @@ int run_device(eses_ctx *c)
         for (int a = 0; a < 3; ++a)
             ck(cudaMemcpyAsync(&tot[a], edge_start + a * nt, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
         ck(cudaMemcpyAsync(&tot[3], edge_start + 3 * nt, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
+        int ov = 0;
+        ck(cudaMemcpyAsync(&ov, ovf, sizeof(ov), cudaMemcpyDeviceToHost, st), "read");
         ck(cudaStreamSynchronize(st), "synchronize");
+        if (ov > 0 && !c->use_big) throw NeedBig{};
         for (int a = 0; a < 3; ++a) c->n_edges[a] = (long long)tot[a + 1] - tot[a];
     }
     EdgeOut eo;
@@ -841,6 +926,7 @@ int run_device(eses_ctx *c)
         ck(cudaMemcpyAsync(need, W.ctr, sizeof(need), cudaMemcpyDeviceToHost, st), "read");
         ck(cudaMemcpyAsync(ov, ovf, sizeof(ov), cudaMemcpyDeviceToHost, st), "read");
         ck(cudaStreamSynchronize(st), "synchronize");
+        if (ov[0] > 0 && !c->use_big) throw NeedBig{};
         if ((long long)need[0] > W.cap_slab || (long long)need[1] > W.cap_sph || (long long)need[2] > W.cap_tor) {
             c->cap_slab = std::max(c->cap_slab, (long long)(need[0] + need[0] / 8));
             c->cap_sph = std::max(c->cap_sph, (long long)(need[1] + need[1] / 8));
@@ -927,6 +1013,7 @@ int finish(eses_ctx *c, int nl)
     c->stats[17] = (long long)rctr[1];
     c->stats[18] = (long long)rctr[2];
     c->stats[19] = (long long)rctr[c->precision == ESES_PREC_FP64 ? 3 : 5];
+    if (hovf > 0 && !c->use_big) throw NeedBig{};
     c->ran = true;
     int derr = hmisc[0];
     if ((long long)rctr[4] > c->cap_jobs) derr |= ERR_CAP_CAND;  // the FP64 job list was full (never planned so)
@@ -1024,11 +1111,6 @@ void apply_box(eses_ctx *c)
     c->ran = false;
 }
 
-// points the allocation-failure countdown at the context for one entry point
-struct AllocScope {
-    explicit AllocScope(eses_ctx *c) { g_fail_countdown = &c->fail_alloc; }
-    ~AllocScope() { g_fail_countdown = nullptr; }
-};
 
 int run_guarded(eses_ctx *c)
 {
@@ -1046,7 +1128,9 @@ int run_guarded(eses_ctx *c)
     } catch (const CudaError &e) {
         return fail(c, ESES_ECUDA, std::string(e.what) + ": " + cudaGetErrorString(e.e));
     } catch (const std::bad_alloc &) {
-        // buffers may be half sized: the next run plans again
+        // buffers may be half sized: the next run plans again; kernels already
+        // enqueued end first (the pool hands their buffers out again)
+        cudaStreamSynchronize(c->stream);
         drop_graph(c);
         c->planned = false;
         return fail(c, ESES_ENOMEM, "device allocation failed");
@@ -1054,6 +1138,11 @@ int run_guarded(eses_ctx *c)
         // a buffer the plan did not size: plan again (eagerly), capture next time
         drop_graph(c);
         c->planned = false;
+        return run_guarded(c);
+    } catch (const NeedBig &) {
+        drop_graph(c);
+        c->planned = false;
+        c->use_big = true;  // (once: with it no run throws this)
         return run_guarded(c);
     } catch (const std::string &m) {
         return fail(c, ESES_EINVAL, m);
@@ -1325,12 +1414,12 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                     cls_tiles(c, q);
                     launch_classify(M, B, c->precision, q, grid_of(c, s, cls_max), labels,
                                     c->precision == ESES_PREC_FP64 ? nullptr : band, misc, (int *)c->ovf.p,
-                                    (unsigned char *)c->big.p, nullptr, st);
+                                    c->use_big ? (unsigned char *)c->big.p : nullptr, nullptr, st);
                 });
                 if (ms < best_cls_ms) best_cls_ms = ms, best_cls = s;
             }
         if (c->precision != ESES_PREC_FP64)
-            launch_band(M, B, labels, band, misc, (int *)c->ovf.p, (unsigned char *)c->big.p, st);
+            launch_band(M, B, labels, band, misc, (int *)c->ovf.p, c->use_big ? (unsigned char *)c->big.p : nullptr, st);
         // root solve: staging CTAs per SM x tiles per pop x root-kernel threads per block
         Shape best_edge = c->edge;
         float best_edge_ms = INFINITY;
@@ -1377,7 +1466,7 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                         q.list_n = (const int *)c->etiles.p;
                         launch_edge_stage(M, B, c->precision, q, grid_of(c, s, edge_max), labels,
                                           (const int *)c->edge_start.p, eo, misc, (int *)c->ovf.p,
-                                          (unsigned char *)c->big.p, W, st);
+                                          c->use_big ? (unsigned char *)c->big.p : nullptr, W, st);
                         launch_edge_roots(M, B, c->precision, threads, eo, (const int *)c->edge_start.p, ne_all,
                                           misc + 1, misc, (long long *)c->fail_log.p, W, st);
                     });
@@ -1482,6 +1571,9 @@ int eses_mol_labels(const eses_ctx *cc, int m, int8_t *out)
     if (!c->sel) {
         const size_t n = (size_t)mol_points(c, m);
         ok = cudaMemcpyAsync(out, src, n, cudaMemcpyDeviceToHost, c->stream) == cudaSuccess;
+    } else if (G.own[1] == G.dims[1] && G.own[2] == G.dims[2]) {  // whole layers: they lie together
+        ok = cudaMemcpyAsync(out, src, (size_t)(G.own[0] * G.own[1] * G.own[2]), cudaMemcpyDeviceToHost, c->stream) ==
+             cudaSuccess;
     } else {  // the owned box out of the computed box, one plane at a time
         for (long long i = 0; i < G.own[0] && ok; ++i)
             ok = cudaMemcpy2DAsync(out + i * G.own[1] * G.own[2], (size_t)G.own[2], src + i * G.dims[1] * G.dims[2],
@@ -1823,6 +1915,10 @@ int eses_mesh_count(eses_ctx *c, int64_t *n_tri)
     AllocScope scope(c);
     try {
         ck(cudaSetDevice(c->device), "cudaSetDevice");
+        if (!c->mesh_ready) {  // the case table, once per context that makes a mesh
+            if (mesh_init() != 0) throw CudaError{cudaErrorInvalidValue, "mesh case table"};
+            c->mesh_ready = true;
+        }
         if (c->n_tri < 0) {
             cudaStream_t st = c->stream;
             const long long nt = c->n_tiles;
@@ -1966,6 +2062,7 @@ void eses_destroy(eses_ctx *c)
     }
     for (int k = 0; k <= NSTAGE; ++k)
         if (c->ev[k]) cudaEventDestroy(c->ev[k]);
+    for (void *b : c->pool.blocks) cudaFree(b);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
     delete c;
 }

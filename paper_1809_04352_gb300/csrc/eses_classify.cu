@@ -572,15 +572,17 @@ int launch_classify(const Model &M, const Batch &B, int precision, const TileSch
     if (precision == 0) {
         k_classify<double, false, CapMid, false><<<grid, CLS_THREADS, cls_bytes<double, CapMid>(), st>>>(
             M, B, Q, labels, band, err, ovf, nullptr, n_tests);
-        k_classify<double, false, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
+        if (big)
+            k_classify<double, false, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
                                                                                big, n_tests);
     } else {
         k_classify<float, true, CapMid, false><<<grid, CLS_THREADS, cls_bytes<float, CapMid>(), st>>>(
             M, B, Q, labels, band, err, ovf, nullptr, n_tests);
-        k_classify<float, true, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
+        if (big)
+            k_classify<float, true, CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, QB, labels, band, err, ovf,
                                                                              big, n_tests);
     }
-    return 2;
+    return big ? 2 : 1;
 }
 
 int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *band, int *err, int *ovf,
@@ -590,8 +592,8 @@ int launch_band(const Model &M, const Batch &B, int8_t *labels, const int *band,
     cudaMemsetAsync(ovf + 1, 0, sizeof(int), st);
     k_band<CapSmall, false><<<(int)grid, CLS_THREADS, band_bytes<CapSmall>(), st>>>(M, B, labels, band, err, ovf,
                                                                                  nullptr);
-    k_band<CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, labels, band, err, ovf, big);
-    return 2;
+    if (big) k_band<CapBig, true><<<g_n_sm, CLS_THREADS, 0, st>>>(M, B, labels, band, err, ovf, big);
+    return big ? 2 : 1;
 }
 
 }  // namespace eses

@@ -2387,6 +2387,7 @@ static void stage_launch(const Model &M, const Batch &B, const TileSched &Q, int
     k_edge_stage<T, FILT, CapMid, false><<<grid, EDGE_THREADS, stage_smem<T>(), st>>>(M, B, Q, labels, edge_start,
                                                                                        out, err, ovf, nullptr, W);
     TileSched QB{nullptr, 1, ovf + 2, ovf + 1};
+    if (!big) return;
     k_edge_stage<T, FILT, CapBig, true><<<g_edge_n_sm, EDGE_THREADS, sizeof(StageSmem), st>>>(
         M, B, QB, labels, edge_start, out, err, ovf, big, W);
 }
@@ -2424,7 +2425,7 @@ int launch_edge_stage(const Model &M, const Batch &B, int precision, const TileS
         stage_launch<double, false>(M, B, Q, grid, labels, edge_start, out, err, ovf, big, W, st);
     else
         stage_launch<float, true>(M, B, Q, grid, labels, edge_start, out, err, ovf, big, W, st);
-    return 2;
+    return big ? 2 : 1;
 }
 
 int launch_edge_roots(const Model &M, const Batch &B, int precision, int threads, EdgeOut out,

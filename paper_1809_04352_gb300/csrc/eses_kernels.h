@@ -59,7 +59,7 @@ int classify_ctas_per_sm(int precision);
 int launch_tile_list(const Model &M, const Batch &B, int *list, cudaStream_t st);
 // ovf: int[2 + tiles] scratch (tiles sent to the global-memory tier over the
 // run, the stage's count, then the tiles that overflowed the shared-memory
-// staging); big: classify_big_bytes() of global scratch for that tier
+// staging); big: classify_big_bytes() of global scratch for that tier (null: it is not launched)
 // band (null: FP64 form): int[1 + tiles], the number of tiles with undecided points, then those tiles;
 // n_tests (may be null): adds up the atom tests of the shell points' witness freeness
 int launch_classify(const Model &M, const Batch &B, int precision, const TileSched &Q, int grid, int8_t *labels,

@@ -94,3 +94,38 @@ def test_circle_with_many_free_end_points():
                 assert np.abs(g["tau"][o] - ref.tau[a]).max() * 1.5 < 1e-6
     finally:
         eses.eses_destroy(ctx)
+
+
+def test_buffers_left_by_grown_ones_are_taken_again():
+    """Runs of changing size in one context (block selections up and down, the
+    whole grid) reuse the memory they gave up: after the first round the
+    device's free memory stays where it is, the results stay the same, and
+    destroying the context gives everything back."""
+    import torch
+
+    libbuild.build()
+    torch.cuda.synchronize()
+    free0, _ = torch.cuda.mem_get_info()
+    xyz, rad = inputs.protein_like(600, 4, inputs.PROTEIN_DENSITY)
+    ctx = eses.eses_create(xyz, rad, 1.4, 0.3, 0.8)
+    try:
+        eses.eses_set_option(ctx, eses.ESES_OPT_BLOCK_PTS, 16)
+        nb = eses.eses_num_blocks(ctx)
+        seen, free = {}, []
+        for cycle in range(4):
+            for cut in (1, int(nb[0]), 2, int(nb[0]) - 1, None):
+                if cut is None:
+                    eses.eses_set_blocks(ctx)
+                else:
+                    eses.eses_set_blocks(ctx, [0, 0, 0], [cut, int(nb[1]), int(nb[2])])
+                eses.eses_run(ctx)
+                got = (eses.eses_labels(ctx).tobytes(), *[eses.eses_intersections(ctx, a)["idx"].tobytes()
+                                                          for a in range(3)], eses.eses_area_volume(ctx))
+                assert seen.setdefault(cut, got) == got
+            free.append(torch.cuda.mem_get_info()[0])
+        assert free[1:] == free[1:2] * 3
+    finally:
+        eses.eses_destroy(ctx)
+    torch.cuda.synchronize()
+    free1, _ = torch.cuda.mem_get_info()
+    assert abs(free1 - free0) <= 1 << 20
