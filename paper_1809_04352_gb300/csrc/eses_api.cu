@@ -210,7 +210,7 @@ struct eses_ctx {
     bool use_big = false;  // a run of this context had a tile for the global-memory tier
     DBuf ovf, big;  // tiles that overflow the shared-memory staging, and the global-memory tier's scratch
     // phased root solve: edge records, candidates, their roots, staged tiles (slabs), counters, hard edges
-    DBuf r_einfo, r_ecnt, r_csph, r_ctor, r_nsph, r_ntor, r_rsph, r_rtor, r_slab, r_ctr, r_hard, r_hard2, r_jobs;
+    DBuf r_einfo, r_ecnt, r_csph, r_ctor, r_nsph, r_ntor, r_rsph, r_rtor, r_slab, r_ctr, r_hard, r_hard2, r_ties, r_jobs;
     long long cap_sph = 0, cap_tor = 0, cap_slab = 0, cap_jobs = 0;  // planned capacities
     DBuf atom_hi, atom_lo, pair_hi, pair_lo, pair_u32, vert_hi, vert_lo;
     // plan: list sizes of the first run (the inputs never change)
@@ -649,6 +649,8 @@ RootWork root_work(eses_ctx *c, long long ne_all)
     W.ecnt = ensure<int>(c->r_ecnt, (size_t)ne);
     W.hard = ensure<int>(c->r_hard, (size_t)ne);
     W.hard2 = ensure<int>(c->r_hard2, (size_t)ne);
+    W.cap_ties = ne / 4 + 1024;  // (about one per 25 edges; a tie that finds no room is settled by its warp)
+    W.ties = ensure<int4>(c->r_ties, (size_t)W.cap_ties);
     W.csph = ensure<int2>(c->r_csph, (size_t)c->cap_sph);
     W.nsph = ensure<uint8_t>(c->r_nsph, (size_t)c->cap_sph);
     W.rsph = ensure<RootRec>(c->r_rsph, 2 * (size_t)c->cap_sph);
@@ -1437,6 +1439,7 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
         W.ecnt = (int *)c->r_ecnt.p;
         W.hard = (int *)c->r_hard.p;
         W.hard2 = (int *)c->r_hard2.p;
+        W.ties = (int4 *)c->r_ties.p;
         W.csph = (int2 *)c->r_csph.p;
         W.nsph = (uint8_t *)c->r_nsph.p;
         W.rsph = (RootRec *)c->r_rsph.p;
@@ -1452,6 +1455,7 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
         W.cap_tor = c->cap_tor;
         const long long ne_all = c->n_edges[0] + c->n_edges[1] + c->n_edges[2];
         W.n_edges = ne_all;
+        W.cap_ties = std::max(ne_all, 1LL) / 4 + 1024;
         for (int k = 1; k <= edge_max; ++k)
             for (int per : {1, 4})
                 for (int threads : {128, 256}) {
@@ -2044,7 +2048,7 @@ void eses_destroy(eses_ctx *c)
                     &c->vbin_cell, &c->vbin_list, &c->labels, &c->band, &c->cls_list, &c->etiles, &c->tile_edges, &c->edge_start,
                     &c->tile_inside, &c->scan_tmp, &c->misc, &c->av, &c->counts, &c->red_d, &c->red_i, &c->fail_log,
                     &c->ovf, &c->big, &c->r_einfo, &c->r_ecnt, &c->r_csph, &c->r_ctor, &c->r_nsph, &c->r_ntor,
-                    &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_hard2, &c->r_jobs, &c->atom_hi,
+                    &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_hard2, &c->r_ties, &c->r_jobs, &c->atom_hi,
                     &c->atom_lo, &c->pair_hi, &c->pair_lo, &c->pair_u32, &c->vert_hi, &c->vert_lo,
                     &c->mlp_params, &c->need, &c->need_pos, &c->tile_list, &c->prop_counts, &c->features,
                     &c->targets, &c->ext, &c->ext_open, &c->ext_misc, &c->mesh_mask, &c->mesh_tile, &c->mesh_off,

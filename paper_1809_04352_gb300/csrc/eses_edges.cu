@@ -33,7 +33,7 @@
 //     inside or one candidate is left and the FP32 bounds order the
 //     candidates; the other edges are listed;
 //   k_edge_settle: one thread per listed edge: the outside end points that the
-//     candidates' own witnesses decide;
+//     candidates' own witnesses decide; k_edge_ties: FP64 roots of near ties;
 //   k_edge_hard: one warp per edge left: near ties broken on FP64 roots; at
 //     an outside end point each earlier candidate tested first against the
 //     later candidates' witnesses, then by the full witness search, whose
@@ -1836,10 +1836,14 @@ __global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Batch B, RootWork W,
 // candidate is strictly outside M and dropped, and the last one left is the
 // root -- warp_select's first test with its tolerances, so an edge takes the
 // same candidate on either path.  A tie that the FP32 bounds cannot order, a
-// test that is not certain, an inside end point or more than SETTLE_MAX
-// candidates leave the edge to the warp selection (W.hard2).
+// test that is not certain or more than SETTLE_MAX candidates leave the edge to
+// the warp selection (W.hard2); the tied candidates are listed (W.ties) and
+// their FP64 roots computed in full warps before it (k_edge_ties).
 // On the 5,000-atom globule 388 k of the warps' 653 k iterations were this
-// test, 545 warp instructions for one lane's work each.
+// test, 545 warp instructions for one lane's work each, and the near ties held
+// the FP64 pipe with two lanes of 32.  Bound by the latency of an edge's
+// dependent reads (eight lanes an edge, one per candidate, took 356 us for the
+// 266 k edges against 250).
 constexpr int SETTLE_MAX = 6;
 constexpr int SETTLE_THREADS = 128;
 
@@ -1861,7 +1865,7 @@ __global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B
             const int ns = cnt & 0xffff, nq = (cnt >> 16) & 0xffff;
             const int pk = inf.y, axis = pk_axis(pk), lab = pk_label(pk), p = pk_point(pk);
             left = true;
-            if (!pk_dropped(pk) && lab != LABEL_IN) {
+            if (!pk_dropped(pk)) {
                 const unsigned char *sl = W.slab + ((size_t)(unsigned)inf.x << 4);
                 const SlabHdr *hd = reinterpret_cast<const SlabHdr *>(sl);
                 const Grid &G = B.grid[__ldg(&hd->mol)];
@@ -1897,6 +1901,7 @@ __global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B
                 }
                 unsigned alive = n >= 1 && n <= SETTLE_MAX ? (1u << n) - 1u : 0u;
                 int pick = -1;
+                float tie_t = INFINITY, tie_e = 0.0f;  // a tie's first candidate
                 while (alive) {
                     // the first candidate left, and whether the bounds order it before the others
                     int k = -1, kk = 0, ki = 0;
@@ -1917,9 +1922,13 @@ __global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B
 #pragma unroll
                     for (int z = 0; z < SETTLE_MAX; ++z)
                         if (((alive >> z) & 1u) && z != k && t[z] - tk <= err[z] + ek + tie) tied = true;
-                    if (tied) break;
+                    if (tied) {
+                        tie_t = tk;
+                        tie_e = ek;
+                        break;
+                    }
                     const unsigned rest = alive & ~(1u << k);
-                    if (rest == 0u) {
+                    if (rest == 0u || lab == LABEL_IN) {
                         pick = k;
                         break;
                     }
@@ -1952,6 +1961,24 @@ __global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B
                     if (!outside) break;  // not certain: the full search decides
                     alive = rest;
                 }
+                if (tie_t < INFINITY) {  // its roots without an FP64 value yet
+                    for (int j = 0; j < ns + nq; ++j) {
+                        const bool sph = j < ns;
+                        const int k = sph ? inf.z + j : inf.w + (j - ns);
+                        const int nr = sph ? W.nsph[k] : W.ntor[k];
+                        for (int r = 0; r < nr; ++r) {
+                            const RootRec c = sph ? W.rsph[(size_t)SPH_SLOTS * k + r] : W.rtor[(size_t)TOR_SLOTS * k + r];
+                            if (!(c.t >= tie_t && c.t < INFINITY) || c.err < 0.0f || c.t64 == c.t64 ||
+                                c.t - tie_t > c.err + tie_e + tie)
+                                continue;
+                            const int it = sph ? W.csph[k].y : W.ctor[k].y;
+                            const unsigned long long z = atomicAdd(W.ctr + 6, 1ull);
+                            if (z < (unsigned long long)W.cap_ties)
+                                W.ties[z] = make_int4(g, k, r | ((sph ? (it < na ? 0 : 2) : 1) << 4),
+                                                      sph && it >= na ? it - na : it);
+                        }
+                    }
+                }
                 if (pick >= 0) {
                     left = false;
                     float tr = 0.0f;
@@ -1973,6 +2000,26 @@ __global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B
         if (lane == 0 && m) base = (int)atomicAdd(W.ctr + 5, (unsigned long long)__popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (left) W.hard2[base + __popc(m & ((1u << lane) - 1))] = g;
+    }
+}
+
+// FP64 roots of the listed tied candidates, one thread each, into their records.
+__global__ void __launch_bounds__(128) k_edge_ties(Model M, Batch B, RootWork W)
+{
+    const long long n = min((long long)W.ctr[6], W.cap_ties);
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
+        const int4 jb = W.ties[q];
+        const int4 inf = W.einfo[jb.x];
+        const int kind = jb.z >> 4, r = jb.z & 15, p = pk_point(inf.y);
+        const unsigned char *sl = W.slab + ((size_t)(unsigned)inf.x << 4);
+        const SlabHdr *hd = reinterpret_cast<const SlabHdr *>(sl);
+        const double x0[3] = {__ldg(&hd->x0[0]), __ldg(&hd->x0[1]), __ldg(&hd->x0[2])};
+        const double h = B.grid[__ldg(&hd->mol)].h;
+        const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
+        const SlabAcc<float> A(sl);
+        const SlabExact<float> X(A, M, x0);
+        RootRec *rec = kind == 1 ? W.rtor + (size_t)TOR_SLOTS * jb.y + r : W.rsph + (size_t)SPH_SLOTS * jb.y + r;
+        rec->t64 = staged_exact_root(X, kind, jb.w, s64, pk_axis(inf.y), M.rp, (double)rec->t);
     }
 }
 
@@ -2401,17 +2448,20 @@ static void roots_launch(const Model &M, const Batch &B, int threads, EdgeOut ou
     const int gs = std::max(g_occ_roots[P][0][ts], 1) * g_edge_n_sm;
     const int gq = std::max(g_occ_roots[P][1][ts], 1) * g_edge_n_sm;
     k_roots_sphere<T, FILT><<<gs, tb, 0, st>>>(M, B, W, err);
-    cudaMemsetAsync(W.ctr + 3, 0, 3 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, hard edges
+    cudaMemsetAsync(W.ctr + 3, 0, 4 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, hard edges, ties
     k_roots_torus<T, FILT><<<gq, tb, 0, st>>>(M, B, W, err);
     if (FILT)
         k_roots_torus_exact<T, FILT><<<std::max(g_occ_exact[P], 1) * g_edge_n_sm, tb, 0, st>>>(M, B, W, err);
     const long long pb = std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, PICK_THREADS), 1),
                                              8LL * g_edge_n_sm);
     k_edge_pick<T><<<(unsigned)pb, PICK_THREADS, 0, st>>>(B, W, edge_start, ne_all, out, err);
-    if (FILT)
+    if (FILT) {
         k_edge_settle<<<(unsigned)std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, 4 * SETTLE_THREADS), 1),
                                                       8LL * g_edge_n_sm),
                         SETTLE_THREADS, 0, st>>>(M, B, W, edge_start, out);
+        k_edge_ties<<<(unsigned)std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, 1024), 1), 8LL * g_edge_n_sm),
+                      128, 0, st>>>(M, B, W);
+    }
     k_edge_hard<T, FILT><<<std::max(g_occ_hard[P], 1) * g_edge_n_sm, HARD_THREADS, 0, st>>>(
         M, B, W, edge_start, out, n_fail, err, fail_log);
 }
@@ -2437,7 +2487,7 @@ int launch_edge_roots(const Model &M, const Batch &B, int precision, int threads
         roots_launch<double, false>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
     else
         roots_launch<float, true>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
-    return precision == 0 ? 4 : 6;
+    return precision == 0 ? 4 : 7;
 }
 
 long long polish_blocks(long long n_edges) { return n_edges > 0 ? ceil_div_ll(n_edges, POLISH_THREADS) : 0; }

@@ -106,7 +106,8 @@ struct RootRec {
 // buffers of the phased root solve; the capacities are planned by the caller
 // from the totals the staging pass adds up in ctr ([0] slab bytes, [1] sphere
 // and [2] torus candidates; [3] edges not picked at once; [4] torus candidates
-// listed for FP64 work; [5] edges left to the warp selection, FP32 form)
+// listed for FP64 work; [5] edges left to the warp selection, [6] tied
+// candidates, FP32 form)
 struct RootWork {
     int4 *einfo;            // per crossing edge: slab (16-byte units), packed point/axis/label/dropped,
                             // first sphere and first torus candidate
@@ -117,8 +118,9 @@ struct RootWork {
     unsigned char *slab;    // staged tiles
     unsigned long long *ctr;  // 8 counters, [4] the torus candidates listed for FP64 work
     int *hard, *hard2;      // edges listed for the selections: not picked at once; left to a warp each (FP32 form)
+    int4 *ties;             // tied candidates for FP64 roots: (edge, record, slot | kind << 4, staged item)
     int2 *jobs;             // torus candidates with FP64 work: (candidate, 1 pending slots / 2 whole)
-    long long cap_slab, cap_sph, cap_tor, cap_jobs;
+    long long cap_slab, cap_sph, cap_tor, cap_jobs, cap_ties;
     long long n_edges;      // crossing edges of the run (all axes)
 };
 void edges_init();
