@@ -505,7 +505,7 @@ __device__ __forceinline__ int free_witness(const Acc &A, T qx, T qy, T qz, int 
 
 // shared memory of the staging pass (beside the staged tile)
 struct StageSmem {
-    int8_t lab[9 * 9 * 9];
+    uint16_t rows[81];         // the tile's labels and the next layer's (tile_row)
     short eptr[3 * TILE_PTS];  // crossing edges of the tile (edge_pack), grouped by axis
     int cs[3 * TILE_PTS + 1];  // per edge: sphere candidates, then their offset in the tile's run
     int ct[3 * TILE_PTS + 1];  // the same for tori
@@ -516,7 +516,7 @@ struct StageSmem {
     long long slab;    // slab offset (16-byte units), -1 when the slab buffer is full
     long long sb, tb;  // the tile's first sphere / torus candidate, -1 when a buffer is full
     long long sb0, tb0;  // the same as reserved (also when a buffer is full)
-    unsigned hmask[HMASK_WORDS];  // prefilter hits, ceil(items / 32) words per edge (when they fit)
+    unsigned hmask[HMASK_WORDS];  // prefilter hits, ceil(items / 32) words per edge (when they fit), two halves a word
 };
 
 // items [0, nsph) are spheres: the bits of 32-item word w that are spheres
@@ -800,6 +800,40 @@ __device__ __forceinline__ bool cand_test(const CandItem &c, const float *s, int
     const float dg = __fdividef(e1 * __fdividef(ma - zc * ua, nw) + zc * ua, D);
     if (gm > fabsf(dg) * H + 0.5f * bend * H + mg) return false;
     return !((inside ? dg : -dg) > bend + 1e-2f);
+}
+
+// Prefilter of the lane's edge (lower point s, axis, label) against 16 staged
+// items from i0 on, the same items on every lane: bit b for item i0 + b.  The
+// warp's edges are neighbours, so an item is mostly near to all of them or to
+// none and the lanes stay together (lanes over items, a warp per edge, ran the
+// sphere and the torus test for every word that held both: 24,000 cycles a tile
+// of 75 edges and 60 items on the globule, half of the staging pass with the
+// writing of the pairs).  Whole warp.
+template <class T, class CP>
+__device__ __forceinline__ unsigned cand_bits(const TileS<T, CP> &S, int i0, int nitem, const float *s, int axis,
+                                              bool inside, float h, float rp)
+{
+    unsigned bits = 0u;
+    const int n = min(16, nitem - i0);
+    CandItem mine;
+    if constexpr (sizeof(T) == sizeof(double)) mine = cand_item<T, CP>(S, i0 + (threadIdx.x & 15), nitem, rp);
+    for (int b = 0; b < n; ++b) {
+        CandItem c;
+        if constexpr (sizeof(T) == sizeof(double)) {  // converted once, by a lane each
+            c.x = __shfl_sync(0xffffffffu, mine.x, b);
+            c.y = __shfl_sync(0xffffffffu, mine.y, b);
+            c.z = __shfl_sync(0xffffffffu, mine.z, b);
+            c.r = __shfl_sync(0xffffffffu, mine.r, b);
+            c.ux = __shfl_sync(0xffffffffu, mine.ux, b);
+            c.uy = __shfl_sync(0xffffffffu, mine.uy, b);
+            c.uz = __shfl_sync(0xffffffffu, mine.uz, b);
+            c.kind = __shfl_sync(0xffffffffu, mine.kind, b);
+        } else {
+            c = cand_item<T, CP>(S, i0 + b, nitem, rp);
+        }
+        if (c.kind >= 0 && cand_test(c, s, axis, inside, h, rp)) bits |= 1u << b;
+    }
+    return bits;
 }
 
 // Roots of one (edge, piece) candidate that can be the surface on that edge:
@@ -1299,39 +1333,35 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
         if (threadIdx.x == 0 && S.flags) atomicOr(err, S.flags);
         int t[3];
         tile_coords(G, tile, t);
-        // labels of the tile and of the next layer (9^3), -1 outside the grid
-        for (int q = threadIdx.x; q < 729; q += EDGE_THREADS) {
-            int li = q / 81, lj = (q / 9) % 9, lk = q % 9;
-            long long g[3] = {(long long)TILE * t[0] + li, (long long)TILE * t[1] + lj, (long long)TILE * t[2] + lk};
-            int8_t v = -1;
-            if (g[0] < G.dims[0] && g[1] < G.dims[1] && g[2] < G.dims[2]) v = labels[g[0] * st0 + g[1] * st1 + g[2]];
-            E.lab[q] = v;
+        if (threadIdx.x < 81) E.rows[threadIdx.x] = tile_row(G, labels_all, t, threadIdx.x);
+        if (threadIdx.x >= 96 && threadIdx.x < 99) {
+            const int a = threadIdx.x - 96;
+            E.gbase[a] = edge_start[a * nt + gt];
+            E.abase[a] = E.gbase[a] - edge_start[a * nt];
         }
-        if (threadIdx.x == 0) E.estart[0] = 0;
         __syncthreads();
-        // the tile's crossing edges, axis by axis, in point order
-        for (int a = 0; a < 3; ++a) {
-            int flag[2], lab[2];
-            for (int k = 0; k < 2; ++k) {
-                int q = 2 * threadIdx.x + k;
-                int l[3] = {q >> 6, (q >> 3) & 7, q & 7};
-                const bool owned = TILE * t[0] + l[0] < G.own[0] && TILE * t[1] + l[1] < G.own[1] &&
-                                   TILE * t[2] + l[2] < G.own[2];
-                int8_t l0 = E.lab[(l[0] * 9 + l[1]) * 9 + l[2]];
-                l[a] += 1;
-                int8_t l1 = E.lab[(l[0] * 9 + l[1]) * 9 + l[2]];
-                flag[k] = (owned && l0 >= 0 && l1 >= 0 && l0 != l1) ? 1 : 0;
-                lab[k] = l0;
+        // the tile's crossing edges, axis by axis, in point order: one thread per
+        // axis and row of 8 points, one scan over all of them
+        {
+            static_assert(EDGE_THREADS >= 192, "a thread per axis and row");
+            const int a = threadIdx.x >> 6, row = threadIdx.x & 63, i = row >> 3, j = row & 7, r = 9 * i + j;
+            unsigned m = 0u, cross = 0u;
+            if (a < 3 && TILE * t[0] + i < G.own[0] && TILE * t[1] + j < G.own[1]) {
+                const long long gk = (long long)TILE * t[2];
+                const int n_on = (int)min(9LL, G.dims[2] - gk), n_own = (int)max(0LL, min(8LL, G.own[2] - gk));
+                unsigned on = (1u << n_own) - 1u;
+                m = E.rows[r];
+                const unsigned x = a == 0 ? E.rows[r + 9] : (a == 1 ? E.rows[r + 1] : (m >> 1) | 0x8000u);
+                if (a == 2) on &= (1u << (n_on - 1)) - 1u;
+                cross = (x & 0x8000u) ? (m ^ x) & on : 0u;
             }
-            int tsum;
-            int rank = block_excl_scan_e(flag[0] + flag[1], E.sh, &tsum);
-            const int eb = E.estart[a];
-            for (int k = 0; k < 2; ++k)
-                if (flag[k]) E.eptr[eb + rank++] = (short)edge_pack(2 * threadIdx.x + k, a, lab[k], 0);
-            if (threadIdx.x == 0) {
-                E.estart[a + 1] = eb + tsum;
-                E.gbase[a] = edge_start[a * nt + gt];
-                E.abase[a] = edge_start[a * nt + gt] - edge_start[a * nt];
+            int tot;
+            int rank = block_excl_scan_e(__popc(cross), E.sh, &tot);
+            if (row == 0 && a < 3) E.estart[a] = rank;
+            if (threadIdx.x == 0) E.estart[3] = tot;
+            for (; cross; cross &= cross - 1) {
+                const int k = __ffs(cross) - 1;
+                E.eptr[rank++] = (short)edge_pack(8 * row + k, a, (m >> k) & 1, 0);
             }
             __syncthreads();
         }
@@ -1350,25 +1380,41 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
                 (long long)(TILE * (t[0] + G.toff[0]) + li) * fst0 + (long long)(TILE * (t[1] + G.toff[1]) + lj) * fst1 +
                 (TILE * (t[2] + G.toff[2]) + lk);
         }
-        // (edge, item) pairs that pass the prefilter, counted: lanes over items,
-        // an item kept in registers while its warp goes through the warp's
-        // edges; the hit masks kept when they fit
-        const int nwd = (nitem + 31) >> 5;
+        // (edge, item) pairs that pass the prefilter, counted: a warp takes 32
+        // edges and 16 items at a time; the hit masks kept when they fit
+        const int nwd = (nitem + 31) >> 5, ngrp = (ne + 31) >> 5;
         const bool keep = (long long)ne * nwd <= HMASK_WORDS;
         const float rpf = (float)M.rp;
-        for (int i0 = 0; i0 < max(nitem, 1); i0 += 32) {
-            const CandItem item = cand_item<T, CP>(S, i0 + lane, nitem, rpf);
-            const unsigned sm = sphere_bits(i0 >> 5, nsph);
-            for (int e = warp; e < ne; e += EDGE_WARPS) {
-                const EdgeRef R = edge_ref(E, e);
-                float s[3], hs;
-                edge_point<float>(G, R.p, s, hs);
-                const unsigned m = __ballot_sync(0xffffffffu, cand_test(item, s, R.axis, R.lab == LABEL_IN, hs, rpf));
-                if (lane == 0) {  // (the same lane for every word of an edge)
-                    E.cs[e] = (i0 ? E.cs[e] : 0) + __popc(m & sm);
-                    E.ct[e] = (i0 ? E.ct[e] : 0) + __popc(m & ~sm);
-                    if (keep) E.hmask[e * nwd + (i0 >> 5)] = m;
-                }
+        uint16_t *half = reinterpret_cast<uint16_t *>(E.hmask);
+        auto test16 = [&](int e, int i0) -> unsigned {  // whole warp, one edge per lane
+            const EdgeRef R = edge_ref(E, e < ne ? e : 0);
+            float s[3], hs;
+            edge_point<float>(G, R.p, s, hs);
+            const unsigned m = cand_bits<T, CP>(S, i0, nitem, s, R.axis, R.lab == LABEL_IN, hs, rpf);
+            return e < ne ? m : 0u;
+        };
+        auto word = [&](int e, int w) -> unsigned {  // the hits of edge e among items 32 w ..
+            return keep ? (e < ne ? E.hmask[e * nwd + w] : 0u) : test16(e, 32 * w) | (test16(e, 32 * w + 16) << 16);
+        };
+        if (keep) {
+            for (int k = warp; k < ngrp * 2 * nwd; k += EDGE_WARPS) {
+                const int hw = k / ngrp, e = 32 * (k - hw * ngrp) + lane;
+                const unsigned m = test16(e, 16 * hw);
+                if (e < ne) half[2 * nwd * e + hw] = (uint16_t)m;
+            }
+            __syncthreads();
+        }
+        for (int e0 = 32 * warp; e0 < ne; e0 += EDGE_THREADS) {
+            const int e = e0 + lane;
+            int cs = 0, ct = 0;
+            for (int w = 0; w < nwd; ++w) {
+                const unsigned m = word(e, w), sm = sphere_bits(w, nsph);
+                cs += __popc(m & sm);
+                ct += __popc(m & ~sm);
+            }
+            if (e < ne) {
+                E.cs[e] = cs;
+                E.ct[e] = ct;
             }
         }
         __syncthreads();
@@ -1430,19 +1476,18 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
             // margin covers the rounding of the staged FP32 positions)
             unsigned *nbm = reinterpret_cast<unsigned *>(sl + L.nbm);
             const int nw = (na + 31) >> 5;
-            for (int it = threadIdx.x; it < na * nw; it += EDGE_THREADS) {
-                const int a = it / nw, w = it - a * nw;
+            for (int it = warp; it < na * nw; it += EDGE_WARPS) {
+                const int a = it / nw, b = ((it - a * nw) << 5) + lane;
                 const P4<T> ca = S.atom[a];
-                const T Ra = ca.w + rpT + T(1e-3);
-                unsigned bits = 0u;
-                const int b0 = w << 5, b1 = min(na, b0 + 32);
-                for (int b = b0; b < b1; ++b) {
+                bool meet = false;
+                if (b < na && b != a) {
                     const P4<T> cb = S.atom[b];
                     const T dx = ca.x - cb.x, dy = ca.y - cb.y, dz = ca.z - cb.z;
-                    const T reach = Ra + cb.w + rpT;
-                    if (b != a && dx * dx + dy * dy + dz * dz < reach * reach) bits |= 1u << (b - b0);
+                    const T reach = ca.w + rpT + T(1e-3) + cb.w + rpT;
+                    meet = dx * dx + dy * dy + dz * dz < reach * reach;
                 }
-                nbm[it] = bits;
+                const unsigned bits = __ballot_sync(0xffffffffu, meet);
+                if (lane == 0) nbm[it] = bits;
             }
             // staged slots of every pair's atoms
             short2 *ps = reinterpret_cast<short2 *>(sl + L.pslot);
@@ -1470,33 +1515,30 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
         // or a second prefilter pass that disagreed with the count) gets a dead
         // record (edge -1), so the root kernels never read an unwritten slot.
         if (ok) {
-            for (int e = warp; e < ne; e += EDGE_WARPS) {
-                const EdgeRef R = edge_ref(E, e);
-                const int g = E.gbase[R.axis] + (e - E.estart[R.axis]);
-                float s[3], hs;
-                edge_point<float>(G, R.p, s, hs);
-                long long ps = E.sb + E.cs[e], pt = E.tb + E.ct[e];
-                const long long ps1 = E.sb + E.cs[e + 1], pt1 = E.tb + E.ct[e + 1];
-                const unsigned below = (1u << lane) - 1;
-                for (int i0 = 0; i0 < nitem; i0 += 32) {
-                    const int it = i0 + lane;
-                    unsigned m;
-                    if (keep) {
-                        m = E.hmask[e * nwd + (i0 >> 5)];
-                    } else {  // tested again
-                        const CandItem item = cand_item<T, CP>(S, it, nitem, rpf);
-                        m = __ballot_sync(0xffffffffu, cand_test(item, s, R.axis, R.lab == LABEL_IN, hs, rpf));
-                    }
-                    const bool hit = (m >> lane) & 1u;
-                    const unsigned sm = sphere_bits(i0 >> 5, nsph), ms = m & sm, mt = m & ~sm;
-                    const long long qs = ps + __popc(ms & below), qt = pt + __popc(mt & below);
-                    if (hit && it < nsph && qs < ps1) W.csph[qs] = make_int2(g, it);
-                    if (hit && it >= nsph && qt < pt1) W.ctor[qt] = make_int2(g, it - nsph);
-                    ps += __popc(ms);
-                    pt += __popc(mt);
+            for (int e0 = 32 * warp; e0 < ne; e0 += EDGE_THREADS) {
+                const int e = e0 + lane;
+                const bool on = e < ne;
+                long long ps = 0, pt = 0, ps1 = 0, pt1 = 0;
+                int g = 0;
+                if (on) {
+                    const EdgeRef R = edge_ref(E, e);
+                    g = E.gbase[R.axis] + (e - E.estart[R.axis]);
+                    ps = E.sb + E.cs[e];
+                    pt = E.tb + E.ct[e];
+                    ps1 = E.sb + E.cs[e + 1];
+                    pt1 = E.tb + E.ct[e + 1];
                 }
-                for (long long q = ps + lane; q < ps1; q += 32) W.csph[q] = make_int2(-1, 0);
-                for (long long q = pt + lane; q < pt1; q += 32) W.ctor[q] = make_int2(-1, 0);
+                for (int w = 0; w < nwd; ++w)
+                    for (unsigned m = word(e, w); m; m &= m - 1) {
+                        const int it = 32 * w + __ffs(m) - 1;
+                        if (it < nsph) {
+                            if (ps < ps1) W.csph[ps++] = make_int2(g, it);
+                        } else if (pt < pt1) {
+                            W.ctor[pt++] = make_int2(g, it - nsph);
+                        }
+                    }
+                for (; ps < ps1; ++ps) W.csph[ps] = make_int2(-1, 0);
+                for (; pt < pt1; ++pt) W.ctor[pt] = make_int2(-1, 0);
             }
         } else {
             const long long s1 = min(E.sb0 + E.cs[ne], W.cap_sph), t1 = min(E.tb0 + E.ct[ne], W.cap_tor);

@@ -142,39 +142,40 @@ __device__ __forceinline__ void tile_coords(const Grid &G, long long tile, int t
     t[0] = (int)(q / n1);
 }
 
-// The labels of a tile and of the next layer along each axis, one warp: row
-// 9 i + j (i, j = 0..8) holds the labels (0 or 1) of its points k = 0..8 as bits
-// 0..8, bit 15 set for a row on the grid.  The nine bytes are read as the three
-// aligned words that hold them and shifted into place (byte by byte where those
-// would pass the molecule's end); bits of points past the row's end hold the
-// next row's labels, for the caller to mask.  Ends with a warp barrier.
+// The labels of a tile and of the next layer along each axis as rows of bits:
+// row r = 9 i + j (i, j = 0..8) holds the labels (0 or 1) of its points k = 0..8
+// as bits 0..8, bit 15 set for a row on the grid.  The nine bytes are read as
+// the three aligned words that hold them and shifted into place (byte by byte
+// where those would pass the molecule's end); bits of points past the row's end
+// hold the next row's labels, for the caller to mask.
+__device__ __forceinline__ uint16_t tile_row(const Grid &G, const int8_t *__restrict__ labels_all, const int t[3],
+                                             int r)
+{
+    const long long d0 = G.dims[0], d1 = G.dims[1], d2 = G.dims[2], np = d0 * d1 * d2, gk = (long long)TILE * t[2];
+    const int i = r / 9, j = r - 9 * i;
+    const long long gi = (long long)TILE * t[0] + i, gj = (long long)TILE * t[1] + j;
+    if (gi >= d0 || gj >= d1) return 0;
+    const long long at = (gi * d1 + gj) * d2 + gk;
+    const uint8_t *p = reinterpret_cast<const uint8_t *>(labels_all) + G.lab0 + at;
+    unsigned m = 0x8000u;
+    if (at + 12 <= np) {
+        const int off = (int)(reinterpret_cast<uintptr_t>(p) & 3);
+        const unsigned *q = reinterpret_cast<const unsigned *>(p - off);
+        const unsigned a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2);
+        const unsigned w0 = __funnelshift_r(a0, a1, 8 * off), w1 = __funnelshift_r(a1, a2, 8 * off);
+        m |= ((w0 & 0x01010101u) * 0x01020408u >> 24) | (((w1 & 0x01010101u) * 0x01020408u >> 24) << 4) |
+             (((a2 >> (8 * off)) & 1u) << 8);
+    } else {
+        for (int k = 0; k < 9 && gk + k < d2; ++k) m |= (unsigned)(p[k] & 1) << k;
+    }
+    return (uint16_t)m;
+}
+
+// every row, one warp; ends with a warp barrier
 __device__ __forceinline__ void tile_rows(const Grid &G, const int8_t *__restrict__ labels_all, const int t[3],
                                           uint16_t *row)
 {
-    const int lane = threadIdx.x & 31;
-    const long long d0 = G.dims[0], d1 = G.dims[1], d2 = G.dims[2], np = d0 * d1 * d2, gk = (long long)TILE * t[2];
-    const uint8_t *__restrict__ labels = reinterpret_cast<const uint8_t *>(labels_all) + G.lab0;
-    for (int r = lane; r < 81; r += 32) {
-        const int i = r / 9, j = r - 9 * i;
-        const long long gi = (long long)TILE * t[0] + i, gj = (long long)TILE * t[1] + j;
-        unsigned m = 0u;
-        if (gi < d0 && gj < d1) {
-            const long long at = (gi * d1 + gj) * d2 + gk;
-            const uint8_t *p = labels + at;
-            if (at + 12 <= np) {
-                const int off = (int)(reinterpret_cast<uintptr_t>(p) & 3);
-                const unsigned *q = reinterpret_cast<const unsigned *>(p - off);
-                const unsigned a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2);
-                const unsigned w0 = __funnelshift_r(a0, a1, 8 * off), w1 = __funnelshift_r(a1, a2, 8 * off);
-                m = ((w0 & 0x01010101u) * 0x01020408u >> 24) | (((w1 & 0x01010101u) * 0x01020408u >> 24) << 4) |
-                    (((a2 >> (8 * off)) & 1u) << 8);
-            } else {
-                for (int k = 0; k < 9 && gk + k < d2; ++k) m |= (unsigned)(p[k] & 1) << k;
-            }
-            m |= 0x8000u;
-        }
-        row[r] = (uint16_t)m;
-    }
+    for (int r = threadIdx.x & 31; r < 81; r += 32) row[r] = tile_row(G, labels_all, t, r);
     __syncwarp();
 }
 
