@@ -87,9 +87,10 @@ __device__ __forceinline__ T pt_coord(const Grid &G, int k)
 // they walk the same atoms.
 template <bool FILT, class T, class CP>
 __device__ __forceinline__ int witness_free(const TileS<T, CP> &S, T qx, T qy, T qz, const unsigned *m0,
-                                            const unsigned *m1, int nw, T rp, T delta, int &nt)
+                                            const unsigned *m1, int nw, T rp, T Rmax, T delta, int &nt)
 {
     int res = 1;
+    const T e = FILT ? T(2) * ((T(2) * Rmax + delta) * delta + T(1e-6) * Rmax * Rmax) : T(0);  // lt_sq's bound at R_max
     for (int w = 0; w < nw; ++w) {
         unsigned bits = m1 ? (m0[w] & m1[w]) : m0[w];
         while (bits) {
@@ -98,10 +99,9 @@ __device__ __forceinline__ int witness_free(const TileS<T, CP> &S, T qx, T qy, T
             ++nt;
             const P4<T> c = S.atom[k];
             const T dx = qx - c.x, dy = qy - c.y, dz = qz - c.z;
-            const T R = c.w + rp;
-            const int t = lt_sq<FILT>(dx * dx + dy * dy + dz * dz, R * R, R, delta);
-            if (t == 1) return 0;
-            if (t < 0) res = -1;
+            const T R = c.w + rp, g = dx * dx + dy * dy + dz * dz - R * R;
+            if (FILT ? g < -e : dx * dx + dy * dy + dz * dz < R * R) return 0;
+            if (FILT && g < e) res = -1;
         }
     }
     return res;
@@ -121,7 +121,7 @@ __device__ __forceinline__ int witness_free(const TileS<T, CP> &S, T qx, T qy, T
 // 0 a free witness within r_p (certain), 2 undecided, 1 none.
 template <bool FILT, class T, class CP>
 __device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem<CP> &C, int code, T x, T y, T z, T rp,
-                                            T d0, float hf, int r, int G, int &nt)
+                                            T Rmax, T d0, float hf, int r, int G, int &nt)
 {
     constexpr unsigned full = 0xffffffffu;
     constexpr int aw = ClsSmem<CP>::AWC;
@@ -163,7 +163,7 @@ __device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem
                     continue;
                 }
                 const int f = witness_free<FILT>(S, qx, qy, qz, C.nbm + a * aw, (const unsigned *)nullptr, nw, rp,
-                                                 dq + d0, nt);
+                                                 Rmax, dq + d0, nt);
                 if (f == 1 && tw == 1) hit = done = true;
                 else if (f != 0) unsure = true;
             }
@@ -206,8 +206,8 @@ __device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem
                     continue;
                 }
                 const short2 sl = C.pslot[p];
-                const int f = witness_free<FILT>(S, qx, qy, qz, C.nbm + sl.x * aw, C.nbm + sl.y * aw, nw, rp, dq + d0,
-                                                 nt);
+                const int f = witness_free<FILT>(S, qx, qy, qz, C.nbm + sl.x * aw, C.nbm + sl.y * aw, nw, rp, Rmax,
+                                                 dq + d0, nt);
                 if (f == 1 && t == 1) hit = done = true;
                 else if (f != 0) unsure = true;
             }
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
     __shared__ long long q_base;
     __shared__ Grid sG;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const T rp = (T)M.rp;
+    const T rp = (T)M.rp, Rmax = (T)M.Rmax, rmax = (T)M.rmax;
     long long iter = 0;
     int ntests = 0;  // this thread's atom tests (witness freeness)
     const long long npos = sched_count(Q, B.n_tiles);
@@ -315,6 +315,9 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
                 T x = pt_coord<T>(G, li), y = pt_coord<T>(G, lj), z = pt_coord<T>(G, lk);
                 bool vdw = false, sas = false, sas_u = false;
                 const int nw = (S.na + 31) >> 5;
+                // lt_sq's bounds at the largest radii
+                const T er = FILT ? T(2) * ((T(2) * rmax + d0) * d0 + T(1e-6) * rmax * rmax) : T(0);
+                const T eR = FILT ? T(2) * ((T(2) * Rmax + d0) * d0 + T(1e-6) * Rmax * Rmax) : T(0);
                 for (int wd = 0; wd < nw && !vdw; ++wd) {
                     unsigned bits = C.bmask[brick][wd];
                     while (bits) {
@@ -324,13 +327,12 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
                         T dx = x - c.x, dy = y - c.y, dz = z - c.z;
                         T d2 = dx * dx + dy * dy + dz * dz;
                         T r = c.w, R = c.w + rp;
-                        if (lt_sq<FILT>(d2, r * r, r, d0) == 1) {
+                        if (FILT ? d2 < r * r - er : d2 < r * r) {
                             vdw = true;
                             break;
                         }
-                        int s = lt_sq<FILT>(d2, R * R, R, d0);
-                        if (s == 1) sas = true;
-                        else if (s < 0) sas_u = true;
+                        if (FILT ? d2 < R * R - eR : d2 < R * R) sas = true;
+                        else if (FILT && d2 < R * R + eR) sas_u = true;
                     }
                 }
                 if (vdw) lab = LABEL_IN;
@@ -370,7 +372,7 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
             const int code = k < nq ? C.queue[k] : -1;
             const int li = (code >> 6) & 7, lj = (code >> 3) & 7, lk = code & 7;
             const T x = pt_coord<T>(G, li), y = pt_coord<T>(G, lj), z = pt_coord<T>(G, lk);
-            const int lab = shell_points<FILT, T, CP>(S, C, code, x, y, z, rp, d0, (float)G.h, r, gs, ntests);
+            const int lab = shell_points<FILT, T, CP>(S, C, code, x, y, z, rp, Rmax, d0, (float)G.h, r, gs, ntests);
             if (r == 0 && code >= 0) {
                 const long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
                                 gk = (long long)TILE * t[2] + lk;

@@ -2282,8 +2282,18 @@ __global__ void __launch_bounds__(POLISH_THREADS) k_edge_polish(Model M, Batch B
 // (m, g) of k_reduce_part sums the terms of molecule m whose index within the
 // molecule's range is g (mod RED_PARTS * blockDim), in a fixed tree;
 // k_reduce_final adds the RED_PARTS partials of each molecule in a fixed tree.
-constexpr int RED_PARTS = 64;  // (16 parts: 192 us on one molecule's 4.9 M terms, 53 us on 1.2 M)
+constexpr int RED_PARTS = 64;  // at most (16 parts: 192 us on one molecule's 4.9 M terms, 53 us on 1.2 M; 58 and 17 now)
 constexpr int RED_THREADS = 512;
+
+// parts of a molecule: its own size decides (a batch's molecule is summed as it
+// is alone), a part for every 8,192 terms and tiles
+__device__ __forceinline__ int red_parts(const Batch &B, const long long *medge, int m)
+{
+    const int nm = B.n_mol;
+    long long n = B.tile_off[m + 1] - B.tile_off[m];
+    for (int a = 0; a < 3; ++a) n += medge[a * (nm + 1) + m + 1] - medge[a * (nm + 1) + m];
+    return (int)max(1LL, min((long long)RED_PARTS, n / 8192));
+}
 
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_part(Batch B, const double2 *__restrict__ term,
                                                              const long long *__restrict__ medge,
@@ -2294,8 +2304,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_part(Batch B, const doub
     __shared__ double sa[32], sv[32];
     __shared__ long long si[32], sp[32];
     const int m = blockIdx.x / RED_PARTS, g = blockIdx.x % RED_PARTS, nm = B.n_mol;
+    const int parts = red_parts(B, medge, m);
+    if (g >= parts) return;
     const long long nt = B.n_tiles;
-    const long long stride = (long long)RED_PARTS * RED_THREADS;
+    const long long stride = (long long)parts * RED_THREADS;
     const long long first = (long long)g * RED_THREADS + threadIdx.x;
     double a = 0.0, v = 0.0;
     long long ie = 0, pin = 0;
@@ -2345,14 +2357,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_part(Batch B, const doub
 
 // out2[2m..] = {area, volume}; counts[2m..] = {inside points, inside edges (all axes)}: a warp per molecule,
 // its parts over the lanes, then a fixed tree
-__global__ void k_reduce_final(Batch B, const double *__restrict__ part_d, const long long *__restrict__ part_i,
+__global__ void k_reduce_final(Batch B, const long long *__restrict__ medge, const double *__restrict__ part_d, const long long *__restrict__ part_i,
                                double *__restrict__ out2, long long *__restrict__ counts)
 {
     const int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (m >= B.n_mol) return;
     double A = 0.0, V = 0.0;
     long long P = 0, IE = 0;
-    for (int g = lane; g < RED_PARTS; g += 32) {
+    const int parts = red_parts(B, medge, m);
+    for (int g = lane; g < parts; g += 32) {
         const int k = m * RED_PARTS + g;
         A += part_d[2 * k];
         V += part_d[2 * k + 1];
@@ -2548,7 +2561,7 @@ int launch_reduce(const Batch &B, const double2 *term, const long long *medge, c
                   long long *part_i, double *out2, long long *counts, cudaStream_t st)
 {
     k_reduce_part<<<B.n_mol * RED_PARTS, RED_THREADS, 0, st>>>(B, term, medge, tile_inside, part_d, part_i);
-    k_reduce_final<<<(B.n_mol + 3) / 4, 128, 0, st>>>(B, part_d, part_i, out2, counts);
+    k_reduce_final<<<(B.n_mol + 3) / 4, 128, 0, st>>>(B, medge, part_d, part_i, out2, counts);
     return 2;
 }
 

@@ -43,7 +43,7 @@ struct alignas(16) P4 {
     T x, y, z, w;
 };
 
-constexpr int STAGE_CELLS = 128;  // cells staged with item-parallel scan (else one thread per cell)
+constexpr int STAGE_RUNS = 64;  // runs of cells staged with item-parallel scan (else one thread per run)
 // words of a set of staged atoms (bit k: staged slot k) for capacity C
 template <class C>
 __host__ __device__ constexpr int atom_words() { return (C::A + 31) / 32; }
@@ -59,8 +59,8 @@ struct TileS {
     int pidx[C::P];         // pair index in the model
     int vidx[C::V];         // triple point index in the model
     uint8_t aface[C::A];    // expanded sphere keeps a free face
-    int cid[STAGE_CELLS];           // cells of the staging range
-    int cs[3][STAGE_CELLS + 1];     // prefix of their atoms / pairs / vertices
+    int rs[3][STAGE_RUNS];          // first atom / pair / vertex of each run of cells along the last axis
+    int cs[3][STAGE_RUNS + 1];      // prefix of their numbers
     double fx0[3], fx1[3];          // tile region (absolute), computed once per tile
     float fh0[3], fl0[3];           // region origin in the grid frame, double-float
     int fc0[3], fc1[3];             // cell range of the region plus halo
@@ -292,8 +292,9 @@ __device__ __forceinline__ void stage_item(const Model &M, TileS<T, C> &S, int l
 
 // Stage the tile's atoms, free-arc pairs and free vertices (whole block of at
 // least 96 threads).
-// The items of every cell in range are numbered by a prefix over the cells
-// and tested one per thread, so all threads share the work.
+// The cells of the range that follow each other along the last axis hold
+// consecutive items: those runs (9 or so) are read, numbered by a prefix over
+// them, and the items tested one per thread, so all threads share the work.
 template <class T, class C>
 __device__ void stage_tile(const Model &M, const Grid &G, int mol, long long tile, TileS<T, C> &S, double x0[3])
 {
@@ -339,15 +340,18 @@ __device__ void stage_tile(const Model &M, const Grid &G, int mol, long long til
         c0[a] = S.fc0[a];
         nc[a] = S.fc1[a] - S.fc0[a] + 1;
     }
-    const int ncell = nc[0] * nc[1] * nc[2];
-    if (ncell <= STAGE_CELLS) {
-        for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-            int cz = c % nc[2], cy = (c / nc[2]) % nc[1], cx = c / (nc[1] * nc[2]);
-            int id = CG.coff + ((c0[0] + cx) * CG.cn[1] + (c0[1] + cy)) * CG.cn[2] + (c0[2] + cz);
-            S.cid[c] = id;
-            S.cs[0][c + 1] = M.cell_start[id + 1] - M.cell_start[id];
-            S.cs[1][c + 1] = M.pcell_start[id + 1] - M.pcell_start[id];
-            S.cs[2][c + 1] = M.vcell_start[id + 1] - M.vcell_start[id];
+    const int nrun = nc[0] * nc[1];
+    const int *const start[3] = {M.cell_start, M.pcell_start, M.vcell_start};
+    auto first_cell = [&](int r) {
+        return CG.coff + ((c0[0] + r / nc[1]) * CG.cn[1] + (c0[1] + r % nc[1])) * CG.cn[2] + c0[2];
+    };
+    if (nrun <= STAGE_RUNS) {
+        for (int t = threadIdx.x; t < 3 * nrun; t += blockDim.x) {
+            const int list = t / nrun, r = t - list * nrun, id = first_cell(r);
+            const int *st = list == 0 ? start[0] : (list == 1 ? start[1] : start[2]);
+            const int s0 = st[id];
+            S.rs[list][r] = s0;
+            S.cs[list][r + 1] = st[id + nc[2]] - s0;
         }
         __syncthreads();
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -355,42 +359,39 @@ __device__ void stage_tile(const Model &M, const Grid &G, int mol, long long til
             int *cs = S.cs[warp];
             int carry = 0;
             if (lane == 0) cs[0] = 0;
-            for (int base = 1; base <= ncell; base += 32) {
+            for (int base = 1; base <= nrun; base += 32) {
                 int k = base + lane;
-                int v = k <= ncell ? cs[k] : 0;
+                int v = k <= nrun ? cs[k] : 0;
                 for (int o = 1; o < 32; o <<= 1) {
                     int u = __shfl_up_sync(0xffffffffu, v, o);
                     if (lane >= o) v += u;
                 }
-                if (k <= ncell) cs[k] = v + carry;
+                if (k <= nrun) cs[k] = v + carry;
                 carry += __shfl_sync(0xffffffffu, v, 31);
             }
         }
         __syncthreads();
-        const int n0 = S.cs[0][ncell], n1 = S.cs[1][ncell], n2 = S.cs[2][ncell];
+        const int n0 = S.cs[0][nrun], n1 = S.cs[1][nrun], n2 = S.cs[2][nrun];
         for (int it = threadIdx.x; it < n0 + n1 + n2; it += blockDim.x) {
             int list = it < n0 ? 0 : (it < n0 + n1 ? 1 : 2);
             int k = it - (list == 0 ? 0 : (list == 1 ? n0 : n0 + n1));
             const int *cs = S.cs[list];
-            int lo = 0, hi = ncell;
+            int lo = 0, hi = nrun;
             while (hi - lo > 1) {
                 int mid = (lo + hi) >> 1;
                 if (cs[mid] <= k) lo = mid;
                 else hi = mid;
             }
-            int id = S.cid[lo];
-            int off = k - cs[lo];
-            int item = list == 0 ? M.cell_start[id] + off : (list == 1 ? M.pcell_start[id] + off : M.vcell_start[id] + off);
-            stage_item<T>(M, S, list, item, F);
+            stage_item<T>(M, S, list, S.rs[list][lo] + k - cs[lo], F);
         }
     } else {
         __syncthreads();
-        for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-            int cz = c % nc[2], cy = (c / nc[2]) % nc[1], cx = c / (nc[1] * nc[2]);
-            int id = CG.coff + ((c0[0] + cx) * CG.cn[1] + (c0[1] + cy)) * CG.cn[2] + (c0[2] + cz);
-            for (int k = M.cell_start[id]; k < M.cell_start[id + 1]; ++k) stage_item<T>(M, S, 0, k, F);
-            for (int k = M.pcell_start[id]; k < M.pcell_start[id + 1]; ++k) stage_item<T>(M, S, 1, k, F);
-            for (int k = M.vcell_start[id]; k < M.vcell_start[id + 1]; ++k) stage_item<T>(M, S, 2, k, F);
+        for (int r = threadIdx.x; r < nrun; r += blockDim.x) {
+            const int id = first_cell(r);
+            for (int list = 0; list < 3; ++list) {
+                const int *st = list == 0 ? start[0] : (list == 1 ? start[1] : start[2]);
+                for (int k = st[id]; k < st[id + nc[2]]; ++k) stage_item<T>(M, S, list, k, F);
+            }
         }
     }
     __syncthreads();
@@ -590,16 +591,18 @@ __device__ __forceinline__ int face_proposal(const Acc &A, int a, T x, T y, T z,
     T d2 = dx * dx + dy * dy + dz * dz;
     T R = c.w + rp;
     if (lt_sq<FILT>(d2, R * R, R, d0) == 0) return 0;
-    T d = sqrt(d2);
+    // (FP32: one reciprocal square root, good to 2e-7; the bounds' 1e-6 R holds it)
+    const T id = FILT ? T(rsqrtf((float)d2)) : T(0);
+    const T d = FILT ? (d2 > T(0) ? d2 * id : T(0)) : sqrt(d2);
     if (d <= T(1e-3)) return FILT ? -2 : 0;  // x at a centre is inside its vdW ball
     T wd = fabs(R - d);                        // distance to the projection
     int tw = lt_lin<FILT>(wd, thr, d0 + T(1e-6) * R);
     if (tw == 0) return 0;
-    T s = R / d;
+    const T s = FILT ? R * id : R / d;
     qx = c.x + s * dx;
     qy = c.y + s * dy;
     qz = c.z + s * dz;
-    dq = FILT ? d0 * (T(1) + T(2) * R / d) + T(1e-6) * R : T(0);
+    dq = FILT ? d0 * (T(1) + T(2) * s) + T(1e-6) * R : T(0);
     e0 = A.agid(a);
     e1 = -1;
     return tw;
@@ -615,7 +618,9 @@ __device__ __forceinline__ int saddle_proposal(const Acc &A, int p, T x, T y, T 
     T zc = yx * u.x + yy * u.y + yz * u.z;
     T wx = yx - zc * u.x, wy = yy - zc * u.y, wz = yz - zc * u.z;
     T w2 = wx * wx + wy * wy + wz * wz;
-    T nw = sqrt(w2);
+    // (FP32: one reciprocal square root, good to 2e-7; dw's 2e-6 |w| holds it)
+    const T iw = FILT ? T(rsqrtf((float)w2)) : T(0);
+    const T nw = FILT ? (w2 > T(0) ? w2 * iw : T(0)) : sqrt(w2);
     T e1d = nw - o.w;
     T dist2 = e1d * e1d + zc * zc;
     T dw = FILT ? T(2) * d0 + T(2e-6) * (nw + fabs(zc)) : T(0);
@@ -623,7 +628,7 @@ __device__ __forceinline__ int saddle_proposal(const Acc &A, int p, T x, T y, T 
     if (t == 0) return 0;
     if (FILT && nw < T(1e-3)) return -2;  // near the circle's axis the nearest point is ill-conditioned
     if constexpr (FILT) {
-        T k = o.w / nw;
+        const T k = o.w * iw;
         qx = o.x + k * wx; qy = o.y + k * wy; qz = o.z + k * wz;
     } else {
         const double yv[3] = {(double)yx, (double)yy, (double)yz}, uv[3] = {(double)u.x, (double)u.y, (double)u.z};
@@ -631,7 +636,7 @@ __device__ __forceinline__ int saddle_proposal(const Acc &A, int p, T x, T y, T 
         axis_normal(yv, uv, wn);
         qx = o.x + o.w * (T)wn[0]; qy = o.y + o.w * (T)wn[1]; qz = o.z + o.w * (T)wn[2];
     }
-    dq = FILT ? o.w * T(2) * dw / nw + d0 + T(1e-6) * o.w : T(0);
+    dq = FILT ? o.w * T(2) * dw * iw + d0 + T(1e-6) * o.w : T(0);
     int2 ij = A.pij(p);
     e0 = ij.x;
     e1 = ij.y;
