@@ -210,7 +210,7 @@ struct eses_ctx {
     bool use_big = false;  // a run of this context had a tile for the global-memory tier
     DBuf ovf, big;  // tiles that overflow the shared-memory staging, and the global-memory tier's scratch
     // phased root solve: edge records, candidates, their roots, staged tiles (slabs), counters, hard edges
-    DBuf r_einfo, r_ecnt, r_csph, r_ctor, r_nsph, r_ntor, r_rsph, r_rtor, r_slab, r_ctr, r_hard, r_hard2, r_ties, r_jobs;
+    DBuf r_einfo, r_ecnt, r_csph, r_ctor, r_nsph, r_ntor, r_rsph, r_rtor, r_slab, r_ctr, r_hard, r_ties, r_jobs;
     long long cap_sph = 0, cap_tor = 0, cap_slab = 0, cap_jobs = 0;  // planned capacities
     DBuf atom_hi, atom_lo, pair_hi, pair_lo, pair_u32, vert_hi, vert_lo;
     // plan: list sizes of the first run (the inputs never change)
@@ -648,7 +648,6 @@ RootWork root_work(eses_ctx *c, long long ne_all)
     W.einfo = ensure<int4>(c->r_einfo, (size_t)ne);
     W.ecnt = ensure<int>(c->r_ecnt, (size_t)ne);
     W.hard = ensure<int>(c->r_hard, (size_t)ne);
-    W.hard2 = ensure<int>(c->r_hard2, (size_t)ne);
     W.cap_ties = ne / 4 + 1024;  // (about one per 25 edges; a tie that finds no room is settled by its warp)
     W.ties = ensure<int4>(c->r_ties, (size_t)W.cap_ties);
     W.csph = ensure<int2>(c->r_csph, (size_t)c->cap_sph);
@@ -978,9 +977,8 @@ int finish(eses_ctx *c, int nl)
     ck(cudaMemcpyAsync(hprop, c->prop_counts.p, sizeof(hprop), cudaMemcpyDeviceToHost, st), "read results");
     int hovf = 0;  // tiles the global-memory staging tier took
     ck(cudaMemcpyAsync(&hovf, c->ovf.p, sizeof(int), cudaMemcpyDeviceToHost, st), "read results");
-    // root solve: slab bytes, sphere and torus candidates, edges not picked at once, torus candidates with FP64
-    // work, edges left to the warp selection (FP32 form)
-    unsigned long long rctr[6] = {0, 0, 0, 0, 0, 0};
+    // root solve: slab bytes, sphere and torus candidates, hard edges, torus candidates with FP64 work
+    unsigned long long rctr[5] = {0, 0, 0, 0, 0};
     if (c->r_ctr.p) ck(cudaMemcpyAsync(rctr, c->r_ctr.p, sizeof(rctr), cudaMemcpyDeviceToHost, st), "read results");
     ck(cudaMemcpyAsync(c->medge_h.data(), c->medge.p, sizeof(long long) * c->medge_h.size(), cudaMemcpyDeviceToHost, st),
        "read results");
@@ -1014,7 +1012,7 @@ int finish(eses_ctx *c, int nl)
     c->stats[16] = (long long)tests;
     c->stats[17] = (long long)rctr[1];
     c->stats[18] = (long long)rctr[2];
-    c->stats[19] = (long long)rctr[c->precision == ESES_PREC_FP64 ? 3 : 5];
+    c->stats[19] = (long long)rctr[3];
     if (hovf > 0 && !c->use_big) throw NeedBig{};
     c->ran = true;
     int derr = hmisc[0];
@@ -1438,7 +1436,6 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
         W.einfo = (int4 *)c->r_einfo.p;
         W.ecnt = (int *)c->r_ecnt.p;
         W.hard = (int *)c->r_hard.p;
-        W.hard2 = (int *)c->r_hard2.p;
         W.ties = (int4 *)c->r_ties.p;
         W.csph = (int2 *)c->r_csph.p;
         W.nsph = (uint8_t *)c->r_nsph.p;
@@ -2048,7 +2045,7 @@ void eses_destroy(eses_ctx *c)
                     &c->vbin_cell, &c->vbin_list, &c->labels, &c->band, &c->cls_list, &c->etiles, &c->tile_edges, &c->edge_start,
                     &c->tile_inside, &c->scan_tmp, &c->misc, &c->av, &c->counts, &c->red_d, &c->red_i, &c->fail_log,
                     &c->ovf, &c->big, &c->r_einfo, &c->r_ecnt, &c->r_csph, &c->r_ctor, &c->r_nsph, &c->r_ntor,
-                    &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_hard2, &c->r_ties, &c->r_jobs, &c->atom_hi,
+                    &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_ties, &c->r_jobs, &c->atom_hi,
                     &c->atom_lo, &c->pair_hi, &c->pair_lo, &c->pair_u32, &c->vert_hi, &c->vert_lo,
                     &c->mlp_params, &c->need, &c->need_pos, &c->tile_list, &c->prop_counts, &c->features,
                     &c->targets, &c->ext, &c->ext_open, &c->ext_misc, &c->mesh_mask, &c->mesh_tile, &c->mesh_off,

@@ -32,8 +32,7 @@
 //   k_edge_pick: one thread per edge: the first root when the end point is
 //     inside or one candidate is left and the FP32 bounds order the
 //     candidates; the other edges are listed;
-//   k_edge_settle: one thread per listed edge: the outside end points that the
-//     candidates' own witnesses decide; k_edge_ties: FP64 roots of near ties;
+//   k_edge_ties: FP64 roots of near ties, one thread each;
 //   k_edge_hard: one warp per edge left: near ties broken on FP64 roots; at
 //     an outside end point each earlier candidate tested first against the
 //     later candidates' witnesses, then by the full witness search, whose
@@ -1762,14 +1761,59 @@ __device__ __forceinline__ void code_out(EdgeOut &out, int axis, long long o, in
     out.code[axis][o] = make_int2(__float_as_int(tr), (kind << 29) | (lab << 28) | (failed << 27) | mid);
 }
 
-// 4. The first root of every edge whose choice needs neither a witness test
-// nor an FP64 tie break -- an inside end point, or a single candidate (the
-// last candidate needs no test) -- with no candidate the FP32 bounds cannot
-// order: one thread per edge, candidates in order (spheres by item, then
-// tori); the other edges are listed for the warp selection.  A dropped edge
-// is recorded as failed (and the run as over capacity).
+// Witness of the accepted root at y of a staged piece (kind as in WCand) and a
+// bound of its error, dy bounding y's; false where it is ill-conditioned.  An
+// accepted root's witness is free.
 template <class T>
-__global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Batch B, RootWork W, const int *__restrict__ edge_start,
+__device__ __forceinline__ bool root_witness(const SlabAcc<T> &A, int kind, int slot, const T *y, T rp, T d0, T dy,
+                                             T *w, T &dw)
+{
+    if (kind == 2) {
+        const P4<T> v = A.vq(slot);
+        w[0] = v.x;
+        w[1] = v.y;
+        w[2] = v.z;
+        dw = d0;
+        return true;
+    }
+    if (kind == 0) {
+        const P4<T> c = A.atom(slot);
+        const T v[3] = {y[0] - c.x, y[1] - c.y, y[2] - c.z}, R = c.w + rp;
+        const T sc = R / sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        w[0] = c.x + sc * v[0];
+        w[1] = c.y + sc * v[1];
+        w[2] = c.z + sc * v[2];
+        dw = d0 + (d0 + dy) * (T(1) + T(2) * sc);
+        return true;
+    }
+    const P4<T> o = A.po(slot), u = A.pu(slot);
+    const T v[3] = {y[0] - o.x, y[1] - o.y, y[2] - o.z};
+    const T z = v[0] * u.x + v[1] * u.y + v[2] * u.z;
+    const T p[3] = {v[0] - z * u.x, v[1] - z * u.y, v[2] - z * u.z};
+    const T nw = sqrt(p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
+    if (!(nw > T(1e-2))) return false;
+    const T k = o.w / nw;
+    w[0] = o.x + k * p[0];
+    w[1] = o.y + k * p[1];
+    w[2] = o.z + k * p[2];
+    dw = d0 + T(2) * k * (d0 + dy + (sizeof(T) == sizeof(float) ? T(2e-6) * (nw + fabs(z)) : T(0)));
+    return true;
+}
+
+// 4. The first root of every edge whose choice needs neither a witness test
+// nor an FP64 tie break, with no candidate the FP32 bounds cannot order: one
+// thread per edge, candidates in order (spheres by item, then tori).
+// From an inside end point it is the first candidate.  From an outside one it
+// is the last if the first lies closer than r_p to the last one's witness: that
+// is a free probe centre, the edge between the two lies in the ball of r_p
+// around it, so every candidate before the last is strictly outside M.  (A
+// single candidate is the last.)  The other edges are listed for the selections:
+// without the rule for several candidates 266 k of 1.2 M edges on the
+// 5,000-atom globule, 23 k with it.  A dropped edge is recorded as failed (and
+// the run as over capacity).
+template <class T>
+__global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Model M, Batch B, RootWork W,
+                                                            const int *__restrict__ edge_start,
                                                             long long ne_all, EdgeOut out, int *__restrict__ err)
 {
     const long long nt = B.n_tiles;
@@ -1797,70 +1841,100 @@ __global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Batch B, RootWork W,
                 const unsigned char *sl = W.slab + ((size_t)(unsigned)inf.x << 4);
                 const SlabHdr *hd = reinterpret_cast<const SlabHdr *>(sl);
                 const int na = __ldg(&hd->na);
-                // smallest FP32 root (ties to the first), its record, and the count
-                int n = 0, kind = -1, slot = 0, kn = -1;
-                float tk = INFINITY, ek = 0.0f;
-                double t64k = 0.0;
-                for (int j = 0; j < ns; ++j) {
-                    const int nr = W.nsph[inf.z + j];
-                    for (int r = 0; r < nr; ++r) {
-                        const RootRec q = W.rsph[(size_t)SPH_SLOTS * (inf.z + j) + r];
-                        if (!(q.t < INFINITY)) continue;
-                        if (q.t < tk) {
-                            const int it = W.csph[inf.z + j].y;
-                            tk = q.t;
-                            ek = q.err;
-                            t64k = q.t64;
-                            kind = it < na ? 0 : 2;
-                            slot = it < na ? it : it - na;
-                            kn = n;
-                        }
-                        ++n;
-                    }
-                }
-                for (int j = 0; j < nq; ++j) {
-                    const int nr = W.ntor[inf.w + j];
-                    for (int r = 0; r < nr; ++r) {
-                        const RootRec q = W.rtor[(size_t)TOR_SLOTS * (inf.w + j) + r];
-                        if (!(q.t < INFINITY) || q.err < 0.0f) continue;  // rejected (or never settled)
-                        if (q.t < tk) {
-                            tk = q.t;
-                            ek = q.err;
-                            t64k = q.t64;
-                            kind = 1;
-                            slot = W.ctor[inf.w + j].y;
-                            kn = n;
-                        }
-                        ++n;
-                    }
-                }
-                hard = !(n >= 1 && n <= WCAND && (lab == LABEL_IN || n == 1) && kn >= 0);
-                if (!hard) {  // every other candidate ordered after it by the FP32 bounds
-                    const float tie = 1e-6f * B.grid[__ldg(&hd->mol)].hl[1];
-                    int m = 0;
-                    for (int j = 0; j < ns && !hard; ++j) {
+                // smallest FP32 root (ties to the first) and largest, their records, and the count
+                struct Root {
+                    float t, err;
+                    double t64;
+                    int kind, slot, n;
+                } first{INFINITY, 0.0f, 0.0, -1, 0, -1}, last{-INFINITY, 0.0f, 0.0, -1, 0, -1};
+                int n = 0;
+                auto roots = [&](auto f) {  // every accepted root in order: f(root, torus?, record, slot, place)
+                    int k = 0;
+                    for (int j = 0; j < ns; ++j) {
                         const int nr = W.nsph[inf.z + j];
                         for (int r = 0; r < nr; ++r) {
                             const RootRec q = W.rsph[(size_t)SPH_SLOTS * (inf.z + j) + r];
-                            if (!(q.t < INFINITY)) continue;
-                            if (m != kn && q.t - tk <= q.err + ek + tie) hard = true;
-                            ++m;
+                            if (q.t < INFINITY) f(q, false, j, r, k++);
                         }
                     }
-                    for (int j = 0; j < nq && !hard; ++j) {
+                    for (int j = 0; j < nq; ++j) {
                         const int nr = W.ntor[inf.w + j];
                         for (int r = 0; r < nr; ++r) {
                             const RootRec q = W.rtor[(size_t)TOR_SLOTS * (inf.w + j) + r];
-                            if (!(q.t < INFINITY) || q.err < 0.0f) continue;
-                            if (m != kn && q.t - tk <= q.err + ek + tie) hard = true;
-                            ++m;
+                            if (q.t < INFINITY && !(q.err < 0.0f)) f(q, true, j, r, k++);  // (else rejected or never settled)
+                        }
+                    }
+                    return k;
+                };
+                n = roots([&](const RootRec &q, bool tor, int j, int, int k) {
+                    if (q.t < first.t) first = Root{q.t, q.err, q.t64, tor ? 1 : 0, j, k};
+                    if (q.t > last.t) last = Root{q.t, q.err, q.t64, tor ? 1 : 0, j, k};
+                });
+                const Grid &G = B.grid[__ldg(&hd->mol)];
+                const float tie = 1e-6f * G.hl[1];
+                const bool in = lab == LABEL_IN || n == 1;
+                hard = !(n >= 1 && n <= WCAND && first.n >= 0);
+                Root &pick = in ? first : last;
+                if (!hard && n > 1) {  // every other candidate certainly after the first, or before the last
+                    roots([&](const RootRec &q, bool, int, int, int k) {
+                        if (k != pick.n && (in ? q.t - pick.t : pick.t - q.t) <= q.err + pick.err + tie) hard = true;
+                    });
+                }
+                const SlabAcc<T> A(sl);
+                if (!hard) {  // the piece: spheres are numbered atoms first, then triple points
+                    if (pick.kind == 0) {
+                        const int it = W.csph[inf.z + pick.slot].y;
+                        pick.kind = it < na ? 0 : 2;
+                        pick.slot = it < na ? it : it - na;
+                    } else {
+                        pick.slot = W.ctor[inf.w + pick.slot].y;
+                    }
+                    if (!in) {
+                        const bool e0 = first.t64 == first.t64, e1 = last.t64 == last.t64;  // exact roots
+                        const T d0 = sizeof(T) == sizeof(float) ? (T)G.d0 : T(0);
+                        T s[3], hT, y0[3], y1[3], w[3], dw;
+                        edge_point<T>(G, pk_point(pk), s, hT);
+                        const T rp = (T)M.rp;
+                        const T t0 = e0 ? (T)first.t64 : (T)first.t, t1 = e1 ? (T)last.t64 : (T)last.t;
+                        for (int a = 0; a < 3; ++a) {
+                            y0[a] = s[a] + (a == axis ? t0 : T(0));
+                            y1[a] = s[a] + (a == axis ? t1 : T(0));
+                        }
+                        const T f0 = (e0 ? T(2e-7) : (T)first.err) + d0, f1 = e1 ? T(2e-7) : (T)last.err;
+                        hard = true;
+                        if (root_witness<T>(A, last.kind, last.slot, y1, rp, d0, f1, w, dw)) {
+                            const T dx = y0[0] - w[0], dy = y0[1] - w[1], dz = y0[2] - w[2];
+                            hard = lt_sq<true>(dx * dx + dy * dy + dz * dz, rp * rp, rp, f0 + dw + T(2e-6)) != 1;
                         }
                     }
                 }
+                if constexpr (sizeof(T) == sizeof(float)) {
+                    // a hard edge's candidates that the bounds cannot order against the first or the last one: their
+                    // FP64 roots are made before the selection
+                    if (hard && n > 1) {
+                        auto near = [&](const Root &e, const RootRec &q, int k) {
+                            return k != e.n && fabsf(q.t - e.t) <= q.err + e.err + tie;
+                        };
+                        bool near_first = false, near_last = false;
+                        roots([&](const RootRec &q, bool, int, int, int k) {
+                            near_first = near_first || near(first, q, k);
+                            near_last = near_last || near(last, q, k);
+                        });
+                        roots([&](const RootRec &q, bool tor, int j, int r, int k) {
+                            const bool tied = near(first, q, k) || near(last, q, k) || (k == first.n && near_first) ||
+                                              (k == last.n && near_last);
+                            if (!tied || q.t64 == q.t64) return;
+                            const unsigned long long z = atomicAdd(W.ctr + 5, 1ull);
+                            if (z >= (unsigned long long)W.cap_ties) return;
+                            const int rec = (tor ? inf.w : inf.z) + j, it = tor ? W.ctor[rec].y : W.csph[rec].y;
+                            W.ties[z] = make_int4((int)g, rec, r | ((tor ? 1 : (it < na ? 0 : 2)) << 4),
+                                                  !tor && it >= na ? it - na : it);
+                        });
+                    }
+                }
                 if (!hard) {
-                    const SlabAcc<T> A(sl);
-                    const float tr = t64k == t64k ? (float)t64k : tk;
-                    code_out(out, axis, o, 0, tr, kind, A.model_index(kind, slot), lab);
+                    const float tr = pick.t64 == pick.t64 ? (float)pick.t64 : pick.t;
+                    code_out(out, axis, o, 0, tr, pick.kind, A.model_index(pick.kind, pick.slot), lab);
                 }
             }
         }
@@ -1872,183 +1946,10 @@ __global__ void __launch_bounds__(PICK_THREADS) k_edge_pick(Batch B, RootWork W,
     }
 }
 
-// 4b. FP32 form only: the listed edges that the targeted test settles, one
-// thread each.  At an outside end point the candidates go in order of t; one
-// whose point is closer than r_p to the free witness of another remaining
-// candidate is strictly outside M and dropped, and the last one left is the
-// root -- warp_select's first test with its tolerances, so an edge takes the
-// same candidate on either path.  A tie that the FP32 bounds cannot order, a
-// test that is not certain or more than SETTLE_MAX candidates leave the edge to
-// the warp selection (W.hard2); the tied candidates are listed (W.ties) and
-// their FP64 roots computed in full warps before it (k_edge_ties).
-// On the 5,000-atom globule 388 k of the warps' 653 k iterations were this
-// test, 545 warp instructions for one lane's work each, and the near ties held
-// the FP64 pipe with two lanes of 32.  Bound by the latency of an edge's
-// dependent reads (eight lanes an edge, one per candidate, took 356 us for the
-// 266 k edges against 250).
-constexpr int SETTLE_MAX = 6;
-constexpr int SETTLE_THREADS = 128;
-
-__global__ void __launch_bounds__(SETTLE_THREADS) k_edge_settle(Model M, Batch B, RootWork W,
-                                                                const int *__restrict__ edge_start, EdgeOut out)
-{
-    const long long nt = B.n_tiles;
-    const int lane = threadIdx.x & 31;
-    const long long nh = (long long)W.ctr[3], stride = (long long)gridDim.x * SETTLE_THREADS;
-    const float rp = (float)M.rp;
-    for (long long q0 = (long long)blockIdx.x * SETTLE_THREADS + (threadIdx.x & ~31); q0 < nh; q0 += stride) {
-        const long long q = q0 + lane;
-        bool left = false;
-        int g = 0;
-        if (q < nh) {
-            g = W.hard[q];
-            const int4 inf = W.einfo[g];
-            const int cnt = W.ecnt[g];
-            const int ns = cnt & 0xffff, nq = (cnt >> 16) & 0xffff;
-            const int pk = inf.y, axis = pk_axis(pk), lab = pk_label(pk), p = pk_point(pk);
-            left = true;
-            if (!pk_dropped(pk)) {
-                const unsigned char *sl = W.slab + ((size_t)(unsigned)inf.x << 4);
-                const SlabHdr *hd = reinterpret_cast<const SlabHdr *>(sl);
-                const Grid &G = B.grid[__ldg(&hd->mol)];
-                float s[3], hT;
-                edge_point<float>(G, p, s, hT);
-                const float d0 = G.d0, tie = 1e-6f * hT;
-                const SlabAcc<float> A(sl);
-                const int na = A.na();
-                // the candidates: root, error bound, best position on the edge and what it adds to d0, piece
-                float t[SETTLE_MAX], err[SETTLE_MAX], tp[SETTLE_MAX], dp[SETTLE_MAX];
-                int kind[SETTLE_MAX], id[SETTLE_MAX];
-                int n = 0;
-                for (int j = 0; j < ns + nq; ++j) {
-                    const bool sph = j < ns;
-                    const int k = sph ? inf.z + j : inf.w + (j - ns);
-                    const int nr = sph ? W.nsph[k] : W.ntor[k];
-                    for (int r = 0; r < nr; ++r) {
-                        const RootRec c = sph ? W.rsph[(size_t)SPH_SLOTS * k + r] : W.rtor[(size_t)TOR_SLOTS * k + r];
-                        if (!(c.t < INFINITY) || c.err < 0.0f) continue;  // rejected (or never settled)
-                        const int it = sph ? W.csph[k].y : W.ctor[k].y;
-#pragma unroll
-                        for (int z = 0; z < SETTLE_MAX; ++z)
-                            if (z == n) {
-                                t[z] = c.t;
-                                err[z] = c.err;
-                                tp[z] = c.t64 == c.t64 ? (float)c.t64 : c.t;
-                                dp[z] = c.t64 == c.t64 ? 2e-7f : c.err;
-                                kind[z] = sph ? (it < na ? 0 : 2) : 1;
-                                id[z] = sph && it >= na ? it - na : it;
-                            }
-                        ++n;
-                    }
-                }
-                unsigned alive = n >= 1 && n <= SETTLE_MAX ? (1u << n) - 1u : 0u;
-                int pick = -1;
-                float tie_t = INFINITY, tie_e = 0.0f;  // a tie's first candidate
-                while (alive) {
-                    // the first candidate left, and whether the bounds order it before the others
-                    int k = -1, kk = 0, ki = 0;
-                    float tk = INFINITY, ek = 0.0f, dk = 0.0f, yk = 0.0f;
-#pragma unroll
-                    for (int z = 0; z < SETTLE_MAX; ++z)
-                        if (((alive >> z) & 1u) && t[z] < tk) {
-                            k = z;
-                            tk = t[z];
-                            ek = err[z];
-                            yk = tp[z];
-                            dk = d0 + dp[z];
-                            kk = kind[z];
-                            ki = id[z];
-                        }
-                    if (k < 0) break;
-                    bool tied = false;
-#pragma unroll
-                    for (int z = 0; z < SETTLE_MAX; ++z)
-                        if (((alive >> z) & 1u) && z != k && t[z] - tk <= err[z] + ek + tie) tied = true;
-                    if (tied) {
-                        tie_t = tk;
-                        tie_e = ek;
-                        break;
-                    }
-                    const unsigned rest = alive & ~(1u << k);
-                    if (rest == 0u || lab == LABEL_IN) {
-                        pick = k;
-                        break;
-                    }
-                    float y[3] = {s[0], s[1], s[2]};
-                    y[0] += axis == 0 ? yk : 0.0f;
-                    y[1] += axis == 1 ? yk : 0.0f;
-                    y[2] += axis == 2 ? yk : 0.0f;
-                    bool outside = false;
-#pragma unroll
-                    for (int z = 0; z < SETTLE_MAX; ++z) {
-                        if (!((rest >> z) & 1u) || outside || (kind[z] == kk && id[z] == ki)) continue;
-                        if (kind[z] == 2) {
-                            const P4<float> v = A.vq(id[z]);
-                            const float dx = y[0] - v.x, dy = y[1] - v.y, dz = y[2] - v.z;
-                            outside = lt_sq<true>(dx * dx + dy * dy + dz * dz, rp * rp, rp, dk) == 1;
-                            continue;
-                        }
-                        float qx, qy, qz, dq;
-                        int e0, e1, tw, sa = id[z], sb = -1;
-                        if (kind[z] == 0) {
-                            tw = face_proposal<true>(A, id[z], y[0], y[1], y[2], rp, rp, dk, qx, qy, qz, dq, e0, e1);
-                        } else {
-                            tw = saddle_proposal<true>(A, id[z], y[0], y[1], y[2], rp, rp, dk, qx, qy, qz, dq, e0, e1);
-                            const short2 ps = A.pslot(id[z]);
-                            sa = ps.x;
-                            sb = ps.y;
-                        }
-                        outside = tw == 1 && free_witness<true>(A, qx, qy, qz, sa, sb, e0, e1, rp, dq + dk) == 1;
-                    }
-                    if (!outside) break;  // not certain: the full search decides
-                    alive = rest;
-                }
-                if (tie_t < INFINITY) {  // its roots without an FP64 value yet
-                    for (int j = 0; j < ns + nq; ++j) {
-                        const bool sph = j < ns;
-                        const int k = sph ? inf.z + j : inf.w + (j - ns);
-                        const int nr = sph ? W.nsph[k] : W.ntor[k];
-                        for (int r = 0; r < nr; ++r) {
-                            const RootRec c = sph ? W.rsph[(size_t)SPH_SLOTS * k + r] : W.rtor[(size_t)TOR_SLOTS * k + r];
-                            if (!(c.t >= tie_t && c.t < INFINITY) || c.err < 0.0f || c.t64 == c.t64 ||
-                                c.t - tie_t > c.err + tie_e + tie)
-                                continue;
-                            const int it = sph ? W.csph[k].y : W.ctor[k].y;
-                            const unsigned long long z = atomicAdd(W.ctr + 6, 1ull);
-                            if (z < (unsigned long long)W.cap_ties)
-                                W.ties[z] = make_int4(g, k, r | ((sph ? (it < na ? 0 : 2) : 1) << 4),
-                                                      sph && it >= na ? it - na : it);
-                        }
-                    }
-                }
-                if (pick >= 0) {
-                    left = false;
-                    float tr = 0.0f;
-                    int pkind = 0, pid = 0;
-#pragma unroll
-                    for (int z = 0; z < SETTLE_MAX; ++z)
-                        if (z == pick) {
-                            tr = tp[z];
-                            pkind = kind[z];
-                            pid = id[z];
-                        }
-                    const int o = g - edge_start[axis * nt];
-                    code_out(out, axis, o, 0, tr, pkind, A.model_index(pkind, pid), lab);
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, left);
-        int base = 0;
-        if (lane == 0 && m) base = (int)atomicAdd(W.ctr + 5, (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (left) W.hard2[base + __popc(m & ((1u << lane) - 1))] = g;
-    }
-}
-
-// FP64 roots of the listed tied candidates, one thread each, into their records.
+// 4b. FP32 form only: FP64 roots of the listed tied candidates, one thread each, into their records.
 __global__ void __launch_bounds__(128) k_edge_ties(Model M, Batch B, RootWork W)
 {
-    const long long n = min((long long)W.ctr[6], W.cap_ties);
+    const long long n = min((long long)W.ctr[5], W.cap_ties);
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const int4 jb = W.ties[q];
         const int4 inf = W.einfo[jb.x];
@@ -2065,8 +1966,7 @@ __global__ void __launch_bounds__(128) k_edge_ties(Model M, Batch B, RootWork W)
     }
 }
 
-// 5. The listed edges: one warp per edge (grid-stride over the list: in the
-// FP32 form those that 4b left).  The
+// 5. The listed edges: one warp per edge (grid-stride over the list).  The
 // edge's accepted roots are gathered in candidate order into the warp's
 // buffer in shared memory (at most WCAND; more is a capacity error), then
 // chosen by warp_select.  A failure is logged with its candidates.
@@ -2079,14 +1979,13 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
     __shared__ WCand cand[HARD_THREADS / 32][WCAND];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long nt = B.n_tiles;
-    const long long nh = (long long)W.ctr[FILT ? 5 : 3];
-    const int *__restrict__ list = FILT ? W.hard2 : W.hard;
+    const long long nh = (long long)W.ctr[3];
     const double rp = M.rp;
     const T rpT = (T)rp;
     WCand *c = cand[warp];
     for (long long q = (long long)blockIdx.x * (HARD_THREADS / 32) + warp; q < nh;
          q += (long long)gridDim.x * (HARD_THREADS / 32)) {
-        const int g = list[q];
+        const int g = W.hard[q];
         const int4 inf = W.einfo[g];
         const int cnt = W.ecnt[g];
         const int ns = cnt & 0xffff, nq = (cnt >> 16) & 0xffff;
@@ -2182,7 +2081,7 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
 // block's edges are first ordered by kind, tori before spheres, so nearly
 // every warp runs one of the two paths instead of both, and 1 / h comes from
 // the host: 513 -> 326 us on 1.2 M edges.
-__global__ void __launch_bounds__(POLISH_THREADS) k_edge_polish(Model M, Batch B, EdgeOut out,
+__global__ void __launch_bounds__(POLISH_THREADS, 4) k_edge_polish(Model M, Batch B, EdgeOut out,
                                                                 const long long *__restrict__ medge,
                                                                 double2 *__restrict__ term)
 {
@@ -2503,20 +2402,16 @@ static void roots_launch(const Model &M, const Batch &B, int threads, EdgeOut ou
     const int gs = std::max(g_occ_roots[P][0][ts], 1) * g_edge_n_sm;
     const int gq = std::max(g_occ_roots[P][1][ts], 1) * g_edge_n_sm;
     k_roots_sphere<T, FILT><<<gs, tb, 0, st>>>(M, B, W, err);
-    cudaMemsetAsync(W.ctr + 3, 0, 4 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, hard edges, ties
+    cudaMemsetAsync(W.ctr + 3, 0, 3 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, ties
     k_roots_torus<T, FILT><<<gq, tb, 0, st>>>(M, B, W, err);
     if (FILT)
         k_roots_torus_exact<T, FILT><<<std::max(g_occ_exact[P], 1) * g_edge_n_sm, tb, 0, st>>>(M, B, W, err);
     const long long pb = std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, PICK_THREADS), 1),
                                              8LL * g_edge_n_sm);
-    k_edge_pick<T><<<(unsigned)pb, PICK_THREADS, 0, st>>>(B, W, edge_start, ne_all, out, err);
-    if (FILT) {
-        k_edge_settle<<<(unsigned)std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, 4 * SETTLE_THREADS), 1),
-                                                      8LL * g_edge_n_sm),
-                        SETTLE_THREADS, 0, st>>>(M, B, W, edge_start, out);
+    k_edge_pick<T><<<(unsigned)pb, PICK_THREADS, 0, st>>>(M, B, W, edge_start, ne_all, out, err);
+    if (FILT)
         k_edge_ties<<<(unsigned)std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, 1024), 1), 8LL * g_edge_n_sm),
                       128, 0, st>>>(M, B, W);
-    }
     k_edge_hard<T, FILT><<<std::max(g_occ_hard[P], 1) * g_edge_n_sm, HARD_THREADS, 0, st>>>(
         M, B, W, edge_start, out, n_fail, err, fail_log);
 }
@@ -2542,7 +2437,7 @@ int launch_edge_roots(const Model &M, const Batch &B, int precision, int threads
         roots_launch<double, false>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
     else
         roots_launch<float, true>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
-    return precision == 0 ? 4 : 7;
+    return precision == 0 ? 4 : 6;
 }
 
 long long polish_blocks(long long n_edges) { return n_edges > 0 ? ceil_div_ll(n_edges, POLISH_THREADS) : 0; }

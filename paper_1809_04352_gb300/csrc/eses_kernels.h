@@ -105,9 +105,8 @@ struct RootRec {
 };
 // buffers of the phased root solve; the capacities are planned by the caller
 // from the totals the staging pass adds up in ctr ([0] slab bytes, [1] sphere
-// and [2] torus candidates; [3] edges not picked at once; [4] torus candidates
-// listed for FP64 work; [5] edges left to the warp selection, [6] tied
-// candidates, FP32 form)
+// and [2] torus candidates; [3] edges listed for the warp selection; [4] torus
+// candidates and [5] tied candidates listed for FP64 work, FP32 form)
 struct RootWork {
     int4 *einfo;            // per crossing edge: slab (16-byte units), packed point/axis/label/dropped,
                             // first sphere and first torus candidate
@@ -117,7 +116,7 @@ struct RootWork {
     RootRec *rsph, *rtor;   // their roots: 2 slots per sphere candidate, 4 per torus candidate
     unsigned char *slab;    // staged tiles
     unsigned long long *ctr;  // 8 counters, [4] the torus candidates listed for FP64 work
-    int *hard, *hard2;      // edges listed for the selections: not picked at once; left to a warp each (FP32 form)
+    int *hard;              // edges listed for the warp selection (at most one per edge)
     int4 *ties;             // tied candidates for FP64 roots: (edge, record, slot | kind << 4, staged item)
     int2 *jobs;             // torus candidates with FP64 work: (candidate, 1 pending slots / 2 whole)
     long long cap_slab, cap_sph, cap_tor, cap_jobs, cap_ties;
