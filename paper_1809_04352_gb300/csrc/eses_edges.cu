@@ -231,26 +231,89 @@ __device__ __noinline__ double exact_root_torus(const double *o, const double *u
     return t;
 }
 
-// unit normal at y (towards the witness, i.e. into the solvent)
-__device__ __forceinline__ void exact_normal(int kind, const double *c, const double *u, double rho, const double *y,
-                                             double *n)
+// The polish's form of the two, with the unit normal (towards the witness, i.e.
+// into the solvent), in as few FP64 instructions as the same accuracy takes: a
+// warp issues one in 16 cycles, a division or square root is about ten of them.
+__device__ __forceinline__ void unit_of(double *n)
 {
-    double v[3];
-    if (kind == 0) {  // convex: radial, outward
-        v[0] = y[0] - c[0]; v[1] = y[1] - c[1]; v[2] = y[2] - c[2];
-    } else if (kind == 2) {  // concave: towards the probe centre
-        v[0] = c[0] - y[0]; v[1] = c[1] - y[1]; v[2] = c[2] - y[2];
-    } else {  // saddle: towards the nearest point of the circle
-        double yo[3] = {y[0] - c[0], y[1] - c[1], y[2] - c[2]};
-        double w[3];
-        axis_normal(yo, u, w);
-        v[0] = rho * w[0] - yo[0]; v[1] = rho * w[1] - yo[1]; v[2] = rho * w[2] - yo[2];
+    const double vv = n[0] * n[0] + n[1] * n[1] + n[2] * n[2];
+    const double iv = vv > 0.0 ? rsqrt(vv) : 0.0;
+    n[0] *= iv;
+    n[1] *= iv;
+    n[2] *= iv;
+}
+
+__device__ __forceinline__ double into_edge(double t, double h) { return t > 0.0 ? (t < h ? t : h) : 0.0; }
+
+// Sphere (`out`: 1 an atom's, its normal radial; -1 a probe's, towards its
+// centre).  The root is -b +- sqrt(rad^2 - the distance^2 of the edge's line),
+// without the b^2 that the quadratic's discriminant adds and takes off again
+// and without a division: its largest and mean error against 80-bit arithmetic
+// are at or below the quadratic formula's (mean 2.8e-16 and 3.3e-16 A at h 0.1).
+__device__ __forceinline__ double polish_sphere(const double *c, double rad, double out, const double *s, int axis,
+                                                double t0, double h, double *n)
+{
+    double d[3] = {s[0] - c[0], s[1] - c[1], s[2] - c[2]};
+    const double b = d[axis];
+    const double p = d[axis == 0 ? 1 : 0], q = d[axis == 2 ? 1 : 2];
+    const double disc = (rad * rad - p * p) - q * q;
+    double t = t0;
+    if (disc >= 0.0) {
+        const double sq = sqrt(disc);
+        t = t0 <= -b ? -b - sq : -b + sq;  // the root on t0's side of their middle
     }
-    double vn = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-    double iv = vn > 0.0 ? 1.0 / vn : 0.0;
-    n[0] = v[0] * iv;
-    n[1] = v[1] * iv;
-    n[2] = v[2] * iv;
+    t = into_edge(t, h);
+    d[axis] += t;
+    n[0] = out * d[0];
+    n[1] = out * d[1];
+    n[2] = out * d[2];
+    unit_of(n);
+    return t;
+}
+
+// Torus: Newton steps on the quartic as exact_root_torus, the slope's inverse
+// in FP32 (the step's relative error, 1e-7, only multiplies the error that is
+// left), ended once a step moves t by less than 1e-11 A (the next would move
+// it by the square of that times the quartic's curvature over its slope, and
+// by 1e-18 A for the slope's rounding); normal towards the nearest point of
+// the circle.
+__device__ __forceinline__ double polish_torus(const double *o, const double *u, double rho, double rp, const double *s,
+                                               int axis, double t0, double h, double *n)
+{
+    double co[5];
+    torus_coeffs(o, u, rho, rp, s, axis, co);
+    const double dc[4] = {co[1], 2.0 * co[2], 3.0 * co[3], 4.0};
+    double t = t0;
+    for (int it = 0; it < 4; ++it) {
+        const double f = horner<double, 4>(co, t);
+        const float df = (float)horner<double, 3>(dc, t);
+        if (fabsf(df) < 1e-30f) break;
+        const double dt = f * (double)(1.0f / df);
+        t -= dt;
+        if (fabs(dt) < 1e-11) break;
+    }
+    t = into_edge(t, h);
+    double y[3] = {s[0] - o[0], s[1] - o[1], s[2] - o[2]}, w[3];
+    y[axis] += t;
+    // the direction from the circle's axis to y, as axis_normal; y on the axis is left to it
+    const double z = y[0] * u[0] + y[1] * u[1] + y[2] * u[2];
+    for (int k = 0; k < 3; ++k) w[k] = y[k] - z * u[k];
+    const double zr = w[0] * u[0] + w[1] * u[1] + w[2] * u[2];
+    for (int k = 0; k < 3; ++k) w[k] -= zr * u[k];
+    const double ww = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+    if ((float)ww > 1e-12f * (1.0f + (float)z * (float)z)) {
+        const double k = rho * rsqrt(ww);
+        n[0] = k * w[0] - y[0];
+        n[1] = k * w[1] - y[1];
+        n[2] = k * w[2] - y[2];
+    } else {
+        axis_normal(y, u, w);
+        n[0] = rho * w[0] - y[0];
+        n[1] = rho * w[1] - y[1];
+        n[2] = rho * w[2] - y[2];
+    }
+    unit_of(n);
+    return t;
 }
 
 // exact root of a staged piece (tile frame, FP64 data from HBM) near t0
@@ -2077,10 +2140,12 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
 
 // One thread per crossing edge, over the three axes: FP64 root of the chosen
 // piece next to the recorded FP32 root, normal, outputs, area/volume terms.
-// Bound by FP64 issue (one warp instruction per 16 cycles per SM).  The
-// block's edges are first ordered by kind, tori before spheres, so nearly
-// every warp runs one of the two paths instead of both, and 1 / h comes from
-// the host: 513 -> 326 us on 1.2 M edges.
+// Bound by FP64 issue (one warp instruction per 16 cycles per SM, 83 % of the
+// time).  The block's edges are first ordered by kind, tori before spheres, so
+// nearly every warp runs one of the two paths instead of both (513 -> 326 us
+// on 1.2 M edges), four blocks stay on an SM (285 us; 82 -> 68 us on 0.1 M
+// edges), and the two paths spend few FP64 divisions and square roots
+// (polish_sphere, polish_torus): 443 -> 305 us on 1.9 M edges, 58 -> 42 us on 0.18 M.
 __global__ void __launch_bounds__(POLISH_THREADS, 4) k_edge_polish(Model M, Batch B, EdgeOut out,
                                                                 const long long *__restrict__ medge,
                                                                 double2 *__restrict__ term)
@@ -2145,23 +2210,15 @@ __global__ void __launch_bounds__(POLISH_THREADS, 4) k_edge_polish(Model M, Batc
         }
         double t = 0.5 * h, n[3] = {0.0, 0.0, 0.0};
         if (!failed && !bad) {
-            double c[3], u[3] = {0.0, 0.0, 0.0}, rho = 0.0;
             if (kind != 1) {
                 const double4 g = kind == 0 ? M.atom[mid] : M.vert[mid];
-                c[0] = g.x; c[1] = g.y; c[2] = g.z;
-                t = exact_root_sphere(c, kind == 0 ? g.w : rp, s, a, (double)t32);
+                const double c[3] = {g.x, g.y, g.z};
+                t = polish_sphere(c, kind == 0 ? g.w : rp, kind == 0 ? 1.0 : -1.0, s, a, (double)t32, h, n);
             } else {
-                double4 g = M.pair_o[mid];
-                double4 q = M.pair_u[mid];
-                c[0] = g.x; c[1] = g.y; c[2] = g.z;
-                u[0] = q.x; u[1] = q.y; u[2] = q.z;
-                rho = g.w;
-                t = exact_root_torus(c, u, rho, rp, s, a, (double)t32);
+                const double4 g = M.pair_o[mid], q = M.pair_u[mid];
+                const double c[3] = {g.x, g.y, g.z}, u[3] = {q.x, q.y, q.z};
+                t = polish_torus(c, u, g.w, rp, s, a, (double)t32, h, n);
             }
-            t = fmin(fmax(t, 0.0), h);
-            double y[3] = {s[0], s[1], s[2]};
-            y[a] += t;
-            exact_normal(kind, c, u, rho, y, n);
         }
         const double tau = t * G.ih;
         out.tau[a][o] = tau;
