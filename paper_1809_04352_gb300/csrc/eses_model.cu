@@ -484,20 +484,76 @@ __device__ __forceinline__ int arc_lt(float d2, float t, float delta)
 // lane takes candidates a = lane, lane + 32, ...: its cover of the circle, its
 // end points and their freeness against every other candidate.  Emitted triple points keep the order (a, end point):
 // the count pass lists them (2 k + end point) for k_verts, which computes them one thread each.
-// Bound by FP64 issue wherever a lane needs an exact end point (one warp
-// instruction per 16 cycles per SM): with FP64 end points past a bound of 2e-4 A
-// about one lane in two circles took them (2.0 ms on 5,000 atoms at 0.1
-// atoms/A^3, 1.4 ms on 32 molecules at h 0.5; 0.62 and 0.52 ms now, bound by
-// issue: half the candidates of a circle cover nothing of it and are dropped
-// before the pairwise tests, each of which is two multiply-adds in the plane).
-constexpr int ARC_WARPS = 4;
-constexpr int ARC_CTAS = 8;  // resident blocks asked for: 64 registers, the FP64 fallbacks' values spilled (106: 4 blocks)
+// Bound by issue and the latency of the neighbours' loads.  FP64 (one warp
+// instruction per 16 cycles per SM) is left to end points that FP32 cannot
+// decide (with FP64 end points past a bound of 2e-4 A about one lane in two
+// circles took them: 2.0 ms on 5,000 atoms at 0.1 atoms/A^3, 1.4 ms on 32
+// molecules at h 0.5).  Half the candidates of a circle cover nothing of it and
+// are dropped as they are gathered (614 and 520 us); a circle covered whole by
+// one ends there (two in three in the dense box), one covered all around by
+// several before any end point is tested against the others, and blocks are
+// one warp, so a long circle holds up no other warp's registers (410 and 537 us
+// with four): 337 and 445 us.
+constexpr int ARC_WARPS = 1;
+constexpr int ARC_CTAS = 32;  // resident blocks asked for: 64 registers, the FP64 fallbacks' values spilled (106: 16)
 
 struct ArcWarp {
     float4 nb[ARC_MAXN];
     int nbk[ARC_MAXN];
     int code[ARC_CODES];
 };
+
+// FP32 end points of a candidate's cover of the circle, in the circle's plane
+// (c: its centre there, num, en + ed; see below): status 1 partial for certain
+// with end points within dq (e = 0 counterclockwise of the centre, e = 1
+// clockwise), 0 it covers nothing for certain, -1 FP64 decides.
+struct ArcEnds {
+    float q1[2], q2[2], dq;
+    float gap;  // half the distance between the end points (0: unknown)
+    int status;
+};
+__device__ __forceinline__ ArcEnds arc_ends(float4 c, float rho, float dlt)
+{
+    ArcEnds r;
+    r.q1[0] = r.q1[1] = r.q2[0] = r.q2[1] = 0.0f;
+    r.dq = 1.0f;
+    r.gap = 0.0f;
+    const float A = sqrtf(c.x * c.x + c.y * c.y);
+    const float num = c.z, den = 2.0f * rho * A, err = 2.0f * c.w;
+    if (num >= den + err) {
+        r.status = 0;
+    } else if (!(num < den - err && num > -den + err)) {
+        r.status = -1;
+    } else {
+        const float T = num / den;
+        const float sT = sqrtf(fmaxf(0.0f, 1.0f - T * T));
+        const float iA = 1.0f / A, e1 = c.x * iA, e2 = c.y * iA;
+        for (int e = 0; e < 2; ++e) {
+            const float sg = e == 0 ? sT : -sT;
+            r.q1[e] = rho * (T * e1 - sg * e2);
+            r.q2[e] = rho * (T * e2 + sg * e1);
+        }
+        // (c.w bounds num's error and den's together, so also |T| of den's)
+        const float dT = c.w / den;
+        float dq = rho * (dT * (1.0f + fabsf(T) / fmaxf(sT, 1e-6f)) + 2.0f * (dlt / fmaxf(A, 1e-6f) + 3e-7f)) + 1e-6f;
+        // past 2e-4 A the bound still holds to a tenth while dT << sT^2 (the second-order part of
+        // the end point's shift is dT / (2 sT^2) of the first-order one)
+        if (dq > 2e-4f) dq = dT < 0.05f * sT * sT && dq < 1.8e-2f ? 1.1f * dq : 1.0f;
+        r.dq = dq;
+        r.gap = rho * sT;
+        r.status = dq > 2e-2f ? -1 : 1;
+    }
+    return r;
+}
+
+// place of a circle point on 64 bins of the circle, increasing counterclockwise
+// (the diamond angle y / (|x| + |y|), unrolled over the half planes; at most
+// one bin for 1/16 of the circle's radius along the circle)
+__device__ __forceinline__ float circle_bin(float x, float y)
+{
+    const float p = __fdividef(y, fabsf(x) + fabsf(y));
+    return 16.0f * (x >= 0.0f ? 1.0f + p : 3.0f - p);
+}
 
 template <bool EMIT>
 __device__ int arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pair_free, int *vert_count,
@@ -521,39 +577,79 @@ __device__ int arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pai
                 djz = (jh.z - oh.z) + (jl.z - ol.z);
     const float rpf = (float)M.rp;
     const float Rj = jh.w + rpf;
-    const double4 cj = M.atom[j];
-    const double Rj64 = cj.w + M.rp;
-    // 1. common neighbours, in list order
+    CircleFrame f;
+    bool have64 = false;
+    // 1. The common neighbours that could cover part of the circle, in list
+    //    order.  One that covers the whole circle ends the work at once (at
+    //    protein packing most circles are buried this way): FP64 when undecided.
+    //    Each is left in the circle's plane: its centre (d1, d2), num
+    //    = rho^2 + |d|^2 - R^2 (a circle point q is covered iff 2 q.d > num)
+    //    and the error bound en + ed of either side.
+    //    One that certainly covers nothing of the circle is dropped: it covers
+    //    no end point either.
+    bool full = false;
+    float amax = 0.0f, emax = 0.0f;  // the lanes' largest |(d1, d2)| and error bound
     int n = 0;
     const int t_end = M.nb_start[i + 1];
-    for (int t0 = M.nb_start[i]; t0 < t_end; t0 += 32) {
-        const int t = t0 + lane;
-        bool keep = false;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        int k = -1;
-        if (t < t_end) {
-            k = M.nb_list[t];
-            if (k != j) {
-                const float4 kh = M.atom_hi[k], kl = M.atom_lo[k];
-                const float dx = (kh.x - oh.x) + (kl.x - ol.x), dy = (kh.y - oh.y) + (kl.y - ol.y),
-                            dz = (kh.z - oh.z) + (kl.z - ol.z);
-                const float Rk = kh.w + rpf;
-                const float ex = dx - djx, ey = dy - djy, ez = dz - djz;
-                const int c = arc_lt(ex * ex + ey * ey + ez * ez, Rk + Rj, 2.0f * dlt);
-                keep = c == 1 || (c < 0 && common_nb(M, k, i, j, cj, Rj64));
-                v = make_float4(dx, dy, dz, Rk);
+    int t = M.nb_start[i] + lane;
+    int k_next = t < t_end ? M.nb_list[t] : j;
+    for (int t0 = t - lane; t0 < t_end && !full; t0 += 32) {
+        const int k = k_next;
+        t += 32;
+        k_next = t < t_end ? M.nb_list[t] : j;
+        bool whole = false, keep = false;
+        float4 flat = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k != j) {
+            const float4 kh = M.atom_hi[k], kl = M.atom_lo[k];
+            const float dx = (kh.x - oh.x) + (kl.x - ol.x), dy = (kh.y - oh.y) + (kl.y - ol.y),
+                        dz = (kh.z - oh.z) + (kl.z - ol.z);
+            const float Rk = kh.w + rpf;
+            const float ex = dx - djx, ey = dy - djy, ez = dz - djz;
+            const int cm = arc_lt(ex * ex + ey * ey + ez * ez, Rk + Rj, 2.0f * dlt);
+            if (cm != 0) {
+                const float d1 = dx * v1x + dy * v1y + dz * v1z;
+                const float d2 = dx * v2x + dy * v2y + dz * v2z;
+                const float dd = dx * dx + dy * dy + dz * dz;
+                const float A = sqrtf(d1 * d1 + d2 * d2);
+                const float num = rho * rho + dd - Rk * Rk, den = 2.0f * rho * A;
+                const float dk = sqrtf(dd);
+                const float en = 2.0f * dk * dlt + 2e-6f * (rho * rho + dd + Rk * Rk);
+                const float ed = 2.0f * rho * (dlt + 3e-7f * dk) + 2e-6f * den;
+                const float err = 2.0f * (en + ed);
+                keep = num < den + err;
+                if (keep && cm < 0) {
+                    const double4 cj = M.atom[j];
+                    keep = common_nb(M, k, i, j, cj, cj.w + M.rp);
+                }
+                if (keep) {
+                    flat = make_float4(d1, d2, num, en + ed);
+                    amax = fmaxf(amax, A);
+                    emax = fmaxf(emax, en + ed);
+                    if (num < -den - err) {
+                        whole = true;
+                    } else if (num < -den + err) {  // undecided near a whole cover: FP64
+                        if (!have64) {
+                            f = frame_of(M.pair_o[p], M.pair_u[p]);
+                            have64 = true;
+                        }
+                        const double4 ck = M.atom[k];
+                        double3 qa, qb;
+                        whole = cover_of(f, ck, ck.w + M.rp, qa, qb) == 2;
+                    }
+                }
             }
         }
+        full = __any_sync(full_mask, whole);
         const unsigned m = __ballot_sync(full_mask, keep);
         const int pos = n + __popc(m & ((1u << lane) - 1));
         if (keep && pos < ARC_MAXN) {
-            W.nb[pos] = v;
+            W.nb[pos] = flat;
             W.nbk[pos] = k;
         }
         n += __popc(m);
     }
     __syncwarp();
-    if (n > ARC_MAXN) {  // very crowded circle: the FP64 form, one lane
+    if (!full && n > ARC_MAXN) {  // very crowded circle: the FP64 form, one lane
         int listed = 0;
         if (lane == 0) {
             arcs_of_pair<EMIT>(M, p, pair_free, vert_count, vert_start, vert);
@@ -561,143 +657,92 @@ __device__ int arcs_of_pair_warp(const Model &M, int p, ArcWarp &W, uint8_t *pai
         }
         return __shfl_sync(full_mask, listed, 0);
     }
-    CircleFrame f;
-    bool have64 = false;
-    // 2. a candidate that covers the whole circle ends the work before any
-    //    end point is tested (at protein packing most circles are buried
-    //    this way): the same cover decisions as below, FP64 when undecided
-    //    Each candidate is left in the circle's plane: its centre (d1, d2), num
-    //    = rho^2 + |d|^2 - R^2 (a circle point q is covered iff 2 q.d > num)
-    //    and the error bound en + ed of either side.
-    //    A candidate that certainly covers nothing of the circle is dropped:
-    //    it covers no end point either.
-    bool full = false;
-    float amax = 0.0f, emax = 0.0f;  // the lanes' largest |(d1, d2)| and error bound
-    const int n_common = n;
-    n = 0;
-    for (int r = 0; r * 32 < n_common && !full; ++r) {
-        const int a = r * 32 + lane;
-        bool whole = false, keep = false;
-        float4 flat = make_float4(0.f, 0.f, 0.f, 0.f);
-        int ka = 0;
-        if (a < n_common) {
-            const float4 c = W.nb[a];
-            const float d1 = c.x * v1x + c.y * v1y + c.z * v1z;
-            const float d2 = c.x * v2x + c.y * v2y + c.z * v2z;
-            const float dd = c.x * c.x + c.y * c.y + c.z * c.z;
-            const float A = sqrtf(d1 * d1 + d2 * d2);
-            const float num = rho * rho + dd - c.w * c.w, den = 2.0f * rho * A;
-            const float dk = sqrtf(dd);
-            const float en = 2.0f * dk * dlt + 2e-6f * (rho * rho + dd + c.w * c.w);
-            const float ed = 2.0f * rho * (dlt + 3e-7f * dk) + 2e-6f * den;
-            const float err = 2.0f * (en + ed);
-            keep = num < den + err;
-            flat = make_float4(d1, d2, num, en + ed);
-            ka = W.nbk[a];
-            if (keep) {
-                amax = fmaxf(amax, A);
-                emax = fmaxf(emax, en + ed);
-            }
-            if (num < -den - err) {
-                whole = true;
-            } else if (num < -den + err) {  // undecided near a whole cover: FP64
-                if (!have64) {
-                    f = frame_of(M.pair_o[p], M.pair_u[p]);
-                    have64 = true;
+    // 2. The bins of the circle that some candidate covers for certain: no end
+    //    point in them is free, and a circle covered all around is buried
+    //    without any end point tested against the others.
+    unsigned cov_lo = 0u, cov_hi = 0u;
+    for (int r = 0; r * 32 < n && !full; ++r) {
+        unsigned long long bins = 0ull;
+        if (r * 32 + lane < n) {
+            const ArcEnds a = arc_ends(W.nb[r * 32 + lane], rho, dlt);
+            const float eps = 16.5f * a.dq / rho + 1e-3f;
+            // (end points further apart than their errors, so that their order on the circle is known)
+            if (a.status == 1 && eps < 0.5f && a.gap > 4.0f * a.dq) {
+                const float b0 = circle_bin(a.q1[0], a.q2[0]), b1 = circle_bin(a.q1[1], a.q2[1]);
+                const int first = (int)ceilf(b1 + eps), last = (int)floorf((b0 < b1 ? b0 + 64.0f : b0) - eps);
+                const int len = min(last - first, 63);
+                if (len > 0) {
+                    const unsigned long long ones = (1ull << len) - 1ull;
+                    const int sh = first & 63;
+                    bins = (ones << sh) | (sh ? ones >> (64 - sh) : 0ull);
                 }
-                const double4 ck = M.atom[ka];
-                double3 qa, qb;
-                whole = cover_of(f, ck, ck.w + M.rp, qa, qb) == 2;
             }
         }
-        full = __any_sync(full_mask, whole);
-        // (places at or below the ones just read: the votes stand between reads and writes)
-        const unsigned m = __ballot_sync(full_mask, keep);
-        if (keep) {
-            const int at = n + __popc(m & ((1u << lane) - 1));
-            W.nb[at] = flat;
-            W.nbk[at] = ka;
-        }
-        n += __popc(m);
-        __syncwarp();
+        cov_lo |= __reduce_or_sync(full_mask, (unsigned)bins);
+        cov_hi |= __reduce_or_sync(full_mask, (unsigned)(bins >> 32));
     }
-    if (full) {
+    if (full || (cov_lo & cov_hi) == 0xffffffffu) {
         if (!EMIT && lane == 0) {
             pair_free[p] = 0;
             vert_count[p] = 0;
         }
         return 0;
     }
+    const unsigned long long covered = ((unsigned long long)cov_hi << 32) | cov_lo;
     for (int o = 16; o > 0; o >>= 1) {
         amax = fmaxf(amax, __shfl_xor_sync(full_mask, amax, o));
         emax = fmaxf(emax, __shfl_xor_sync(full_mask, emax, o));
     }
     __syncwarp();
     // 3. candidates a = lane + 32 r: covers, end points and their freeness.  An
-    //    end point q (in the plane) is tested against every other candidate with
-    //    two multiply-adds and one bound for all of them: 2 q.d - num against
-    //    2 |dq| max |d| + 2 max(en + ed).  Only an end point that no candidate
-    //    covers for certain and some could is taken to FP64.
+    //    end point q (in the plane) outside the covered bins is tested against
+    //    every other candidate with two multiply-adds and one bound for all of
+    //    them: 2 q.d - num against 2 |dq| max |d| + 2 max(en + ed).  Only an end
+    //    point that no candidate covers for certain and some could is taken to
+    //    FP64.
     int n_partial = 0, n_free_end = 0, n_emit_total = 0;
     const int w0 = EMIT ? vert_start[p] : 0;
     for (int r = 0; r * 32 < n; ++r) {
         const int a = r * 32 + lane;
         int status = 0;  // 0 none, 1 partial, 2 full
-        bool fr[2] = {false, false};
+        bool fr[2] = {false, false}, open[2] = {true, true};
         double3 qe[2];
         bool e64 = false;
         if (a < n) {
-            const float4 c = W.nb[a];
-            const float A = sqrtf(c.x * c.x + c.y * c.y);
-            const float num = c.z, den = 2.0f * rho * A, err = 2.0f * c.w;
-            float q1[2] = {0.0f, 0.0f}, q2[2] = {0.0f, 0.0f};
-            float dq = 1.0f;
-            if (num >= den + err) {
-                status = 0;
-            } else if (num < -den - err) {
-                status = 2;
-            } else {
-                status = 1;
-                if (num < den - err && num > -den + err) {  // partial for certain: FP32 end points
-                    const float T = num / den;
-                    const float sT = sqrtf(fmaxf(0.0f, 1.0f - T * T));
-                    const float iA = 1.0f / A, e1 = c.x * iA, e2 = c.y * iA;
-                    for (int e = 0; e < 2; ++e) {
-                        const float sg = e == 0 ? sT : -sT;
-                        q1[e] = rho * (T * e1 - sg * e2);
-                        q2[e] = rho * (T * e2 + sg * e1);
-                    }
-                    // (c.w bounds num's error and den's together, so also |T| of den's)
-                    const float dT = c.w / den;
-                    dq = rho * (dT * (1.0f + fabsf(T) / fmaxf(sT, 1e-6f)) + 2.0f * (dlt / fmaxf(A, 1e-6f) + 3e-7f)) +
-                         1e-6f;
-                    // past 2e-4 A the bound still holds to a tenth while dT << sT^2 (the second-order part of
-                    // the end point's shift is dT / (2 sT^2) of the first-order one)
-                    if (dq > 2e-4f) dq = dT < 0.05f * sT * sT && dq < 1.8e-2f ? 1.1f * dq : 1.0f;
+            const ArcEnds ar = arc_ends(W.nb[a], rho, dlt);
+            float q1[2] = {ar.q1[0], ar.q1[1]}, q2[2] = {ar.q2[0], ar.q2[1]};
+            float dq = ar.dq;
+            status = ar.status;
+            if (status < 0) {  // undecided cover or loose FP32 end points: FP64
+                if (!have64) {
+                    f = frame_of(M.pair_o[p], M.pair_u[p]);
+                    have64 = true;
                 }
-                if (dq > 2e-2f) {  // undecided cover or loose FP32 end points: FP64
-                    if (!have64) {
-                        f = frame_of(M.pair_o[p], M.pair_u[p]);
-                        have64 = true;
+                const double4 ck = M.atom[W.nbk[a]];
+                const int cov = cover_of(f, ck, ck.w + M.rp, qe[0], qe[1]);
+                status = cov;
+                if (cov == 1) {
+                    for (int e = 0; e < 2; ++e) {
+                        const float qx = (float)(qe[e].x - f.o.x), qy = (float)(qe[e].y - f.o.y),
+                                    qz = (float)(qe[e].z - f.o.z);
+                        q1[e] = qx * v1x + qy * v1y + qz * v1z;
+                        q2[e] = qx * v2x + qy * v2y + qz * v2z;
                     }
-                    const double4 ck = M.atom[W.nbk[a]];
-                    const int cov = cover_of(f, ck, ck.w + M.rp, qe[0], qe[1]);
-                    status = cov;
-                    if (cov == 1) {
-                        for (int e = 0; e < 2; ++e) {
-                            const float qx = (float)(qe[e].x - f.o.x), qy = (float)(qe[e].y - f.o.y),
-                                        qz = (float)(qe[e].z - f.o.z);
-                            q1[e] = qx * v1x + qy * v1y + qz * v1z;
-                            q2[e] = qx * v2x + qy * v2y + qz * v2z;
-                        }
-                        dq = 1e-6f + 1e-6f * rho;
-                        e64 = true;
-                    }
+                    dq = 1e-6f + 1e-6f * rho;
+                    e64 = true;
                 }
             }
             if (status == 1) {
+                const float eps = 16.5f * dq / rho + 1e-3f;
+                for (int e = 0; e < 2 && eps < 0.5f; ++e) {
+                    const float b = circle_bin(q1[e], q2[e]);
+                    const int lo = (int)floorf(b - eps) & 63, hi = (int)floorf(b + eps) & 63;
+                    open[e] = !((covered >> lo) & (covered >> hi) & 1ull);
+                }
+            }
+            if (status == 1 && (open[0] || open[1])) {
                 const float E = 2.0f * (dq * amax + emax);
-                bool cov0 = false, cov1 = false, und0 = false, und1 = false;
+                bool cov0 = !open[0], cov1 = !open[1], und0 = false, und1 = false;
                 const float x0 = 2.0f * q1[0], y0 = 2.0f * q2[0], x1 = 2.0f * q1[1], y1 = 2.0f * q2[1];
                 for (int b = 0; b < n && !(cov0 && cov1); ++b) {
                     const float4 cb = W.nb[b];

@@ -96,6 +96,29 @@ def test_circle_with_many_free_end_points():
         eses.eses_destroy(ctx)
 
 
+@pytest.mark.parametrize("k", [2, 3, 5, 8, 31, 32, 33, 40])
+def test_circle_covered_all_around(k):
+    """The circle of two large balls under a ring of k others: neighbours that
+    miss each other by a thousandth leave two free triple points each, that
+    overlap by a thousandth none, and two where one of the ring is missing."""
+    libbuild.build()
+    rho = np.sqrt((30.0 + 1.4) ** 2 - 10.0 ** 2)
+    phi = 0.3 + 2.0 * np.pi * np.arange(k) / k
+    for delta, drop, expect in ((-1e-3, 0, 2 * k), (1e-3, 0, 0), (1e-3, 1, 2)):
+        ring = np.stack([np.zeros(k), rho * np.cos(phi), rho * np.sin(phi)], 1)[drop:]
+        reach = 2.0 * rho * np.sin(0.5 * np.pi / k * (1.0 + delta))  # covers pi / k (1 + delta) to either side
+        xyz = np.concatenate([[[-10.0, 0.0, 0.0], [10.0, 0.0, 0.0]], ring])
+        rad = np.concatenate([[30.0, 30.0], np.full(k - drop, reach - 1.4)])
+        ctx = eses.eses_create(xyz, rad, 1.4, 3.0, 3.1)
+        try:
+            eses.eses_run(ctx)
+            v = eses.eses_patch_data(ctx)["vertices"]
+            d = np.abs(np.linalg.norm(v[:, None, :] - xyz[None, :2], axis=2) - 31.4) if len(v) else np.zeros((0, 2))
+            assert int((d.max(1) < 1e-9).sum() if len(d) else 0) == expect
+        finally:
+            eses.eses_destroy(ctx)
+
+
 def test_buffers_left_by_grown_ones_are_taken_again():
     """Runs of changing size in one context (block selections up and down, the
     whole grid) reuse the memory they gave up: after the first round the
