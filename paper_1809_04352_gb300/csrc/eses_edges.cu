@@ -72,6 +72,13 @@ __device__ __forceinline__ double root_eps<double>() { return 1e-15; }
 template <>
 __device__ __forceinline__ float root_eps<float>() { return 2e-7f; }
 
+template <class R>
+__device__ __forceinline__ R fp_eps();
+template <>
+__device__ __forceinline__ double fp_eps<double>() { return 2.3e-16; }
+template <>
+__device__ __forceinline__ float fp_eps<float>() { return 1.2e-7f; }
+
 template <class R, int DEG>
 __device__ __forceinline__ R horner(const R *c, R t)
 {
@@ -88,7 +95,13 @@ __device__ R mono_root(const R *c, R a, R b, R fa)
     R dc[DEG];
 #pragma unroll
     for (int k = 0; k < DEG; ++k) dc[k] = (R)(k + 1) * c[k + 1];
-    R t = R(0.5) * (a + b);
+    // rounding of c's value on [a, b]
+    const R m = fmax(fabs(a), fabs(b));
+    R noise = fabs(c[DEG]);
+#pragma unroll
+    for (int k = DEG - 1; k >= 0; --k) noise = noise * m + fabs(c[k]);
+    noise *= fp_eps<R>();
+    R t = R(0.5) * (a + b), step = INFINITY;
     for (int it = 0; it < 100; ++it) {
         R f = horner<R, DEG>(c, t);
         if (f == R(0)) return t;
@@ -96,8 +109,15 @@ __device__ R mono_root(const R *c, R a, R b, R fa)
         else b = t;
         R df = horner<R, DEG - 1>(dc, t);
         R tn = (df != R(0)) ? t - f / df : R(0.5) * (a + b);
-        if (!(tn > a && tn < b)) tn = R(0.5) * (a + b);
-        if (fabs(tn - t) <= root_eps<R>() * fmax(R(1), fabs(t))) return tn;
+        const bool out = !(tn > a && tn < b);
+        // at its rounding f gives no better t once the steps leave the bracket
+        // or no longer shrink (without this the search goes back to the middle of
+        // the bracket, again and again until that has closed or for 100 steps)
+        if (fabs(f) <= noise && (out || fabs(tn - t) >= R(0.75) * step)) return out ? t : tn;
+        if (out) tn = R(0.5) * (a + b);
+        const R d = fabs(tn - t);
+        if (d <= root_eps<R>() * fmax(R(1), fabs(t))) return tn;
+        step = d;
         t = tn;
         if (b - a <= root_eps<R>() * fmax(R(1), fabs(a))) return R(0.5) * (a + b);
     }
@@ -213,21 +233,23 @@ __device__ __forceinline__ void torus_coeffs(const double *o, const double *u, d
 // is within 1e-3 A and the root simple, else the warp solve already took it in
 // FP64): quadratic convergence, so the steps stop once one moves t by less
 // than 1e-13 A (the next would move it by about the square of that)
+// (`last`: the last step's length)
 __device__ __noinline__ double exact_root_torus(const double *o, const double *u, double rho, double rp,
-                                                   const double *s, int axis, double t0)
+                                                   const double *s, int axis, double t0, double *last = nullptr)
 {
     double co[5];
     torus_coeffs(o, u, rho, rp, s, axis, co);
     double dc[4] = {co[1], 2.0 * co[2], 3.0 * co[3], 4.0};
-    double t = t0;
+    double t = t0, dt = INFINITY;
     for (int it = 0; it < 4; ++it) {
         double f = horner<double, 4>(co, t);
         double df = horner<double, 3>(dc, t);
         if (df == 0.0) break;
-        const double dt = f / df;
+        dt = f / df;
         t -= dt;
         if (fabs(dt) < 1e-13) break;
     }
+    if (last) *last = fabs(dt);
     return t;
 }
 
@@ -518,8 +540,9 @@ struct SlabExact {
     const SlabAcc<T> &S;
     const Model &M;
     double x0, y0, z0;
-    __device__ SlabExact(const SlabAcc<T> &s, const Model &m, const double *o)
-        : S(s), M(m), x0(o[0]), y0(o[1]), z0(o[2]) {}
+    float d0;  // bound of the tile frame's FP32 rounding
+    __device__ SlabExact(const SlabAcc<T> &s, const Model &m, const double *o, float d)
+        : S(s), M(m), x0(o[0]), y0(o[1]), z0(o[2]), d0(d) {}
     __device__ int na() const { return S.na(); }
     __device__ int np() const { return S.np(); }
     __device__ int nv() const { return S.nv(); }
@@ -580,6 +603,57 @@ struct StageSmem {
     long long sb0, tb0;  // the same as reserved (also when a buffer is full)
     unsigned hmask[HMASK_WORDS];  // prefilter hits, ceil(items / 32) words per edge (when they fit), two halves a word
 };
+
+// Freeness of an FP64 saddle witness: free_witness<false>.
+template <class Acc>
+__device__ __forceinline__ bool exact_free(const Acc &A, const double *q, short2 sl, int2 ij, double rp)
+{
+    return free_witness<false>(A, q[0], q[1], q[2], (int)sl.x, (int)sl.y, ij.x, ij.y, rp, 0.0) == 1;
+}
+
+// The same answer where the staged copies are FP32: an atom whose FP32 distance
+// is certain needs no FP64 one (2 d0 + 1e-6 A covers the rounding of q and of
+// the atom).  One thread walks the atoms one after the other, so the latency of
+// their loads is the time: four independent FP32 loads at once instead of an
+// index and then an FP64 load for each (k_roots_torus_exact 116 -> 73 us on the
+// packed box, 90 -> 66 us on 3,000 atoms).
+__device__ __noinline__ bool exact_free(const SlabExact<float> &X, const double *q, short2 sl, int2 ij, double rp)
+{
+    const SlabAcc<float> &S = X.S;
+    const float qx = (float)q[0], qy = (float)q[1], qz = (float)q[2], rpf = (float)rp;
+    const float delta = 2.0f * X.d0 + 1e-6f;
+    const bool sets = sl.x >= 0 && sl.y >= 0;
+    const unsigned *m0 = sets ? S.nb(sl.x) : nullptr, *m1 = sets ? S.nb(sl.y) : nullptr;
+    const int na = S.na();
+    for (int w = 0; w * 32 < na; ++w) {
+        unsigned bits = sets ? m0[w] & m1[w] : (na - w * 32 >= 32 ? 0xffffffffu : (1u << (na - w * 32)) - 1u);
+        while (bits) {
+            int k[4];
+            P4<float> c[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                k[u] = bits ? (w << 5) + __ffs(bits) - 1 : -1;
+                bits &= bits - 1;
+                c[u] = S.atom(max(k[u], 0));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float dx = qx - c[u].x, dy = qy - c[u].y, dz = qz - c[u].z, R = c[u].w + rpf;
+                const int t = lt_sq<true>(dx * dx + dy * dy + dz * dz, R * R, R, delta);
+                if (k[u] < 0 || t == 0) continue;
+                if (!sets) {
+                    const int g = S.agid(k[u]);
+                    if (g == ij.x || g == ij.y) continue;
+                }
+                if (t == 1) return false;
+                const P4<double> e = X.atom(k[u]);
+                const double ex = q[0] - e.x, ey = q[1] - e.y, ez = q[2] - e.z, R64 = e.w + rp;
+                if (ex * ex + ey * ey + ez * ez < R64 * R64) return false;
+            }
+        }
+    }
+    return true;
+}
 
 // items [0, nsph) are spheres: the bits of 32-item word w that are spheres
 __device__ __forceinline__ unsigned sphere_bits(int w, int nsph)
@@ -773,9 +847,8 @@ __device__ __noinline__ void torus_root_exact(const Acc &X, RootSink &out, int p
     if (inside ? rate > 0.0 : rate < 0.0) return;
     const int2 ij = X.pij(pi);
     const short2 sl = X.pslot(pi);
-    const int f = free_witness<false>(X, oo[0] + oe.w * wd[0], oo[1] + oe.w * wd[1], oo[2] + oe.w * wd[2], (int)sl.x,
-                                      (int)sl.y, ij.x, ij.y, rp, 0.0);
-    if (f == 1) out.push((float)t64, 0.0f, t64);
+    const double q[3] = {oo[0] + oe.w * wd[0], oo[1] + oe.w * wd[1], oo[2] + oe.w * wd[2]};
+    if (exact_free(X, q, sl, ij, rp)) out.push((float)t64, 0.0f, t64);
 }
 
 // Every root of a torus piece in [0, h] from the quartic, each decided in FP64.
@@ -1645,7 +1718,7 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_sphere(Model M, Batc
         T s[3], hT;
         edge_point<T>(B.grid[mol], p, s, hT);
         const SlabAcc<T> A(sl);
-        const SlabExact<T> X(A, M, x0);
+        const SlabExact<T> X(A, M, x0, B.grid[mol].d0);
         RootSink out{W.rsph + (size_t)SPH_SLOTS * k, 0, SPH_SLOTS};
         sphere_roots<T, FILT>(A, X, c.y, s, s64, pk_axis(pk), pk_label(pk) == LABEL_IN, hT, rpT, h, rp, d0, out);
         if (out.n > SPH_SLOTS) atomicOr(err, ERR_CAP_CAND);
@@ -1736,16 +1809,29 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus(Model M, Batch
             job = torus_roots_fp32(A, c.y, s, pk_axis(pk), pk_label(pk) == LABEL_IN, hT, rpf, (float)d0, out);
         } else {
             const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
-            const SlabExact<T> X(A, M, x0);
-            // (a candidate that the certified isolation finds without a root near the edge has none in FP64)
+            // The certified isolation leaves the edge's roots as single ones: Newton steps in
+            // FP64 from there, and every decision in FP64 (47 k candidates of 200 atoms: the quartic
+            // on its derivative chain for each 472 us, 282 us so, 126 us with mono_root's stop).  The quartic where the
+            // isolation is undecided or the steps do not settle.
+            const int axis = pk_axis(pk);
+            const bool inside = pk_label(pk) == LABEL_IN;
             const P4<T> o = A.po(c.y), u = A.pu(c.y);
             const float q0[3] = {(float)(s64[0] - o.x), (float)(s64[1] - o.y), (float)(s64[2] - o.z)};
             const float uu[3] = {(float)u.x, (float)u.y, (float)u.z};
+            const double oo[3] = {o.x, o.y, o.z}, u64[3] = {u.x, u.y, u.z};
             float rt[4];
             int nr = 0;
-            if (!torus_roots32(q0, uu, (float)o.w, rpf, pk_axis(pk), -1e-4f, (float)h + 1e-4f, B.grid[mol].d0, rt, nr) ||
-                nr > 0)
-            torus_roots<T, FILT>(A, X, c.y, s64, pk_axis(pk), pk_label(pk) == LABEL_IN, h, rp, d0, out);
+            bool whole = !torus_roots32(q0, uu, (float)o.w, rpf, axis, -1e-4f, (float)h + 1e-4f, B.grid[mol].d0, rt, nr);
+            for (int j = 0; j < nr && !whole; ++j) {
+                double last = 0.0;
+                const double t64 = exact_root_torus(oo, u64, o.w, rp, s64, axis, (double)rt[j], &last);
+                if (last < 1e-10) torus_root_exact(A, out, c.y, s64, axis, h, rp, inside, t64);
+                else whole = true;
+            }
+            if (whole) {
+                out.n = 0;
+                torus_piece_exact(A, out, c.y, s64, axis, h, rp, inside);
+            }
         }
         if (out.n > TOR_SLOTS) atomicOr(err, ERR_CAP_CAND);
         W.ntor[k] = (uint8_t)min(out.n, TOR_SLOTS);
@@ -1792,7 +1878,7 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus_exact(Model M,
         const bool inside = pk_label(pk) == LABEL_IN;
         const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
         const SlabAcc<T> A(sl);
-        const SlabExact<T> X(A, M, x0);
+        const SlabExact<T> X(A, M, x0, B.grid[mol].d0);
         RootRec *slots = W.rtor + (size_t)TOR_SLOTS * k;
         if (jb.y == 2) {
             RootSink out{slots, 0, TOR_SLOTS};
@@ -2023,7 +2109,7 @@ __global__ void __launch_bounds__(128) k_edge_ties(Model M, Batch B, RootWork W)
         const double h = B.grid[__ldg(&hd->mol)].h;
         const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
         const SlabAcc<float> A(sl);
-        const SlabExact<float> X(A, M, x0);
+        const SlabExact<float> X(A, M, x0, B.grid[hd->mol].d0);
         RootRec *rec = kind == 1 ? W.rtor + (size_t)TOR_SLOTS * jb.y + r : W.rsph + (size_t)SPH_SLOTS * jb.y + r;
         rec->t64 = staged_exact_root(X, kind, jb.w, s64, pk_axis(inf.y), M.rp, (double)rec->t);
     }
@@ -2064,7 +2150,7 @@ __global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, Ro
         T s[3], hT;
         edge_point<T>(B.grid[mol], p, s, hT);
         const SlabAcc<T> A(sl);
-        const SlabExact<T> X(A, M, x0);
+        const SlabExact<T> X(A, M, x0, B.grid[mol].d0);
         const int na = A.na();
         // gather: lanes over candidates, each lane's roots at its prefix of the counts
         int n = 0;

@@ -64,6 +64,29 @@ def test_noalloc_rows_at_every_alignment(dims, shift):
         assert np.array_equal(got[:-1], ref[a]) and got[-1] == -1, a
 
 
+@pytest.mark.parametrize("prec", [eses.ESES_PREC_FP32_FILTERED, eses.ESES_PREC_FP64])
+@pytest.mark.parametrize("h,r_p", [(0.2, 1.4), (0.45, 0.3), (0.95, 1.4), (0.5, 4.0)])
+def test_torus_roots_from_short_to_long_edges(h, r_p, prec):
+    """Edges from a seventh of the probe to more than it, tori from thin ones to
+    those that meet themselves: every root next to the oracle's."""
+    libbuild.build()
+    xyz, rad = inputs.protein_like(30, 91, inputs.PROTEIN_DENSITY)
+    margin = 1.5 * h + 0.3
+    ref = oracle.run(xyz, rad, r_p, h, margin)
+    ctx = eses.eses_create(xyz, rad, r_p, h, margin)
+    try:
+        eses.eses_set_option(ctx, eses.ESES_OPT_PRECISION, prec)
+        eses.eses_run(ctx)
+        assert np.array_equal(eses.eses_labels(ctx), ref.labels)
+        for a in range(3):
+            g = eses.eses_intersections(ctx, a)
+            o = np.argsort(g["idx"])
+            assert np.array_equal(g["idx"][o], ref.idx[a])
+            assert np.abs(g["tau"][o] - ref.tau[a]).max() * h < 1e-6
+    finally:
+        eses.eses_destroy(ctx)
+
+
 def test_circle_with_many_free_end_points():
     """Two large balls whose circle carries 35 small ones, none touching the
     next: 70 free triple points on one circle, more than the arc kernel lists
