@@ -3,8 +3,7 @@
 //
 // k_classify<T, FILT>:
 //   1. stages the tile's atoms, free-arc pairs and free triple points in
-//      shared memory (tile frame) and lists, for every staged atom, the staged
-//      pairs it belongs to;
+//      shared memory (tile frame);
 //   2. splits the tile into 16 bricks of 2x4x4 points, one warp per brick:
 //      the lanes test the staged atoms against the brick's box and ballots
 //      give the set of atoms whose expanded ball reaches the brick.  A warp
@@ -21,9 +20,10 @@
 //   Bound by instruction issue and the latency of a tile's slowest points.  One
 //   thread per point walking its own balls' circles (12.9 active lanes, 65 % of
 //   the kernel in this phase, 59,000 cycles a tile on the 5,000-atom globule at
-//   h 0.25) became all lanes on one patch at a time: 2.19 -> 1.30 ms there,
-//   8.2 -> 5.0 ms at 20,000 atoms, 3.6 -> 2.2 ms on 32 molecules at h 0.5,
-//   1.30 -> 0.64 ms in FP64 on 200 atoms (single-tile queue pops included).
+//   h 0.25) became all lanes on one patch at a time: 2.19 -> 1.12 ms there,
+//   8.2 -> 4.4 ms at 20,000 atoms, 3.6 -> 1.75 ms on 32 molecules at h 0.5,
+//   1.30 -> 0.64 ms in FP64 on 200 atoms (single-tile queue pops, staging by
+//   runs of cells and five CTAs an SM included).
 //   T = double, FILT = false is the plain FP64 form; T = float, FILT = true
 //   is the filtered form, whose undecided points get LABEL_BAND and whose
 //   tiles with such points are listed.
@@ -47,11 +47,11 @@ constexpr int CLS_SPLIT = 2 * CLS_THREADS;
 template <class CP>
 struct ClsSmem {
     static constexpr int HS = slot_hash_size<CP>(), AWC = atom_words<CP>();
-    int hkey[HS];                  // staged-atom lookup (pair_slots)
-    short hval[HS];
     short2 pslot[CP::P];           // staged slots of each pair's atoms (-1: not staged)
     unsigned bmask[NBRICK][AWC];   // per-brick sets of the atoms whose expanded ball reaches the brick
-    unsigned nbm[CP::A * AWC];     // neighbour set of every staged atom (build_neighbour_sets)
+    unsigned nbm[CP::A * AWC];     // neighbour set of every staged atom (build_neighbour_sets); before that
+                                   // the staged-atom lookup of pair_slots (HS keys, HS slots)
+    static_assert(CP::A * AWC * sizeof(unsigned) >= HS * (sizeof(int) + sizeof(short)), "lookup in nbm");
     short queue[TILE_PTS];         // shell points, brick by brick
     int nq, band, next;            // queue length, band points, next queue position to take
 };
@@ -226,12 +226,16 @@ __host__ __device__ constexpr size_t cls_bytes()
     return (((sizeof(TileS<T, CP>) + 15) & ~(size_t)15) + sizeof(ClsSmem<CP>) + 255) & ~(size_t)255;
 }
 
+// Five CTAs an SM in FP32 (48 registers, 42 KB: the lookup of pair_slots lies in
+// the neighbour sets' place, else 48 KB and four): 1,808 -> 1,749 us on 32
+// molecules, and in FP64, three CTAs either way, what is left to L1 takes
+// 1.50 -> 1.37 ms off the run of 200 atoms.
 // CP = CapMid: the staged lists in shared memory; a tile that overflows
 // them goes to ovf.  CP = CapBig (BIG): the tiles listed in ovf, with the
 // staged lists in this CTA's slice of the global scratch `big`; overflowing
 // that too is a capacity error.
 template <class T, bool FILT, class CP, bool BIG>
-__global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, TileSched Q, int8_t *__restrict__ labels_all,
+__global__ void __launch_bounds__(CLS_THREADS, sizeof(T) == sizeof(float) && !BIG ? 5 : 1) k_classify(Model M, Batch B, TileSched Q, int8_t *__restrict__ labels_all,
                                                           int *__restrict__ band, int *__restrict__ err,
                                                           int *__restrict__ ovf, unsigned char *__restrict__ big,
                                                           unsigned long long *__restrict__ n_tests)
@@ -356,8 +360,10 @@ __global__ void __launch_bounds__(CLS_THREADS) k_classify(Model M, Batch B, Tile
         __syncthreads();
         const int nq = C.nq;
         if (nq > 0) {  // neighbour sets and pair slots for the witnesses' freeness tests
+            int *hkey = reinterpret_cast<int *>(C.nbm);
+            pair_slots<T>(S, hkey, reinterpret_cast<short *>(hkey + C.HS), C.pslot);
             build_neighbour_sets<T, CP>(S, C.nbm, rp);
-            pair_slots<T>(S, C.hkey, C.hval, C.pslot);
+            __syncthreads();
         }
         // phase 2: shell points, 32 / gs at a time per warp from a block counter
         int gs = 1;

@@ -1857,9 +1857,12 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus(Model M, Batch
 // only): job 1 settles the pending slots (the FP64 root next to the FP32 one,
 // kept or rejected as torus_roots does), job 2 solves the whole candidate
 // with torus_roots (the quartic on its derivative chain, FP64 where needed).
+// Bound by the latency of its chains of loads and FP64 instructions: three
+// blocks on an SM rather than the two of its 126 registers (178 -> 157 us on the
+// 20,000-atom globule).
 template <class T, bool FILT>
-__global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus_exact(Model M, Batch B, RootWork W,
-                                                                        int *__restrict__ err)
+__global__ void __launch_bounds__(ROOT_THREADS_MAX, 3) k_roots_torus_exact(Model M, Batch B, RootWork W,
+                                                                           int *__restrict__ err)
 {
     const long long n = min((long long)W.ctr[4], W.cap_jobs);
     const double rp = M.rp;
@@ -2119,8 +2122,10 @@ __global__ void __launch_bounds__(128) k_edge_ties(Model M, Batch B, RootWork W)
 // edge's accepted roots are gathered in candidate order into the warp's
 // buffer in shared memory (at most WCAND; more is a capacity error), then
 // chosen by warp_select.  A failure is logged with its candidates.
+// Bound by latency (a warp's witness searches, one after the other): three
+// blocks on an SM rather than two at 118 registers, 422 -> 390 us on 38 k edges.
 template <class T, bool FILT>
-__global__ void __launch_bounds__(HARD_THREADS) k_edge_hard(Model M, Batch B, RootWork W,
+__global__ void __launch_bounds__(HARD_THREADS, FILT ? 3 : 1) k_edge_hard(Model M, Batch B, RootWork W,
                                                             const int *__restrict__ edge_start, EdgeOut out,
                                                             int *__restrict__ n_fail, int *__restrict__ err,
                                                             long long *__restrict__ fail_log)

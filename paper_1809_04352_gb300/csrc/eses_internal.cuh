@@ -33,8 +33,8 @@ struct CapBig {
     static constexpr int A = 1024, P = 2048, V = 2048;
 };
 // the shared-memory tier of the classification and of the root solve's
-// staging pass: lists sized so that four CTAs fit an SM (the tiles past them
-// take the global-memory tier)
+// staging pass: lists sized so that four CTAs fit an SM, five of the
+// classification's in FP32 (the tiles past them take the global-memory tier)
 struct CapMid {
     static constexpr int A = 256, P = 384, V = 384;
 };
