@@ -14,13 +14,13 @@
 //   (falling from an inside end, rising from an outside end), is a candidate.
 //   From an inside end point the first candidate is the first root; from an
 //   outside end point the first candidate that is not strictly outside M is.
-//   Five launches linked by lists in HBM:
+//   Seven launches linked by lists in HBM:
 //   k_edge_stage: persistent CTAs take tiles from the work queue; per tile
 //     the pieces are staged (shared memory, or the global-memory tier for a
 //     tile that overflows it), the crossing edges listed, and written out:
 //     the staged lists (the tile's slab), an edge record per edge, and the
-//     (edge, piece) pairs that pass a prefilter (one warp per edge, lanes over
-//     the staged pieces), spheres and tori in separate lists;
+//     (edge, piece) pairs that pass a prefilter (32 edges a warp, a lane each,
+//     against the same pieces), spheres and tori in separate lists;
 //   k_roots_sphere / k_roots_torus: one thread per pair, no block barrier:
 //     sphere roots from the quadratic; torus roots of
 //          (|y-o|^2 + rho^2 - r_p^2)^2 = 4 rho^2 (|y-o|^2 - ((y-o).u)^2)
@@ -29,9 +29,11 @@
 //     refined by Newton (undecided: the quartic on its derivative chain, then
 //     FP64); every FP32 root carries an error bound; the accepted roots go to
 //     the pair's slots;
+//   k_roots_torus_exact: the tori's FP64 work that those leave, one thread each;
 //   k_edge_pick: one thread per edge: the first root when the end point is
-//     inside or one candidate is left and the FP32 bounds order the
-//     candidates; the other edges are listed;
+//     inside, the last one when it is outside and the first lies within r_p of
+//     the last one's witness, where the FP32 bounds order the candidates; the
+//     other edges are listed, with the candidates that are nearly tied;
 //   k_edge_ties: FP64 roots of near ties, one thread each;
 //   k_edge_hard: one warp per edge left: near ties broken on FP64 roots; at
 //     an outside end point each earlier candidate tested first against the
@@ -1274,7 +1276,7 @@ __device__ int warp_select(const AccT &A, const AccX &X, WCand *c, int n, const 
 // is read as three aligned words (byte by byte where those would pass the
 // molecule's end) and kept as 9 bits, bit 15 set for a row on the grid; the
 // counts are then popcounts of rows against their neighbours.  Byte loads per
-// point and axis took 153 us on 38 M points (250 GB/s) and 939 us on 198 M.
+// point and axis took 153 us on 38 M points (250 GB/s) and 939 us on 198 M; 45 and 243 us now.
 constexpr int COUNT_WARPS = 8;
 
 __global__ void __launch_bounds__(COUNT_WARPS * 32) k_edge_count(Batch B, const int8_t *__restrict__ labels_all,
