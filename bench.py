@@ -60,10 +60,10 @@ WORKLOAD = 2
 # (profiles/k_classify_globule-5000.md); reported only while the kernels'
 # sources are the ones that were captured
 TRAFFIC = {
-    "edge_solve": (739_858_432, {"eses_edges.cu": "caf97df99fe6129f", "eses_tile.cuh": "0665160bfe8f347d",
-                                 "eses_internal.cuh": "9c0bf5106d8efdeb"}),
-    "classify": (10_196_736, {"eses_classify.cu": "71fc2607bb299d7e", "eses_tile.cuh": "0665160bfe8f347d",
-                              "eses_internal.cuh": "9c0bf5106d8efdeb"}),
+    "edge_solve": (644_018_944, {"eses_edges.cu": "c7aeb5039a91dceb", "eses_tile.cuh": "9e7d65712438136b",
+                                 "eses_internal.cuh": "85eea755cbda79ad"}),
+    "classify": (9_741_056, {"eses_classify.cu": "04754d6e89d4d447", "eses_tile.cuh": "9e7d65712438136b",
+                             "eses_internal.cuh": "85eea755cbda79ad"}),
 }
 
 
