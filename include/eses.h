@@ -115,7 +115,7 @@ typedef struct eses_ctx eses_ctx;
 
 #define ESES_MLP_NPARAM 6337     /* parameters of the proposer MLP (layout at eses_set_proposer) */
 
-#define ESES_PREC_FP64 0           /* every step in FP64 */
+#define ESES_PREC_FP64 0           /* every decision and root in FP64 (certified FP32 tests only leave candidates out or bracket a root) */
 #define ESES_PREC_FP32_FILTERED 1  /* FP32 with a forward-error filter, FP64 inside the filter band */
 
 /* Create a context for one molecule.  xyz: host, n_atoms*3 doubles (x,y,z per
