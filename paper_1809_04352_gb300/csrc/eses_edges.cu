@@ -913,6 +913,9 @@ __device__ __forceinline__ CandItem cand_item(const TileS<T, CP> &S, int it, int
 __device__ __forceinline__ bool cand_test(const CandItem &c, const float *s, int axis, bool inside, float h, float rp)
 {
     constexpr float mg = 2e-3f;
+    // (edges longer than any use of the grid: a squared distance's rounding, 2 |d| d0 with
+    // |d| up to h and d0 = 6e-7 of the tile, would near 2 r mg, so every piece is a candidate)
+    if (h > 4.0f) return c.kind >= 0;
     const float d0 = s[0] - c.x, d1 = s[1] - c.y, d2 = s[2] - c.z;
     if (c.kind < 2) {
         const float dd = d0 * d0 + d1 * d1 + d2 * d2;

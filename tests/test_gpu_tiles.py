@@ -65,9 +65,9 @@ def test_noalloc_rows_at_every_alignment(dims, shift):
 
 
 @pytest.mark.parametrize("prec", [eses.ESES_PREC_FP32_FILTERED, eses.ESES_PREC_FP64])
-@pytest.mark.parametrize("h,r_p", [(0.2, 1.4), (0.45, 0.3), (0.95, 1.4), (0.5, 4.0)])
+@pytest.mark.parametrize("h,r_p", [(0.2, 1.4), (0.45, 0.3), (0.95, 1.4), (0.5, 4.0), (3.9, 1.4), (4.1, 1.4), (12.0, 0.4)])
 def test_torus_roots_from_short_to_long_edges(h, r_p, prec):
-    """Edges from a seventh of the probe to more than it, tori from thin ones to
+    """Edges from a seventh of the probe to past the molecule, tori from thin ones to
     those that meet themselves: every root next to the oracle's."""
     libbuild.build()
     xyz, rad = inputs.protein_like(30, 91, inputs.PROTEIN_DENSITY)
