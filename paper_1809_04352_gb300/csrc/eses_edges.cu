@@ -281,10 +281,12 @@ __device__ __forceinline__ double polish_sphere(const double *c, double rad, dou
     const double b = d[axis];
     const double p = d[axis == 0 ? 1 : 0], q = d[axis == 2 ? 1 : 2];
     const double disc = (rad * rad - p * p) - q * q;
-    double t = t0;
-    if (disc >= 0.0) {
+    double t;
+    if (disc > 1e-4) {
         const double sq = sqrt(disc);
         t = t0 <= -b ? -b - sq : -b + sq;  // the root on t0's side of their middle
+    } else {  // near a tangent a root moves by the square root of the rounding: the selection's form
+        t = exact_root_sphere(c, rad, s, axis, t0);
     }
     t = into_edge(t, h);
     d[axis] += t;
@@ -311,7 +313,10 @@ __device__ __forceinline__ double polish_torus(const double *o, const double *u,
     for (int it = 0; it < 4; ++it) {
         const double f = horner<double, 4>(co, t);
         const float df = (float)horner<double, 3>(dc, t);
-        if (fabsf(df) < 1e-30f) break;
+        if (fabsf(df) < 5e-2f) {  // nearly a double root: the selection's form, as for spheres
+            t = exact_root_torus(o, u, rho, rp, s, axis, t0);
+            break;
+        }
         const double dt = f * (double)(1.0f / df);
         t -= dt;
         if (fabs(dt) < 1e-11) break;
