@@ -60,9 +60,9 @@ WORKLOAD = 2
 # (profiles/k_classify_globule-5000.md); reported only while the kernels'
 # sources are the ones that were captured
 TRAFFIC = {
-    "edge_solve": (644_018_944, {"eses_edges.cu": "c7aeb5039a91dceb", "eses_tile.cuh": "9e7d65712438136b",
+    "edge_solve": (644_276_992, {"eses_edges.cu": "e666d46675dc5cc0", "eses_tile.cuh": "9e7d65712438136b",
                                  "eses_internal.cuh": "85eea755cbda79ad"}),
-    "classify": (9_741_056, {"eses_classify.cu": "04754d6e89d4d447", "eses_tile.cuh": "9e7d65712438136b",
+    "classify": (9_756_416, {"eses_classify.cu": "04754d6e89d4d447", "eses_tile.cuh": "9e7d65712438136b",
                              "eses_internal.cuh": "85eea755cbda79ad"}),
 }
 
