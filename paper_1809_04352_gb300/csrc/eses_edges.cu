@@ -376,6 +376,18 @@ struct WCand {
     int kind, id;  // kind 0: van der Waals sphere (atom slot), 1: torus (pair slot), 2: probe sphere (vertex slot)
 };
 
+// A surface point on a grid point is a root at an end of its edges, which
+// rounding leaves on either side of the end (Newton's limit from an exact tie
+// is 1e-28 A off, a sphere's root an ulp); dropped there, the edge has no root
+// or takes a later one.  Roots that far outside [0, h] are taken at the end;
+// the crossing's direction keeps the neighbouring edge's root out.
+constexpr double END_TOL = 1e-11;
+__device__ __forceinline__ double at_end(double t, double h)
+{
+    if (t < 0.0 && t >= -END_TOL) return 0.0;
+    return t > h && t <= h + END_TOL ? h : t;
+}
+
 // Accepted roots of one (edge, piece) candidate, written to the candidate's
 // slots in HBM (at most SPH_SLOTS for a sphere, whose two roots cross in
 // opposite directions; at most TOR_SLOTS, the quartic's degree, for a torus).
@@ -837,6 +849,7 @@ template <class Acc>
 __device__ __noinline__ void torus_root_exact(const Acc &X, RootSink &out, int pi, const double *s64, int axis,
                                               double h, double rp, bool inside, double t64)
 {
+    t64 = at_end(t64, h);
     if (!(t64 >= 0.0 && t64 <= h)) return;
     const P4<double> oe = X.po(pi);
     const P4<double> ue = X.pu(pi);
@@ -858,7 +871,8 @@ __device__ __noinline__ void torus_root_exact(const Acc &X, RootSink &out, int p
     if (exact_free(X, q, sl, ij, rp)) out.push((float)t64, 0.0f, t64);
 }
 
-// Every root of a torus piece in [0, h] from the quartic, each decided in FP64.
+// Every root of a torus piece in [0, h] (or END_TOL past an end) from the
+// quartic, each decided in FP64.
 template <class Acc>
 __device__ __noinline__ void torus_piece_exact(const Acc &X, RootSink &out, int pi, const double *s64, int axis,
                                                double h, double rp, bool inside)
@@ -870,6 +884,14 @@ __device__ __noinline__ void torus_piece_exact(const Acc &X, RootSink &out, int 
     torus_coeffs(oo, u64, oe.w, rp, s64, axis, co);
     const int n = PolyRoots<double, 4>::run(co, 0.0, h, r64);
     for (int k = 0; k < n; ++k) torus_root_exact(X, out, pi, s64, axis, h, rp, inside, r64[k]);
+    // a simple root just past an end
+    const double dc[4] = {co[1], 2.0 * co[2], 3.0 * co[3], 4.0};
+    for (int e = 0; e < 2; ++e) {
+        const double t = e == 0 ? 0.0 : h, f = horner<double, 4>(co, t), df = horner<double, 3>(dc, t);
+        if (f == 0.0 || !(fabs(f) <= END_TOL * fabs(df))) continue;
+        if (e == 0 ? (f > 0.0) == (df > 0.0) : (f > 0.0) != (df > 0.0))  // t - f / df lies outside
+            torus_root_exact(X, out, pi, s64, axis, h, rp, inside, t);
+    }
 }
 
 // Can item `it` (staged atom, vertex or pair, in that order) put an accepted
@@ -997,7 +1019,8 @@ __device__ void sphere_roots(const AccT &A, const AccX &X, int item, const T *s,
                              bool inside, T hT, T rpT, double h, double rp, T d0, RootSink &out)
 {
     const int na = A.na();
-    const T lo = FILT ? T(-1e-4) : T(0), hi = hT + (FILT ? T(1e-4) : T(0));
+    const T past = FILT ? T(1e-4) : T(END_TOL);
+    const T lo = -past, hi = hT + past;
     const T tmax = T(1e-3);  // FP32 root error beyond which FP64 decides (grazing pieces)
     const double NaN = __longlong_as_double(0x7ff8000000000000LL);
     const bool vdw = item < na;
@@ -1015,7 +1038,7 @@ __device__ void sphere_roots(const AccT &A, const AccX &X, int item, const T *s,
         nr = (-b >= lo && -b <= hi) ? 1 : 0;
     }
     for (int k = 0; k < nr; ++k) {
-        T t = rt32[k];
+        T t = FILT ? rt32[k] : (T)at_end((double)rt32[k], h);
         T vA = d[axis] + t;  // +-sqrt(disc) at a root: the rate of |y - c|
         T terr = T(0);
         if (FILT) {
@@ -1028,7 +1051,7 @@ __device__ void sphere_roots(const AccT &A, const AccX &X, int item, const T *s,
             const P4<double> ce = vdw ? X.atom(slot) : X.vq(slot);
             const double cc[3] = {ce.x, ce.y, ce.z};
             const double r64 = vdw ? ce.w : rp;
-            t64 = exact_root_sphere(cc, r64, s64, axis, (double)t);
+            t64 = at_end(exact_root_sphere(cc, r64, s64, axis, (double)t), h);
             double dv[3] = {s64[0] - cc[0], s64[1] - cc[1], s64[2] - cc[2]};
             dv[axis] += t64;
             const double f = dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2] - r64 * r64;
