@@ -2614,6 +2614,9 @@ int launch_edge_roots(const Model &M, const Batch &B, int precision, int threads
                       const RootWork &W, cudaStream_t st)
 {
     if (!root_threads_valid(threads) || threads == 0) threads = ROOT_THREADS_MAX;
+    // the failures of these launches only: planning runs them again when the FP64 job list was full, and what
+    // it lacked then counted as failed edges
+    cudaMemsetAsync(n_fail, 0, sizeof(int), st);
     if (precision == 0)
         roots_launch<double, false>(M, B, threads, out, edge_start, ne_all, n_fail, err, fail_log, W, st);
     else
