@@ -443,6 +443,7 @@ int setup(eses_ctx *c, const double *xyz, const double *r, const int64_t *counts
         // point one, a difference of two of them one more: 5 * 2^-24 L per
         // coordinate, 5.2e-7 L for the vector; d0 rounds that up
         G.d0 = (float)(6e-7 * L);
+        G.mg = (float)(2e-3 + 12.0 * 6e-7 * L);
         for (int k = 0; k <= TILE; ++k) G.hl[k] = (float)((double)k * c->h);
         G.ht_hi = (float)(TILE * c->h);
         G.ht_lo = (float)(TILE * c->h - (double)G.ht_hi);

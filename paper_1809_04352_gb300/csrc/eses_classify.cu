@@ -117,11 +117,12 @@ __device__ __forceinline__ int witness_free(const TileS<T, CP> &S, T qx, T qy, T
 // first culled against the box of the points still undecided, lanes over
 // circles; a circle that meets no containing ball of a point is no nearer
 // than r_p with a free witness unless the point is outside, so testing it
-// changes no decision.  Returns the point's label on each of its lanes:
+// changes no decision.  df: FP32 error bound of a staged difference (also in
+// the FP64 form, whose cull is FP32).  Returns the point's label on each of its lanes:
 // 0 a free witness within r_p (certain), 2 undecided, 1 none.
 template <bool FILT, class T, class CP>
 __device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem<CP> &C, int code, T x, T y, T z, T rp,
-                                            T Rmax, T d0, float hf, int r, int G, int &nt)
+                                            T Rmax, T d0, float hf, float df, int r, int G, int &nt)
 {
     constexpr unsigned full = 0xffffffffu;
     constexpr int aw = ClsSmem<CP>::AWC;
@@ -178,8 +179,9 @@ __device__ __forceinline__ int shell_points(const TileS<T, CP> &S, const ClsSmem
         const float hh = 0.5f * hf;
         const float cx = hh * (float)(i0 + i1), cy = hh * (float)(j0 + j1), cz = hh * (float)(k0 + k1);
         const float ex = (float)(i1 - i0), ey = (float)(j1 - j0), ez = (float)(k1 - k0);
-        // 2e-3 A covers the FP32 rounding of the distance (as in the prefilters)
-        const float reach = (float)rp + hh * sqrtf(ex * ex + ey * ey + ez * ez) + 2e-3f;
+        // 4 df covers the FP32 rounding of the distance at the molecule's lengths (2e-3 A alone does not for
+        // radii of 1e4 A)
+        const float reach = (float)rp + hh * sqrtf(ex * ex + ey * ey + ez * ez) + 2e-3f + 4.0f * df;
         for (int p0 = 0; p0 < S.np; p0 += 32) {
             bool near = false;
             if (p0 + lane < S.np) {
@@ -378,7 +380,8 @@ __global__ void __launch_bounds__(CLS_THREADS, sizeof(T) == sizeof(float) && !BI
             const int code = k < nq ? C.queue[k] : -1;
             const int li = (code >> 6) & 7, lj = (code >> 3) & 7, lk = code & 7;
             const T x = pt_coord<T>(G, li), y = pt_coord<T>(G, lj), z = pt_coord<T>(G, lk);
-            const int lab = shell_points<FILT, T, CP>(S, C, code, x, y, z, rp, Rmax, d0, (float)G.h, r, gs, ntests);
+            const int lab = shell_points<FILT, T, CP>(S, C, code, x, y, z, rp, Rmax, d0, (float)G.h, G.d0, r, gs,
+                                                      ntests);
             if (r == 0 && code >= 0) {
                 const long long gi = (long long)TILE * t[0] + li, gj = (long long)TILE * t[1] + lj,
                                 gk = (long long)TILE * t[2] + lk;

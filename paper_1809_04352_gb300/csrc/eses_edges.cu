@@ -906,8 +906,14 @@ __device__ __noinline__ void torus_piece_exact(const Acc &X, RootSink &out, int 
 // its axis stay away (|g''| <= C = 1 / min(D, |w|) over the edge) |g| is at
 // most |g'| h/2 + C h^2/8, and g' keeps its sign when |g'| > C h/2, which must
 // be falling after an inside end, rising after an outside one.
-// The test is FP32 in either form (a superset of the pieces with roots: every
-// comparison is widened by 2e-3 A).  (The Lipschitz test alone, and spheres by
+// The test is FP32 in either form and a superset of the pieces with roots at
+// any scale: every length is compared with a margin mg = 2e-3 A + 12 d0, d0 the
+// bound of a staged difference's rounding, which grows with the molecule's
+// lengths.  Squares are formed from components across the edge or the axis, never as
+// differences of squares, so a length is off by 4 d0 at most, and g' by
+// 5 d0 over the smaller of D and |w| (2e-3 A alone and differences of squares
+// lost roots on balls of 1e5, and tests that were given up on edges above
+// 4 A took every piece there).  (The Lipschitz test alone, and spheres by
 // their distance range only, left 1.50 M sphere and 4.31 M torus candidates on
 // 1.14 M edges of the 5,000-atom globule, 1.0 M and 1.6 M now.)
 struct CandItem {  // one staged piece, held by a lane over many edges
@@ -937,39 +943,34 @@ __device__ __forceinline__ CandItem cand_item(const TileS<T, CP> &S, int it, int
     return c;
 }
 
-__device__ __forceinline__ bool cand_test(const CandItem &c, const float *s, int axis, bool inside, float h, float rp)
+// m: the edge's middle, half: half its length
+__device__ __forceinline__ bool cand_test(const CandItem &c, const float *m, int axis, bool inside, float half,
+                                          float rp, float mg)
 {
-    constexpr float mg = 2e-3f;
-    // (edges longer than any use of the grid: a squared distance's rounding, 2 |d| d0 with
-    // |d| up to h and d0 = 6e-7 of the tile, would near 2 r mg, so every piece is a candidate)
-    if (h > 4.0f) return c.kind >= 0;
-    const float d0 = s[0] - c.x, d1 = s[1] - c.y, d2 = s[2] - c.z;
+    const float d0 = m[0] - c.x, d1 = m[1] - c.y, d2 = m[2] - c.z;
     if (c.kind < 2) {
-        const float dd = d0 * d0 + d1 * d1 + d2 * d2;
-        const float da = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
-        const float tc = fminf(fmaxf(-da, 0.0f), h);         // nearest point of the segment
-        const float dmin2 = dd + tc * (tc + 2.0f * da);
-        const float end2 = (c.kind == 0) == inside ? dd + h * (h + 2.0f * da) : dd;
+        const float a = axis == 0 ? d0 : (axis == 1 ? d1 : d2), p = axis == 0 ? d1 : d0, q = axis == 2 ? d1 : d2;
+        const float pp = p * p + q * q;
+        const float vn = a + fminf(fmaxf(-a, -half), half);         // nearest point of the segment
+        const float ve = (c.kind == 0) == inside ? a + half : a - half;
         const float rhi = c.r + mg, rlo = fmaxf(c.r - mg, 0.0f);
-        return c.kind >= 0 && dmin2 <= rhi * rhi && end2 >= rlo * rlo;
+        return c.kind >= 0 && pp + vn * vn <= rhi * rhi && pp + ve * ve >= rlo * rlo;
     }
-    const float half = 0.5f * h;
-    const float m0 = axis == 0 ? d0 + half : d0, m1 = axis == 1 ? d1 + half : d1, m2 = axis == 2 ? d2 + half : d2;
-    const float zc = m0 * c.ux + m1 * c.uy + m2 * c.uz;
-    const float w2 = fmaxf(m0 * m0 + m1 * m1 + m2 * m2 - zc * zc, 0.0f);
-    const float nw = sqrtf(w2), e1 = nw - c.r;
+    const float zc = d0 * c.ux + d1 * c.uy + d2 * c.uz;
+    const float w0 = d0 - zc * c.ux, w1 = d1 - zc * c.uy, w2 = d2 - zc * c.uz;
+    const float nw = sqrtf(w0 * w0 + w1 * w1 + w2 * w2), e1 = nw - c.r;
     const float D = sqrtf(e1 * e1 + zc * zc), gm = fabsf(D - rp), H = half + mg;
     if (gm > H) return false;
     const float low = fminf(D, nw) - H;
-    if (low < 0.1f) return true;
-    const float ua = axis == 0 ? c.ux : (axis == 1 ? c.uy : c.uz), ma = axis == 0 ? m0 : (axis == 1 ? m1 : m2);
+    if (low < 50.0f * mg) return true;
+    const float ua = axis == 0 ? c.ux : (axis == 1 ? c.uy : c.uz), wa = axis == 0 ? w0 : (axis == 1 ? w1 : w2);
     const float bend = __fdividef(H, low);  // C h/2: g' moves by at most this over the edge
-    const float dg = __fdividef(e1 * __fdividef(ma - zc * ua, nw) + zc * ua, D);
+    const float dg = __fdividef(e1 * __fdividef(wa, nw) + zc * ua, D);
     if (gm > fabsf(dg) * H + 0.5f * bend * H + mg) return false;
     return !((inside ? dg : -dg) > bend + 1e-2f);
 }
 
-// Prefilter of the lane's edge (lower point s, axis, label) against 16 staged
+// Prefilter of the lane's edge (middle m, axis, label) against 16 staged
 // items from i0 on, the same items on every lane: bit b for item i0 + b.  The
 // warp's edges are neighbours, so an item is mostly near to all of them or to
 // none and the lanes stay together (lanes over items, a warp per edge, ran the
@@ -977,8 +978,8 @@ __device__ __forceinline__ bool cand_test(const CandItem &c, const float *s, int
 // of 75 edges and 60 items on the globule, half of the staging pass with the
 // writing of the pairs).  Whole warp.
 template <class T, class CP>
-__device__ __forceinline__ unsigned cand_bits(const TileS<T, CP> &S, int i0, int nitem, const float *s, int axis,
-                                              bool inside, float h, float rp)
+__device__ __forceinline__ unsigned cand_bits(const TileS<T, CP> &S, int i0, int nitem, const float *m, int axis,
+                                              bool inside, float half, float rp, float mg)
 {
     unsigned bits = 0u;
     const int n = min(16, nitem - i0);
@@ -998,7 +999,7 @@ __device__ __forceinline__ unsigned cand_bits(const TileS<T, CP> &S, int i0, int
         } else {
             c = cand_item<T, CP>(S, i0 + b, nitem, rp);
         }
-        if (c.kind >= 0 && cand_test(c, s, axis, inside, h, rp)) bits |= 1u << b;
+        if (c.kind >= 0 && cand_test(c, m, axis, inside, half, rp, mg)) bits |= 1u << b;
     }
     return bits;
 }
@@ -1558,7 +1559,9 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
             const EdgeRef R = edge_ref(E, e < ne ? e : 0);
             float s[3], hs;
             edge_point<float>(G, R.p, s, hs);
-            const unsigned m = cand_bits<T, CP>(S, i0, nitem, s, R.axis, R.lab == LABEL_IN, hs, rpf);
+            const float half = 0.5f * hs;
+            for (int a = 0; a < 3; ++a) s[a] += a == R.axis ? half : 0.0f;
+            const unsigned m = cand_bits<T, CP>(S, i0, nitem, s, R.axis, R.lab == LABEL_IN, half, rpf, G.mg);
             return e < ne ? m : 0u;
         };
         auto word = [&](int e, int w) -> unsigned {  // the hits of edge e among items 32 w ..

@@ -126,6 +126,7 @@ struct Grid {
     double rp;
     double halo;                  // r_max + 2 r_p
     float d0;                     // FP32 error bound of a staged position difference
+    float mg;                     // margin of the staging pass' prefilter (eses_edges.cu, cand_test)
     float hl[TILE + 1];           // k * h rounded to FP32, k = 0..8 (tile-frame point coordinates)
     float ht_hi, ht_lo;           // TILE * h as a double-float
 };
