@@ -232,9 +232,9 @@ struct eses_ctx {
     bool exterior = false;
     DBuf ext, ext_open, ext_misc;
     // triangle mesh of the last run (eses_mesh_count / eses_mesh)
-    DBuf mesh_mask, mesh_tile, mesh_off, mesh_keys, mesh_xyz, mesh_err, mesh_tot;
+    DBuf mesh_table, mesh_mask, mesh_tile, mesh_off, mesh_keys, mesh_xyz, mesh_err, mesh_tot;
     long long n_tri = -1;  // -1: not made for the current results
-    bool mesh_ready = false;
+    bool mesh_ready = false;  // mesh_table is filled
     long long n_cavity = 0;
     int ext_sweeps = 0;
     // learned tile proposer
@@ -1917,12 +1917,13 @@ int eses_mesh_count(eses_ctx *c, int64_t *n_tri)
     AllocScope scope(c);
     try {
         ck(cudaSetDevice(c->device), "cudaSetDevice");
-        if (!c->mesh_ready) {  // the case table, once per context that makes a mesh
-            if (mesh_init() != 0) throw CudaError{cudaErrorInvalidValue, "mesh case table"};
-            c->mesh_ready = true;
-        }
         if (c->n_tri < 0) {
             cudaStream_t st = c->stream;
+            uint8_t *table = ensure<uint8_t>(c->mesh_table, mesh_table_bytes());
+            if (!c->mesh_ready) {  // once per context that makes a mesh
+                if (mesh_table_copy(table, st) != 0) throw CudaError{cudaErrorInvalidValue, "mesh case table"};
+                c->mesh_ready = true;
+            }
             const long long nt = c->n_tiles;
             const Batch &B = c->B;
             uint32_t *mask = ensure<uint32_t>(c->mesh_mask, mesh_mask_words(nt));
@@ -1931,7 +1932,7 @@ int eses_mesh_count(eses_ctx *c, int64_t *n_tri)
             int *derr = ensure<int>(c->mesh_err, 1);
             // the total in 64 bits first: the offsets are 32-bit
             unsigned long long *dtot = ensure<unsigned long long>(c->mesh_tot, 1), total = 0;
-            launch_mesh_count(B, (const int8_t *)c->labels.p, mask, tile, dtot, st);
+            launch_mesh_count(B, table, (const int8_t *)c->labels.p, mask, tile, dtot, st);
             ck(cudaMemcpyAsync(&total, dtot, sizeof(total), cudaMemcpyDeviceToHost, st), "read");
             ck(cudaStreamSynchronize(st), "synchronize");
             if (total >= (1ULL << 31)) return fail(c, ESES_EINVAL, "mesh of 2^31 triangles or more");
@@ -1942,8 +1943,8 @@ int eses_mesh_count(eses_ctx *c, int64_t *n_tri)
             long long *keys = ensure<long long>(c->mesh_keys, 3 * (size_t)std::max(tot, 1));
             double *xyz = ensure<double>(c->mesh_xyz, 9 * (size_t)std::max(tot, 1));
             ck(cudaMemsetAsync(derr, 0, sizeof(int), st), "memset");
-            launch_mesh_emit(B, (const int8_t *)c->labels.p, mask, (const int *)c->edge_start.p, eo, off, keys, xyz,
-                             derr, st);
+            launch_mesh_emit(B, table, (const int8_t *)c->labels.p, mask, (const int *)c->edge_start.p, eo, off, keys,
+                             xyz, derr, st);
             int herr = 0;
             ck(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, st), "read");
             ck(cudaStreamSynchronize(st), "synchronize");
@@ -2049,7 +2050,7 @@ void eses_destroy(eses_ctx *c)
                     &c->r_rsph, &c->r_rtor, &c->r_slab, &c->r_ctr, &c->r_hard, &c->r_ties, &c->r_jobs, &c->atom_hi,
                     &c->atom_lo, &c->pair_hi, &c->pair_lo, &c->pair_u32, &c->vert_hi, &c->vert_lo,
                     &c->mlp_params, &c->need, &c->need_pos, &c->tile_list, &c->prop_counts, &c->features,
-                    &c->targets, &c->ext, &c->ext_open, &c->ext_misc, &c->mesh_mask, &c->mesh_tile, &c->mesh_off,
+                    &c->targets, &c->ext, &c->ext_open, &c->ext_misc, &c->mesh_table, &c->mesh_mask, &c->mesh_tile, &c->mesh_off,
                     &c->mesh_keys, &c->mesh_xyz, &c->mesh_err, &c->mesh_tot};
     if (c->own_stream) cudaStreamSynchronize(c->own_stream);
     drop_graph(c);

@@ -15,7 +15,7 @@
 // is reversed after its first vertex if its Newell normal (from the edge
 // midpoints) points on the whole from outside corners to inside ones, and is
 // cut into the fan (v0, v_k, v_k+1).  The 256-case table is built on the host
-// at library set-up.
+// once, at the first mesh.
 //
 // Kernels (one warp per 8x8x8 tile, cubes by their lower corner; the tile's
 // labels and the next layer's as rows of bits, tile_rows):
@@ -34,6 +34,7 @@
 //                 after the other: 382 us for the three kernels on 3,000 atoms at
 //                 h 0.4 (5.6 M points, 0.5 M triangles).
 #include <cstring>
+#include <memory>
 #include <vector>
 
 #include "eses_kernels.h"
@@ -44,9 +45,14 @@ namespace eses {
 constexpr int MESH_WARPS = 8;
 constexpr int MC_MAXT = 12;  // triangles per cube at most (the rule gives at most 5)
 
-__constant__ int8_t c_mc_tri[256][3 * MC_MAXT];
-__constant__ uint8_t c_mc_n[256];
-__constant__ int8_t c_mc_edge[12][4];  // axis, offsets of the lower corner
+// The case table as the kernels read it, from a buffer of the context that its
+// first mesh fills on its own stream: no other context or thread writes it,
+// and the copy is ordered before the kernels.
+struct MeshTable {
+    int8_t tri[256][3 * MC_MAXT];
+    uint8_t n[256];
+    int8_t edge[12][4];  // axis, offsets of the lower corner
+};
 
 // ---------------------------------------------------------------------------
 // the case table (host)
@@ -164,34 +170,41 @@ static bool mc_table(int8_t (*tri)[3 * MC_MAXT], uint8_t *n)
     return true;
 }
 
+// built once, by whichever thread asks first (null if the rule fails)
+static const MeshTable *mesh_table_build()
+{
+    static const std::unique_ptr<const MeshTable> table = [] {
+        auto t = std::make_unique<MeshTable>();
+        if (!mc_table(t->tri, t->n)) return std::unique_ptr<const MeshTable>();
+        const std::vector<CubeEdge> E = cube_edges();
+        for (int e = 0; e < 12; ++e) {
+            t->edge[e][0] = (int8_t)E[e].axis;
+            for (int a = 0; a < 3; ++a) t->edge[e][1 + a] = (int8_t)corner_off(E[e].lo, a);
+        }
+        return std::unique_ptr<const MeshTable>(std::move(t));
+    }();
+    return table.get();
+}
+
 int mesh_table_host(int8_t *tri, uint8_t *n, int max_tri)
 {
-    static int8_t T[256][3 * MC_MAXT];
-    static uint8_t N[256];
-    if (!mc_table(T, N)) return -1;
+    const MeshTable *T = mesh_table_build();
+    if (!T) return -1;
     for (int cs = 0; cs < 256; ++cs) {
-        if (N[cs] > max_tri) return -1;
-        n[cs] = N[cs];
-        for (int k = 0; k < 3 * max_tri; ++k) tri[cs * 3 * max_tri + k] = k < 3 * MC_MAXT ? T[cs][k] : (int8_t)-1;
+        if (T->n[cs] > max_tri) return -1;
+        n[cs] = T->n[cs];
+        for (int k = 0; k < 3 * max_tri; ++k) tri[cs * 3 * max_tri + k] = k < 3 * MC_MAXT ? T->tri[cs][k] : (int8_t)-1;
     }
     return 0;
 }
 
-int mesh_init()
+size_t mesh_table_bytes() { return sizeof(MeshTable); }
+
+int mesh_table_copy(void *table, cudaStream_t st)
 {
-    static int8_t T[256][3 * MC_MAXT];
-    static uint8_t N[256];
-    if (!mc_table(T, N)) return -1;
-    int8_t ed[12][4];
-    const std::vector<CubeEdge> E = cube_edges();
-    for (int e = 0; e < 12; ++e) {
-        ed[e][0] = (int8_t)E[e].axis;
-        for (int a = 0; a < 3; ++a) ed[e][1 + a] = (int8_t)corner_off(E[e].lo, a);
-    }
-    if (cudaMemcpyToSymbol(c_mc_tri, T, sizeof(T)) != cudaSuccess) return -1;
-    if (cudaMemcpyToSymbol(c_mc_n, N, sizeof(N)) != cudaSuccess) return -1;
-    if (cudaMemcpyToSymbol(c_mc_edge, ed, sizeof(ed)) != cudaSuccess) return -1;
-    return 0;
+    const MeshTable *T = mesh_table_build();
+    if (!T) return -1;
+    return cudaMemcpyAsync(table, T, sizeof(*T), cudaMemcpyHostToDevice, st) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -218,7 +231,8 @@ __device__ __forceinline__ int cube_case(const uint16_t *row, int p, int k_on)
     return (int)(((a >> k) & 3u) | (((b >> k) & 3u) << 2) | (((c >> k) & 3u) << 4) | (((d >> k) & 3u) << 6));
 }
 
-__global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_count(Batch B, const int8_t *__restrict__ labels,
+__global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_count(Batch B, const MeshTable *__restrict__ Tb,
+                                                                const int8_t *__restrict__ labels,
                                                                uint32_t *__restrict__ mask,
                                                                int *__restrict__ tile_tri,
                                                                unsigned long long *__restrict__ total)
@@ -259,7 +273,7 @@ __global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_count(Batch B, const i
         int n = 0;
         for (int p = lane; p < TILE_PTS; p += 32) {
             const int cs = cube_case(row, p, n_on);
-            if (cs > 0) n += c_mc_n[cs];
+            if (cs > 0) n += Tb->n[cs];
         }
         n = __reduce_add_sync(0xffffffffu, n);
         if (lane == 0) tile_tri[gt] = n;
@@ -269,7 +283,8 @@ __global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_count(Batch B, const i
     if (lane == 0 && sum) atomicAdd(total, sum);
 }
 
-__global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_emit(Batch B, const int8_t *__restrict__ labels,
+__global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_emit(Batch B, const MeshTable *__restrict__ Tb,
+                                                               const int8_t *__restrict__ labels,
                                                               const uint32_t *__restrict__ mask,
                                                               const int *__restrict__ edge_start, EdgeOut out,
                                                               const int *__restrict__ tile_off,
@@ -294,7 +309,7 @@ __global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_emit(Batch B, const in
         const int n_on = (int)min(9LL, d[2] - (long long)TILE * t[2]);
         for (int r = 0; r < TILE_PTS / 32; ++r) {
             const int cs = cube_case(row, 32 * r + lane, n_on);
-            const int cnt = cs > 0 ? c_mc_n[cs] : 0;
+            const int cnt = cs > 0 ? Tb->n[cs] : 0;
             int inc = cnt;  // cubes in local order: inclusive warp scan
             for (int o = 1; o < 32; o <<= 1) {
                 const int u = __shfl_up_sync(0xffffffffu, inc, o);
@@ -310,10 +325,10 @@ __global__ void __launch_bounds__(MESH_WARPS * 32) k_mesh_emit(Batch B, const in
                 const int c = __shfl_sync(0xffffffffu, cs, src);
                 if (q >= 3 * tot) continue;
                 const int p = 32 * r + src;
-                const int e = c_mc_tri[c][3 * k + v];
-                const int a = c_mc_edge[e][0];
-                const int l[3] = {(p >> 6) + c_mc_edge[e][1], ((p >> 3) & 7) + c_mc_edge[e][2],
-                                  (p & 7) + c_mc_edge[e][3]};
+                const int e = Tb->tri[c][3 * k + v];
+                const int a = Tb->edge[e][0];
+                const int l[3] = {(p >> 6) + Tb->edge[e][1], ((p >> 3) & 7) + Tb->edge[e][2],
+                                  (p & 7) + Tb->edge[e][3]};
                 // the edge's rank in its tile's run of axis a's output
                 const long long tl = ((long long)(t[0] + (l[0] >> 3)) * G.tiles[1] + (t[1] + (l[1] >> 3))) * G.tiles[2] +
                                      (t[2] + (l[2] >> 3));
@@ -348,19 +363,21 @@ static int warp_grid(long long n_tiles)
 
 size_t mesh_mask_words(long long n_tiles) { return (size_t)n_tiles * 3 * MASK_STRIDE; }
 
-int launch_mesh_count(const Batch &B, const int8_t *labels, uint32_t *mask, int *tile_tri, unsigned long long *total,
-                      cudaStream_t st)
+int launch_mesh_count(const Batch &B, const void *table, const int8_t *labels, uint32_t *mask, int *tile_tri,
+                      unsigned long long *total, cudaStream_t st)
 {
     cudaMemsetAsync(total, 0, sizeof(*total), st);
-    k_mesh_count<<<warp_grid(B.n_tiles), MESH_WARPS * 32, 0, st>>>(B, labels, mask, tile_tri, total);
+    k_mesh_count<<<warp_grid(B.n_tiles), MESH_WARPS * 32, 0, st>>>(B, (const MeshTable *)table, labels, mask,
+                                                                   tile_tri, total);
     return 1;
 }
 
-int launch_mesh_emit(const Batch &B, const int8_t *labels, const uint32_t *mask, const int *edge_start,
-                     const EdgeOut &out, const int *tile_off, long long *keys, double *xyz, int *err, cudaStream_t st)
+int launch_mesh_emit(const Batch &B, const void *table, const int8_t *labels, const uint32_t *mask,
+                     const int *edge_start, const EdgeOut &out, const int *tile_off, long long *keys, double *xyz,
+                     int *err, cudaStream_t st)
 {
-    k_mesh_emit<<<warp_grid(B.n_tiles), MESH_WARPS * 32, 0, st>>>(B, labels, mask, edge_start, out, tile_off, keys,
-                                                                  xyz, err);
+    k_mesh_emit<<<warp_grid(B.n_tiles), MESH_WARPS * 32, 0, st>>>(B, (const MeshTable *)table, labels, mask,
+                                                                  edge_start, out, tile_off, keys, xyz, err);
     return 1;
 }
 
