@@ -668,6 +668,49 @@ RootWork root_work(eses_ctx *c, long long ne_all)
     return W;
 }
 
+// Exterior-only surface: cavities filled, sweeps until one reaches nothing new
+// (never under capture).  Returns the number of kernels launched.
+int fill_cavities(eses_ctx *c, int8_t *labels)
+{
+    if (g_capturing) throw std::string("the exterior-only surface is not captured in a graph");
+    cudaStream_t st = c->stream;
+    const Batch &B = c->B;
+    const long long nt = c->n_tiles;
+    int nl = 0;
+    uint16_t *ext = ensure<uint16_t>(c->ext, 64 * (size_t)nt);
+    uint8_t *open = ensure<uint8_t>(c->ext_open, nt);
+    // em[0..1]: four ints (three sweep flags, the sweep count), em[2]: filled points
+    unsigned long long *em = ensure<unsigned long long>(c->ext_misc, 3);
+    int *flags = reinterpret_cast<int *>(em);
+    c->ext_sweeps = 0;
+    ck(cudaMemsetAsync(em, 0, 3 * sizeof(unsigned long long), st), "memset");
+    nl += launch_ext_init(B, labels, ext, open, st);
+    // a sweep reaches at least one more tile, or nothing: at most nt + 1 sweeps
+    const int coop = launch_ext_fill(B, ext, open, flags, nt + 1, st);
+    if (coop < 0) throw CudaError{cudaGetLastError(), "cooperative launch"};
+    if (coop == 1) {  // one launch for every sweep
+        ++nl;
+    } else {  // no cooperative launch on this device: one launch per sweep, driven from the host
+        const int sweep_grid = (int)std::min<long long>(std::max<long long>(ceil_div_ll(nt, 8), 1), 8LL * c->n_sm);
+        for (long long it = 0; it <= nt; ++it) {
+            ck(cudaMemsetAsync(flags, 0, sizeof(int), st), "memset");
+            nl += launch_ext_sweep(B, ext, open, flags, sweep_grid, st);
+            int changed = 0;
+            ck(cudaMemcpyAsync(&changed, flags, sizeof(changed), cudaMemcpyDeviceToHost, st), "read");
+            ck(cudaStreamSynchronize(st), "synchronize");
+            ++c->ext_sweeps;
+            if (!changed) break;
+        }
+    }
+    nl += launch_ext_apply(B, labels, ext, em + 2, st);
+    unsigned long long misc[3] = {0, 0, 0};
+    ck(cudaMemcpyAsync(misc, em, sizeof(misc), cudaMemcpyDeviceToHost, st), "read");
+    ck(cudaStreamSynchronize(st), "synchronize");
+    if (coop == 1) c->ext_sweeps = reinterpret_cast<const int *>(misc)[3];
+    c->n_cavity = (long long)misc[2];
+    return nl;
+}
+
 // The device path of one run.  Planning (not capturing): reads list totals
 // and sizes every buffer; capturing: uses the planned sizes and touches no
 // host memory.  Returns the number of kernels launched.
@@ -845,39 +888,7 @@ int run_device(eses_ctx *c)
     if (c->precision != ESES_PREC_FP64) nl += launch_band(M, B, labels, band, d_err, ovf, big, st);
     c->n_cavity = 0;
     c->ext_sweeps = 0;
-    if (c->exterior) {  // cavities filled: sweeps until one reaches nothing new (never under capture)
-        if (g_capturing) throw std::string("the exterior-only surface is not captured in a graph");
-        uint16_t *ext = ensure<uint16_t>(c->ext, 64 * (size_t)nt);
-        uint8_t *open = ensure<uint8_t>(c->ext_open, nt);
-        // em[0..1]: four ints (three sweep flags, the sweep count), em[2]: filled points
-        unsigned long long *em = ensure<unsigned long long>(c->ext_misc, 3);
-        int *flags = reinterpret_cast<int *>(em);
-        ck(cudaMemsetAsync(em, 0, 3 * sizeof(unsigned long long), st), "memset");
-        nl += launch_ext_init(B, labels, ext, open, st);
-        // a sweep reaches at least one more tile, or nothing: at most nt + 1 sweeps
-        const int coop = launch_ext_fill(B, ext, open, flags, nt + 1, st);
-        if (coop < 0) throw CudaError{cudaGetLastError(), "cooperative launch"};
-        if (coop == 1) {  // one launch for every sweep
-            ++nl;
-        } else {  // no cooperative launch on this device: one launch per sweep, driven from the host
-            const int sweep_grid = (int)std::min<long long>(std::max<long long>(ceil_div_ll(nt, 8), 1), 8LL * c->n_sm);
-            for (long long it = 0; it <= nt; ++it) {
-                ck(cudaMemsetAsync(flags, 0, sizeof(int), st), "memset");
-                nl += launch_ext_sweep(B, ext, open, flags, sweep_grid, st);
-                int changed = 0;
-                ck(cudaMemcpyAsync(&changed, flags, sizeof(changed), cudaMemcpyDeviceToHost, st), "read");
-                ck(cudaStreamSynchronize(st), "synchronize");
-                ++c->ext_sweeps;
-                if (!changed) break;
-            }
-        }
-        nl += launch_ext_apply(B, labels, ext, em + 2, st);
-        unsigned long long misc[3] = {0, 0, 0};
-        ck(cudaMemcpyAsync(misc, em, sizeof(misc), cudaMemcpyDeviceToHost, st), "read");
-        ck(cudaStreamSynchronize(st), "synchronize");
-        if (coop == 1) c->ext_sweeps = reinterpret_cast<const int *>(misc)[3];
-        c->n_cavity = (long long)misc[2];
-    }
+    if (c->exterior) nl += fill_cavities(c, labels);
 
     // 8. crossing edges, roots, area and volume
     int *tile_edges = ensure<int>(c->tile_edges, 3 * nt);
@@ -1421,6 +1432,8 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
             }
         if (c->precision != ESES_PREC_FP64)
             launch_band(M, B, labels, band, misc, (int *)c->ovf.p, c->use_big ? (unsigned char *)c->big.p : nullptr, st);
+        // the edge lists hold the filled labels' edges: staging the unfilled ones would write past them
+        if (c->exterior) fill_cavities(c, labels);
         // root solve: staging CTAs per SM x tiles per pop x root-kernel threads per block
         Shape best_edge = c->edge;
         float best_edge_ms = INFINITY;
