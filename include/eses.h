@@ -82,10 +82,9 @@ typedef struct eses_ctx eses_ctx;
 #define ESES_OPT_QUEUE 7       /* 1 (default): persistent tile kernels take tiles from a device work queue;
                                   0: fixed grid-stride order */
 #define ESES_OPT_CLS_CTAS 8    /* classification CTAs per SM (0 = occupancy limit, default) */
-#define ESES_OPT_CLS_TILES 9   /* classification tiles per queue pop (default 4, read as an upper bound: until the
-                                  option is set or the autotuner has run, the library takes single tiles) */
+#define ESES_OPT_CLS_TILES 9   /* classification tiles per queue pop (default 1) */
 #define ESES_OPT_EDGE_CTAS 10  /* root-solve staging pass: CTAs per SM (0 = occupancy limit, default) */
-#define ESES_OPT_EDGE_TILES 11 /* root-solve staging pass: tiles per queue pop (default 4, as above) */
+#define ESES_OPT_EDGE_TILES 11 /* root-solve staging pass: tiles per queue pop (default 1) */
 #define ESES_OPT_ROOT_THREADS 12 /* root solve: threads per block of the per-candidate root kernels
                                     (0 = 256, default; 64, 128 or 256) */
 #define ESES_OPT_EXTERIOR 13   /* 1: exterior-only surface -- outside points that no path of outside grid points

@@ -159,15 +159,13 @@ struct MolInfo {
 // launch shape of a persistent tile kernel
 struct Shape {
     int ctas_per_sm = 0;  // 0: the occupancy limit
-    // tiles per queue pop as set (ESES_OPT_*_TILES, the autotuner); until then
-    // single tiles: a pop of four neighbouring tiles leaves them to one CTA one
-    // after the other, and the tiles near the surface are neighbours (at h 0.4,
-    // 3,000 atoms: classification 520 us with pops of 4, 375 us with single
-    // tiles, staging pass 1,034 -> 943 us for the root solve; on 2e8 points the
-    // queue's atomics still cost nothing that shows)
-    int tiles_per_pop = 4;
-    bool pop_set = false;
-    int pop() const { return pop_set ? std::max(tiles_per_pop, 1) : 1; }
+    // tiles per queue pop (ESES_OPT_*_TILES, the autotuner).  Single tiles: a pop
+    // of four neighbouring tiles leaves them to one CTA one after the other, and
+    // the tiles near the surface are neighbours (at h 0.4, 3,000 atoms:
+    // classification 520 us with pops of 4, 375 us with single tiles, staging
+    // pass 1,034 -> 943 us for the root solve; on 2e8 points the queue's
+    // atomics still cost nothing that shows)
+    int tiles_per_pop = 1;
     int threads = 0;      // root solve: threads per block of the per-candidate root kernels (0: 256)
 };
 
@@ -605,7 +603,7 @@ int grid_of(const eses_ctx *c, const Shape &s, int max_per_sm)
 {
     int k = s.ctas_per_sm > 0 ? std::min(s.ctas_per_sm, max_per_sm) : max_per_sm;
     long long g = (long long)std::max(k, 1) * c->n_sm;
-    long long need = ceil_div_ll(std::max(c->n_tiles, 1LL), s.pop());
+    long long need = ceil_div_ll(std::max(c->n_tiles, 1LL), s.tiles_per_pop);
     return (int)std::max(1LL, std::min(g, need));
 }
 
@@ -613,7 +611,7 @@ TileSched sched_of(eses_ctx *c, const Shape &s, int which)
 {
     TileSched q;
     q.head = c->use_queue ? (unsigned long long *)c->queue.p + which : nullptr;
-    q.per = s.pop();
+    q.per = s.tiles_per_pop;
     q.list = nullptr;
     q.list_n = nullptr;
     return q;
@@ -1307,7 +1305,6 @@ int eses_set_option(eses_ctx *c, int key, int64_t value)
         if (value < 1 || value > 64) return fail(c, ESES_EINVAL, "tiles per pop must be in [1, 64]");
         drop_graph(c);
         (key == ESES_OPT_CLS_TILES ? c->cls : c->edge).tiles_per_pop = (int)value;
-        (key == ESES_OPT_CLS_TILES ? c->cls : c->edge).pop_set = true;
         return ESES_OK;
     case ESES_OPT_ROOT_THREADS:
         if (value < 0 || value > 256 || !root_threads_valid((int)value))
@@ -1419,7 +1416,6 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                 Shape s;
                 s.ctas_per_sm = k;
                 s.tiles_per_pop = per;
-                s.pop_set = true;
                 float ms = time_it([&] {
                     ck(cudaMemsetAsync(c->queue.p, 0, 4 * sizeof(unsigned long long), st), "memset");
                     TileSched q = sched_of(c, s, 0);
@@ -1473,8 +1469,7 @@ int eses_autotune(eses_ctx *c, int reps, double *ms_out)
                     Shape s;
                     s.ctas_per_sm = k;
                     s.tiles_per_pop = per;
-                    s.pop_set = true;
-                    s.threads = threads;
+                        s.threads = threads;
                     float ms = time_it([&] {
                         TileSched q = sched_of(c, s, 1);
                         q.list = (const int *)c->etiles.p + 1;
