@@ -1098,81 +1098,77 @@ __device__ void sphere_roots(const AccT &A, const AccX &X, int item, const T *s,
 // Tori (saddle pieces) around the free-arc circle of staged pair pi: roots on
 // the near branch, isolated in FP32 (certified) with the quartic on its
 // derivative chain and FP64 where that cannot decide.
-template <class T, bool FILT, class AccT, class AccX>
+template <class AccT, class AccX>
 __device__ void torus_roots(const AccT &A, const AccX &X, int pi, const double *s64, int axis, bool inside, double h,
-                            double rp, T d0, RootSink &out)
+                            double rp, float d0, RootSink &out)
 {
-    if constexpr (!FILT) {
-        torus_piece_exact(A, out, pi, s64, axis, h, rp, inside);
-    } else {
-        const T s[3] = {(T)s64[0], (T)s64[1], (T)s64[2]};
-        const T hT = (T)h, rpT = (T)rp;
-        const T lo = T(-1e-4), hi = hT + T(1e-4);
-        const T tmax = T(1e-3);
-        const double NaN = __longlong_as_double(0x7ff8000000000000LL);
-        const P4<T> o = A.po(pi);
-        const P4<T> u = A.pu(pi);
-        const float q0[3] = {s[0] - o.x, s[1] - o.y, s[2] - o.z};
-        const float uu[3] = {u.x, u.y, u.z};
-        float rt[4];
-        int nr = 0;
-        if (!torus_roots32(q0, uu, o.w, rpT, axis, lo, hi, d0, rt, nr)) {
-            // sampling undecided (near-tangent line, or close to the circle's axis): the
-            // quartic's roots on the derivative chain
-            const float P = q0[0] * q0[0] + q0[1] * q0[1] + q0[2] * q0[2];
-            const float z0 = q0[0] * uu[0] + q0[1] * uu[1] + q0[2] * uu[2];
-            const float pe = q0[axis], eu = uu[axis];
-            const float K = P + o.w * o.w - rpT * rpT, r2 = o.w * o.w;
-            const float co32[5] = {K * K - 4.0f * r2 * (P - z0 * z0), 4.0f * pe * K - 8.0f * r2 * (pe - z0 * eu),
-                                   4.0f * pe * pe + 2.0f * K - 4.0f * r2 * (1.0f - eu * eu), 4.0f * pe, 1.0f};
-            float rq[4];
-            const int nq = PolyRoots<float, 4>::run(co32, lo, hi, rq);
-            nr = 0;
-            for (int k = 0; k < nq; ++k) {
-                float D, dD, nw, yy, zy, wv[3];
-                circle_dist32(q0, uu, o.w, axis, rq[k], D, dD, nw, yy, zy, wv);
-                // near branch: A = |y|^2 + rho^2 - r_p^2 >= 0; undecided signs go to FP64
-                const float Ay = yy + r2 - rpT * rpT;
-                if (fabsf(Ay) < 1e-3f * (yy + r2 + rpT * rpT)) nr = -1;
-                else if (Ay > 0.0f && nr >= 0) rt[nr++] = rq[k];
-            }
-            if (nr < 0) {
-                torus_piece_exact(X, out, pi, s64, axis, h, rp, inside);
-                return;
-            }
+    const float s[3] = {(float)s64[0], (float)s64[1], (float)s64[2]};
+    const float hT = (float)h, rpT = (float)rp;
+    const float lo = -1e-4f, hi = hT + 1e-4f;
+    const float tmax = 1e-3f;
+    const double NaN = __longlong_as_double(0x7ff8000000000000LL);
+    const P4<float> o = A.po(pi);
+    const P4<float> u = A.pu(pi);
+    const float q0[3] = {s[0] - o.x, s[1] - o.y, s[2] - o.z};
+    const float uu[3] = {u.x, u.y, u.z};
+    float rt[4];
+    int nr = 0;
+    if (!torus_roots32(q0, uu, o.w, rpT, axis, lo, hi, d0, rt, nr)) {
+        // sampling undecided (near-tangent line, or close to the circle's axis): the
+        // quartic's roots on the derivative chain
+        const float P = q0[0] * q0[0] + q0[1] * q0[1] + q0[2] * q0[2];
+        const float z0 = q0[0] * uu[0] + q0[1] * uu[1] + q0[2] * uu[2];
+        const float pe = q0[axis], eu = uu[axis];
+        const float K = P + o.w * o.w - rpT * rpT, r2 = o.w * o.w;
+        const float co32[5] = {K * K - 4.0f * r2 * (P - z0 * z0), 4.0f * pe * K - 8.0f * r2 * (pe - z0 * eu),
+                               4.0f * pe * pe + 2.0f * K - 4.0f * r2 * (1.0f - eu * eu), 4.0f * pe, 1.0f};
+        float rq[4];
+        const int nq = PolyRoots<float, 4>::run(co32, lo, hi, rq);
+        nr = 0;
+        for (int k = 0; k < nq; ++k) {
+            float D, dD, nw, yy, zy, wv[3];
+            circle_dist32(q0, uu, o.w, axis, rq[k], D, dD, nw, yy, zy, wv);
+            // near branch: A = |y|^2 + rho^2 - r_p^2 >= 0; undecided signs go to FP64
+            const float Ay = yy + r2 - rpT * rpT;
+            if (fabsf(Ay) < 1e-3f * (yy + r2 + rpT * rpT)) nr = -1;
+            else if (Ay > 0.0f && nr >= 0) rt[nr++] = rq[k];
         }
-        const int2 ij = A.pij(pi);
-        const short2 sl = A.pslot(pi);
-        for (int k = 0; k < nr; ++k) {
-            const float t = rt[k];
-            float D, rate, nw, yy, zy, wv[3];
-            circle_dist32(q0, uu, o.w, axis, t, D, rate, nw, yy, zy, wv);
-            // root error: residual plus rounding of g over |g'| (g' varies little within terr)
-            const float terr =
-                (fabsf(D - rpT) + circle_dist_err(d0, yy, nw, o.w, rpT)) / fmax(fabs(rate), 1e-20f) + d0;
-            if (terr > tmax || t < terr + 1e-6f || t > hT - terr - 1e-6f || fabs(rate) < 1e-3f ||
-                nw < 1e-3f) {  // grazing or at an end point: the FP64 root decides
-                const P4<double> oe = X.po(pi);
-                const P4<double> ue = X.pu(pi);
-                const double oo[3] = {oe.x, oe.y, oe.z}, u64[3] = {ue.x, ue.y, ue.z};
-                const double t64 = exact_root_torus(oo, u64, oe.w, rp, s64, axis, (double)t);
-                torus_root_exact(X, out, pi, s64, axis, h, rp, inside, t64);
-                continue;
-            }
-            if (inside ? rate > 0.0f : rate < 0.0f) continue;
-            const float kk = o.w / nw;
-            const float delta = d0 + terr * (1.0f + 2.0f * o.w / nw) + 2e-6f;
-            const int f = free_witness<true>(A, o.x + kk * wv[0], o.y + kk * wv[1], o.z + kk * wv[2], (int)sl.x,
-                                             (int)sl.y, ij.x, ij.y, rpT, delta);
-            if (f == 1) {
-                out.push(t, terr, NaN);
-            } else if (f < 0) {
-                const P4<double> oe = X.po(pi);
-                const P4<double> ue = X.pu(pi);
-                const double oo[3] = {oe.x, oe.y, oe.z}, u64[3] = {ue.x, ue.y, ue.z};
-                const double t64 = exact_root_torus(oo, u64, oe.w, rp, s64, axis, (double)t);
-                torus_root_exact(X, out, pi, s64, axis, h, rp, inside, t64);
-            }
+        if (nr < 0) {
+            torus_piece_exact(X, out, pi, s64, axis, h, rp, inside);
+            return;
+        }
+    }
+    const int2 ij = A.pij(pi);
+    const short2 sl = A.pslot(pi);
+    for (int k = 0; k < nr; ++k) {
+        const float t = rt[k];
+        float D, rate, nw, yy, zy, wv[3];
+        circle_dist32(q0, uu, o.w, axis, t, D, rate, nw, yy, zy, wv);
+        // root error: residual plus rounding of g over |g'| (g' varies little within terr)
+        const float terr =
+            (fabsf(D - rpT) + circle_dist_err(d0, yy, nw, o.w, rpT)) / fmax(fabs(rate), 1e-20f) + d0;
+        if (terr > tmax || t < terr + 1e-6f || t > hT - terr - 1e-6f || fabs(rate) < 1e-3f ||
+            nw < 1e-3f) {  // grazing or at an end point: the FP64 root decides
+            const P4<double> oe = X.po(pi);
+            const P4<double> ue = X.pu(pi);
+            const double oo[3] = {oe.x, oe.y, oe.z}, u64[3] = {ue.x, ue.y, ue.z};
+            const double t64 = exact_root_torus(oo, u64, oe.w, rp, s64, axis, (double)t);
+            torus_root_exact(X, out, pi, s64, axis, h, rp, inside, t64);
+            continue;
+        }
+        if (inside ? rate > 0.0f : rate < 0.0f) continue;
+        const float kk = o.w / nw;
+        const float delta = d0 + terr * (1.0f + 2.0f * o.w / nw) + 2e-6f;
+        const int f = free_witness<true>(A, o.x + kk * wv[0], o.y + kk * wv[1], o.z + kk * wv[2], (int)sl.x,
+                                         (int)sl.y, ij.x, ij.y, rpT, delta);
+        if (f == 1) {
+            out.push(t, terr, NaN);
+        } else if (f < 0) {
+            const P4<double> oe = X.po(pi);
+            const P4<double> ue = X.pu(pi);
+            const double oo[3] = {oe.x, oe.y, oe.z}, u64[3] = {ue.x, ue.y, ue.z};
+            const double t64 = exact_root_torus(oo, u64, oe.w, rp, s64, axis, (double)t);
+            torus_root_exact(X, out, pi, s64, axis, h, rp, inside, t64);
         }
     }
 }
@@ -1721,13 +1717,6 @@ __global__ void __launch_bounds__(EDGE_THREADS) k_edge_stage(Model M, Batch B, T
     }
 }
 
-// slab, grid and edge geometry of global edge g's record
-struct EdgeView {
-    const unsigned char *slab;
-    int axis, p, lab;
-    double s64[3];  // lower point in the tile frame
-};
-
 // 2. Roots of the sphere candidates, one thread each (grid-stride).
 template <class T, bool FILT>
 __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_sphere(Model M, Batch B, RootWork W,
@@ -1896,7 +1885,6 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX) k_roots_torus(Model M, Batch
 // Bound by the latency of its chains of loads and FP64 instructions: three
 // blocks on an SM rather than the two of its 126 registers (178 -> 157 us on the
 // 20,000-atom globule).
-template <class T, bool FILT>
 __global__ void __launch_bounds__(ROOT_THREADS_MAX, 3) k_roots_torus_exact(Model M, Batch B, RootWork W,
                                                                            int *__restrict__ err)
 {
@@ -1912,16 +1900,16 @@ __global__ void __launch_bounds__(ROOT_THREADS_MAX, 3) k_roots_torus_exact(Model
         const int mol = __ldg(&hd->mol);
         const double x0[3] = {__ldg(&hd->x0[0]), __ldg(&hd->x0[1]), __ldg(&hd->x0[2])};
         const double h = B.grid[mol].h;
-        const T d0 = FILT ? (T)B.grid[mol].d0 : T(0);
+        const float d0 = B.grid[mol].d0;
         const int pk = inf.y, p = pk_point(pk), axis = pk_axis(pk);
         const bool inside = pk_label(pk) == LABEL_IN;
         const double s64[3] = {(double)(p >> 6) * h, (double)((p >> 3) & 7) * h, (double)(p & 7) * h};
-        const SlabAcc<T> A(sl);
-        const SlabExact<T> X(A, M, x0, B.grid[mol].d0);
+        const SlabAcc<float> A(sl);
+        const SlabExact<float> X(A, M, x0, d0);
         RootRec *slots = W.rtor + (size_t)TOR_SLOTS * k;
         if (jb.y == 2) {
             RootSink out{slots, 0, TOR_SLOTS};
-            torus_roots<T, FILT>(A, X, c.y, s64, axis, inside, h, rp, d0, out);
+            torus_roots(A, X, c.y, s64, axis, inside, h, rp, d0, out);
             if (out.n > TOR_SLOTS) atomicOr(err, ERR_CAP_CAND);
             W.ntor[k] = (uint8_t)min(out.n, TOR_SLOTS);
         } else {
@@ -2363,8 +2351,9 @@ __global__ void __launch_bounds__(POLISH_THREADS, 4) k_edge_polish(Model M, Batc
 
 // Area/volume reduction in two fixed-order levels (deterministic): block
 // (m, g) of k_reduce_part sums the terms of molecule m whose index within the
-// molecule's range is g (mod RED_PARTS * blockDim), in a fixed tree;
-// k_reduce_final adds the RED_PARTS partials of each molecule in a fixed tree.
+// molecule's range is g (mod parts * blockDim), in a fixed tree, for the
+// molecule's number of parts (red_parts; the blocks past it return);
+// k_reduce_final adds those partials of each molecule in a fixed tree.
 constexpr int RED_PARTS = 64;  // at most (16 parts: 192 us on one molecule's 4.9 M terms, 53 us on 1.2 M; 58 and 17 now)
 constexpr int RED_THREADS = 512;
 
@@ -2502,7 +2491,7 @@ static int g_edge_n_sm = 1;  // SMs: the grid of the global-memory tier and of t
 // resident blocks per SM: [FP64, FP32][sphere roots, torus roots][64, 128, 256 threads]; hard selection
 static int g_occ_roots[2][2][3];
 static int g_occ_hard[2];
-static int g_occ_exact[2];
+static int g_occ_exact;
 
 static int threads_slot(int threads) { return threads <= 64 ? 0 : (threads <= 128 ? 1 : 2); }
 
@@ -2528,7 +2517,7 @@ void edges_init()
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_roots[1][0][k], k_roots_sphere<float, true>, tb[k], 0);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_roots[1][1][k], k_roots_torus<float, true>, tb[k], 0);
     }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_exact[1], k_roots_torus_exact<float, true>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_exact, k_roots_torus_exact, 256, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_hard[0], k_edge_hard<double, false>, HARD_THREADS, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_occ_hard[1], k_edge_hard<float, true>, HARD_THREADS, 0);
 }
@@ -2589,7 +2578,7 @@ static void roots_launch(const Model &M, const Batch &B, int threads, EdgeOut ou
     cudaMemsetAsync(W.ctr + 3, 0, 3 * sizeof(unsigned long long), st);  // listed edges, FP64 jobs, ties
     k_roots_torus<T, FILT><<<gq, tb, 0, st>>>(M, B, W, err);
     if (FILT)
-        k_roots_torus_exact<T, FILT><<<std::max(g_occ_exact[P], 1) * g_edge_n_sm, tb, 0, st>>>(M, B, W, err);
+        k_roots_torus_exact<<<std::max(g_occ_exact, 1) * g_edge_n_sm, tb, 0, st>>>(M, B, W, err);
     const long long pb = std::min<long long>(std::max<long long>(ceil_div_ll(ne_all, PICK_THREADS), 1),
                                              8LL * g_edge_n_sm);
     k_edge_pick<T><<<(unsigned)pb, PICK_THREADS, 0, st>>>(M, B, W, edge_start, ne_all, out, err);

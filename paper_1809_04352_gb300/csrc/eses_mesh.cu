@@ -210,13 +210,6 @@ int mesh_table_copy(void *table, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // kernels (one molecule: B.grid[0], tiles 0 .. n_tiles - 1)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void tile_point(const int *t, int p, long long *g)
-{
-    g[0] = (long long)TILE * t[0] + (p >> 6);
-    g[1] = (long long)TILE * t[1] + ((p >> 3) & 7);
-    g[2] = (long long)TILE * t[2] + (p & 7);
-}
-
 constexpr int MASK_WORDS = TILE_PTS / 32;
 // per tile and axis: the mask, then 16-bit prefix counts (two to a word)
 constexpr int MASK_STRIDE = MASK_WORDS + MASK_WORDS / 2;
