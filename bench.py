@@ -55,15 +55,15 @@ WORKLOAD = 2
 
 
 # DRAM bytes per step (dram__bytes_read.sum + dram__bytes_write.sum) from one
-# ncu capture of the globule workload: the root solve's six launches summed
+# ncu capture of the globule workload: the root solve's seven launches summed
 # (profiles/root-solve_globule-5000.md), the classification's two tiers
 # (profiles/k_classify_globule-5000.md); reported only while the kernels'
 # sources are the ones that were captured
 TRAFFIC = {
-    "edge_solve": (644_276_992, {"eses_edges.cu": "e666d46675dc5cc0", "eses_tile.cuh": "9e7d65712438136b",
-                                 "eses_internal.cuh": "85eea755cbda79ad"}),
-    "classify": (9_756_416, {"eses_classify.cu": "04754d6e89d4d447", "eses_tile.cuh": "9e7d65712438136b",
-                             "eses_internal.cuh": "85eea755cbda79ad"}),
+    "edge_solve": (644_538_368, {"eses_edges.cu": "1074de99dc0e2615", "eses_tile.cuh": "9e7d65712438136b",
+                                 "eses_internal.cuh": "5039a9ab6fd28ac6"}),
+    "classify": (9_754_624, {"eses_classify.cu": "7de98a9b06aa8a70", "eses_tile.cuh": "9e7d65712438136b",
+                             "eses_internal.cuh": "5039a9ab6fd28ac6"}),
 }
 
 
